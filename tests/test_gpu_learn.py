@@ -126,3 +126,26 @@ def test_learning_run_descends_and_matches_the_oracle_objective():
     codes, d_best, _ = oracle.encode(x.numpy(), cb2.cpu().numpy(), c, b)
     _, d_init, _ = oracle.encode(x.numpy(), oracle.kmeanspp_init(x.numpy(), w.numpy(), u, c, b)[0], c, b)
     assert (w.numpy() * d_best).sum() < 0.8 * (w.numpy() * d_init).sum()
+
+
+@pytest.mark.parametrize("c,n_vec,weighted", [(8, 1, False), (8, 31, True), (4, 513, True), (8, 4096, True), (2, 4097, False),
+                                              (8, 16385, True), (4, 32768, False), (8, 32769, True)])
+def test_kmeanspp_and_one_iteration_at_the_edges_of_the_split(c, n_vec, weighted):
+    # one to eight CTAs per problem, their last vectors, and one vector more than a cluster holds (the plain kernels);
+    # half of the vectors equal, so that one centroid has most of the members of the update
+    b, G = 3, 128 // c
+    x = calib(360 + c, n_vec, 1, False, c)
+    x[::2] = x[0].clone()
+    w = fisher_like_weights(c + b, n_vec, 1, G) if weighted else None
+    u = torch.rand(1, G, 1 << b, dtype=torch.float64, generator=torch.Generator().manual_seed(n_vec))
+    u[0, :, 1] = 0.0
+    u[0, ::2, 2] = 1.0 - 2.0 ** -53
+    wn = None if w is None else w.numpy()
+    want, _ = oracle.kmeanspp_init(x.numpy(), wn, u.numpy(), c, b)
+    wd = None if w is None else w.to(DEV)
+    got = cq.cq_kmeanspp_init(x.to(DEV), wd, u.to(DEV), c, b)
+    assert np.array_equal(got.cpu().numpy(), want)
+    new, _, obj = oracle.lloyd_step(x.numpy(), wn, want, c, b)
+    got_new, got_obj = cq.cq_lloyd_step(x.to(DEV), wd, got, c, b)
+    assert np.allclose(got_new.cpu().numpy(), new, rtol=0, atol=2e-5 * max(1.0, np.abs(new).max()))
+    assert np.allclose(got_obj.cpu().numpy(), obj, rtol=1e-5, atol=1e-9)
