@@ -144,7 +144,7 @@ int cq_encode_variant(const void* x_fp16, const float* codebooks, const int32_t*
     if (n_tokens == 0) return CQ_OK;
     const bool tuned_ok = encode_tuned_supported(sh);
     if (variant == 2 && !tuned_ok) return CQ_ERR_UNSUPPORTED;
-    if (variant == 4 && !encode_tc_supported(sh)) return CQ_ERR_UNSUPPORTED;
+    if (variant == 4 && (b != 8 || !encode_tc_supported(sh))) return CQ_ERR_UNSUPPORTED;
     const bool small_ok = encode_small_supported(sh);
     if (variant == 3 && !small_ok) return CQ_ERR_UNSUPPORTED;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);

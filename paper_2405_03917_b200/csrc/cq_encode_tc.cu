@@ -1,5 +1,5 @@
 // Bulk encode on the fifth-generation tensor cores (tcgen05, accumulators in tensor memory) for
-// head_dim 128, b = 8, c in {2, 4, 8}: the kernel for prefill-sized inputs.
+// head_dim 128, b in {8, 9, 10}, c in {2, 4, 8}.
 //
 // CQ encode (Section 3.2 of the paper, the map CQ(.) of Eq. 5): every group of c contiguous
 // channels of a vector is replaced by the index of its nearest centroid in L2 distance, lowest
@@ -16,18 +16,22 @@
 //     c = 8   two K steps: (x x x x | x x x x) against (t0 | t1), then (x x x x | (1,1), X, (1,0), 0)
 //             against (t2 | N, (1,1), (N_lo2,0), 0)
 // What differs is where the scores go.  The accumulator tile lives in tensor memory, row i in
-// lane i, and a thread reads the 256 scores of ITS row with tcgen05.ld: no accumulator registers
-// to clear, no B fragments to fetch in the selecting warps, no quad to merge, and - because the
-// winner is found by exact re-evaluation anyway - no index packed into every score.  A thread
-// keeps the minimum of each of 16 subsets of the centroids (index mod 16), one 3-input min per
-// two scores; the subset with the smallest minimum is evaluated exactly (16 centroids, direct form
-// sum (x - C)^2 in fp32, lowest index on ties) and the second smallest subset minimum bounds
-// every other centroid from below.  The exact winner is accepted if that bound is farther away
-// than a bound on the evaluation error; otherwise (near-ties, ties across subsets, codebooks
-// fp16 cannot carry) the warp recomputes that row over all 256 centroids exactly.
+// lane i, and a thread reads the scores of ITS row with tcgen05.ld: no accumulator registers to
+// clear, no B fragments to fetch in the selecting warps, no quad to merge.  The 256 scores of a
+// (vector, group) are a 16 x 16 grid, and a thread keeps the minimum of every row and of every
+// column: 1.25 operations per score, no index packed into it.  The row and the column with the smallest minima name
+// the winner, and whatever else there is lies in another row or in another column, so the second
+// smallest minima bound it from below.  The winner is accepted if that bound is farther away than a
+// bound on the evaluation error; otherwise (near-ties, ties, codebooks fp16 cannot carry) the warp
+// recomputes that row over all centroids exactly: sum (x - C)^2 in fp32, lowest index on ties.
+// (Before, the winning column's 16 centroids were evaluated exactly from shared memory: at c = 8 the bank
+// conflicts of those reads kept the shared-memory pipe 74 % busy.  8192 vectors x 32 heads: c = 8
+// 350 -> 217 us.)  More than 256 centroids (b = 9, 10) come in chunks of 256 whose operands all
+// stay in shared memory while a row tile passes them; the grid then has 32 or 64 rows.  (CQ-8c10b,
+// 32768 vectors x 8 heads: 3.1 -> 1.2 ms against the mma.sync kernel.)
 //
 // A CTA is one tile of 128 vectors of one head: 4 warps, warp w owning the tensor memory lanes
-// 32 w ... 32 w + 31, and 128 tensor-memory columns, so that four CTAs (three for c = 8, whose
+// 32 w ... 32 w + 31, and 128 tensor-memory columns, so that four CTAs (fewer for wide codes, whose
 // operands take more shared memory) live on an SM and fill each other's waits.  The accumulator is
 // therefore 128 x 128: the scores of a step arrive in two halves (centroids 0-127, then 128-255)
 // through the same columns, and the operand preparation and the row finishing are placed behind
@@ -43,7 +47,8 @@ constexpr int kTcThreads = 128;
 constexpr int kTcTileVecs = 128;          // vectors of a row tile
 constexpr float kTcInf = __builtin_huge_valf();
 
-template <int kC>
+// kChunks: 256-centroid chunks per group (b = 8, 9, 10: 1, 2, 4)
+template <int kC, int kChunks>
 struct TcCfg {
     static constexpr int G = 128 / kC;
     static constexpr int kSteps = (kC == 8) ? 2 : 1;              // K steps (16 fp16 slots each)
@@ -51,34 +56,25 @@ struct TcCfg {
     static constexpr int kBTile = 256 * 32;
     static constexpr int kABuf = kSteps * kATile;
     static constexpr int kBBuf = kSteps * kBTile;
-    static constexpr int kCbf = 256 * kC * 4;                     // the group's centroids as fp32
-    static constexpr int kMaxLogRt = (kC == 8) ? 2 : 3;           // up to 2^kMaxLogRt row tiles per CTA
-    static constexpr int kCtasPerSm = (kC == 8) ? 3 : 4;
+    static constexpr int kBSlots = kChunks == 1 ? 2 : kChunks;    // prepared chunks: this group's and the next one's, or all of a group's
+    static constexpr int kMaxLogRt = (kC == 8 || kChunks > 1) ? 2 : 3;    // up to 2^kMaxLogRt row tiles per CTA
+    static constexpr int kCtasPerSm = (kC == 8 && kChunks == 4) ? 2 : (kC == 8 && kChunks == 2) ? 3 : 4;
     static constexpr int kAOff = 0;                               // [2 buffers]
-    static constexpr int kBOff = kAOff + 2 * kABuf;               // [2 buffers]
-    static constexpr int kCbfOff = kBOff + 2 * kBBuf;             // [2 slots]
-    static constexpr int kRowOff = kCbfOff + 2 * kCbf;            // [row tiles][128 threads] row records
-    static constexpr int kCtlOff = kRowOff + (1 << kMaxLogRt) * kTcThreads * 16;
-    static constexpr int kUsedBytes = kCtlOff + 256;
+    static constexpr int kBOff = kAOff + 2 * kABuf;               // [kBSlots]
+    static constexpr int kRowOff = kBOff + kBSlots * kBBuf;       // [row tiles][128 threads] code offset of the row
+    static constexpr int kCtlOff = kRowOff + (1 << kMaxLogRt) * kTcThreads * 8;
+    static constexpr int kUsedBytes = kCtlOff + 512;
     // at least 46 KiB, so that a fifth CTA (for which no tensor memory would be left) never fits an SM
     static constexpr int kSmemBytes = kUsedBytes > 46 * 1024 ? kUsedBytes : 46 * 1024;
     static_assert(kCtasPerSm * (kSmemBytes + 1024) <= 228 * 1024, "shared memory of an SM");
-    static_assert((kCtasPerSm + 1) * (kSmemBytes + 1024) > 228 * 1024, "one CTA too many would fit");
+    static_assert(5 * (kSmemBytes + 1024) > 228 * 1024, "one CTA too many would fit");
 };
 
 constexpr int kTcColumns = 128;            // tensor-memory columns of a CTA
 
-// What a thread needs of one of its rows, worked out once: where the vector's head slice starts and where its code of
-// group 0 goes (the code of group g follows kTokenBlock * g bytes on).
-struct TcRow {
-    const __half* x;           // null: no such vector
-    int64_t code_offset;       // negative: the token has no position in the cache
-};
-static_assert(sizeof(TcRow) == 16, "row record");
-
 struct TcCtl {
-    int range_flag[2][8];      // per warp and pass, non-zero: those centroids of the prepared group hold values fp16 cannot carry
-    float nmax[2][8];          // per warp and pass, the largest ||C_j||^2 among those centroids
+    int range_flag[4][8];      // per slot, warp and pass, non-zero: those centroids of the prepared chunk hold values fp16 cannot carry
+    float nmax[4][8];          // per slot, warp and pass, the largest ||C_j||^2 among those centroids
     uint32_t tmem_base;
     int wait_failed;           // a wait on an MMA barrier gave up
     uint64_t bar[2];           // completion of the MMA of the low / high half of a step
@@ -160,35 +156,6 @@ __device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity)
     return false;
 }
 
-// Exact nearest centroid of one group of one vector, computed by the whole warp:
-// d_j = sum_i (x_i - C_ji)^2 in fp32 (same operation order as the generic kernel), lowest j on ties.
-template <int kC>
-__device__ __forceinline__ int tc_exact_code(const float (&xg)[kC], const float* cbf, int lane, float* dist)
-{
-    float best = kTcInf;
-    int arg = 0;
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-        const int j = t * 32 + lane;
-        float d = 0.f;
-#pragma unroll
-        for (int i = 0; i < kC; ++i) {
-            const float diff = xg[i] - cbf[j * kC + i];
-            d = fmaf(diff, diff, d);
-        }
-        if (d < best) { best = d; arg = j; }        // j increases with t: strict < keeps the lowest index
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oa = __shfl_xor_sync(0xffffffffu, arg, o);
-        if (ob < best || (ob == best && oa < arg)) { best = ob; arg = oa; }
-    }
-    *dist = best;
-    return arg;
-}
-
-
 // Centroid j of a group, from global memory into registers.
 template <int kC>
 __device__ __forceinline__ void tc_fetch_centroid(const float* __restrict__ cb_g, int j, float (&cv)[kC])
@@ -206,19 +173,43 @@ __device__ __forceinline__ void tc_fetch_centroid(const float* __restrict__ cb_g
     }
 }
 
-// B operand of one group, one centroid: K slots as in the header comment; keeps the fp32 centroid for the exact
-// evaluations; every warp leaves its largest squared norm and its range flag of this pass in the control block.
+// Exact nearest centroid of one group of one vector, computed by the whole warp:
+// d_j = sum_i (x_i - C_ji)^2 in fp32 (same operation order as the generic kernel), centroids from
+// global memory (rare, and in L1 after the first), lowest j on ties.
 template <int kC>
-__device__ __forceinline__ void tc_prepare_b(const float (&cv)[kC], int j, unsigned char* bbuf, float* cbf, TcCtl* ctl, int slot, int pass)
+__device__ __noinline__ int tc_exact_code(const float* __restrict__ cb_g, int n_centroids, float x0, float x1, float x2, float x3,
+                                          float x4, float x5, float x6, float x7)
 {
-    using C = TcCfg<kC>;
-    if (kC == 2) {
-        *reinterpret_cast<float2*>(cbf + j * 2) = make_float2(cv[0], cv[1]);
-    } else {
+    const float xs[8] = {x0, x1, x2, x3, x4, x5, x6, x7};
+    const int lane = threadIdx.x & 31;
+    float best = kTcInf;
+    int arg = 0;
+#pragma unroll 4
+    for (int j = lane; j < n_centroids; j += 32) {
+        float cv[kC];
+        tc_fetch_centroid<kC>(cb_g, j, cv);
+        float d = 0.f;
 #pragma unroll
-        for (int w = 0; w < kC; w += 4)
-            *reinterpret_cast<float4*>(cbf + j * kC + w) = make_float4(cv[w], cv[w + 1], cv[(w + 2) % kC], cv[(w + 3) % kC]);
+        for (int i = 0; i < kC; ++i) {
+            const float diff = xs[i] - cv[i];
+            d = fmaf(diff, diff, d);
+        }
+        if (d < best) { best = d; arg = j; }        // j increases: strict < keeps the lowest index
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oa = __shfl_xor_sync(0xffffffffu, arg, o);
+        if (ob < best || (ob == best && oa < arg)) { best = ob; arg = oa; }
+    }
+    return arg;
+}
+
+// B operand of one chunk, one centroid: K slots as in the header comment; every warp leaves its largest squared norm and its range flag of this pass in the control block.
+template <int kC>
+__device__ __forceinline__ void tc_prepare_b(const float (&cv)[kC], int j, unsigned char* bbuf, TcCtl* ctl, int slot, int pass)
+{
+    using C = TcCfg<kC, 1>;
     float nrm = 0.f, amax = 0.f;
     float t0[kC], t1[kC], t2[kC];
 #pragma unroll
@@ -296,7 +287,7 @@ __device__ __forceinline__ void tc_fetch_x(const __half* gp, uint32_t (&xw)[kC /
 template <int kC>
 __device__ __forceinline__ void tc_build_a(const uint32_t (&xw)[kC / 2], float X, unsigned char* atile, int row)
 {
-    using C = TcCfg<kC>;
+    using C = TcCfg<kC, 1>;
     const uint32_t ones = 0x3c003c00u, one_zero = 0x00003c00u;   // half2(1, 1), half2(1, 0)
     const float x0 = __half2float(__float2half_rn(X));
     const uint32_t xn = tc_pack_half2(x0, X - x0);
@@ -323,12 +314,12 @@ __device__ __forceinline__ void tc_build_a(const uint32_t (&xw)[kC / 2], float X
     }
 }
 
-static_assert(sizeof(TcCtl) <= 256, "control block");
+static_assert(sizeof(TcCtl) <= 512, "control block");
 
-// One step = one row tile (128 vectors) against one group.  A CTA takes 2^log_rt row tiles through its groups;
-// blockIdx.x = (block of row tiles, head, group split).
-template <int kC>
-__global__ void __launch_bounds__(kTcThreads, TcCfg<kC>::kCtasPerSm)
+// One step = one row tile (128 vectors) against one chunk of 256 centroids of a group.  A CTA takes 2^log_rt row tiles
+// through its groups, all chunks of a group per row tile; blockIdx.x = (block of row tiles, head, group split).
+template <int kC, int kChunks>
+__global__ void __launch_bounds__(kTcThreads, TcCfg<kC, kChunks>::kCtasPerSm)
 encode_tc_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, const int32_t* __restrict__ seq_offsets,
                  Shape sh, int64_t n_tokens, int64_t token_offset, uint8_t* __restrict__ codes1, int groups_per_cta, int log_rt,
                  const __half* __restrict__ x2, const float* __restrict__ cb2, uint8_t* __restrict__ codes2)
@@ -336,7 +327,7 @@ encode_tc_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, c
     const __half* x = blockIdx.y ? x2 : x1;
     const float* cb = blockIdx.y ? cb2 : cb1;
     uint8_t* codes = blockIdx.y ? codes2 : codes1;
-    using C = TcCfg<kC>;
+    using C = TcCfg<kC, kChunks>;
     constexpr int G = C::G;
     extern __shared__ __align__(1024) unsigned char tc_smem[];
     TcCtl* ctl = reinterpret_cast<TcCtl*>(tc_smem + C::kCtlOff);
@@ -353,7 +344,8 @@ encode_tc_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, c
     const int g_begin = gs * groups_per_cta;
     const int g_end = g_begin + groups_per_cta < G ? g_begin + groups_per_cta : G;
     const int rt_mask = (1 << log_rt) - 1;
-    const int n_steps = (g_end - g_begin) << log_rt;     // step st: group g_begin + (st >> log_rt), row tile st & rt_mask
+    // step st: row step st / kChunks (group g_begin + (rs >> log_rt), row tile rs & rt_mask), chunk st % kChunks
+    const int n_steps = ((g_end - g_begin) << log_rt) * kChunks;
 
     // tensor memory (warp 0 allocates the CTA's columns and frees them at the end), the MMA barriers
     if (warp == 0) {
@@ -372,44 +364,47 @@ encode_tc_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, c
     const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(&ctl->tmem_base);
     const uint32_t taddr = tmem_base + ((uint32_t)(warp * 32) << 16);
 
-    auto a_buf = [&](int buf) { return tc_smem + C::kAOff + buf * C::kABuf; };
-    auto b_buf = [&](int buf) { return tc_smem + C::kBOff + buf * C::kBBuf; };
-    auto cbf_slot = [&](int slot) { return reinterpret_cast<float*>(tc_smem + C::kCbfOff + slot * C::kCbf); };
-    TcRow* rows = reinterpret_cast<TcRow*>(tc_smem + C::kRowOff) + threadIdx.x;      // record of row tile r: rows[r * kTcThreads]
+    auto a_buf = [&](int rs) { return tc_smem + C::kAOff + (rs & 1) * C::kABuf; };
+    auto slot_of = [&](int st) { return kChunks == 1 ? (st >> log_rt) & 1 : st % kChunks; };
+    auto b_buf = [&](int slot) { return tc_smem + C::kBOff + slot * C::kBBuf; };
+    // Where the code of group 0 of this thread's row of row tile r goes (the low byte of group g follows kTokenBlock * g
+    // bytes on): offsets[r * kTcThreads], worked out once; -1: no position in the cache, -2: no such vector.
+    int64_t* offsets = reinterpret_cast<int64_t*>(tc_smem + C::kRowOff) + threadIdx.x;
+    const int64_t v_first = tile_block * (rt_mask + 1) * kTcTileVecs + row;
     for (int r = 0; r <= rt_mask; ++r) {
-        const int64_t v = (tile_block * (rt_mask + 1) + r) * kTcTileVecs + row;
-        TcRow rec;
-        rec.x = nullptr;
-        rec.code_offset = -1;
+        const int64_t v = v_first + r * kTcTileVecs;
+        int64_t off = -2;
         if (v < n_vec) {
-            rec.x = x + (v * n_heads + h) * 128;
             const int64_t s = v / n_tokens, i = v % n_tokens;
             const int64_t pos = token_offset + (seq_offsets ? seq_offsets[s] : 0) + i;
-            if (pos >= 0 && pos < sh.max_tokens) rec.code_offset = code_word_offset(sh, n_heads, s, h, pos / kTokenBlock, 0) + pos % kTokenBlock;
+            off = pos >= 0 && pos < sh.max_tokens ? code_word_offset(sh, n_heads, s, h, pos / kTokenBlock, 0) + pos % kTokenBlock : -1;
         }
-        rows[r * kTcThreads] = rec;                      // read back by this thread only
+        offsets[r * kTcThreads] = off;                   // read back by this thread only
     }
 
     // The vector's words travel global memory -> registers (fetch, half a step ahead) -> shared memory (build).
     uint32_t xw_pf[kC / 2];
-    auto fetch = [&](int st) {
-        const __half* xr = rows[(st & rt_mask) * kTcThreads].x;
+    auto fetch = [&](int rs) {
+        const int64_t v = v_first + (rs & rt_mask) * kTcTileVecs;
 #pragma unroll
         for (int w = 0; w < kC / 2; ++w) xw_pf[w] = 0u;
-        if (xr) tc_fetch_x<kC>(xr + (g_begin + (st >> log_rt)) * kC, xw_pf);
+        if (v < n_vec) tc_fetch_x<kC>(x + (v * n_heads + h) * 128 + (g_begin + (rs >> log_rt)) * kC, xw_pf);
     };
     uint32_t xw_nxt[kC / 2];
-    float X_nxt;
+    float X_nxt = 0.f;
+    // what step st needs and its predecessor has not left: the chunk's centroids (first row tile of a group), the row
+    // tile's vectors (first chunk)
     auto build = [&](int st) {
-        const int gslot = (st >> log_rt) & 1;
-        if ((st & rt_mask) == 0) {                       // a new group: centroids threadIdx.x and threadIdx.x + 128
-            const float* cb_g = cb + ((int64_t)h * G + g_begin + (st >> log_rt)) * 256 * kC;
+        const int rs = st / kChunks, ch = st % kChunks, slot = slot_of(st);
+        if ((rs & rt_mask) == 0) {                       // centroids threadIdx.x and threadIdx.x + 128 of the chunk
+            const float* cb_g = cb + (((int64_t)h * G + g_begin + (rs >> log_rt)) * kChunks + ch) * 256 * kC;
             float cv[2][kC];
             tc_fetch_centroid<kC>(cb_g, threadIdx.x, cv[0]);
             tc_fetch_centroid<kC>(cb_g, threadIdx.x + 128, cv[1]);
-            tc_prepare_b<kC>(cv[0], threadIdx.x, b_buf(gslot), cbf_slot(gslot), ctl, gslot, 0);
-            tc_prepare_b<kC>(cv[1], threadIdx.x + 128, b_buf(gslot), cbf_slot(gslot), ctl, gslot, 1);
+            tc_prepare_b<kC>(cv[0], threadIdx.x, b_buf(slot), ctl, slot, 0);
+            tc_prepare_b<kC>(cv[1], threadIdx.x + 128, b_buf(slot), ctl, slot, 1);
         }
+        if (ch != 0) return;
         X_nxt = 0.f;
 #pragma unroll
         for (int w = 0; w < kC / 2; ++w) {
@@ -418,36 +413,51 @@ encode_tc_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, c
             X_nxt = fmaf(f.x, f.x, X_nxt);
             X_nxt = fmaf(f.y, f.y, X_nxt);
         }
-        tc_build_a<kC>(xw_pf, X_nxt, a_buf(st & 1), row);
+        tc_build_a<kC>(xw_pf, X_nxt, a_buf(rs), row);
     };
     // the MMA of one half of step st (half 1 = centroids 128 ... 255), then the commit that arrives on that half's
     // barrier when it is done
     auto issue = [&](int st, int half) {
-        const uint32_t a0 = tc_smem_u32(a_buf(st & 1)), b0 = tc_smem_u32(b_buf((st >> log_rt) & 1)) + half * (128 * 16);
+        const uint32_t a0 = tc_smem_u32(a_buf(st / kChunks)), b0 = tc_smem_u32(b_buf(slot_of(st))) + half * (128 * 16);
 #pragma unroll
         for (int s = 0; s < C::kSteps; ++s)
             tc_mma(tmem_base, tc_desc(a0 + s * C::kATile, 128 * 16), tc_desc(b0 + s * C::kBTile, 256 * 16), s > 0 ? 1u : 0u);
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(tc_smem_u32(&ctl->bar[half])) : "memory");
     };
-    // minima of the 16 subsets (centroid index mod 16) over the 128 scores of the half that is in tensor memory
-    auto scan_half = [&](float (&sb)[16]) {
+
+    // Selection state of this thread's row: minima over the columns of the 16-wide grid of scores (centroid index mod
+    // 16), and the smallest and second smallest minimum over its rows (index / 16, carried in the low mantissa bits)
+    constexpr uint32_t kRowBits = kChunks == 1 ? 15u : 63u;
+    float sb[16], m1 = kTcInf, m2 = kTcInf, nmax = 0.f;
+    bool out_of_range = false, scores_valid = true;
+    auto scan_half = [&](int row0) {
         float va[32], vb[32];
-        auto consume = [&](const float (&v)[32]) {
+        auto consume = [&](const float (&v)[32], int first) {
 #pragma unroll
             for (int q = 0; q < 16; ++q) sb[q] = tc_min3(sb[q], v[q], v[q + 16]);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                float t[5];
+#pragma unroll
+                for (int k = 0; k < 5; ++k) t[k] = tc_min3(v[16 * e + 3 * k], v[16 * e + 3 * k + 1], v[16 * e + 3 * k + 2]);
+                const float r = fminf(tc_min3(t[0], t[1], t[2]), tc_min3(t[3], t[4], v[16 * e + 15]));
+                const float rt = __uint_as_float((__float_as_uint(r) & ~kRowBits) | (uint32_t)(first + e));
+                m2 = fminf(m2, fmaxf(m1, rt));
+                m1 = fminf(m1, rt);
+            }
         };
         tc_ld32_issue(va, taddr);
         tc_ld_wait(va);
         tc_ld32_issue(vb, taddr + 32);
-        consume(va);
+        consume(va, row0);
         tc_ld_wait(vb);
         tc_ld32_issue(va, taddr + 64);
-        consume(vb);
+        consume(vb, row0 + 2);
         tc_ld_wait(va);
         tc_ld32_issue(vb, taddr + 96);
-        consume(va);
+        consume(va, row0 + 4);
         tc_ld_wait(vb);
-        consume(vb);
+        consume(vb, row0 + 6);
     };
 
     fetch(0);
@@ -460,24 +470,31 @@ encode_tc_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, c
         issue(0, 0);
     }
 
+    uint32_t xw[kC / 2];
+    float X = 0.f;
     for (int st = 0; st < n_steps; ++st) {
-        const int g = g_begin + (st >> log_rt), slot = (st >> log_rt) & 1;
-        uint32_t xw[kC / 2];
+        const int rs = st / kChunks, ch = st % kChunks, slot = slot_of(st);
+        const int g = g_begin + (rs >> log_rt);
+        if (ch == 0) {
 #pragma unroll
-        for (int w = 0; w < kC / 2; ++w) xw[w] = xw_nxt[w];
-        const float X = X_nxt;
-        if (st + 1 < n_steps) fetch(st + 1);
+            for (int w = 0; w < kC / 2; ++w) xw[w] = xw_nxt[w];
+            X = X_nxt;
+#pragma unroll
+            for (int q = 0; q < 16; ++q) sb[q] = kTcInf;
+            m1 = m2 = kTcInf;
+            nmax = 0.f;
+            out_of_range = false;
+            scores_valid = true;
+        }
+        if (ch == kChunks - 1 && st + 1 < n_steps) fetch(rs + 1);
 
-        bool scores_valid = *reinterpret_cast<volatile int*>(&ctl->wait_failed) == 0;
+        scores_valid = scores_valid && *reinterpret_cast<volatile int*>(&ctl->wait_failed) == 0;
         if (scores_valid && !tc_wait(&ctl->bar[0], (uint32_t)(st & 1))) {
             ctl->wait_failed = 1;                        // never expected: every row of this CTA goes the exact way from here on
             scores_valid = false;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        float sb[16];
-#pragma unroll
-        for (int q = 0; q < 16; ++q) sb[q] = kTcInf;
-        scan_half(sb);
+        scan_half(ch * 16);
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();                                 // the low half has been read: its columns take the high half
         if (threadIdx.x == 0 && *reinterpret_cast<volatile int*>(&ctl->wait_failed) == 0) {
@@ -491,7 +508,7 @@ encode_tc_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, c
             scores_valid = false;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        scan_half(sb);
+        scan_half(ch * 16 + 8);
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();                                 // tensor memory is free again; the operands of step st + 1 are complete
@@ -500,22 +517,20 @@ encode_tc_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, c
             issue(st + 1, 0);
         }
 
-        // control words of this step's group
-        bool out_of_range;
-        float nmax;
+        // control words of this step's chunk
         {
             const int4 f0 = *reinterpret_cast<const int4*>(&ctl->range_flag[slot][0]);
             const int4 f1 = *reinterpret_cast<const int4*>(&ctl->range_flag[slot][4]);
-            out_of_range = (f0.x | f0.y | f0.z | f0.w | f1.x | f1.y | f1.z | f1.w) != 0;
-            const float4 m0 = *reinterpret_cast<const float4*>(&ctl->nmax[slot][0]);
-            const float4 m1 = *reinterpret_cast<const float4*>(&ctl->nmax[slot][4]);
-            nmax = fmaxf(fmaxf(fmaxf(m0.x, m0.y), fmaxf(m0.z, m0.w)), fmaxf(fmaxf(m1.x, m1.y), fmaxf(m1.z, m1.w)));
+            out_of_range = out_of_range || (f0.x | f0.y | f0.z | f0.w | f1.x | f1.y | f1.z | f1.w) != 0;
+            const float4 n0 = *reinterpret_cast<const float4*>(&ctl->nmax[slot][0]);
+            const float4 n1 = *reinterpret_cast<const float4*>(&ctl->nmax[slot][4]);
+            nmax = fmaxf(nmax, fmaxf(fmaxf(fmaxf(n0.x, n0.y), fmaxf(n0.z, n0.w)), fmaxf(fmaxf(n1.x, n1.y), fmaxf(n1.z, n1.w))));
         }
-        const float* cbf = cbf_slot(slot);
+        if (ch != kChunks - 1) continue;
 
-        // smallest and second smallest subset minimum (a tournament of (smallest, second) pairs); the subset number
-        // rides in the low four mantissa bits, which also makes the 16 values differ
-        float m1v, s2;
+        // smallest and second smallest column minimum (a tournament of (smallest, second) pairs); the column rides in
+        // the low four mantissa bits, which also makes the 16 values differ
+        float c1, c2;
         {
             float lo[8], hi[8];
 #pragma unroll
@@ -533,84 +548,63 @@ encode_tc_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, c
                     hi[i] = tc_min3(fmaxf(lo[i], lo[i + n]), hi[i], hi[i + n]);
                     lo[i] = m;
                 }
-            m1v = lo[0];
-            s2 = hi[0];
+            c1 = lo[0];
+            c2 = hi[0];
         }
-        const int qw = (int)(__float_as_uint(m1v) & 15u);
-        float xg[kC];
-#pragma unroll
-        for (int w = 0; w < kC / 2; ++w) {
-            const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&xw[w]));
-            xg[2 * w] = f.x;
-            xg[2 * w + 1] = f.y;
-        }
-        // the winner's subset, exactly: centroids qw, qw + 16, ..., qw + 240; the smallest distance by a tournament in
-        // which the lower index wins ties
-        float dk[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            const int j = qw + 16 * k;
-            float cc[kC];
-            if (kC == 2) {
-                const float2 t2 = *reinterpret_cast<const float2*>(cbf + j * 2);
-                cc[0] = t2.x; cc[1] = t2.y;
-            } else {
-#pragma unroll
-                for (int w = 0; w < kC; w += 4) {
-                    const float4 t4 = *reinterpret_cast<const float4*>(cbf + j * kC + w);
-                    cc[w] = t4.x; cc[w + 1] = t4.y; cc[(w + 2) % kC] = t4.z; cc[(w + 3) % kC] = t4.w;
-                }
-            }
-            float dd = 0.f;
-#pragma unroll
-            for (int i = 0; i < kC; ++i) {
-                const float diff = xg[i] - cc[i];
-                dd = fmaf(diff, diff, dd);
-            }
-            dk[k] = dd;
-        }
-        int ik[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const bool right = dk[2 * i + 1] < dk[2 * i];        // strict: the lower index keeps a tie
-            ik[i] = right ? 2 * i + 1 : 2 * i;
-            dk[i] = right ? dk[2 * i + 1] : dk[2 * i];
-        }
-#pragma unroll
-        for (int n = 4; n >= 1; n >>= 1)
-#pragma unroll
-            for (int i = 0; i < n; ++i) {
-                const bool right = dk[2 * i + 1] < dk[2 * i];
-                ik[i] = right ? ik[2 * i + 1] : ik[2 * i];
-                dk[i] = right ? dk[2 * i + 1] : dk[2 * i];
-            }
-        float dbest = dk[0];
-        int code = qw + 16 * ik[0];
-        // Evaluation error of a score: fp32 accumulation of up to ~20 terms bounded by 2 (X + N) in magnitude, plus
-        // the four mantissa bits given to the subset number.  dbest is exact.
-        const float ss = __uint_as_float(__float_as_uint(s2) & ~15u);
-        const float tau = 1.6e-5f * (X + nmax) + 4e-6f * fabsf(ss);
-        const bool certain = scores_valid && !out_of_range && (ss - dbest > tau);
-        const TcRow rec = rows[(st & rt_mask) * kTcThreads];
-        const bool live = rec.x != nullptr;
+        int code = (int)((__float_as_uint(m1) & kRowBits) << 4) | (int)(__float_as_uint(c1) & 15u);
+        // Every centroid but the named one lies in another row or another column of the grid, so its score is at least
+        // the smaller of the two second minima.  tau bounds the evaluation error of two scores: an MMA adds 17 exact
+        // terms of at most X + N each, aligned to the largest and cut below its last fp32 bit (17 x 2^-23 (X + N); two
+        // MMAs for c = 8), plus the mantissa bits given to the indexes.
+        const float gap = fminf(m2, c2) - fmaxf(m1, c1);
+        const float tau = (kC == 8 ? 1.2e-5f : 6e-6f) * (X + nmax) + (kRowBits == 15u ? 2.1e-6f : 8e-6f) * (fabsf(m2) + fabsf(m1));
+        const bool certain = scores_valid && !out_of_range && gap > tau;
+        const int64_t off = offsets[(rs & rt_mask) * kTcThreads];
         // exact recomputation of the uncertain rows, one row at a time by the whole warp
-        unsigned pending = __ballot_sync(0xffffffffu, !certain && live);
+        unsigned pending = __ballot_sync(0xffffffffu, !certain && off != -2);
         while (pending) {
             const int src = __ffs(pending) - 1;
             pending &= pending - 1;
-            float xs[kC];
+            float xs[8];
 #pragma unroll
-            for (int w = 0; w < kC / 2; ++w) {
-                const uint32_t ww = __shfl_sync(0xffffffffu, xw[w], src);
-                const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&ww));
-                xs[2 * w] = f.x;
-                xs[2 * w + 1] = f.y;
+            for (int w = 0; w < 4; ++w) {
+                xs[2 * w] = xs[2 * w + 1] = 0.f;
+                if (w < kC / 2) {
+                    const uint32_t ww = __shfl_sync(0xffffffffu, xw[w % (kC / 2)], src);
+                    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&ww));
+                    xs[2 * w] = f.x;
+                    xs[2 * w + 1] = f.y;
+                }
             }
-            float ed;
-            const int ec = tc_exact_code<kC>(xs, cbf, lane, &ed);
-            if (lane == src) { code = ec; dbest = ed; }
+            const int ec = tc_exact_code<kC>(cb + ((int64_t)h * G + g) * (kChunks * 256) * kC, kChunks * 256, xs[0], xs[1], xs[2],
+                                             xs[3], xs[4], xs[5], xs[6], xs[7]);
+            if (lane == src) code = ec;
         }
-        if (rec.code_offset >= 0) codes[rec.code_offset + g * kTokenBlock] = (uint8_t)code;
+        if (off >= 0) codes[off + g * kTokenBlock] = (uint8_t)code;
+        if (kChunks > 1) {
+            // Upper bits: 16 tokens share a word of 2 hb bytes.  Where a half warp holds the 16 tokens of one block it
+            // writes the word; otherwise the bits are replaced in the aligned 32-bit word that other tokens share.
+            constexpr int kHb = kChunks == 2 ? 1 : 2;
+            const int64_t block = off >= 0 ? off & ~(int64_t)15 : -1;
+            const int64_t block0 = __shfl_sync(0xffffffffu, block, lane & 16);
+            const unsigned whole = __ballot_sync(0xffffffffu, off >= 0 && block == block0 && (int)(off & 15) == (lane & 15));
+            const unsigned half_mask = 0xffffu << (lane & 16);
+            if ((whole & half_mask) == half_mask) {
+                const uint32_t word = __reduce_or_sync(half_mask, ((uint32_t)code >> 8) << (kHb * (lane & 15)));
+                unsigned char* dst = codes + block + G * kTokenBlock + g * 2 * kHb;
+                if ((lane & 15) == 0) {
+                    if (kHb == 2) *reinterpret_cast<uint32_t*>(dst) = word;
+                    else *reinterpret_cast<uint16_t*>(dst) = (uint16_t)word;
+                }
+            } else if (off >= 0) {
+                const int bit = (int)(off & 15) * kHb;
+                const uintptr_t a = reinterpret_cast<uintptr_t>(codes) + (uintptr_t)(block + G * kTokenBlock + g * 2 * kHb + (bit >> 3));
+                unsigned int* w = reinterpret_cast<unsigned int*>(a & ~(uintptr_t)3);
+                const int shift = (int)(a & 3) * 8 + (bit & 7);
+                atomicAnd(w, ~((unsigned int)((1 << kHb) - 1) << shift));
+                atomicOr(w, (unsigned int)(code >> 8) << shift);
+            }
+        }
     }
 
     // every MMA that was issued has been waited for (or the wait gave up); hand the tensor memory back
@@ -622,11 +616,11 @@ encode_tc_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, c
     }
 }
 
-template <int kC>
+template <int kC, int kChunks>
 cudaError_t launch_enc_tc(const __half* x, const float* cb, const int32_t* seq_offsets, const Shape& sh, int64_t n_tokens,
                           int64_t token_offset, uint8_t* codes, cudaStream_t st, const __half* x2, const float* cb2, uint8_t* codes2)
 {
-    using C = TcCfg<kC>;
+    using C = TcCfg<kC, kChunks>;
     const int64_t n_vec = sh.n_seq * n_tokens;
     const int64_t tiles = (n_vec + kTcTileVecs - 1) / kTcTileVecs;
     const int64_t slots = C::kCtasPerSm * (int64_t)device_sm_count();          // CTAs in flight
@@ -642,10 +636,12 @@ cudaError_t launch_enc_tc(const __half* x, const float* cb, const int32_t* seq_o
     n_gsplit = (C::G + groups_per_cta - 1) / groups_per_cta;
     const int64_t grid = blocks * sh.n_kv_heads * n_gsplit;
     if (grid > 0x7fffffff) return cudaErrorInvalidConfiguration;
-    constexpr int kSlot = 44 + (kC == 2 ? 0 : kC == 4 ? 1 : 2);       // call-site slots 44 ... 46 of ensure_dynamic_smem
-    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(encode_tc_kernel<kC>), C::kSmemBytes, kSlot);
+    // call-site slots 38, 39, 43 ... 47, 62, 63 of ensure_dynamic_smem
+    constexpr int kSlots[9] = {38, 39, 43, 44, 45, 46, 47, 62, 63};
+    constexpr int kSlot = kSlots[3 * (kC == 2 ? 0 : kC == 4 ? 1 : 2) + (kChunks == 1 ? 0 : kChunks == 2 ? 1 : 2)];
+    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(encode_tc_kernel<kC, kChunks>), C::kSmemBytes, kSlot);
     if (e != cudaSuccess) return e;
-    encode_tc_kernel<kC><<<dim3((unsigned)grid, x2 ? 2u : 1u), kTcThreads, C::kSmemBytes, st>>>(
+    encode_tc_kernel<kC, kChunks><<<dim3((unsigned)grid, x2 ? 2u : 1u), kTcThreads, C::kSmemBytes, st>>>(
         x, cb, seq_offsets, sh, n_tokens, token_offset, codes, groups_per_cta, log_rt, x2, cb2, codes2);
     return cudaGetLastError();
 }
@@ -654,19 +650,24 @@ cudaError_t launch_enc_tc(const __half* x, const float* cb, const int32_t* seq_o
 
 bool encode_tc_supported(const Shape& sh)
 {
-    return sh.head_dim == 128 && sh.b == 8 && (sh.c == 2 || sh.c == 4 || sh.c == 8);
+    return sh.head_dim == 128 && (sh.b == 8 || sh.b == 9 || sh.b == 10) && (sh.c == 2 || sh.c == 4 || sh.c == 8);
 }
 
 cudaError_t launch_encode_tc(const __half* x, const float* cb, const int32_t* seq_offsets, const Shape& sh, int64_t n_tokens,
                              int64_t token_offset, uint8_t* codes, cudaStream_t st, const __half* x2, const float* cb2, uint8_t* codes2)
 {
     if (sh.n_seq * n_tokens == 0) return cudaSuccess;
+#define CQ_TC(C_)                                                                                                              \
+    return sh.b == 8   ? launch_enc_tc<C_, 1>(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2)    \
+           : sh.b == 9 ? launch_enc_tc<C_, 2>(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2)    \
+                       : launch_enc_tc<C_, 4>(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2)
     switch (sh.c) {
-        case 2: return launch_enc_tc<2>(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2);
-        case 4: return launch_enc_tc<4>(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2);
-        case 8: return launch_enc_tc<8>(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2);
+        case 2: CQ_TC(2);
+        case 4: CQ_TC(4);
+        case 8: CQ_TC(8);
         default: return cudaErrorNotSupported;
     }
+#undef CQ_TC
 }
 
 }  // namespace cq
