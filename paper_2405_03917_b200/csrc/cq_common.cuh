@@ -100,6 +100,11 @@ bool encode_tc_supported(const Shape& sh);
 cudaError_t launch_encode_tc(const __half* x, const float* cb, const int32_t* seq_offsets, const Shape& sh, int64_t n_tokens,
                              int64_t token_offset, uint8_t* codes, cudaStream_t st, const __half* x2, const float* cb2,
                              uint8_t* codes2);
+// boxes of the plane with their possible nearest centroids (cq_encode_grid.cu): c = 2, b = 8, many vectors per head
+bool encode_grid_pays(const Shape& sh, int64_t n_tokens, int n_tensors);
+cudaError_t launch_encode_grid(const __half* x, const float* cb, const int32_t* seq_offsets, const Shape& sh, int64_t n_tokens,
+                               int64_t token_offset, uint8_t* codes, cudaStream_t st, const __half* x2, const float* cb2,
+                               uint8_t* codes2);
 bool encode_tuned_supported(const Shape& sh);
 // (x2, cb2, codes2): an optional second tensor of the same shape, encoded by the same launch.
 // allow_tc: bulk inputs of byte codes go to the tensor-memory kernel (false: always the mma.sync kernels).

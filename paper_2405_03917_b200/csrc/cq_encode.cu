@@ -513,7 +513,9 @@ cudaError_t launch_encode_tuned(const __half* x, const float* cb, const int32_t*
 {
     const int64_t n_vec = sh.n_seq * n_tokens;
     if (n_vec == 0) return cudaSuccess;
-    // Byte codes: the tensor-memory kernel at every size.  (8 heads, c = 8: 1665 vectors 70 -> 30 us, 8192 253 -> 114 us;
+    if (allow_tc && encode_grid_pays(sh, n_tokens, x2 ? 2 : 1))
+        return launch_encode_grid(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2);
+    // Up to 1024 centroids: the tensor-memory kernel at every size.  (8 heads, c = 8: 1665 vectors 70 -> 30 us, 8192 253 -> 114 us;
     // the two are level below some 300 vectors, where the launch is what takes the time.)
     if (allow_tc && encode_tc_supported(sh))
         return launch_encode_tc(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2);

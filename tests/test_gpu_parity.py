@@ -509,3 +509,38 @@ def test_both_tuned_kernels_for_four_heads_per_kv_head(n_q, n_kv):
         got, ref = attn_both(q, kc_rm, vc_rm, kcb, vcb, lens, 128 ** -0.5, 8, 8, variant)
         for s_ in range(len(lens)):
             H.check_attn(got[s_], ref[s_], f"variant {variant} seq {s_}")
+
+
+@pytest.mark.parametrize("kind,n_seq,n_tokens,n_heads", [("source", 1, 60000, 2), ("source", 9, 7777, 2), ("ties", 1, 99999, 1), ("far", 3, 33000, 1),
+                                                        ("flat", 1, 98001, 1), ("clumps", 1, 50033, 2)])
+def test_two_channel_bulk_encode_equals_the_generic_kernel(kind, n_seq, n_tokens, n_heads):
+    # the kernel that looks up boxes of the plane: equal distances, points far outside the centroids, a codebook without
+    # extent along one axis, dense clumps (boxes with more centroids than a list holds); codes equal bit for bit
+    # (enough vectors that the dispatch takes it; half of the least would not be)
+    xk, _, kcb, _, _ = H.generic_case(1200 + n_tokens, n_seq, n_tokens, n_heads, n_heads, 128, 2, 8)
+    if kind == "ties":                                                  # a lattice of centroids, each twice; points on lattice and midpoints
+        g = torch.arange(128)
+        cb = torch.stack([(g % 16).float(), (g // 16).float()], 1).repeat_interleave(2, 0)
+        kcb = cb.expand(n_heads, 64, 256, 2).contiguous()
+        xk = (torch.randint(0, 40, xk.shape, generator=torch.Generator().manual_seed(3)).float() / 2 - 1).to(torch.float16)
+    if kind == "far":
+        xk[:, ::3] *= 50
+        xk[:, 1::7] = -60000.0
+    if kind == "flat":
+        kcb[..., 1] = 0.25
+        kcb[:, 5] = kcb[:, 5, :1]
+    if kind == "clumps":
+        kcb = kcb * (torch.arange(256).view(1, 1, 256, 1) % 8 == 0) * 0.01 + 3.0 * kcb[:, :, :1]
+    cap = n_tokens + 30
+    offs = torch.arange(n_seq, dtype=torch.int32, device=DEV) * 11
+    nbytes = cq.cq_codes_bytes(n_seq, cap, n_heads, 128, 2, 8)
+    want, got = (torch.zeros(nbytes, dtype=torch.uint8, device=DEV) for _ in range(2))
+    x, cb = xk.to(DEV), kcb.to(DEV)
+    cq.cq_encode(x, cb, 2, 8, want, cap, seq_offsets=offs, variant=1)
+    cq.cq_encode(x, cb, 2, 8, got, cap, seq_offsets=offs)
+    assert torch.equal(got, want)
+    k2, v2 = torch.zeros_like(got), torch.zeros_like(got)
+    cq.cq_encode_kv(x, x.flip(1).contiguous(), cb, cb, 2, 8, k2, v2, cap, seq_offsets=offs)
+    assert torch.equal(k2, want)
+    cq.cq_encode(x.flip(1).contiguous(), cb, 2, 8, want.zero_(), cap, seq_offsets=offs, variant=1)
+    assert torch.equal(v2, want)
