@@ -1,4 +1,4 @@
-// Tuned decode-attention kernels for head_dim 128, b = 8 (one byte per code).
+// Tuned decode-attention kernels for head_dim 128 (c = 2, 4, 8) and 64 (c = 4, 8), b = 8 (one byte per code).
 //
 // Formulation (an exact re-association of Eq. 1 of the paper with K and V replaced by
 // their CQ reconstructions, Section 3.2):
@@ -25,7 +25,7 @@
 //   row j (256 bytes) of a table holds, for code value j, 32-word "planes"; word w of a
 //   plane belongs to one (group, query head | replica) pair, and lane (r, p) = (lane/4,
 //   lane%4) of a warp uses word  16*(r/4) + 4*((r+m)%4) + p  (16 groups) or
-//   4*((r+m)%8) + p  (32 groups) for its m-th code word, which is a bijection lanes ->
+//   4*((r+m)%8) + p  (32 groups; 8 groups: 8*(r/2) + 4*((r+m)%2) + p) for its m-th code word, which is a bijection lanes ->
 //   banks for every m.
 // A lane quad r owns one 16-token block; lane p of the quad owns the groups congruent to
 // p mod 4.  Table entries are stored as half2 (hi, lo) pairs, so a looked-up word is
@@ -39,19 +39,24 @@ namespace cq {
 namespace {
 
 
-template <int G, int R>
+// kD: head_dim, G: groups, R: query heads a CTA serves.  A table row has one or two planes of 32 words.  A plane is
+// cut into runs of G words (32 / G of them for 8 and 16 groups), each of which holds one query head, or a copy of it
+// where there are fewer heads than runs; the lane rows r = lane / 4 are dealt to the runs.
+template <int kD, int G, int R>
 struct Cfg {
-    static_assert(G == 16 || G == 32 || (G == 64 && R == 1), "tuned decode kernels cover 16, 32 and (one query head) 64 groups");
-    static constexpr int kC = 128 / G;                                  // channels per group
+    static_assert(G == 8 || G == 16 || G == 32 || (G == 64 && R == 1), "tuned decode kernels cover 8, 16, 32 and (one query head) 64 groups");
+    static constexpr int kC = kD / G;                                   // channels per group
     // 64 groups: the two half warps take the same four 16-token blocks, quads 0-3 the groups 0-31 and quads
     // 4-7 the groups 32-63 (second plane of a table row); they exchange their partial scores with one shuffle.
     static constexpr bool kHalfGroups = (G == 64);
-    static constexpr bool kHalfRows = (G == 16);                         // quads 0-3 / 4-7 use different 16-word halves
-    static constexpr bool kReplica = (G == 16 && R == 1);                // the two halves are copies of one table
-    static constexpr int kLaneHeads = (G == 16 && R >= 2) ? R / 2 : R;   // query heads a lane serves
+    static constexpr int kRuns = G == 8 ? 4 : G == 16 ? 2 : 1;          // runs of a plane
+    static constexpr int kPlaneHeads = R < kRuns ? R : kRuns;           // query heads of a plane
+    static constexpr int kCopies = kRuns / kPlaneHeads;                 // runs that hold the same query head
+    static constexpr int kRowsPerHead = 8 / kPlaneHeads;                // lane rows that serve the same head of a plane
+    static constexpr int kLaneHeads = R / kPlaneHeads;                  // query heads a lane serves
     static constexpr int kPlanes = kHalfGroups ? 2 : kLaneHeads;         // 32-word planes per table row
     static constexpr int kSlots = kHalfGroups ? 8 : G / 4;               // code words (16 tokens each) per lane
-    static constexpr int kBlocksPerIter = ((G == 16 && R >= 2) || kHalfGroups) ? 4 : 8;   // 16-token blocks per warp iteration
+    static constexpr int kBlocksPerIter = kHalfGroups ? 4 : kRowsPerHead;   // 16-token blocks per warp iteration
     static constexpr int kWarps = (kPlanes == 1) ? 8 : 16;
     static constexpr int kThreads = kWarps * 32;
     static constexpr int kMinBlocks = (kPlanes == 1) ? 2 : 1;     // 128 registers per thread in every configuration
@@ -60,33 +65,31 @@ struct Cfg {
     // One plane: K and V planes share a row (K at +0, V at +128).  Two planes: separate tables.
     static constexpr int kVOffset = (kPlanes == 1) ? 128 : kRows * kRowBytes;
     static constexpr int kTableBytes = (kPlanes == 1) ? kRows * kRowBytes : 2 * kRows * kRowBytes;
-    static constexpr int kNewOffset = 128 + R * 128 * 4;                 // codes of an appended token: [key | value][64 groups]
+    static constexpr int kNewOffset = 128 + R * kD * 4;                  // codes of an appended token: [key | value][64 groups]
     static constexpr int kCtlBytes = kNewOffset + 128;                   // control words + scaled query + those codes
     static constexpr int kSmemBytes = kTableBytes + kCtlBytes;
 
-    // word inside a plane that lane (r, p) uses for its m-th code word
+    // word inside a plane that lane (r, p) uses for its m-th code word: run r / (8 / kRuns), a bijection lanes -> banks
+    // for every m
     __device__ static __forceinline__ int word(int r, int p, int m)
     {
-        return kHalfRows ? 16 * (r >> 2) + 4 * ((r + m) & 3) + p : 4 * ((r + m) & 7) + p;
+        return G == 8 ? 8 * (r >> 1) + 4 * ((r + m) & 1) + p : G == 16 ? 16 * (r >> 2) + 4 * ((r + m) & 3) + p : 4 * ((r + m) & 7) + p;
     }
-    // group of a table word, and the (plane, word) that holds (group g, query head h of the KV head)
-    __device__ static __forceinline__ int group_of(int w) { return kHalfRows ? (w & 15) : w; }
-    __device__ static __forceinline__ int plane_of(int g, int h)
-    {
-        return kHalfGroups ? g >> 5 : (kHalfRows ? (R <= 2 ? 0 : h >> 1) : h);
-    }
+    // group of a table word, and the (plane, word) that holds (group g, query head h of the KV head; first copy)
+    __device__ static __forceinline__ int group_of(int w) { return kRuns > 1 ? (w & (G - 1)) : w; }
+    __device__ static __forceinline__ int plane_of(int g, int h) { return kHalfGroups ? g >> 5 : h / kPlaneHeads; }
     __device__ static __forceinline__ int word_of(int g, int h)
     {
-        return kHalfGroups ? (g & 31) : (kHalfRows ? (R == 1 ? 0 : (h & 1) * 16) + g : g);
+        return kHalfGroups ? (g & 31) : (h % kPlaneHeads) * (kCopies * G) % 32 + g;
     }
     // byte offset, inside a table row, of the plane that lane row r uses by itself (64 groups only)
     __device__ static __forceinline__ unsigned lane_plane_bytes(int r) { return kHalfGroups ? 128u * (unsigned)(r >> 2) : 0u; }
     // query head (of the KV head) that lane row r serves as its u-th head, and the head a table word belongs to
-    __device__ static __forceinline__ int lane_head(int u, int r) { return kHalfRows ? (R == 1 ? 0 : 2 * u + (r >> 2)) : u; }
+    __device__ static __forceinline__ int lane_head(int u, int r) { return u * kPlaneHeads + r / kRowsPerHead; }
     __device__ static __forceinline__ int head_of_word(int word_in_row)
     {
         const int plane = word_in_row >> 5, w = word_in_row & 31;
-        return kHalfGroups ? 0 : (kHalfRows ? (R == 1 ? 0 : 2 * plane + (w >> 4)) : plane);
+        return kHalfGroups ? 0 : plane * kPlaneHeads + w / (32 / kPlaneHeads);
     }
     // v[lane_head(u, r)] without indexing a register array by a run-time value
     template <int N>
@@ -99,7 +102,7 @@ struct Cfg {
     }
     static constexpr int kLog2Groups = kWarps == 16 ? 4 : 3;             // log2 of the warps that add to a head's bins per round
     static constexpr int kGroupsPerWarp = G / kWarps;
-    static_assert(G % kWarps == 0 && kSlots % 4 == 0, "ownership of groups by warps; four code words per MMA");
+    static_assert(G % kWarps == 0 && kSlots % 2 == 0, "ownership of groups by warps; two code words per MMA");
 };
 
 struct Ctl {
@@ -246,8 +249,8 @@ __device__ __noinline__ void encode_new_value_tuned(uint8_t* newcode, const __ha
 
 // kAppend: the launch also encodes and appends one token per sequence (a second instance, so that the plain attention
 // carries none of that code)
-template <int G, int R, bool kShared, bool kAppend>
-__global__ void __launch_bounds__(Cfg<G, R>::kThreads, Cfg<G, R>::kMinBlocks)
+template <int kD, int G, int R, bool kShared, bool kAppend>
+__global__ void __launch_bounds__(Cfg<kD, G, R>::kThreads, Cfg<kD, G, R>::kMinBlocks)
 decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, const uint8_t* __restrict__ vc,
                     const float* __restrict__ kcb, const float* __restrict__ vcb,
                     const int32_t* __restrict__ seq_lens, float scale_log2e, Shape sh, int chunk_tokens, int n_parts,
@@ -257,7 +260,7 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
     // out: non-null only when every item is one part; the CTA then normalises its partial itself (no merge launch).
     // R is the number of query heads one CTA serves.  A KV head with more query heads than that
     // (kv_share groups of R; kShared) is served by kv_share CTAs, which read the same codes and codebooks.
-    using C = Cfg<G, R>;
+    using C = Cfg<kD, G, R>;
     constexpr int kC = C::kC;
     extern __shared__ __align__(1024) uint8_t smem[];
     Ctl* ctl = reinterpret_cast<Ctl*>(smem + C::kTableBytes);
@@ -293,7 +296,7 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
     if (has_new) ++n;
     const int64_t t_begin = (int64_t)part * chunk_tokens;
     const int64_t t_end = (whole || t_begin + chunk_tokens >= n) ? n : t_begin + chunk_tokens;
-    const int stride = partial_stride(128);
+    const int stride = partial_stride(kD);
     float* part_base = partials + ((s * sh.n_q_heads + (int64_t)head_group * R) * n_parts + part) * stride;
     // partial of query head head_group*R + h: part_base + h * n_parts * stride
     if (whole)          // the other partial slots of this item hold the neutral element of the merge
@@ -307,7 +310,7 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
             part_base[(int64_t)h * n_parts * stride + d] = d == 0 ? -INFINITY : 0.f;
         }
         if (out)            // nothing to attend: the zero row of the merge
-            for (int i = threadIdx.x; i < R * 128; i += C::kThreads) out[(s * sh.n_q_heads + (int64_t)head_group * R) * 128 + i] = 0.f;
+            for (int i = threadIdx.x; i < R * kD; i += C::kThreads) out[(s * sh.n_q_heads + (int64_t)head_group * R) * kD + i] = 0.f;
         return;
     }
 
@@ -315,7 +318,7 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
     const int64_t blk0 = t_begin / kTokenBlock;
     const int64_t blk_lim = (t_end + kTokenBlock - 1) / kTokenBlock;       // blocks holding a valid token
     const int n_iters = (int)((t_end - t_begin + C::kRoundTokens - 1) / C::kRoundTokens);
-    const int qb = (C::kBlocksPerIter == 8) ? r : (r & 3);                 // block of this quad inside the warp's iteration
+    const int qb = r % C::kBlocksPerIter;                 // block of this quad inside the warp's iteration
     // The new token, when its position is in this CTA's range: the CTA works its codes out itself (so do the CTAs of
     // the other query heads that share the KV head) and puts them into the code words it loads of that block; one
     // CTA per KV head also writes them to the cache.
@@ -351,7 +354,7 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
 
     // Codebooks are read in units of kJb * 32 centroids (32 registers per lane): a warp owns whole
     // groups, its lanes walk the code values, and the next unit is loaded while the current one is used.
-    constexpr int kJb = (kC == 8) ? 4 : 8;
+    constexpr int kJb = (kC == 8 || C::kGroupsPerWarp == 1) ? 4 : 8;
     constexpr int kUnitsPerGroup = (kRows / 32) / kJb;
     constexpr int kUnits = C::kGroupsPerWarp * kUnitsPerGroup;
     static_assert(kUnits % 2 == 0, "units are taken in pairs");
@@ -372,8 +375,8 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
         ctl->req_need[threadIdx.x] = kUnset;
     }
     if (threadIdx.x == 4) { ctl->want = 0; ctl->lut_absmax = 0.f; }
-    for (int i = threadIdx.x; i < R * 128; i += C::kThreads)
-        qs[i] = __half2float(q[(s * sh.n_q_heads + (int64_t)head_group * R) * 128 + i]) * scale_log2e;
+    for (int i = threadIdx.x; i < R * kD; i += C::kThreads)
+        qs[i] = __half2float(q[(s * sh.n_q_heads + (int64_t)head_group * R) * kD + i]) * scale_log2e;
     // bins start at zero (16-byte stores over the V planes)
     for (int i = threadIdx.x; i < kRows * 8 * C::kPlanes; i += C::kThreads)
         *reinterpret_cast<uint4*>(smem + C::kVOffset + (i / (8 * C::kPlanes)) * kRowBytes + (i % (8 * C::kPlanes)) * 16) =
@@ -409,7 +412,7 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
 #pragma unroll
             for (int h = 0; h < R; ++h)
 #pragma unroll
-                for (int i = 0; i < kC; ++i) qreg[h][i] = qs[h * 128 + g * kC + i] * inv;
+                for (int i = 0; i < kC; ++i) qreg[h][i] = qs[h * kD + g * kC + i] * inv;
 #pragma unroll
             for (int jb = 0; jb < kJb; ++jb) {
                 const int j = ((u % kUnitsPerGroup) * kJb + jb) * 32 + lane;
@@ -422,7 +425,9 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
                     const uint32_t e = pack_hi_lo(dot);
                     uint8_t* row = smem + j * kRowBytes + C::plane_of(g, h) * 128;
                     *reinterpret_cast<uint32_t*>(row + ((C::word_of(g, h) + j) & 31) * 4) = e;
-                    if (C::kReplica) *reinterpret_cast<uint32_t*>(row + ((16 + g + j) & 31) * 4) = e;
+                    #pragma unroll
+                    for (int copy = 1; copy < C::kCopies; ++copy)
+                        *reinterpret_cast<uint32_t*>(row + ((copy * G + C::word_of(g, h) + j) & 31) * 4) = e;
                 }
                 if (kAppend && find_key) {
                     float d = 0.f;
@@ -560,9 +565,11 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
         }
         event_barrier(C::kThreads);                         // the new state is visible
     };
-    constexpr bool kSplit = C::kHalfRows && R >= 2;      // the two half warps serve different query heads
-    const unsigned grp_mask = kSplit ? (lane < 16 ? 0x0000ffffu : 0xffff0000u) : 0xffffffffu;
-    const bool grp_leader = kSplit ? (lane & 15) == 0 : lane == 0;
+    // lanes that serve the same query heads: the warp, or a half or a quarter of it
+    constexpr int kHeadLanes = 32 / C::kPlaneHeads;
+    constexpr bool kSplit = C::kPlaneHeads > 1;
+    const unsigned grp_mask = kSplit ? ((1u << (kHeadLanes % 32)) - 1u) << (lane & ~(kHeadLanes - 1)) : 0xffffffffu;
+    const bool grp_leader = lane % kHeadLanes == 0;
     load_words(kw, kbase, blk0 + (int64_t)warp * C::kBlocksPerIter + qb);
 
     for (int it = 0; it < n_iters; ++it) {
@@ -642,7 +649,7 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
             }
 #pragma unroll
             // (with 64 groups both half warps hold the same tokens: each counts them once)
-            for (int o = (kSplit || C::kHalfGroups) ? 8 : 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+            for (int o = C::kHalfGroups ? 8 : kHeadLanes / 2; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
             zsum[u] = z;
         }
         any_tokens = __any_sync(0xffffffffu, any_tokens);
@@ -680,7 +687,7 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
                 unsigned int old = 0u;
                 if (grp_leader) old = atomicAdd(&ctl->total[h], ci);
                 // (group mask: with two heads per warp the other half warp may have left this iteration)
-                old = __shfl_sync(grp_mask, old, kSplit ? (lane & 16) : 0);
+                old = __shfl_sync(grp_mask, old, lane & ~(kHeadLanes - 1));
                 mine[u] = ci;
                 if (old + ci >= kBinLimit256) ok = false;
             }
@@ -779,7 +786,9 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
             for (int h = 0; h < R; ++h) {
                 const uint8_t* row = smem + C::kVOffset + j * kRowBytes + C::plane_of(g, h) * 128;
                 uint32_t bi = *reinterpret_cast<const uint32_t*>(row + ((C::word_of(g, h) + j) & 31) * 4);
-                if (C::kReplica) bi += *reinterpret_cast<const uint32_t*>(row + ((16 + g + j) & 31) * 4);
+                #pragma unroll
+                for (int copy = 1; copy < C::kCopies; ++copy)
+                    bi += *reinterpret_cast<const uint32_t*>(row + ((copy * G + C::word_of(g, h) + j) & 31) * 4);
                 const float bv = (float)bi;
                 if (gi == 0) lsum[h] += bv;
 #pragma unroll
@@ -828,11 +837,11 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
     }
     if (out) {
         __syncthreads();
-        for (int i = threadIdx.x; i < R * 128; i += C::kThreads) {
-            const int h = i >> 7, d = i & 127;
+        for (int i = threadIdx.x; i < R * kD; i += C::kThreads) {
+            const int h = i / kD, d = i % kD;
             const float* ph = part_base + (int64_t)h * n_parts * stride;
             const float l = ph[1];
-            out[(s * sh.n_q_heads + (int64_t)head_group * R + h) * 128 + d] = l > 0.f ? ph[2 + d] / l : 0.f;
+            out[(s * sh.n_q_heads + (int64_t)head_group * R + h) * kD + d] = l > 0.f ? ph[2 + d] / l : 0.f;
         }
     }
 }
@@ -1298,38 +1307,44 @@ Plan plan_from(const Shape& sh, int64_t round, int min_blocks, int64_t items)
     return pl;
 }
 
-template <int G, int R>
+template <int kD, int G, int R>
 Plan plan_for(const Shape& sh)
 {
-    return plan_from(sh, Cfg<G, R>::kRoundTokens, Cfg<G, R>::kMinBlocks, sh.n_seq * sh.n_kv_heads * (sh.R / R));
+    return plan_from(sh, Cfg<kD, G, R>::kRoundTokens, Cfg<kD, G, R>::kMinBlocks, sh.n_seq * sh.n_kv_heads * (sh.R / R));
 }
 
-template <int G, int R>
+template <int kD, int G, int R>
 cudaError_t launch_cfg(const __half* q, const uint8_t* kc, const uint8_t* vc, const float* kcb, const float* vcb,
                        const int32_t* seq_lens, float scale, const Shape& sh, const Plan& pl, float* partials,
                        cudaStream_t st, float* out, const AppendArgs& app)
 {
-    using C = Cfg<G, R>;
+    using C = Cfg<kD, G, R>;
     const int kv_share = sh.R / R;
-    // call-site slots of ensure_dynamic_smem: 1 is the wide kernel, 2 ... 13 the template instances
-    constexpr int kSlot = 2 + 2 * ((G == 16 ? 0 : G == 32 ? 3 : 5) + (R == 1 ? 0 : R == 2 ? 1 : 2));
+    // call-site slots of ensure_dynamic_smem: 1 is the wide kernel, 2 ... 13 the template instances of head_dim 128,
+    // 78 ... 89 those of head_dim 64
+    constexpr int kSlot = (kD == 128 ? 2 : 78) + 2 * ((G == 16 ? 0 : G == 64 ? 5 : 3) + (R == 1 ? 0 : R == 2 ? 1 : 2));
     const bool append = app.k_new != nullptr;
+    if (append && kD != 128) return cudaErrorNotSupported;
     // one launch per (shared KV head or not, appending or not) instance; smem call-site slots kSlot, kSlot + 1 and 64 + those
 #define CQ_LAUNCH_TUNED(SHARED, APPEND, SLOT)                                                                                   \
     do {                                                                                                                        \
-        cudaError_t e_ = ensure_dynamic_smem(reinterpret_cast<const void*>(decode_tuned_kernel<G, R, SHARED, APPEND>),           \
+        cudaError_t e_ = ensure_dynamic_smem(reinterpret_cast<const void*>(decode_tuned_kernel<kD, G, R, SHARED, APPEND>),           \
                                              C::kSmemBytes, SLOT);                                                              \
         if (e_ != cudaSuccess) return e_;                                                                                       \
-        decode_tuned_kernel<G, R, SHARED, APPEND><<<pl.grid, C::kThreads, C::kSmemBytes, st>>>(                                  \
+        decode_tuned_kernel<kD, G, R, SHARED, APPEND><<<pl.grid, C::kThreads, C::kSmemBytes, st>>>(                                  \
             q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, pl.chunk, pl.n_parts, pl.tail_first, aligned32(kcb, vcb),         \
             kv_share, partials, pl.n_parts == 1 ? out : nullptr, app);                                                          \
     } while (0)
     if (kv_share > 1) {
-        if (append) CQ_LAUNCH_TUNED(true, true, 62 + kSlot);
-        else CQ_LAUNCH_TUNED(true, false, kSlot);
+        if constexpr (kD == 128) {
+            if (append) CQ_LAUNCH_TUNED(true, true, 62 + kSlot);
+        }
+        if (!append) CQ_LAUNCH_TUNED(true, false, kSlot);
     } else {
-        if (append) CQ_LAUNCH_TUNED(false, true, 62 + kSlot + 1);
-        else CQ_LAUNCH_TUNED(false, false, kSlot + 1);
+        if constexpr (kD == 128) {
+            if (append) CQ_LAUNCH_TUNED(false, true, 62 + kSlot + 1);
+        }
+        if (!append) CQ_LAUNCH_TUNED(false, false, kSlot + 1);
     }
 #undef CQ_LAUNCH_TUNED
     return cudaGetLastError();
@@ -1341,22 +1356,33 @@ bool wide_shape(const Shape& sh) { return sh.head_dim == 128 && sh.c == 8 && sh.
 // the number of query heads per KV head (16 groups: 4, 2, 1; 32 groups: 2, 1; 64 groups: 1).
 int heads_per_cta(const Shape& sh)
 {
-    if (sh.G == 16) return sh.R % 4 == 0 ? 4 : (sh.R % 2 == 0 ? 2 : 1);
+    if (sh.G <= 16) return sh.R % 4 == 0 ? 4 : (sh.R % 2 == 0 ? 2 : 1);
     if (sh.G == 32) return sh.R % 2 == 0 ? 2 : 1;
     return 1;
+}
+
+// f(head_dim, groups, query heads per CTA) as integral constants, for the instance that serves the shape
+template <int kD, int G, int R>
+struct Instance {
+    static constexpr int D = kD, groups = G, heads = R;
+};
+template <typename F>
+auto with_instance(const Shape& sh, F&& f)
+{
+    const int w = heads_per_cta(sh);
+    if (sh.head_dim == 64) {
+        if (sh.G == 8) return w == 1 ? f(Instance<64, 8, 1>()) : w == 2 ? f(Instance<64, 8, 2>()) : f(Instance<64, 8, 4>());
+        return w == 1 ? f(Instance<64, 16, 1>()) : w == 2 ? f(Instance<64, 16, 2>()) : f(Instance<64, 16, 4>());
+    }
+    if (sh.G == 16) return w == 1 ? f(Instance<128, 16, 1>()) : w == 2 ? f(Instance<128, 16, 2>()) : f(Instance<128, 16, 4>());
+    if (sh.G == 32) return w == 1 ? f(Instance<128, 32, 1>()) : f(Instance<128, 32, 2>());
+    return f(Instance<128, 64, 1>());
 }
 
 Plan plan_dispatch(const Shape& sh)
 {
     if (wide_shape(sh)) return plan_from(sh, WideCfg::kRoundTokens, 1, sh.n_seq * sh.n_q_heads);
-    const int w = heads_per_cta(sh);
-    if (sh.G == 16 && w == 1) return plan_for<16, 1>(sh);
-    if (sh.G == 16 && w == 2) return plan_for<16, 2>(sh);
-    if (sh.G == 16 && w == 4) return plan_for<16, 4>(sh);
-    if (sh.G == 32 && w == 1) return plan_for<32, 1>(sh);
-    if (sh.G == 32 && w == 2) return plan_for<32, 2>(sh);
-    if (sh.G == 64) return plan_for<64, 1>(sh);
-    return Plan{0, 1, -1, 0u};
+    return with_instance(sh, [&](auto i) { return plan_for<i.D, i.groups, i.heads>(sh); });
 }
 
 }  // namespace
@@ -1365,7 +1391,9 @@ bool decode_tuned_supported(const Shape& sh)
 {
     if (sh.max_tokens > ((int64_t)1 << 30)) return false;
     if (wide_shape(sh)) return true;
-    if (sh.head_dim != 128 || sh.b != 8) return false;
+    if (sh.b != 8) return false;
+    if (sh.head_dim == 64) return sh.c == 4 || sh.c == 8;
+    if (sh.head_dim != 128) return false;
     return sh.G == 16 || sh.G == 32 || sh.G == 64;      // any number of query heads per KV head
 }
 
@@ -1378,7 +1406,7 @@ int decode_tuned_parts(const Shape& sh)
     return pair > own ? pair : own;
 }
 
-bool decode_fused_append_supported(const Shape& sh) { return decode_tuned_supported(sh) && !wide_shape(sh); }
+bool decode_fused_append_supported(const Shape& sh) { return decode_tuned_supported(sh) && !wide_shape(sh) && sh.head_dim == 128; }
 
 int decode_step_fused_launches(const Shape& sh)
 {
@@ -1416,12 +1444,11 @@ cudaError_t launch_decode_tuned(const __half* q, const uint8_t* kc, const uint8_
             partials);
         e = cudaGetLastError();
     }
-    else if (sh.G == 16 && heads_per_cta(sh) == 1) e = launch_cfg<16, 1>(q, kc, vc, kcb, vcb, seq_lens, scale, sh, pl, partials, st, out, app);
-    else if (sh.G == 16 && heads_per_cta(sh) == 2) e = launch_cfg<16, 2>(q, kc, vc, kcb, vcb, seq_lens, scale, sh, pl, partials, st, out, app);
-    else if (sh.G == 16 && heads_per_cta(sh) == 4) e = launch_cfg<16, 4>(q, kc, vc, kcb, vcb, seq_lens, scale, sh, pl, partials, st, out, app);
-    else if (sh.G == 32 && heads_per_cta(sh) == 1) e = launch_cfg<32, 1>(q, kc, vc, kcb, vcb, seq_lens, scale, sh, pl, partials, st, out, app);
-    else if (sh.G == 32 && heads_per_cta(sh) == 2) e = launch_cfg<32, 2>(q, kc, vc, kcb, vcb, seq_lens, scale, sh, pl, partials, st, out, app);
-    else if (sh.G == 64) e = launch_cfg<64, 1>(q, kc, vc, kcb, vcb, seq_lens, scale, sh, pl, partials, st, out, app);
+    else {
+        e = with_instance(sh, [&](auto i) {
+            return launch_cfg<i.D, i.groups, i.heads>(q, kc, vc, kcb, vcb, seq_lens, scale, sh, pl, partials, st, out, app);
+        });
+    }
     if (e != cudaSuccess) return e;
     if (pl.n_parts == 1 && !wide_shape(sh)) return e;           // one part per item: the kernel wrote the output itself
     return launch_merge(partials, pl.n_parts, sh, out, st);

@@ -544,3 +544,18 @@ def test_two_channel_bulk_encode_equals_the_generic_kernel(kind, n_seq, n_tokens
     assert torch.equal(k2, want)
     cq.cq_encode(x.flip(1).contiguous(), cb, 2, 8, want.zero_(), cap, seq_offsets=offs, variant=1)
     assert torch.equal(v2, want)
+
+
+@pytest.mark.parametrize("c", [4, 8])
+@pytest.mark.parametrize("n_q,n_kv,lens", [(1, 1, [1, 15, 16, 17, 0, 333]), (2, 1, [700, 2049]), (4, 1, [257, 31, 1500]), (8, 1, [90, 200]),
+                                           (3, 3, [515]), (12, 2, [1300, 64])])
+def test_attention_head_dim_64_tuned(c, n_q, n_kv, lens):
+    # 8 and 16 groups, one to four query heads per table plane, contexts that end inside a block and inside a round
+    cap = max(lens) + 3
+    xk, xv, kcb, vcb, q = H.generic_case(1300 + n_q + c, len(lens), cap, n_q, n_kv, 64, c, 8)
+    kc_rm, _ = H.oracle_encode_rowmajor(xk, kcb, c, 8)
+    vc_rm, _ = H.oracle_encode_rowmajor(xv, vcb, c, 8)
+    for variant in (2, 1):
+        out, ref = attn_both(q, kc_rm, vc_rm, kcb, vcb, lens, 64 ** -0.5, c, 8, variant)
+        err, rel = H.check_attn(out, ref, f"head_dim 64 c={c} R={n_q // n_kv} variant={variant}")
+        assert rel < 2e-6
