@@ -1,8 +1,12 @@
-"""ctypes binding of `libcq.so`: argument marshalling only, same names as the C ABI.
+"""Binding of `libcq.so`: argument marshalling only, same names as the C ABI.
 
 Every function takes torch tensors (device tensors for device pointers, CPU tensors for
 the `_host` arguments), checks dtype / contiguity / device, and forwards raw pointers and
 sizes.  A non-zero cq_status raises CQError.  Work is enqueued on torch's current stream.
+
+The calls of a serving loop go through `_cq_native` (csrc/cq_binding.cpp), which makes the same checks in native code;
+it returns None without calling the library where an argument is missing or wrong, and the code here then names the
+error or fills in the default.  Everything else goes through ctypes.
 """
 from __future__ import annotations
 
@@ -100,6 +104,21 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+_native_module = None
+
+
+def _native():
+    global _native_module
+    if _native_module is None:
+        lib()
+        try:
+            from . import _cq_native
+        except ImportError as e:
+            raise ImportError(f"{e}; run `python -m paper_2405_03917_b200.build`") from e
+        _native_module = _cq_native
+    return _native_module
+
+
 def _dev(t: torch.Tensor, dtype, name: str) -> int:
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name}: CUDA tensor expected")
@@ -141,6 +160,11 @@ def cq_encode(x: torch.Tensor, codebooks: torch.Tensor, c: int, b: int, codes_ou
               token_offset: int = 0, seq_offsets: Optional[torch.Tensor] = None, variant: int = 0) -> torch.Tensor:
     """x fp16 (n_seq, n_tokens, n_heads, head_dim); codebooks fp32 (n_heads, G, 2^b, c);
     codes_out uint8 buffer of cq_codes_bytes(...) bytes, updated in place and returned."""
+    st = (_native_module or _native()).encode(x, codebooks, seq_offsets, c, b, codes_out, max_tokens, token_offset, variant)
+    if st is not None:
+        if st:
+            raise CQError(st, "cq_encode")
+        return codes_out
     n_seq, n_tokens, n_heads, head_dim = x.shape
     if tuple(codebooks.shape) != (n_heads, head_dim // max(c, 1), 1 << b, c):
         raise ValueError(f"codebooks shape {tuple(codebooks.shape)} does not match heads/groups/centroids")
@@ -161,6 +185,11 @@ def cq_encode_kv(k: torch.Tensor, v: torch.Tensor, k_cb: torch.Tensor, v_cb: tor
                  k_codes_out: torch.Tensor, v_codes_out: torch.Tensor, max_tokens: int, token_offset: int = 0,
                  seq_offsets: Optional[torch.Tensor] = None) -> None:
     """cq_encode of the key and the value embeddings of the same tokens; k, v fp16 (n_seq, n_tokens, n_heads, head_dim)."""
+    st = (_native_module or _native()).encode_kv(k, v, k_cb, v_cb, seq_offsets, c, b, k_codes_out, v_codes_out, max_tokens, token_offset)
+    if st is not None:
+        if st:
+            raise CQError(st, "cq_encode_kv")
+        return None
     n_seq, n_tokens, n_heads, head_dim = k.shape
     if tuple(v.shape) != tuple(k.shape):
         raise ValueError("k and v must have the same shape")
@@ -206,6 +235,11 @@ def cq_decode_attn(q: torch.Tensor, k_codes: torch.Tensor, v_codes: torch.Tensor
                    variant: int = 0) -> torch.Tensor:
     """q fp16 (n_seq, Hq, head_dim); codes in the library layout; codebooks fp32
     (Hkv, G, 2^b, c); seq_lens int32 (n_seq,).  Returns out fp32 (n_seq, Hq, head_dim)."""
+    st = (_native_module or _native()).decode_attn(q, k_codes, v_codes, k_cb, v_cb, seq_lens, scale, c, b, max_tokens, out, workspace, variant)
+    if st is not None:
+        if st:
+            raise CQError(st, "cq_decode_attn")
+        return out
     n_seq, n_q_heads, head_dim = q.shape
     n_kv_heads = k_cb.shape[0]
     for nm, cb in (("k_cb", k_cb), ("v_cb", v_cb)):
@@ -236,6 +270,11 @@ def cq_prefill_attn(q: torch.Tensor, k_codes: torch.Tensor, v_codes: torch.Tenso
                     out: Optional[torch.Tensor] = None, variant: int = 0) -> torch.Tensor:
     """Causal attention of the n_q newest cached tokens.  q fp16 (n_seq, n_q, Hq, head_dim); seq_lens counts
     the cached tokens including the new ones.  Returns out fp32 (n_seq, n_q, Hq, head_dim)."""
+    st = (_native_module or _native()).prefill_attn(q, k_codes, v_codes, k_cb, v_cb, seq_lens, scale, c, b, max_tokens, out, variant)
+    if st is not None:
+        if st:
+            raise CQError(st, "cq_prefill_attn")
+        return out
     n_seq, n_q, n_q_heads, head_dim = q.shape
     n_kv_heads = k_cb.shape[0]
     for nm, cb in (("k_cb", k_cb), ("v_cb", v_cb)):
@@ -270,6 +309,12 @@ def cq_decode_attn_rope(q: torch.Tensor, k_codes: torch.Tensor, v_codes: torch.T
                         variant: int = 0) -> torch.Tensor:
     """cq_decode_attn for key codes taken before RoPE: rope_cos / rope_sin fp32 (max_tokens, head_dim / 2).
     variant 0 = automatic, 1 = generic kernel, 2 = tuned kernel."""
+    st = (_native_module or _native()).decode_attn_rope(q, k_codes, v_codes, k_cb, v_cb, seq_lens, rope_cos, rope_sin, scale, c, b, max_tokens, pairing,
+                                                        out, workspace, variant)
+    if st is not None:
+        if st:
+            raise CQError(st, "cq_decode_attn_rope")
+        return out
     n_seq, n_q_heads, head_dim = q.shape
     n_kv_heads = k_cb.shape[0]
     for nm, t in (("rope_cos", rope_cos), ("rope_sin", rope_sin)):
@@ -338,6 +383,12 @@ def cq_decode_step(q: torch.Tensor, k_new: torch.Tensor, v_new: torch.Tensor, se
     """One decode step on device buffers: q fp16 (n_seq, n_q_heads, D), k_new / v_new fp16 (n_seq, n_kv_heads, D),
     seq_lens int32 (n_seq,) = tokens cached before the step.  The caches take the new token's codes; returns the
     attention output fp32 (n_seq, n_q_heads, D) over seq_lens + 1 tokens."""
+    st = (_native_module or _native()).decode_step(q, k_new, v_new, seq_lens, k_codes, v_codes, k_cb, v_cb, scale, c, b, max_tokens, out,
+                                                   workspace)
+    if st is not None:
+        if st:
+            raise CQError(st, "cq_decode_step")
+        return out
     n_seq, n_q_heads, head_dim = q.shape
     n_kv_heads = k_cb.shape[0]
     if tuple(k_new.shape) != (n_seq, n_kv_heads, head_dim) or tuple(v_new.shape) != (n_seq, n_kv_heads, head_dim):
@@ -372,6 +423,12 @@ def cq_decode_step_host(q_host: torch.Tensor, k_new_host: torch.Tensor, v_new_ho
                         k_cb: torch.Tensor, v_cb: torch.Tensor, scale: float, c: int, b: int, max_tokens: int,
                         out_host: torch.Tensor, workspace: torch.Tensor) -> torch.Tensor:
     """One decode step from host buffers: H2D copies, append-encode, attention, D2H copy, stream sync."""
+    st = (_native_module or _native()).decode_step_host(q_host, k_new_host, v_new_host, seq_lens_host, k_codes, v_codes, k_cb, v_cb, scale, c, b,
+                                                        max_tokens, out_host, workspace)
+    if st is not None:
+        if st:
+            raise CQError(st, "cq_decode_step_host")
+        return out_host
     n_seq, n_q_heads, head_dim = q_host.shape
     n_kv_heads = k_cb.shape[0]
     st = lib().cq_decode_step_host(_host(q_host, torch.float16, "q_host"), _host(k_new_host, torch.float16, "k_new_host"),
