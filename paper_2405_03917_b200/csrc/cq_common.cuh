@@ -175,7 +175,11 @@ cudaError_t launch_lloyd_step(const __half* x, const float* weights, const float
 cudaError_t launch_learn(const __half* x, const float* weights, const double* uniforms, const Shape& sh, int64_t n_vec,
                          int n_iters, float* codebooks, double* objective, void* workspace, cudaStream_t st);
 
-// Merge of split-K partials into out (shared by both decode variants).
+// Configuration of a launch that may start before the kernel ahead of it in the stream has ended (its kernel executes
+// griddepcontrol.wait before it touches memory); `attr` is the caller's and outlives the launch.
+cudaLaunchConfig_t overlapped_config(unsigned grid, unsigned threads, size_t smem, cudaStream_t st, cudaLaunchAttribute* attr);
+
+// Merge of split-K partials into out (shared by the decode kernels).
 cudaError_t launch_merge(const float* partials, int n_parts, const Shape& sh, float* out, cudaStream_t st);
 
 }  // namespace cq

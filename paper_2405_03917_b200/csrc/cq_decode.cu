@@ -294,6 +294,7 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
     // the attention covers n + 1 tokens (a sequence at capacity gets no new token).
     const bool has_new = kAppend && app.k_new != nullptr && n < sh.max_tokens;
     if (has_new) ++n;
+    if (tail_first == kEvenShares) chunk_tokens = share_of_context(n, n_parts, chunk_tokens);
     const int64_t t_begin = (int64_t)part * chunk_tokens;
     const int64_t t_end = (whole || t_begin + chunk_tokens >= n) ? n : t_begin + chunk_tokens;
     const int stride = partial_stride(kD);
@@ -921,6 +922,7 @@ decode_wide_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc,
 
     int64_t n = seq_lens[s];
     n = n < 0 ? 0 : (n > sh.max_tokens ? sh.max_tokens : n);
+    if (tail_first == kEvenShares) chunk_tokens = share_of_context(n, n_parts, chunk_tokens);
     const int64_t t_begin = (int64_t)part * chunk_tokens;
     const int64_t t_end = (whole || t_begin + chunk_tokens >= n) ? n : t_begin + chunk_tokens;
     const int stride = partial_stride(128);
@@ -1292,8 +1294,8 @@ Plan plan_from(const Shape& sh, int64_t round, int min_blocks, int64_t items)
         chunk = (chunk / 2 + round - 1) / round * round;
     pl.chunk = (int)chunk;
     pl.n_parts = (int)((sh.max_tokens + chunk - 1) / chunk);
-    pl.tail_first = -1;
     pl.grid = (unsigned)(items * pl.n_parts);
+    pl.tail_first = pl.n_parts > 1 && (int64_t)pl.grid <= slots ? kEvenShares : -1;
     const int64_t rest = items % slots;               // CTAs of the last wave
     if (min_blocks == 1 && pl.n_parts == 1 && items > slots && rest > 0 && 2 * rest <= slots && chunk >= 2 * 2048) {
         int64_t k = slots / rest;

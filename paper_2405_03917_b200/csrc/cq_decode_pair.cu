@@ -404,6 +404,7 @@ decode_pair_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc,
     // the attention covers n + 1 tokens (a sequence at capacity gets no new token).
     const bool has_new = app.k_new != nullptr && n < sh.max_tokens;
     if (has_new) ++n;
+    if (tail_first == kEvenShares) chunk_tokens = share_of_context(n, n_parts, chunk_tokens);
     const int64_t t_begin = (int64_t)part * chunk_tokens;
     const int64_t t_end = (whole || t_begin + chunk_tokens >= n) ? n : t_begin + chunk_tokens;
     const int stride = partial_stride(128);
@@ -958,8 +959,8 @@ DecodePlan decode_pair_plan(const Shape& sh)
         chunk = (chunk / 2 + round - 1) / round * round;
     pl.chunk = (int)chunk;
     pl.n_parts = (int)((sh.max_tokens + chunk - 1) / chunk);
-    pl.tail_first = -1;
     pl.grid = (unsigned)(items * pl.n_parts);
+    pl.tail_first = pl.n_parts > 1 && (int64_t)pl.grid <= slots ? kEvenShares : -1;
     // Last wave.  Splitting an item over k CTAs shortens it, but every CTA pays the table build and
     // the bins x centroids product, which cost about as much as seven loop iterations (measured), and
     // a CTA that has an SM to itself runs at about 1 / 0.62 of the rate of two that share one.  Take

@@ -105,6 +105,22 @@ __device__ __forceinline__ int seq_by_rank(const int32_t* __restrict__ seq_lens,
     return hit ? __ffs(hit) - 1 : rank;
 }
 
+// Tokens per CTA of a context of n tokens that is split over n_parts CTAs.  The plan knows only the capacity of the cache
+// (planned = its share).  Where all CTAs run at once (tail_first = kEvenShares) a shorter context is split evenly too, down
+// to kLeastShare tokens, instead of leaving the last parts without any: CQ-8c8b, one sequence of 20011 tokens in a cache
+// for 32768, 32 query heads on 8, 16 parts: 39.1 -> 33.0 us with the merge.  (With more CTAs than run at once the even
+// split only adds table builds: 12 ragged sequences at head_dim 64 24.3 -> 26.9 us.)
+constexpr int kEvenShares = -2;
+constexpr int kLeastShare = 512;
+__device__ __forceinline__ int share_of_context(int64_t n, int n_parts, int planned)
+{
+    if (n_parts == 1) return planned;
+    int share = (int)((n + n_parts - 1) / n_parts);
+    share = (share + kTokenBlock - 1) / kTokenBlock * kTokenBlock;
+    share = share < kLeastShare ? kLeastShare : share;
+    return share < planned ? share : planned;
+}
+
 // byte `k` (0..15) of a 16-byte code word
 __device__ __forceinline__ uint32_t word32(const uint4& w, int k)
 {

@@ -568,39 +568,78 @@ int decode_generic_splits(const Shape& sh)
 }
 
 // out[d] = sum_p 2^(m_p - M) acc_p[d] / sum_p 2^(m_p - M) l_p,  M = max_p m_p  (log-sum-exp merge)
-__global__ void merge_kernel(const float* __restrict__ partials, int n_parts, Shape sh, float* __restrict__ out)
+// The parts are dealt to the lanes for the references and normalisers, so that their loads are in flight together, and
+// eight accumulators at a time are; 16 parts of one sequence's 32 heads, with the launch: 10 -> 4 us.
+constexpr int kMergeThreads = 128;
+__global__ void __launch_bounds__(kMergeThreads)
+merge_kernel(const float* __restrict__ partials, int n_parts, Shape sh, float* __restrict__ out)
 {
+    const int lane = threadIdx.x & 31;
     const int hq = blockIdx.x % sh.n_q_heads;
     const int64_t s = blockIdx.x / sh.n_q_heads;
     const int stride = partial_stride(sh.head_dim);
     const float* base = partials + (s * sh.n_q_heads + hq) * (int64_t)n_parts * stride;
-    float M = -INFINITY;
-    for (int p = 0; p < n_parts; ++p) M = fmaxf(M, base[p * stride]);
     float* o = out + (s * sh.n_q_heads + hq) * (int64_t)sh.head_dim;
+    asm volatile("griddepcontrol.wait;" ::: "memory");      // launched ahead of the end of the kernel that writes the partials
+    float M = -INFINITY;
+    for (int p = lane; p < n_parts; p += 32) M = fmaxf(M, base[p * stride]);
+    for (int d = 16; d > 0; d >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, d));
     if (M == -INFINITY) {           // empty context
-        for (int d = threadIdx.x; d < sh.head_dim; d += blockDim.x) o[d] = 0.f;
+        for (int d = threadIdx.x; d < sh.head_dim; d += kMergeThreads) o[d] = 0.f;
         return;
     }
-    float L = 0.f;
-    for (int p = 0; p < n_parts; ++p) {
-        const float m = base[p * stride];
-        if (m != -INFINITY) L += exp2f(m - M) * base[p * stride + 1];
-    }
-    for (int d = threadIdx.x; d < sh.head_dim; d += blockDim.x) {
-        float a = 0.f;
-        for (int p = 0; p < n_parts; ++p) {
-            const float m = base[p * stride];
-            if (m != -INFINITY) a = fmaf(exp2f(m - M), base[p * stride + 2 + d], a);
+    float L = 0.f, a[2] = {0.f, 0.f};                        // (head_dim <= 256)
+    const int d0 = threadIdx.x, d1 = threadIdx.x + kMergeThreads;
+    for (int p0 = 0; p0 < n_parts; p0 += 32) {
+        const float m = p0 + lane < n_parts ? base[(p0 + lane) * stride] : -INFINITY;
+        const float w = m == -INFINITY ? 0.f : exp2f(m - M);
+        if (w != 0.f) L = fmaf(w, base[(p0 + lane) * stride + 1], L);
+        const int n = n_parts - p0 < 32 ? n_parts - p0 : 32;
+        for (int q0 = 0; q0 < n; q0 += 8) {
+            float v0[8], v1[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const float* part = base + (p0 + q0 + q) * stride + 2;
+                v0[q] = q0 + q < n && d0 < sh.head_dim ? part[d0] : 0.f;
+                v1[q] = q0 + q < n && d1 < sh.head_dim ? part[d1] : 0.f;
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const float wq = __shfl_sync(0xffffffffu, w, (q0 + q) & 31);
+                // (a part without tokens has weight zero; its accumulators may hold anything)
+                if (wq != 0.f) {
+                    a[0] = fmaf(wq, v0[q], a[0]);
+                    a[1] = fmaf(wq, v1[q], a[1]);
+                }
+            }
         }
-        o[d] = a / L;
     }
+    for (int d = 16; d > 0; d >>= 1) L += __shfl_xor_sync(0xffffffffu, L, d);
+    if (d0 < sh.head_dim) o[d0] = a[0] / L;
+    if (d1 < sh.head_dim) o[d1] = a[1] / L;
+}
+
+// A launch that may start before the kernel ahead of it in the stream has ended (its kernel waits for that end itself,
+// with griddepcontrol.wait, before it touches memory): the launch's own latency passes behind that kernel.
+cudaLaunchConfig_t overlapped_config(unsigned grid, unsigned threads, size_t smem, cudaStream_t st, cudaLaunchAttribute* attr)
+{
+    attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr->val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
 }
 
 cudaError_t launch_merge(const float* partials, int n_parts, const Shape& sh, float* out, cudaStream_t st)
 {
-    const unsigned grid = (unsigned)(sh.n_q_heads * sh.n_seq);
-    merge_kernel<<<grid, 128, 0, st>>>(partials, n_parts, sh, out);
-    return cudaGetLastError();
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = overlapped_config((unsigned)(sh.n_q_heads * sh.n_seq), kMergeThreads, 0, st, &attr);
+    return cudaLaunchKernelEx(&cfg, merge_kernel, partials, n_parts, sh, out);
 }
 
 cudaError_t launch_decode_generic(const __half* q, const uint8_t* kc, const uint8_t* vc, const float* kcb,
