@@ -906,6 +906,7 @@ decode_wide_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc,
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int r = lane >> 2, p = lane & 3;
 
+    asm volatile("griddepcontrol.wait;" ::: "memory");      // launched ahead of the end of the append that writes the codes
     // work item: (context part, sequence, query head), with the same tail rule as decode_tuned_kernel
     const int n_items = (int)(sh.n_q_heads * sh.n_seq);
     int item = blockIdx.x % n_items;
@@ -1441,10 +1442,10 @@ cudaError_t launch_decode_tuned(const __half* q, const uint8_t* kc, const uint8_
         if (app.k_new) return cudaErrorNotSupported;          // this kernel does not append
         e = ensure_dynamic_smem(reinterpret_cast<const void*>(decode_wide_kernel), WideCfg::kSmemBytes, 1);
         if (e != cudaSuccess) return e;
-        decode_wide_kernel<<<pl.grid, WideCfg::kThreads, WideCfg::kSmemBytes, st>>>(
-            q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, pl.chunk, pl.n_parts, pl.tail_first, aligned32(kcb, vcb),
-            partials);
-        e = cudaGetLastError();
+        cudaLaunchAttribute attr;
+        const cudaLaunchConfig_t cfg = overlapped_config(pl.grid, WideCfg::kThreads, WideCfg::kSmemBytes, st, &attr);
+        e = cudaLaunchKernelEx(&cfg, decode_wide_kernel, q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, pl.chunk, pl.n_parts, pl.tail_first,
+                               aligned32(kcb, vcb), partials);
     }
     else {
         e = with_instance(sh, [&](auto i) {

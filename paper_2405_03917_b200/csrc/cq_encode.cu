@@ -472,6 +472,113 @@ encode_tuned_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1
     }
 }
 
+// Few vectors per head (the append of a decode step): one CTA per (head, group) reads the group's codebook once, a thread
+// holding kPer of its 256 * kPer centroids in registers, and takes the vectors past them sixteen at a time.
+// Distances are the direct form sum (x - C)^2 in fp32 in the order of the generic kernel, lowest index on ties.  What
+// it takes is one pass over the codebooks (16 vectors x 32 heads of CQ-8c10b, key and value: 33 MB; 52 us on the
+// tensor-memory kernel, which walks its steps one after the other with 16 of 128 rows in use, 17 us here; one vector of
+// CQ-8c8b, 8 heads: 5.6 -> 1.9 us).
+constexpr int kFewVecs = 16;
+constexpr int kFewMost = 32;          // vectors per head up to which it is the faster one (32 heads, key and value of CQ-8c10b: 31 against 45 us; 64: 59 against 46)
+template <int kC, int kPer>
+__global__ void __launch_bounds__(256)
+encode_few_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, const int32_t* __restrict__ seq_offsets, Shape sh,
+                  int n_vec, int n_tokens, int64_t token_offset, uint8_t* __restrict__ codes1, const __half* __restrict__ x2,
+                  const float* __restrict__ cb2, uint8_t* __restrict__ codes2)
+{
+    const __half* x = blockIdx.y ? x2 : x1;
+    const float* cb = blockIdx.y ? cb2 : cb1;
+    uint8_t* codes = blockIdx.y ? codes2 : codes1;
+    constexpr int G = 128 / kC;
+    __shared__ float xs[kFewVecs][kC];
+    __shared__ unsigned long long near[kFewVecs][8];          // per vector and warp: (distance, centroid)
+    const int g = blockIdx.x % G, h = blockIdx.x / G, n_heads = sh.n_kv_heads;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float cv[kPer][kC];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        const float* src = cb + (((int64_t)h * G + g) * (256 * kPer) + u * 256 + threadIdx.x) * kC;
+        if (kC == 2) {
+            const float2 a = *reinterpret_cast<const float2*>(src);
+            cv[u][0] = a.x; cv[u][1 % kC] = a.y;
+        } else {
+#pragma unroll
+            for (int w = 0; w < kC; w += 4) {
+                const float4 a = *reinterpret_cast<const float4*>(src + w);
+                cv[u][w] = a.x; cv[u][(w + 1) % kC] = a.y; cv[u][(w + 2) % kC] = a.z; cv[u][(w + 3) % kC] = a.w;
+            }
+        }
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");       // (the codebooks are never written by the kernel ahead)
+    for (int v0 = 0; v0 < n_vec; v0 += kFewVecs) {
+        const int nv = n_vec - v0 < kFewVecs ? n_vec - v0 : kFewVecs;
+        if (threadIdx.x < kFewVecs * kC) {
+            const int v = threadIdx.x / kC, e = threadIdx.x % kC;
+            xs[v][e] = v < nv ? __half2float(x[((int64_t)(v0 + v) * n_heads + h) * 128 + g * kC + e]) : 0.f;
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int v = 0; v < nv; ++v) {
+            float xv[kC];
+#pragma unroll
+            for (int e = 0; e < kC; ++e) xv[e] = xs[v][e];
+            float best = kInfBits;
+            int arg = 0;
+#pragma unroll
+            for (int u = 0; u < kPer; ++u) {
+                float d = 0.f;
+#pragma unroll
+                for (int e = 0; e < kC; ++e) {
+                    const float diff = xv[e] - cv[u][e];
+                    d = fmaf(diff, diff, d);
+                }
+                if (d < best) { best = d; arg = u * 256 + (int)threadIdx.x; }      // ascending: strict < keeps the lowest index
+            }
+            // (distances are not negative: their bits order as they do)
+            const unsigned db = __float_as_uint(best), dm = __reduce_min_sync(0xffffffffu, db);
+            const unsigned jm = __reduce_min_sync(0xffffffffu, db == dm ? (unsigned)arg : 0xffffffffu);
+            if (lane == 0) near[v][warp] = ((unsigned long long)dm << 32) | jm;
+        }
+        __syncthreads();
+        if ((int)threadIdx.x < nv) {
+            unsigned long long key = near[threadIdx.x][0];
+#pragma unroll
+            for (int w = 1; w < 8; ++w) key = near[threadIdx.x][w] < key ? near[threadIdx.x][w] : key;
+            const int code = (int)(key & 0xffffffffu), v = v0 + (int)threadIdx.x;
+            const int s = v / n_tokens, i = v - s * n_tokens;
+            const int64_t pos = token_offset + (seq_offsets ? seq_offsets[s] : 0) + i;
+            if (pos >= 0 && pos < sh.max_tokens) {
+                const int k = (int)(pos % kTokenBlock);
+                codes[code_word_offset(sh, n_heads, s, h, pos / kTokenBlock, g) + k] = (uint8_t)code;
+                if (kPer > 1) {            // upper bits: replaced in the 32-bit word that other tokens share
+                    const int bit = k * sh.hb;
+                    const uintptr_t a = reinterpret_cast<uintptr_t>(codes) +
+                                        (uintptr_t)code_high_offset(sh, n_heads, s, h, pos / kTokenBlock, g) + (bit >> 3);
+                    unsigned int* w = reinterpret_cast<unsigned int*>(a & ~(uintptr_t)3);
+                    const int shift = (int)(a & 3) * 8 + (bit & 7);
+                    atomicAnd(w, ~((unsigned int)((1 << sh.hb) - 1) << shift));
+                    atomicOr(w, (unsigned int)(code >> 8) << shift);
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
+template <int kC>
+cudaError_t launch_few(const __half* x, const float* cb, const int32_t* seq_offsets, const Shape& sh, int64_t n_tokens, int64_t token_offset,
+                       uint8_t* codes, cudaStream_t st, const __half* x2, const float* cb2, uint8_t* codes2)
+{
+    cudaLaunchAttribute attr;
+    cudaLaunchConfig_t cfg = overlapped_config((unsigned)(sh.n_kv_heads * EncCfg<kC>::G), 256, 0, st, &attr);
+    cfg.gridDim.y = x2 ? 2 : 1;
+    const int n_vec = (int)(sh.n_seq * n_tokens);
+    auto go = [&](auto kernel) {
+        return cudaLaunchKernelEx(&cfg, kernel, x, cb, seq_offsets, sh, n_vec, (int)n_tokens, token_offset, codes, x2, cb2, codes2);
+    };
+    return sh.b == 8 ? go(encode_few_kernel<kC, 1>) : sh.b == 9 ? go(encode_few_kernel<kC, 2>) : go(encode_few_kernel<kC, 4>);
+}
+
 template <int kC, int kMT, bool kWide = false>
 cudaError_t launch_enc(const __half* x, const float* cb, const int32_t* seq_offsets, const Shape& sh, int64_t n_tokens,
                        int64_t token_offset, uint8_t* codes, cudaStream_t st, const __half* x2 = nullptr,
@@ -513,6 +620,13 @@ cudaError_t launch_encode_tuned(const __half* x, const float* cb, const int32_t*
 {
     const int64_t n_vec = sh.n_seq * n_tokens;
     if (n_vec == 0) return cudaSuccess;
+    if (allow_tc && n_vec <= kFewMost && (sh.b == 8 || sh.b == 9 || sh.b == 10)) {
+        switch (sh.c) {
+            case 2: return launch_few<2>(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2);
+            case 4: return launch_few<4>(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2);
+            default: return launch_few<8>(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2);
+        }
+    }
     if (allow_tc && encode_grid_pays(sh, n_tokens, x2 ? 2 : 1))
         return launch_encode_grid(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2);
     // Up to 1024 centroids: the tensor-memory kernel at every size.  (8 heads, c = 8: 1665 vectors 70 -> 30 us, 8192 253 -> 114 us;

@@ -207,3 +207,22 @@ def test_centroid_learning_with_1024_centroids():
     close = np.abs(got - want) <= 2e-5 * np.abs(want).max() + 2e-5 * np.abs(want)
     assert close.mean() > 0.999
     np.testing.assert_allclose(gobj, obj, rtol=1e-5)
+
+
+@pytest.mark.parametrize("c,b", [(2, 8), (4, 8), (8, 8), (8, 9), (4, 10), (8, 10)])
+@pytest.mark.parametrize("n_seq", [1, 16, 17, 32, 33])
+def test_few_vectors_equal_the_generic_kernel(c, b, n_seq):
+    # one vector per sequence appended at ragged positions: one and two passes of sixteen vectors, and one vector more
+    # than the few-vector kernel takes; positions beyond the capacity are skipped, neighbours' upper bits are kept
+    n_heads, cap = 3, 40
+    xk, xv, kcb, vcb, _ = H.generic_case(1400 + c * b + n_seq, n_seq, 1, n_heads, n_heads, 128, c, b)
+    offs = (torch.arange(n_seq, dtype=torch.int32) * 7 % 43).to(DEV)
+    nbytes = cq.cq_codes_bytes(n_seq, cap, n_heads, 128, c, b)
+    start = torch.randint(0, 256, (nbytes,), dtype=torch.uint8, generator=torch.Generator().manual_seed(n_seq)).to(DEV)
+    want, got_k, got_v = start.clone(), start.clone(), start.clone()
+    cq.cq_encode(xk.to(DEV), kcb.to(DEV), c, b, want, cap, seq_offsets=offs, variant=1)
+    cq.cq_encode_kv(xk.to(DEV), xv.to(DEV), kcb.to(DEV), vcb.to(DEV), c, b, got_k, got_v, cap, seq_offsets=offs)
+    assert torch.equal(got_k, want)
+    want = start.clone()
+    cq.cq_encode(xv.to(DEV), vcb.to(DEV), c, b, want, cap, seq_offsets=offs, variant=1)
+    assert torch.equal(got_v, want)
