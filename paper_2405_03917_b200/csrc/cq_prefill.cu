@@ -104,49 +104,39 @@ prefill_generic_kernel(const __half* __restrict__ q, const uint8_t* __restrict__
 // tensor-core kernel
 // ------------------------------------------------------------------------------------------
 struct PfCfg {
-    static constexpr int kWarps = 8;                                    // warps that multiply (16 rows each)
-    static constexpr int kProducerWarps = 4;                            // warps that dequantise the tiles
-    static constexpr int kThreads = (kWarps + kProducerWarps) * 32;
-    // Registers: the CTA is launched with 168 per thread (the most 384 threads can have); the producers go down to
-    // 40, the multiplying warps up to 232.  The registers the producers give back must cover what the others ask
-    // for, or the increase waits for ever (48 for the producers does: 4 x 120 < 8 x 64).
-    static constexpr int kLaunchRegs = 168, kProducerRegs = 40, kMultiplierRegs = 232;
-    static_assert((kLaunchRegs - kProducerRegs) * kProducerWarps >= (kMultiplierRegs - kLaunchRegs) * kWarps,
-                  "setmaxnreg: the producers must release what the multiplying warps take");
-    static constexpr int kRows = 128;             // (query, head) rows per CTA: 16 per warp
+    static constexpr int kRows = 256;             // (query, head) rows per CTA: two tiles of 128, one tensor-memory lane each
+    static constexpr int kMmaWarp = 8;            // one thread issues the MMAs; the warps before it: softmax, four per row tile, a thread per row
+    static constexpr int kProducerWarp0 = 9, kProducerWarps = 4;       // dequantise the tiles
+    static constexpr int kThreads = (kProducerWarp0 + kProducerWarps) * 32;
     static constexpr int kTile = 64;              // cached tokens per step
-    static constexpr int kRowBytes = 256;         // 128 fp16 channels
-    static constexpr int kCbBytes = 128 * 256 * 2;                     // one codebook as fp16: [G][256][c]
+    static constexpr int kStages = 3;
+    static constexpr int kCbBytes = 128 * 256 * 2;                     // one codebook as fp16, code-major
     static constexpr int kKcbOffset = 0, kVcbOffset = kCbBytes;
-    static constexpr int kQOffset = 2 * kCbBytes;
-    static constexpr int kKtOffset = kQOffset + kRows * kRowBytes;     // K tiles, two buffers
-    static constexpr int kVtOffset = kKtOffset + 2 * kTile * kRowBytes; // V tiles, two buffers
-    static constexpr int kTileBytes = kTile * kRowBytes;
-    static constexpr int kSmemBytes = kVtOffset + 2 * kTile * kRowBytes;   // 224 KiB
+    static constexpr int kHalfBytes = kTile * 128;                     // 64 channels of a tile: rows of 128 bytes, one per token
+    static constexpr int kTileBytes = 2 * kHalfBytes;
+    static constexpr int kVtOffset = 2 * kCbBytes;                     // [stages]
+    static constexpr int kKtOffset = kVtOffset + kStages * kTileBytes; // [stages]
+    static constexpr int kCtlOffset = kKtOffset + kStages * kTileBytes;
+    static constexpr int kSmemBytes = kCtlOffset + 256;                // 224.25 KiB
+    // tensor-memory columns: output accumulators (fp32), queries (fp16, two per column), scores (fp32) with the weights
+    // (fp16) in their place
+    static constexpr int kOCol = 0, kQCol = 256, kSCol = 384;
+    static_assert(kKtOffset % 1024 == 0 && kTileBytes % 1024 == 0, "swizzled tiles");
+    static_assert(kSmemBytes <= 227 * 1024, "shared memory");
 };
 
+struct PfCtl {
+    uint64_t full[PfCfg::kStages];        // K and V tile of the stage are written (one arrival per producer warp)
+    uint64_t empty[PfCfg::kStages];       // the MMAs that read the stage are done
+    uint64_t s_full[2];                   // scores of the row tile are in tensor memory (and the sums before them are done)
+    uint64_t p_full[2];                   // its weights are (one arrival per warp); also: its queries are, before the first tile
+    uint64_t o_full;                      // all sums are done
+    uint32_t tmem_base;
+    int failed;                           // a wait gave up
+};
+static_assert(sizeof(PfCtl) <= 256, "control block");
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// byte offset of 16-byte chunk `chunk` (0..15) of row `row` in a tile of 256-byte rows; the chunk index is
-// XOR-ed with the low row bits so that eight consecutive rows of one chunk column fall into different banks
-__device__ __forceinline__ uint32_t tile_off(int row, int chunk) { return (uint32_t)(row * 256 + ((chunk ^ (row & 7)) << 4)); }
-
-__device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t addr)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], uint32_t addr)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-__device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
-{
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
 __device__ __forceinline__ uint32_t pack_half2(float lo, float hi)
 {
     const __half2 h = __floats2half2_rn(lo, hi);
@@ -160,21 +150,94 @@ __device__ __forceinline__ float ex2_approx(float x)
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+__device__ __forceinline__ float max3(float a, float b, float c)
+{
+    float d;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+
+__device__ __forceinline__ void pf_init(uint64_t* bar, int arrivals)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(arrivals) : "memory");
+}
+__device__ __forceinline__ void pf_arrive(uint64_t* bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+// Waits for the phase with the given parity; gives up after a bounded number of polls, or when another wait has, and then
+// returns false: every role leaves its loop and the CTA ends.
+__device__ __forceinline__ bool pf_wait(PfCtl* ctl, uint64_t* bar, uint32_t parity)
+{
+    for (int poll = 0; poll < (1 << 17); ++poll) {
+        uint32_t done;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(done) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+        if (done) return true;
+        if ((poll & 63) == 63 && *reinterpret_cast<volatile int*>(&ctl->failed)) return false;
+    }
+    ctl->failed = 1;
+    return false;
+}
+
+// Shared-memory matrix descriptor of a tile of 128-byte rows with the 128-byte swizzle (16-byte chunk index XOR row mod 8).
+// Rows = tokens.  As keys (contraction along the row) eight rows are one core matrix group of 1024 bytes; as values (the
+// row is the N dimension) the next 64 channels are kHalfBytes on and the next eight tokens 1024 bytes.
+__device__ __forceinline__ uint64_t pf_desc(uint32_t saddr, uint32_t leading_bytes)
+{
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr >> 4) & 0x3fffu);
+    d |= (uint64_t)((leading_bytes >> 4) & 0x3fffu) << 16;
+    d |= (uint64_t)((1024u >> 4) & 0x3fffu) << 32;
+    d |= (uint64_t)1 << 46;                      // descriptor version of sm_100
+    d |= (uint64_t)2 << 61;                      // 128-byte swizzle
+    return d;
+}
+// D[128 x N] (+)= A[128 x 16] * B, A (fp16) from tensor memory, B (fp16) from shared memory, fp32 accumulator
+__device__ __forceinline__ void pf_mma(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, {%5, %5, %5, %5}, p;\n\t}"
+                 ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(0) : "memory");
+}
+__device__ __forceinline__ void pf_commit(uint64_t* bar)
+{
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+#define CQ_R32(u) "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]), "=r"(u[8]), "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15]), "=r"(u[16]), "=r"(u[17]), "=r"(u[18]), "=r"(u[19]), "=r"(u[20]), "=r"(u[21]), "=r"(u[22]), "=r"(u[23]), "=r"(u[24]), "=r"(u[25]), "=r"(u[26]), "=r"(u[27]), "=r"(u[28]), "=r"(u[29]), "=r"(u[30]), "=r"(u[31])
+#define CQ_RW32(u) "+r"(u[0]), "+r"(u[1]), "+r"(u[2]), "+r"(u[3]), "+r"(u[4]), "+r"(u[5]), "+r"(u[6]), "+r"(u[7]), "+r"(u[8]), "+r"(u[9]), "+r"(u[10]), "+r"(u[11]), "+r"(u[12]), "+r"(u[13]), "+r"(u[14]), "+r"(u[15]), "+r"(u[16]), "+r"(u[17]), "+r"(u[18]), "+r"(u[19]), "+r"(u[20]), "+r"(u[21]), "+r"(u[22]), "+r"(u[23]), "+r"(u[24]), "+r"(u[25]), "+r"(u[26]), "+r"(u[27]), "+r"(u[28]), "+r"(u[29]), "+r"(u[30]), "+r"(u[31])
+#define CQ_IN32(u) "r"(u[0]), "r"(u[1]), "r"(u[2]), "r"(u[3]), "r"(u[4]), "r"(u[5]), "r"(u[6]), "r"(u[7]), "r"(u[8]), "r"(u[9]), "r"(u[10]), "r"(u[11]), "r"(u[12]), "r"(u[13]), "r"(u[14]), "r"(u[15]), "r"(u[16]), "r"(u[17]), "r"(u[18]), "r"(u[19]), "r"(u[20]), "r"(u[21]), "r"(u[22]), "r"(u[23]), "r"(u[24]), "r"(u[25]), "r"(u[26]), "r"(u[27]), "r"(u[28]), "r"(u[29]), "r"(u[30]), "r"(u[31])
+// 32 consecutive columns of this thread's row (the values are there after pf_ld_wait, whose registers pass through it)
+__device__ __forceinline__ void pf_ld32(uint32_t (&u)[32], uint32_t taddr)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+                 : CQ_R32(u) : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void pf_ld_wait(uint32_t (&u)[32]) { asm volatile("tcgen05.wait::ld.sync.aligned;" : CQ_RW32(u)::"memory"); }
+__device__ __forceinline__ void pf_st32(uint32_t taddr, const uint32_t (&u)[32])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};"
+                 ::"r"(taddr), CQ_IN32(u) : "memory");
+}
+__device__ __forceinline__ void pf_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void pf_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void pf_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 template <int kC>
 __global__ void __launch_bounds__(PfCfg::kThreads, 1)
-prefill_mma_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, const uint8_t* __restrict__ vc,
-                   const float* __restrict__ kcb, const float* __restrict__ vcb,
-                   const int32_t* __restrict__ seq_lens, float scale_log2e, Shape sh, int n_q, int row_tiles,
-                   float* __restrict__ out)
+prefill_tc_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, const uint8_t* __restrict__ vc,
+                  const float* __restrict__ kcb, const float* __restrict__ vcb,
+                  const int32_t* __restrict__ seq_lens, float scale_log2e, Shape sh, int n_q, int row_tiles,
+                  float* __restrict__ out)
 {
     using C = PfCfg;
     constexpr int G = 128 / kC;
     extern __shared__ __align__(1024) uint8_t smem[];
+    PfCtl* ctl = reinterpret_cast<PfCtl*>(smem + C::kCtlOffset);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int r = lane >> 2, p = lane & 3;
     const int R = sh.R;
-    const int q_per_tile = C::kRows / R;                                 // query tokens of one row tile
+    const int q_per_tile = C::kRows / R;                                   // query tokens of one row tile
 
     const int tile = row_tiles - 1 - blockIdx.x % row_tiles;               // later queries attend more tokens: they start first
     const int hkv = (blockIdx.x / row_tiles) % sh.n_kv_heads;
@@ -183,284 +246,310 @@ prefill_mma_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc,
     n = n < 0 ? 0 : (n > sh.max_tokens ? sh.max_tokens : n);
     const int qi0 = tile * q_per_tile;
     // row rho of the CTA: query qi0 + rho / R, head hkv * R + rho % R, position n - n_q + query
-    const int64_t pos0 = n - n_q + qi0;                                  // position of the tile's first query (may be negative)
+    const int64_t pos0 = n - n_q + qi0;                                    // position of the tile's first query (may be negative)
     int q_last = qi0 + q_per_tile - 1;
     if (q_last > n_q - 1) q_last = n_q - 1;
-    const int64_t pos_last = n - n_q + q_last;                           // largest position of the tile
+    const int64_t pos_last = n - n_q + q_last;                             // largest position of the tile
+    const int n_tiles = pos_last < 0 ? 0 : (int)(pos_last / C::kTile + 1);
+    const int n_halves = (q_last - qi0 + 1) * R > 128 ? 2 : 1;             // row tiles of 128 in use
+    // (a negative scale: the queries change sign instead; a zero one: they become zero; both are exact)
+    const uint32_t q_sign = scale_log2e < 0.f ? 0x80008000u : 0u, q_keep = scale_log2e == 0.f ? 0u : 0xffffffffu;
+    const float scale = scale_log2e == 0.f ? 1.f : fabsf(scale_log2e);
 
-    // ---- codebooks as fp16, the query tile
+    // ---- barriers, tensor memory
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < C::kStages; ++i) {
+            pf_init(&ctl->full[i], C::kProducerWarps);
+            pf_init(&ctl->empty[i], 1);
+        }
+        for (int t = 0; t < 2; ++t) {
+            pf_init(&ctl->s_full[t], 1);
+            pf_init(&ctl->p_full[t], 4);
+        }
+        pf_init(&ctl->o_full, 1);
+        ctl->failed = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == C::kMmaWarp) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&ctl->tmem_base)) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    // ---- codebooks as fp16, code-major ([code][group][channel]): the lanes of a gather take different groups, so they
+    // meet in no bank whatever the codes are.  For c = 2 (one word per centroid) group g sits in column
+    // 16 (g mod 4) + g / 4.
     for (int i = threadIdx.x; i < 128 * 256 / 2; i += C::kThreads) {
         const float2 a = *reinterpret_cast<const float2*>(kcb + (int64_t)hkv * 128 * 256 + 2 * i);
         const float2 b = *reinterpret_cast<const float2*>(vcb + (int64_t)hkv * 128 * 256 + 2 * i);
-        // code-major ([code][group][channel]): the lanes of a gather take different groups, so they meet in no bank
-        // whatever the codes are.  For c = 2 (one word per centroid, a lane gathers the groups 4 chunk + i) group g
-        // sits in column 16 (g mod 4) + g / 4, so that the 16 chunks of one gather fall into 16 different banks.
-        int w;
-        {
-            const int g = (2 * i) / (256 * kC), code = ((2 * i) / kC) % 256, ch = (2 * i) % kC;
-            w = kC == 2 ? code * G + 16 * (g & 3) + (g >> 2) : ((code * G + g) * kC + ch) / 2;
-        }
+        const int g = (2 * i) / (256 * kC), code = ((2 * i) / kC) % 256, ch = (2 * i) % kC;
+        const int w = kC == 2 ? code * G + 16 * (g & 3) + (g >> 2) : ((code * G + g) * kC + ch) / 2;
         *reinterpret_cast<uint32_t*>(smem + C::kKcbOffset + 4 * w) = pack_half2(a.x, a.y);
         *reinterpret_cast<uint32_t*>(smem + C::kVcbOffset + 4 * w) = pack_half2(b.x, b.y);
     }
-    for (int i = threadIdx.x; i < C::kRows * 16; i += C::kThreads) {
-        const int rho = i >> 4, chunk = i & 15;
-        const int qi = qi0 + rho / R, h = hkv * R + rho % R;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (qi < n_q) v = *reinterpret_cast<const uint4*>(q + (((s * n_q + qi) * sh.n_q_heads + h) * 128 + chunk * 8));
-        *reinterpret_cast<uint4*>(smem + C::kQOffset + tile_off(rho, chunk)) = v;
-    }
+    pf_fence_before();
     __syncthreads();
+    pf_fence_after();
+    const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&ctl->tmem_base);
 
-    float o[16][4];
+    if (warp >= C::kProducerWarp0) {
+        // ---------------------------------------------------------------- producers: codes -> fp16 tiles of 64 tokens
+        // A warp takes one 16-token block of the tile.  16-byte chunk `ch` (channels 8 ch ... + 7) of token t goes to byte
+        // (ch / 8) * kHalfBytes + t * 128 + ((ch % 8) ^ (t % 8)) * 16: eight lanes of a store hold the chunks of one token,
+        // so they meet in no bank either.
+        const int pw = warp - C::kProducerWarp0;
+        const uint8_t* kbase = kc + code_word_offset(sh, sh.n_kv_heads, s, hkv, 0, 0);
+        const uint8_t* vbase = vc + code_word_offset(sh, sh.n_kv_heads, s, hkv, 0, 0);
+        constexpr int kW = kC == 8 ? 2 : kC == 4 ? 4 : 8;                   // code words a lane takes of a block, per tensor
+        uint32_t kw[kW], vw[kW];
+        auto load_codes = [&](int jt) {
+            const int64_t blk = (int64_t)jt * (C::kTile / kTokenBlock) + pw;
 #pragma unroll
-    for (int nt = 0; nt < 16; ++nt)
+            for (int i = 0; i < kW; ++i) kw[i] = vw[i] = 0u;
+            if (jt >= n_tiles || blk >= sh.n_blocks) return;
+            const uint8_t* kp = kbase + blk * (G * kTokenBlock);
+            const uint8_t* vp = vbase + blk * (G * kTokenBlock);
+            if (kC == 8) {                              // lane = (token half, group)
+                const int off = (lane & 15) * kTokenBlock + 8 * (lane >> 4);
+                const uint2 a = *reinterpret_cast<const uint2*>(kp + off), b = *reinterpret_cast<const uint2*>(vp + off);
+                kw[0] = a.x; kw[1] = a.y; vw[0] = b.x; vw[1] = b.y;
+            } else if (kC == 4) {                       // lane = group
+                const uint4 a = *reinterpret_cast<const uint4*>(kp + lane * kTokenBlock), b = *reinterpret_cast<const uint4*>(vp + lane * kTokenBlock);
+                kw[0] = a.x; kw[1] = a.y; kw[2 % kW] = a.z; kw[3 % kW] = a.w;
+                vw[0] = b.x; vw[1] = b.y; vw[2 % kW] = b.z; vw[3 % kW] = b.w;
+            } else {                                    // lane = (token half, chunk of four groups, taken in another order by the other half)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) o[nt][j] = 0.f;
-    float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};     // rows r and r + 8 of the warp
-    // positions of this thread's two rows
-    const int rho_a = warp * 16 + r, rho_b = rho_a + 8;
-    const int64_t pos_a = pos0 + rho_a / R, pos_b = pos0 + rho_b / R;
-    const int64_t pos_warp = pos0 + (warp * 16) / R;                      // smallest position among the warp's rows
-
-    const int64_t n_tiles = pos_last < 0 ? 0 : pos_last / C::kTile + 1;
-    const uint8_t* kbase = kc + code_word_offset(sh, sh.n_kv_heads, s, hkv, 0, 0);
-    const uint8_t* vbase = vc + code_word_offset(sh, sh.n_kv_heads, s, hkv, 0, 0);
-    const uint32_t q_s = smem_u32(smem + C::kQOffset), kt_s = smem_u32(smem + C::kKtOffset), vt_s = smem_u32(smem + C::kVtOffset);
-
-    // codes -> fp16 tiles of the 64 tokens from j0 on, into buffer `buf`, by the 128 producer threads: a work item
-    // is (8 tokens, one group), 8 G items per tile (one per thread for c = 8, two for c = 4)
-    auto dequantise_groups = [&](int64_t j0, int buf) {
-        for (int item = threadIdx.x - C::kWarps * 32; item < 8 * G; item += C::kProducerWarps * 32) {
-            const int g = item % G, oct = item / G;                      // tokens 8 oct .. 8 oct + 7 of the tile
-            const int64_t blk = j0 / kTokenBlock + (oct >> 1);
-            uint2 kw = make_uint2(0u, 0u), vw = make_uint2(0u, 0u);
-            if (blk < sh.n_blocks) {
-                kw = *reinterpret_cast<const uint2*>(kbase + blk * (G * kTokenBlock) + g * kTokenBlock + 8 * (oct & 1));
-                vw = *reinterpret_cast<const uint2*>(vbase + blk * (G * kTokenBlock) + g * kTokenBlock + 8 * (oct & 1));
-            }
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const uint32_t kcode = ((k < 4 ? kw.x : kw.y) >> (8 * (k & 3))) & 0xffu;
-                const uint32_t vcode = ((k < 4 ? vw.x : vw.y) >> (8 * (k & 3))) & 0xffu;
-                const int tok = 8 * oct + k;
-                const uint32_t dst = tile_off(tok, (g * kC) >> 3) + (uint32_t)((g * kC) & 7) * 2u;
-                if (kC == 8) {
-                    *reinterpret_cast<uint4*>(smem + C::kKtOffset + buf * C::kTileBytes + dst) = *reinterpret_cast<const uint4*>(smem + C::kKcbOffset + (kcode * G + g) * 16);
-                    *reinterpret_cast<uint4*>(smem + C::kVtOffset + buf * C::kTileBytes + dst) = *reinterpret_cast<const uint4*>(smem + C::kVcbOffset + (vcode * G + g) * 16);
-                } else if (kC == 4) {
-                    *reinterpret_cast<uint2*>(smem + C::kKtOffset + buf * C::kTileBytes + dst) = *reinterpret_cast<const uint2*>(smem + C::kKcbOffset + (kcode * G + g) * 8);
-                    *reinterpret_cast<uint2*>(smem + C::kVtOffset + buf * C::kTileBytes + dst) = *reinterpret_cast<const uint2*>(smem + C::kVcbOffset + (vcode * G + g) * 8);
-                } else {
-                    *reinterpret_cast<uint32_t*>(smem + C::kKtOffset + buf * C::kTileBytes + dst) = *reinterpret_cast<const uint32_t*>(smem + C::kKcbOffset + (g * 256 + kcode) * 4);
-                    *reinterpret_cast<uint32_t*>(smem + C::kVtOffset + buf * C::kTileBytes + dst) = *reinterpret_cast<const uint32_t*>(smem + C::kVcbOffset + (g * 256 + vcode) * 4);
+                for (int i = 0; i < 4; ++i) {
+                    const int off = (4 * (lane & 15) + (i ^ (lane >> 4))) * kTokenBlock + 8 * (lane >> 4);
+                    const uint2 a = *reinterpret_cast<const uint2*>(kp + off), b = *reinterpret_cast<const uint2*>(vp + off);
+                    kw[(2 * i) % kW] = a.x; kw[(2 * i + 1) % kW] = a.y; vw[(2 * i) % kW] = b.x; vw[(2 * i + 1) % kW] = b.y;
                 }
             }
-        }
-    };
-    // The same with work items of (8 tokens, one 16-byte chunk of the row = 8 channels = 8 / c groups): 128 items,
-    // one per producer thread, which gathers the chunk's centroids per token and stores the 16 bytes at once.
-    // Measured (4 x 2048 queries over 8192 tokens, 32 heads on 8 KV heads): c = 2 5.24 -> 3.91 ms, but c = 4 3.55 -> 3.66 and c = 8
-    // 3.32 -> 3.56 ms, so only c = 2 takes this form.
-    auto dequantise_chunks = [&](int64_t j0, int buf) {
-        constexpr int kGpi = 8 / kC;                                     // groups per item
-        const int item = threadIdx.x - C::kWarps * 32;
-        const int chunk = item & 15, oct = item >> 4;                    // tokens 8 oct .. 8 oct + 7 of the tile
-        const int64_t blk = j0 / kTokenBlock + (oct >> 1);
-        uint2 kw[kGpi], vw[kGpi];
+        };
+        auto fill = [&](const uint32_t (&w)[kW], int book, int tile_off) {
+            if (kC == 4) {
 #pragma unroll
-        for (int i = 0; i < kGpi; ++i) {
-            kw[i] = make_uint2(0u, 0u);
-            vw[i] = make_uint2(0u, 0u);
-            if (blk < sh.n_blocks) {
-                const int64_t off = blk * (G * kTokenBlock) + (chunk * kGpi + i) * kTokenBlock + 8 * (oct & 1);
-                kw[i] = *reinterpret_cast<const uint2*>(kbase + off);
-                vw[i] = *reinterpret_cast<const uint2*>(vbase + off);
-            }
-        }
+                for (int k = 0; k < 16; ++k) {
+                    const uint32_t code = (w[(k >> 2) % kW] >> (8 * (k & 3))) & 0xffu;
+                    const int tok = 16 * pw + k;
+                    const uint32_t dst = (uint32_t)((lane >> 4) * C::kHalfBytes + tok * 128 + ((((lane >> 1) & 7) ^ (k & 7)) << 4) + 8 * (lane & 1));
+                    *reinterpret_cast<uint2*>(smem + tile_off + dst) = *reinterpret_cast<const uint2*>(smem + book + (code * G + lane) * 8);
+                }
+            } else {
+                const int ch = lane & 15;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            uint32_t kv[4], vv[4];
+                for (int k = 0; k < 8; ++k) {
+                    const int tok = 16 * pw + 8 * (lane >> 4) + k;
+                    const uint32_t dst = (uint32_t)((ch >> 3) * C::kHalfBytes + tok * 128 + (((ch & 7) ^ k) << 4));
+                    uint4 v;
+                    if (kC == 8) {
+                        const uint32_t code = (w[(k >> 2) % kW] >> (8 * (k & 3))) & 0xffu;
+                        v = *reinterpret_cast<const uint4*>(smem + book + (code * G + ch) * 16);
+                    } else {
+                        // (the halves' gathers fall into different halves of the banks)
+                        const int hb = lane >> 4;
+                        uint32_t e[4];
 #pragma unroll
-            for (int i = 0; i < kGpi; ++i) {
-                const uint32_t kcode = ((k < 4 ? kw[i].x : kw[i].y) >> (8 * (k & 3))) & 0xffu;
-                const uint32_t vcode = ((k < 4 ? vw[i].x : vw[i].y) >> (8 * (k & 3))) & 0xffu;
-                // (the c = 2 placement of the codebooks; the other sizes do not take this form)
-                const uint32_t krow = (kcode * G + 16 * i + chunk) * 4;
-                const uint32_t vrow = (vcode * G + 16 * i + chunk) * 4;
-                if (kC == 8) {
-                    const uint4 a = *reinterpret_cast<const uint4*>(smem + C::kKcbOffset + krow);
-                    const uint4 b2 = *reinterpret_cast<const uint4*>(smem + C::kVcbOffset + vrow);
-                    kv[0] = a.x; kv[1] = a.y; kv[2] = a.z; kv[3] = a.w;
-                    vv[0] = b2.x; vv[1] = b2.y; vv[2] = b2.z; vv[3] = b2.w;
-                } else if (kC == 4) {
-                    const uint2 a = *reinterpret_cast<const uint2*>(smem + C::kKcbOffset + krow);
-                    const uint2 b2 = *reinterpret_cast<const uint2*>(smem + C::kVcbOffset + vrow);
-                    kv[(2 * i) & 3] = a.x; kv[(2 * i + 1) & 3] = a.y;
-                    vv[(2 * i) & 3] = b2.x; vv[(2 * i + 1) & 3] = b2.y;
-                } else {
-                    kv[i & 3] = *reinterpret_cast<const uint32_t*>(smem + C::kKcbOffset + krow);
-                    vv[i & 3] = *reinterpret_cast<const uint32_t*>(smem + C::kVcbOffset + vrow);
+                        for (int i = 0; i < 4; ++i) {
+                            const uint32_t code = (w[(2 * i + (k >> 2)) % kW] >> (8 * (k & 3))) & 0xffu;
+                            e[i] = *reinterpret_cast<const uint32_t*>(smem + book + (code * G + 16 * (i ^ hb) + ch) * 4);
+                        }
+                        v = hb ? make_uint4(e[1], e[0], e[3], e[2]) : make_uint4(e[0], e[1], e[2], e[3]);
+                    }
+                    *reinterpret_cast<uint4*>(smem + tile_off + dst) = v;
                 }
             }
-            const uint32_t dst = tile_off(8 * oct + k, chunk);
-            *reinterpret_cast<uint4*>(smem + C::kKtOffset + buf * C::kTileBytes + dst) = make_uint4(kv[0], kv[1], kv[2], kv[3]);
-            *reinterpret_cast<uint4*>(smem + C::kVtOffset + buf * C::kTileBytes + dst) = make_uint4(vv[0], vv[1], vv[2], vv[3]);
+        };
+        load_codes(0);
+        for (int jt = 0; jt < n_tiles; ++jt) {
+            const int stage = jt % C::kStages;
+            if (jt >= C::kStages && !pf_wait(ctl, &ctl->empty[stage], (uint32_t)(jt / C::kStages - 1) & 1u)) break;
+            fill(kw, C::kKcbOffset, C::kKtOffset + stage * C::kTileBytes);
+            fill(vw, C::kVcbOffset, C::kVtOffset + stage * C::kTileBytes);
+            load_codes(jt + 1);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) pf_arrive(&ctl->full[stage]);
         }
-    };
-    auto dequantise = [&](int64_t j0, int buf) {
-        if (kC == 2) dequantise_chunks(j0, buf);
-        else dequantise_groups(j0, buf);
-    };
-    // Producer warps fill the two tile buffers, the other warps multiply; named barriers 1 + buf ("buffer free") and
-    // 3 + buf ("buffer full") hand a buffer back and forth, registers move from the producers to the multipliers.
-    constexpr int kAll = C::kThreads;
-    if (warp >= C::kWarps) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
-        for (int64_t jt = 0; jt < n_tiles; ++jt) {
-            const int buf = (int)(jt & 1);
-            if (jt >= 2) asm volatile("bar.sync %0, %1;" ::"r"(1 + buf), "n"(kAll) : "memory");
-            dequantise(jt * C::kTile, buf);
-            __threadfence_block();
-            asm volatile("bar.arrive %0, %1;" ::"r"(3 + buf), "n"(kAll) : "memory");
-        }
-        return;
-    }
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 232;");
-    // the warp's query rows as A fragments, kept in registers for the whole context
-    uint32_t qf[8][4];
+    } else if (warp == C::kMmaWarp) {
+        // ---------------------------------------------------------------- one thread issues every MMA
+        if (lane == 0 && n_tiles > 0) {
+            // instruction descriptors: D fp32, A and B fp16, M = 128; scores: N = 64, sums: N = 128 with B's rows along N
+            constexpr uint32_t kScores = (1u << 4) | ((64u >> 3) << 17) | ((128u >> 4) << 24);
+            constexpr uint32_t kSums = (1u << 4) | (1u << 16) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
+            const uint32_t kt = smem_u32(smem + C::kKtOffset), vt = smem_u32(smem + C::kVtOffset);
+            auto scores = [&](int t, int jt) {
+                const uint32_t base = kt + (jt % C::kStages) * C::kTileBytes;
 #pragma unroll
-    for (int ks = 0; ks < 8; ++ks) {
-        const int mi = lane >> 3;
-        ldmatrix_x4(qf[ks], q_s + tile_off(warp * 16 + (lane & 7) + 8 * (mi & 1), 2 * ks + (mi >> 1)));
-    }
-
-    for (int64_t jt = 0; jt < n_tiles; ++jt) {
-        const int64_t j0 = jt * C::kTile;
-        const int buf = (int)(jt & 1);
-        asm volatile("bar.sync %0, %1;" ::"r"(3 + buf), "n"(kAll) : "memory");
-
-        // ---- S = Q Khat^T for the warp's 16 rows and the tile's 64 tokens
-        float sc[8][4];
+                for (int ks = 0; ks < 8; ++ks)           // 16 channels = 32 bytes of the 128-byte rows
+                    pf_mma(tmem + C::kSCol + 64 * t, tmem + C::kQCol + 64 * t + 8 * ks,
+                           pf_desc(base + (ks >> 2) * C::kHalfBytes + (ks & 3) * 32, 16), kScores, ks > 0 ? 1u : 0u);
+                pf_commit(&ctl->s_full[t]);
+            };
+            auto sums = [&](int t, int jt) {
+                const uint32_t base = vt + (jt % C::kStages) * C::kTileBytes;
 #pragma unroll
-        for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) sc[nt][j] = 0.f;
-#pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
-            const uint32_t (&a)[4] = qf[ks];
-#pragma unroll
-            for (int ntp = 0; ntp < 4; ++ntp) {
-                uint32_t b[4];
-                const int mi = lane >> 3;
-                ldmatrix_x4(b, kt_s + buf * C::kTileBytes + tile_off(16 * ntp + (lane & 7) + 8 * (mi >> 1), 2 * ks + (mi & 1)));
-                mma_f16(sc[2 * ntp], a, b[0], b[1]);
-                mma_f16(sc[2 * ntp + 1], a, b[2], b[3]);
+                for (int ks = 0; ks < 4; ++ks)           // 16 tokens = 2048 bytes
+                    pf_mma(tmem + C::kOCol + 128 * t, tmem + C::kSCol + 64 * t + 8 * ks, pf_desc(base + ks * 2048, C::kHalfBytes), kSums,
+                           (jt > 0 || ks > 0) ? 1u : 0u);
+            };
+            bool ok = pf_wait(ctl, &ctl->full[0], 0u);
+            for (int t = 0; ok && t < n_halves; ++t) {
+                ok = pf_wait(ctl, &ctl->p_full[t], 0u);  // the queries
+                if (!ok) break;
+                pf_fence_after();
+                scores(t, 0);
             }
-        }
-        // ---- running maximum and P.  A tile that lies wholly below every row's causal limit needs no mask: the
-        // maximum is taken over the raw scores and the scale folded into the exponent's multiply-add.
-        float corr[2];
-        uint32_t pa[4][4];                                               // P as A fragments: one per 16 tokens
-        if (j0 + C::kTile - 1 <= pos_warp && scale_log2e > 0.f) {
-            float mx[2] = {-INFINITY, -INFINITY};
-#pragma unroll
-            for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) mx[j >> 1] = fmaxf(mx[j >> 1], sc[nt][j]);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 1));
-                mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 2));
-                const float m_new = fmaxf(m_run[h], mx[h] * scale_log2e);      // finite: the tile has no masked score
-                corr[h] = exp2f(m_run[h] - m_new);
-                m_run[h] = m_new;
-                l_run[h] *= corr[h];
-            }
-#pragma unroll
-            for (int nt = 0; nt < 8; ++nt) {
-                float pv[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    pv[j] = ex2_approx(fmaf(sc[nt][j], scale_log2e, -m_run[j >> 1]));
-                    l_run[j >> 1] += pv[j];
+            for (int jt = 0; ok && jt < n_tiles; ++jt) {
+                for (int t = 0; t < n_halves; ++t) {
+                    ok = pf_wait(ctl, &ctl->p_full[t], (uint32_t)(jt + 1) & 1u);
+                    if (!ok) break;
+                    pf_fence_after();
+                    sums(t, jt);
+                    if (t == n_halves - 1) pf_commit(&ctl->empty[jt % C::kStages]);
+                    if (jt + 1 < n_tiles) {
+                        if (t == 0) ok = pf_wait(ctl, &ctl->full[(jt + 1) % C::kStages], (uint32_t)((jt + 1) / C::kStages) & 1u);
+                        if (!ok) break;
+                        pf_fence_after();
+                        scores(t, jt + 1);
+                    }
                 }
-                pa[nt >> 1][(nt & 1) * 2 + 0] = pack_half2(pv[0], pv[1]);
-                pa[nt >> 1][(nt & 1) * 2 + 1] = pack_half2(pv[2], pv[3]);
             }
-        } else {
-            float mx[2] = {-INFINITY, -INFINITY};
-#pragma unroll
-            for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int64_t tok = j0 + 8 * nt + 2 * p + (j & 1);
-                    const int64_t pos = (j < 2) ? pos_a : pos_b;
-                    const float v = tok <= pos ? sc[nt][j] * scale_log2e : -INFINITY;
-                    sc[nt][j] = v;
-                    mx[j >> 1] = fmaxf(mx[j >> 1], v);
-                }
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 1));
-                mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 2));
-                const float m_new = fmaxf(m_run[h], mx[h]);
-                corr[h] = m_new == -INFINITY ? 1.f : exp2f(m_run[h] - m_new);
-                m_run[h] = m_new;
-                l_run[h] *= corr[h];
-            }
-#pragma unroll
-            for (int nt = 0; nt < 8; ++nt) {
-                float pv[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float mrow = m_run[j >> 1];
-                    pv[j] = mrow == -INFINITY ? 0.f : exp2f(sc[nt][j] - mrow);
-                    l_run[j >> 1] += pv[j];
-                }
-                pa[nt >> 1][(nt & 1) * 2 + 0] = pack_half2(pv[0], pv[1]);
-                pa[nt >> 1][(nt & 1) * 2 + 1] = pack_half2(pv[2], pv[3]);
-            }
+            pf_commit(&ctl->o_full);
         }
-        if (__any_sync(0xffffffffu, corr[0] != 1.f || corr[1] != 1.f)) {   // most tiles leave every maximum as it was
-#pragma unroll
-            for (int nt = 0; nt < 16; ++nt) {
-                o[nt][0] *= corr[0];
-                o[nt][1] *= corr[0];
-                o[nt][2] *= corr[1];
-                o[nt][3] *= corr[1];
-            }
-        }
-        // ---- O += P Vhat
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks)
-#pragma unroll
-            for (int ntp = 0; ntp < 8; ++ntp) {
-                uint32_t b[4];
-                const int mi = lane >> 3;
-                ldmatrix_x4_trans(b, vt_s + buf * C::kTileBytes + tile_off(16 * ks + (lane & 7) + 8 * (mi & 1), 2 * ntp + (mi >> 1)));
-                mma_f16(o[2 * ntp], pa[ks], b[0], b[1]);
-                mma_f16(o[2 * ntp + 1], pa[ks], b[2], b[3]);
-            }
-        if (jt + 2 < n_tiles) asm volatile("bar.arrive %0, %1;" ::"r"(1 + buf), "n"(kAll) : "memory");   // the buffer is free again
-    }
-
-    // ---- normalise and write (l is spread over the quad)
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], 1);
-        l_run[h] += __shfl_xor_sync(0xffffffffu, l_run[h], 2);
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int rho = h == 0 ? rho_a : rho_b;
+    } else if (warp < 4 * n_halves) {
+        // ---------------------------------------------------------------- softmax: a thread per row
+        const int t = warp >> 2, rho = threadIdx.x;
+        const uint32_t lanes = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        const uint32_t s_addr = lanes + C::kSCol + 64 * t, o_addr = lanes + C::kOCol + 128 * t;
         const int qi = qi0 + rho / R;
-        if (qi >= n_q) continue;
-        const float inv = l_run[h] > 0.f ? 1.f / l_run[h] : 0.f;        // no position: zero row
-        float* orow = out + ((s * n_q + qi) * sh.n_q_heads + hkv * R + rho % R) * 128;
+        const bool live = qi < n_q;
+        const int64_t row = (s * n_q + qi) * sh.n_q_heads + hkv * R + rho % R;
+        const int64_t pos = live ? pos0 + rho / R : -1;
+        const int64_t pos_warp = pos0 + (warp * 32) / R;                   // smallest position among the warp's rows
+        {
+            uint32_t u[32];
 #pragma unroll
-        for (int nt = 0; nt < 16; ++nt)
-            *reinterpret_cast<float2*>(orow + 8 * nt + 2 * p) = make_float2(o[nt][2 * h] * inv, o[nt][2 * h + 1] * inv);
+            for (int half = 0; half < 2; ++half) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                    if (live) v = *reinterpret_cast<const uint4*>(q + row * 128 + half * 64 + i * 8);
+                    u[4 * i] = (v.x ^ q_sign) & q_keep; u[4 * i + 1] = (v.y ^ q_sign) & q_keep;
+                    u[4 * i + 2] = (v.z ^ q_sign) & q_keep; u[4 * i + 3] = (v.w ^ q_sign) & q_keep;
+                }
+                pf_st32(lanes + C::kQCol + 64 * t + 32 * half, u);
+            }
+            pf_st_wait();
+            pf_fence_before();
+            __syncwarp();
+            if (lane == 0) pf_arrive(&ctl->p_full[t]);
+        }
+        float m = -INFINITY, l = 0.f;                                       // reference of the weights (log2 domain), their sum
+        bool ok = true;
+        for (int jt = 0; jt < n_tiles; ++jt) {
+            if (!pf_wait(ctl, &ctl->s_full[t], (uint32_t)jt & 1u)) { ok = false; break; }
+            pf_fence_after();
+            uint32_t a[32], b[32];
+            pf_ld32(a, s_addr);
+            pf_ld32(b, s_addr + 32);
+            pf_ld_wait(a);
+            pf_ld_wait(b);
+            float* sa = reinterpret_cast<float*>(a);
+            float* sb = reinterpret_cast<float*>(b);
+            const int64_t j0 = (int64_t)jt * C::kTile;
+            if (j0 + C::kTile - 1 > pos_warp) {                             // some row's causal limit lies in the tile
+                const int64_t left = pos - j0;                              // columns 0 ... left are attended
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    if (i > left) sa[i] = -INFINITY;
+                    if (i + 32 > left) sb[i] = -INFINITY;
+                }
+            }
+            float mx[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) mx[i] = max3(sa[i], sb[i], sa[i + 4]);
+#pragma unroll
+            for (int i = 8; i < 32; i += 8)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) mx[k] = max3(mx[k], sa[i + k], sa[i + 4 + k]);
+#pragma unroll
+            for (int i = 4; i < 28; i += 8)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) mx[k] = max3(mx[k], sb[i + k], sb[i + 4 + k]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) mx[k] = fmaxf(mx[k], sb[28 + k]);
+            const float top = max3(fmaxf(mx[0], mx[1]), mx[2], mx[3]);
+            const float m_tile = top * scale;                               // (-inf: the row attends nothing of the tile)
+            // The weights' reference follows the maximum only when it is more than 8 (a factor of 256) behind: the sums
+            // rarely have to be rescaled, and fp16 weights up to 256 are as precise as weights up to 1.
+            const bool move = m_tile > m + 8.f || (m == -INFINITY && m_tile > -INFINITY);
+            if (__any_sync(0xffffffffu, move)) {
+                const float m_new = fmaxf(m, m_tile);
+                const float f = m == -INFINITY ? 0.f : exp2f(m - m_new);
+                m = m_new;
+                l *= f;
+                if (jt > 0) {                                               // (the sums so far are done: the scores came after them)
+#pragma unroll 1
+                    for (int c0 = 0; c0 < 128; c0 += 32) {
+                        uint32_t o[32];
+                        pf_ld32(o, o_addr + c0);
+                        pf_ld_wait(o);
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f);
+                        pf_st32(o_addr + c0, o);
+                    }
+                }
+            }
+            const float mm = m == -INFINITY ? 0.f : m;
+            uint32_t p[32];
+            float l0 = 0.f, l1 = 0.f;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const float x0 = ex2_approx(fmaf(sa[2 * i], scale, -mm)), x1 = ex2_approx(fmaf(sa[2 * i + 1], scale, -mm));
+                l0 += x0;
+                l1 += x1;
+                p[i] = pack_half2(x0, x1);
+            }
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const float x0 = ex2_approx(fmaf(sb[2 * i], scale, -mm)), x1 = ex2_approx(fmaf(sb[2 * i + 1], scale, -mm));
+                l0 += x0;
+                l1 += x1;
+                p[16 + i] = pack_half2(x0, x1);
+            }
+            l += l0 + l1;
+            pf_st32(s_addr, p);
+            pf_st_wait();
+            pf_fence_before();
+            __syncwarp();
+            if (lane == 0) pf_arrive(&ctl->p_full[t]);
+        }
+        // ---- normalise and write
+        if (n_tiles > 0) ok = ok && pf_wait(ctl, &ctl->o_full, 0u);
+        pf_fence_after();
+        const float inv = ok && l > 0.f ? 1.f / l : 0.f;                    // no position: zero row
+#pragma unroll 1
+        for (int c0 = 0; c0 < 128; c0 += 32) {
+            uint32_t o[32];
+            if (n_tiles > 0) {
+                pf_ld32(o, o_addr + c0);
+                pf_ld_wait(o);
+            }
+            if (live) {
+                float4* dst = reinterpret_cast<float4*>(out + row * 128 + c0);
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    dst[i] = inv == 0.f ? make_float4(0.f, 0.f, 0.f, 0.f)
+                                        : make_float4(__uint_as_float(o[4 * i]) * inv, __uint_as_float(o[4 * i + 1]) * inv,
+                                                      __uint_as_float(o[4 * i + 2]) * inv, __uint_as_float(o[4 * i + 3]) * inv);
+            }
+        }
+        pf_fence_before();
+    }
+    // every MMA that was issued has been waited for (or a wait gave up); hand the tensor memory back
+    __syncthreads();
+    if (warp == C::kMmaWarp) {
+        pf_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
     }
 }
 
@@ -484,19 +573,19 @@ cudaError_t launch_prefill(const __half* q, const uint8_t* kc, const uint8_t* vc
         cudaError_t e = cudaSuccess;
         switch (sh.c) {
             case 8:
-                e = ensure_dynamic_smem(reinterpret_cast<const void*>(prefill_mma_kernel<8>), C::kSmemBytes, 40);
+                e = ensure_dynamic_smem(reinterpret_cast<const void*>(prefill_tc_kernel<8>), C::kSmemBytes, 40);
                 if (e != cudaSuccess) return e;
-                prefill_mma_kernel<8><<<(unsigned)grid, C::kThreads, C::kSmemBytes, st>>>(q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, n_q, row_tiles, out);
+                prefill_tc_kernel<8><<<(unsigned)grid, C::kThreads, C::kSmemBytes, st>>>(q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, n_q, row_tiles, out);
                 break;
             case 4:
-                e = ensure_dynamic_smem(reinterpret_cast<const void*>(prefill_mma_kernel<4>), C::kSmemBytes, 41);
+                e = ensure_dynamic_smem(reinterpret_cast<const void*>(prefill_tc_kernel<4>), C::kSmemBytes, 41);
                 if (e != cudaSuccess) return e;
-                prefill_mma_kernel<4><<<(unsigned)grid, C::kThreads, C::kSmemBytes, st>>>(q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, n_q, row_tiles, out);
+                prefill_tc_kernel<4><<<(unsigned)grid, C::kThreads, C::kSmemBytes, st>>>(q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, n_q, row_tiles, out);
                 break;
             default:
-                e = ensure_dynamic_smem(reinterpret_cast<const void*>(prefill_mma_kernel<2>), C::kSmemBytes, 42);
+                e = ensure_dynamic_smem(reinterpret_cast<const void*>(prefill_tc_kernel<2>), C::kSmemBytes, 42);
                 if (e != cudaSuccess) return e;
-                prefill_mma_kernel<2><<<(unsigned)grid, C::kThreads, C::kSmemBytes, st>>>(q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, n_q, row_tiles, out);
+                prefill_tc_kernel<2><<<(unsigned)grid, C::kThreads, C::kSmemBytes, st>>>(q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, n_q, row_tiles, out);
                 break;
         }
         return cudaGetLastError();
