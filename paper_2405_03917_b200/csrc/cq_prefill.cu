@@ -8,18 +8,22 @@
 // With many queries per cached token the per-query lookup tables of the decode kernels no longer
 // pay (one table per query); the codes are turned back into vectors instead and the two
 // contractions run on the tensor cores:
-//   prefill_mma_kernel (head_dim 128, one byte per code, c = 2, 4 or 8): one CTA per (sequence,
-//     KV head, tile of 128 (query, head of the KV head's group) rows).  Both codebooks are kept
-//     in shared memory as fp16, code-major, so that the lanes of a gather (one group each) meet
-//     in no bank whatever the codes are; per tile of 64 cached tokens the K and V codes are gathered into
-//     fp16 tiles, S = Q Khat^T and O += P Vhat are m16n8k16 MMAs with fp32 accumulators, and the
-//     softmax is the usual running-maximum form in the log2 domain.  Four producer warps do the
-//     gathering into two tile buffers while eight warps (16 rows each) multiply; named barriers
-//     hand a buffer back and forth, and the producers give most of their registers to the others.
-//     The multiplying warps hold their query fragments in registers; a tile wholly below the
-//     causal limit of a warp's rows skips the mask and folds the scale into the exponent.
+//   prefill_tc_kernel (head_dim 128, one byte per code, c = 2, 4 or 8): one CTA per (sequence, KV
+//     head, 256 (query, head of the KV head's group) rows), as two row tiles of 128, one row per lane
+//     of tensor memory.  Both codebooks are kept in shared memory as fp16, code-major, so that the
+//     lanes of a gather (one group each) meet in no bank whatever the codes are.  Four producer warps
+//     gather the codes of 64 cached tokens into swizzled fp16 tiles (three stages); S = Q Khat^T and
+//     O += P Vhat are tcgen05 MMAs with fp32 accumulators, Q and P read from tensor memory, issued by
+//     a warp each; eight softmax warps take a row per thread (running maximum, log2 domain).
+//     What bounds it: per 64 tokens and 256 rows the MMAs take 1024 cycles and the exponentials 1024
+//     (two per clock and SM quarter); each waits for the other in turn through the two row tiles.
+//     4 x 2048 queries over 8192 tokens, 32 heads on 8, CQ-8c8b: 3.20 ms with m16n8k16 MMAs and the
+//     tiles' fragments in registers, 1.36 ms with one MMA-issuing thread that did scores and sums in
+//     turn, 0.98 ms now, 0.57 ms being the contractions at the measured GEMM rate.
 //   prefill_generic_kernel: any supported shape, one CTA per (sequence, query, head), plain loops.
 #include "cq_common.cuh"
+
+#include <type_traits>
 
 namespace cq {
 
@@ -107,7 +111,8 @@ struct PfCfg {
     static constexpr int kRows = 256;             // (query, head) rows per CTA: two tiles of 128, one tensor-memory lane each
     static constexpr int kMmaWarp = 8;            // one thread issues the MMAs; the warps before it: softmax, four per row tile, a thread per row
     static constexpr int kProducerWarp0 = 9, kProducerWarps = 4;       // dequantise the tiles
-    static constexpr int kThreads = (kProducerWarp0 + kProducerWarps) * 32;
+    static constexpr int kSumWarp = kProducerWarp0 + kProducerWarps;
+    static constexpr int kThreads = (kSumWarp + 1) * 32;
     static constexpr int kTile = 64;              // cached tokens per step
     static constexpr int kStages = 3;
     static constexpr int kCbBytes = 128 * 256 * 2;                     // one codebook as fp16, code-major
@@ -118,9 +123,13 @@ struct PfCfg {
     static constexpr int kKtOffset = kVtOffset + kStages * kTileBytes; // [stages]
     static constexpr int kCtlOffset = kKtOffset + kStages * kTileBytes;
     static constexpr int kSmemBytes = kCtlOffset + 256;                // 224.25 KiB
-    // tensor-memory columns: output accumulators (fp32), queries (fp16, two per column), scores (fp32) with the weights
-    // (fp16) in their place
-    static constexpr int kOCol = 0, kQCol = 256, kSCol = 384;
+    // tensor-memory columns: output accumulators (fp32) and queries (fp16, two per column) of both row tiles, ONE tile of
+    // scores (fp32) that the row tiles use in turn, weights (fp16) of both row tiles
+    static constexpr int kOCol = 0, kQCol = 256, kSCol = 384, kPCol = 448;
+    // where the set-up leaves the queries: behind stage 0, which the producers fill while they are read
+    static constexpr int kOutStride = 144;        // bytes between the rows of a warp's 32 x 32 block of results (in the codebooks' place)
+    __host__ __device__ static constexpr int q_offset(int rho) { return (rho < 128 ? kVtOffset : kKtOffset) + kTileBytes + (rho & 127) * 256; }
+    static_assert(kStages >= 3 && 8 * 32 * kOutStride <= 2 * kCbBytes, "room");
     static_assert(kKtOffset % 1024 == 0 && kTileBytes % 1024 == 0, "swizzled tiles");
     static_assert(kSmemBytes <= 227 * 1024, "shared memory");
 };
@@ -128,9 +137,11 @@ struct PfCfg {
 struct PfCtl {
     uint64_t full[PfCfg::kStages];        // K and V tile of the stage are written (one arrival per producer warp)
     uint64_t empty[PfCfg::kStages];       // the MMAs that read the stage are done
-    uint64_t s_full[2];                   // scores of the row tile are in tensor memory (and the sums before them are done)
-    uint64_t p_full[2];                   // its weights are (one arrival per warp); also: its queries are, before the first tile
-    uint64_t o_full;                      // all sums are done
+    uint64_t s_full[2];                   // scores of the row tile are in tensor memory
+    uint64_t s_free[2];                   // they have been read (one arrival per warp): their columns take the other row tile's
+    uint64_t q_full[2];                   // queries of the row tile are in tensor memory (one arrival per warp)
+    uint64_t p_full[2];                   // its weights are (one arrival per warp)
+    uint64_t pv_done[2];                  // the sums with those weights are done
     uint32_t tmem_base;
     int failed;                           // a wait gave up
 };
@@ -182,23 +193,24 @@ __device__ __forceinline__ bool pf_wait(PfCtl* ctl, uint64_t* bar, uint32_t pari
 
 // Shared-memory matrix descriptor of a tile of 128-byte rows with the 128-byte swizzle (16-byte chunk index XOR row mod 8).
 // Rows = tokens.  As keys (contraction along the row) eight rows are one core matrix group of 1024 bytes; as values (the
-// row is the N dimension) the next 64 channels are kHalfBytes on and the next eight tokens 1024 bytes.
-__device__ __forceinline__ uint64_t pf_desc(uint32_t saddr, uint32_t leading_bytes)
-{
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr >> 4) & 0x3fffu);
-    d |= (uint64_t)((leading_bytes >> 4) & 0x3fffu) << 16;
-    d |= (uint64_t)((1024u >> 4) & 0x3fffu) << 32;
-    d |= (uint64_t)1 << 46;                      // descriptor version of sm_100
-    d |= (uint64_t)2 << 61;                      // 128-byte swizzle
-    return d;
-}
+// row is the N dimension) the next 64 channels are kHalfBytes on and the next eight tokens 1024 bytes.  Low word: start
+// address and leading offset in 16-byte units; high word: stride offset, descriptor version of sm_100, swizzle.
+__device__ __forceinline__ uint32_t pf_desc_lo(uint32_t saddr, uint32_t leading_bytes) { return (saddr >> 4) | ((leading_bytes >> 4) << 16); }
+constexpr uint32_t kPfDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
 // D[128 x N] (+)= A[128 x 16] * B, A (fp16) from tensor memory, B (fp16) from shared memory, fp32 accumulator
-__device__ __forceinline__ void pf_mma(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
+__device__ __forceinline__ void pf_mma(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t idesc, bool accumulate)
 {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, {%5, %5, %5, %5}, p;\n\t}"
-                 ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(0) : "memory");
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 d;\n\tsetp.ne.b32 p, %5, 0;\n\tmov.b64 d, {%2, %3};\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], d, %4, p;\n\t}"
+                 ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(kPfDescHi), "r"(idesc), "r"(accumulate ? 1u : 0u) : "memory");
+}
+// One lane of the warp, the same one every time.  (A branch on this, unlike one on the lane number, lets the compiler keep
+// the operands of the MMAs in uniform registers: an issue costs some ten cycles instead of seventy.)
+__device__ __forceinline__ bool pf_elect()
+{
+    uint32_t is;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(is));
+    return is != 0;
 }
 __device__ __forceinline__ void pf_commit(uint64_t* bar)
 {
@@ -264,9 +276,11 @@ prefill_tc_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, 
         }
         for (int t = 0; t < 2; ++t) {
             pf_init(&ctl->s_full[t], 1);
+            pf_init(&ctl->s_free[t], 4);
+            pf_init(&ctl->q_full[t], 4);
             pf_init(&ctl->p_full[t], 4);
+            pf_init(&ctl->pv_done[t], 1);
         }
-        pf_init(&ctl->o_full, 1);
         ctl->failed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -274,23 +288,55 @@ prefill_tc_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, 
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&ctl->tmem_base)) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    // ---- queries, coalesced, into the tile buffers of stages 1 and 2 (row tile 0: the values', 1: the keys'); 16-byte chunk
+    // i of row rho goes to chunk i XOR (rho mod 8) of its 256 bytes, so that a thread per row can read them without conflicts
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n_halves * 128 * 16; i += C::kThreads) {
+        const int rho = i >> 4, qi = qi0 + rho / R;
+        uint4 x = make_uint4(0u, 0u, 0u, 0u);
+        if (qi < n_q) x = reinterpret_cast<const uint4*>(q + ((s * n_q + qi) * sh.n_q_heads + hkv * R + rho % R) * 128)[i & 15];
+        *reinterpret_cast<uint4*>(smem + C::q_offset(rho) + (((i & 15) ^ (rho & 7)) << 4)) = x;
+    }
     // ---- codebooks as fp16, code-major ([code][group][channel]): the lanes of a gather take different groups, so they
     // meet in no bank whatever the codes are.  For c = 2 (one word per centroid) group g sits in column
-    // 16 (g mod 4) + g / 4.
-    for (int i = threadIdx.x; i < 128 * 256 / 2; i += C::kThreads) {
-        const float2 a = *reinterpret_cast<const float2*>(kcb + (int64_t)hkv * 128 * 256 + 2 * i);
-        const float2 b = *reinterpret_cast<const float2*>(vcb + (int64_t)hkv * 128 * 256 + 2 * i);
-        const int g = (2 * i) / (256 * kC), code = ((2 * i) / kC) % 256, ch = (2 * i) % kC;
-        const int w = kC == 2 ? code * G + 16 * (g & 3) + (g >> 2) : ((code * G + g) * kC + ch) / 2;
-        *reinterpret_cast<uint32_t*>(smem + C::kKcbOffset + 4 * w) = pack_half2(a.x, a.y);
-        *reinterpret_cast<uint32_t*>(smem + C::kVcbOffset + 4 * w) = pack_half2(b.x, b.y);
+    // 16 (g mod 4) + g / 4.  A warp takes 64 bytes of eight groups at a time: eight lines of memory per load, and at most
+    // 1, 2 or 4 lanes (c = 8, 4, 2) that meet in a bank of a store.  (Straight copies, whose stores met eight at a time,
+    // took 12.7 thousand cycles per CTA; 4 thousand are what the L2 takes to deliver 256 KB.)
+    {
+        constexpr int kTasks = 2 * 256, kBatch = 6, kWarps = C::kThreads / 32;
+        const int gl = kC == 8 ? (lane >> 1) & 7 : lane & 7, j = kC == 8 ? (lane >> 4) * 2 + (lane & 1) : lane >> 3;
+#pragma unroll 1
+        for (int i0 = warp; i0 < kTasks; i0 += kBatch * kWarps) {
+            float4 x[kBatch];
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) {
+                const int i = i0 + u * kWarps, o = (i & 255) % (G / 8), seg = (i & 255) / (G / 8);
+                const int g = kC == 2 ? 4 * (8 * (o >> 2) + gl) + (o & 3) : 8 * o + gl;
+                if (i < kTasks)
+                    x[u] = reinterpret_cast<const float4*>((i < 256 ? kcb : vcb) + (int64_t)hkv * 128 * 256)[(g * 16 * kC + seg) * 4 + j];
+            }
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) {
+                const int i = i0 + u * kWarps, o = (i & 255) % (G / 8), seg = (i & 255) / (G / 8);
+                if (i >= kTasks) break;
+                uint8_t* book = smem + (i < 256 ? C::kKcbOffset : C::kVcbOffset);
+                const uint32_t lo = pack_half2(x[u].x, x[u].y), hi = pack_half2(x[u].z, x[u].w);
+                if (kC == 8) *reinterpret_cast<uint2*>(book + (seg * 2 + (j >> 1)) * 256 + (8 * o + gl) * 16 + (j & 1) * 8) = make_uint2(lo, hi);
+                if (kC == 4) *reinterpret_cast<uint2*>(book + (seg * 4 + j) * 256 + (8 * o + gl) * 8) = make_uint2(lo, hi);
+                if (kC == 2) {
+                    uint8_t* dst = book + (seg * 8 + 2 * j) * 256 + (16 * (o & 3) + 8 * (o >> 2) + gl) * 4;
+                    *reinterpret_cast<uint32_t*>(dst) = lo;
+                    *reinterpret_cast<uint32_t*>(dst + 256) = hi;
+                }
+            }
+        }
     }
     pf_fence_before();
     __syncthreads();
     pf_fence_after();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&ctl->tmem_base);
 
-    if (warp >= C::kProducerWarp0) {
+    if (warp >= C::kProducerWarp0 && warp < C::kSumWarp) {
         // ---------------------------------------------------------------- producers: codes -> fp16 tiles of 64 tokens
         // A warp takes one 16-token block of the tile.  16-byte chunk `ch` (channels 8 ch ... + 7) of token t goes to byte
         // (ch / 8) * kHalfBytes + t * 128 + ((ch % 8) ^ (t % 8)) * 16: eight lanes of a store hold the chunks of one token,
@@ -299,8 +345,8 @@ prefill_tc_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, 
         const uint8_t* kbase = kc + code_word_offset(sh, sh.n_kv_heads, s, hkv, 0, 0);
         const uint8_t* vbase = vc + code_word_offset(sh, sh.n_kv_heads, s, hkv, 0, 0);
         constexpr int kW = kC == 8 ? 2 : kC == 4 ? 4 : 8;                   // code words a lane takes of a block, per tensor
-        uint32_t kw[kW], vw[kW];
-        auto load_codes = [&](int jt) {
+        uint32_t kw[kW], vw[kW], kn[kW], vn[kW];        // this tile's and the next one's, loaded a whole tile ahead of their use
+        auto load_codes = [&](int jt, uint32_t (&kw)[kW], uint32_t (&vw)[kW]) {
             const int64_t blk = (int64_t)jt * (C::kTile / kTokenBlock) + pw;
 #pragma unroll
             for (int i = 0; i < kW; ++i) kw[i] = vw[i] = 0u;
@@ -358,71 +404,96 @@ prefill_tc_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, 
                 }
             }
         };
-        load_codes(0);
+        load_codes(0, kn, vn);
         for (int jt = 0; jt < n_tiles; ++jt) {
             const int stage = jt % C::kStages;
-            if (jt >= C::kStages && !pf_wait(ctl, &ctl->empty[stage], (uint32_t)(jt / C::kStages - 1) & 1u)) break;
+#pragma unroll
+            for (int i = 0; i < kW; ++i) { kw[i] = kn[i]; vw[i] = vn[i]; }
+            load_codes(jt + 1, kn, vn);
+            bool ok = jt < C::kStages || pf_wait(ctl, &ctl->empty[stage], (uint32_t)(jt / C::kStages - 1) & 1u);
+            if (jt == 1) ok = ok && pf_wait(ctl, &ctl->q_full[lane % n_halves], 0u);      // the queries lay there
+            if (!__all_sync(0xffffffffu, ok)) break;
             fill(kw, C::kKcbOffset, C::kKtOffset + stage * C::kTileBytes);
             fill(vw, C::kVcbOffset, C::kVtOffset + stage * C::kTileBytes);
-            load_codes(jt + 1);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0) pf_arrive(&ctl->full[stage]);
         }
     } else if (warp == C::kMmaWarp) {
-        // ---------------------------------------------------------------- one thread issues every MMA
-        if (lane == 0 && n_tiles > 0) {
-            // instruction descriptors: D fp32, A and B fp16, M = 128; scores: N = 64, sums: N = 128 with B's rows along N
-            constexpr uint32_t kScores = (1u << 4) | ((64u >> 3) << 17) | ((128u >> 4) << 24);
-            constexpr uint32_t kSums = (1u << 4) | (1u << 16) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
-            const uint32_t kt = smem_u32(smem + C::kKtOffset), vt = smem_u32(smem + C::kVtOffset);
-            auto scores = [&](int t, int jt) {
-                const uint32_t base = kt + (jt % C::kStages) * C::kTileBytes;
+        // ---------------------------------------------------------------- scores: Q Khat^T of (tile, row tile) 0, 1, 2, ...
+        // (All lanes of the warp go round the loop, a turn of which goes once round the stages, and different lanes wait for
+        // different barriers: with everything in a one-thread branch an MMA took some 60 cycles to issue and a wait, behind
+        // the exponentials in the queue that it shares with them, 200.)
+        constexpr uint32_t kScores = (1u << 4) | ((64u >> 3) << 17) | ((128u >> 4) << 24);       // D fp32, A and B fp16, M = 128, N = 64
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0), kdesc = pf_desc_lo(smem_u32(smem + C::kKtOffset), 16);
+        const int n_work = __shfl_sync(0xffffffffu, n_tiles * n_halves, 0);
+        auto go = [&](auto halves_in_use) {
+            constexpr int kHalves = decltype(halves_in_use)::value, kTurn = kHalves * C::kStages;
+            if (!__all_sync(0xffffffffu, pf_wait(ctl, &ctl->q_full[lane % kHalves], 0u))) return;                // the queries
+            for (int o = 0; o * kTurn < n_work; ++o) {
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks)           // 16 channels = 32 bytes of the 128-byte rows
-                    pf_mma(tmem + C::kSCol + 64 * t, tmem + C::kQCol + 64 * t + 8 * ks,
-                           pf_desc(base + (ks >> 2) * C::kHalfBytes + (ks & 3) * 32, 16), kScores, ks > 0 ? 1u : 0u);
-                pf_commit(&ctl->s_full[t]);
-            };
-            auto sums = [&](int t, int jt) {
-                const uint32_t base = vt + (jt % C::kStages) * C::kTileBytes;
-#pragma unroll
-                for (int ks = 0; ks < 4; ++ks)           // 16 tokens = 2048 bytes
-                    pf_mma(tmem + C::kOCol + 128 * t, tmem + C::kSCol + 64 * t + 8 * ks, pf_desc(base + ks * 2048, C::kHalfBytes), kSums,
-                           (jt > 0 || ks > 0) ? 1u : 0u);
-            };
-            bool ok = pf_wait(ctl, &ctl->full[0], 0u);
-            for (int t = 0; ok && t < n_halves; ++t) {
-                ok = pf_wait(ctl, &ctl->p_full[t], 0u);  // the queries
-                if (!ok) break;
-                pf_fence_after();
-                scores(t, 0);
-            }
-            for (int jt = 0; ok && jt < n_tiles; ++jt) {
-                for (int t = 0; t < n_halves; ++t) {
-                    ok = pf_wait(ctl, &ctl->p_full[t], (uint32_t)(jt + 1) & 1u);
-                    if (!ok) break;
+                for (int u = 0; u < kTurn; ++u) {
+                    if (o * kTurn + u >= n_work) break;
+                    const int t = u % kHalves, stage = u / kHalves, jt = o * C::kStages + stage;
+                    // even lanes: the scores of the work before have been read; odd lanes: the tile is there
+                    const bool first = o == 0 && u == 0;
+                    uint64_t* bar = (lane & 1) || first ? &ctl->full[stage] : &ctl->s_free[t == 0 ? kHalves - 1 : 0];
+                    const uint32_t parity = (lane & 1) || first ? (uint32_t)o & 1u : (uint32_t)(t == 0 ? jt - 1 : jt) & 1u;
+                    if (!__all_sync(0xffffffffu, pf_wait(ctl, bar, parity))) return;
                     pf_fence_after();
-                    sums(t, jt);
-                    if (t == n_halves - 1) pf_commit(&ctl->empty[jt % C::kStages]);
-                    if (jt + 1 < n_tiles) {
-                        if (t == 0) ok = pf_wait(ctl, &ctl->full[(jt + 1) % C::kStages], (uint32_t)((jt + 1) / C::kStages) & 1u);
-                        if (!ok) break;
-                        pf_fence_after();
-                        scores(t, jt + 1);
+                    if (pf_elect()) {
+#pragma unroll
+                        for (int ks = 0; ks < 8; ++ks)               // 16 channels = 32 bytes of the 128-byte rows
+                            pf_mma(tm + C::kSCol, tm + C::kQCol + 64 * t + 8 * ks,
+                                   kdesc + (stage * C::kTileBytes + (ks >> 2) * C::kHalfBytes + (ks & 3) * 32) / 16, kScores, ks > 0);
+                        pf_commit(&ctl->s_full[t]);
                     }
                 }
             }
-            pf_commit(&ctl->o_full);
+        };
+        if (n_work > 0) {
+            if (n_halves == 2) go(std::integral_constant<int, 2>());
+            else go(std::integral_constant<int, 1>());
+        }
+    } else if (warp == C::kSumWarp) {
+        // ---------------------------------------------------------------- sums: P Vhat, in the same order
+        constexpr uint32_t kSums = (1u << 4) | (1u << 16) | ((128u >> 3) << 17) | ((128u >> 4) << 24);   // N = 128, B's rows along N
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0), vdesc = pf_desc_lo(smem_u32(smem + C::kVtOffset), C::kHalfBytes);
+        const int n_work = __shfl_sync(0xffffffffu, n_tiles * n_halves, 0);
+        auto go = [&](auto halves_in_use) {
+            constexpr int kHalves = decltype(halves_in_use)::value, kTurn = kHalves * C::kStages;
+            for (int o = 0; o * kTurn < n_work; ++o) {
+#pragma unroll
+                for (int u = 0; u < kTurn; ++u) {
+                    if (o * kTurn + u >= n_work) break;
+                    const int t = u % kHalves, stage = u / kHalves, jt = o * C::kStages + stage;
+                    uint64_t* bar = lane & 1 ? &ctl->full[stage] : &ctl->p_full[t];
+                    const uint32_t parity = lane & 1 ? (uint32_t)o & 1u : (uint32_t)jt & 1u;
+                    if (!__all_sync(0xffffffffu, pf_wait(ctl, bar, parity))) return;
+                    pf_fence_after();
+                    const bool more = jt > 0;
+                    if (pf_elect()) {
+#pragma unroll
+                        for (int ks = 0; ks < 4; ++ks)               // 16 tokens = 2048 bytes
+                            pf_mma(tm + C::kOCol + 128 * t, tm + C::kPCol + 32 * t + 8 * ks,
+                                   vdesc + (stage * C::kTileBytes + ks * 2048) / 16, kSums, more || ks > 0);
+                        pf_commit(&ctl->pv_done[t]);
+                        if (t == kHalves - 1) pf_commit(&ctl->empty[stage]);
+                    }
+                }
+            }
+        };
+        if (n_work > 0) {
+            if (n_halves == 2) go(std::integral_constant<int, 2>());
+            else go(std::integral_constant<int, 1>());
         }
     } else if (warp < 4 * n_halves) {
         // ---------------------------------------------------------------- softmax: a thread per row
         const int t = warp >> 2, rho = threadIdx.x;
         const uint32_t lanes = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-        const uint32_t s_addr = lanes + C::kSCol + 64 * t, o_addr = lanes + C::kOCol + 128 * t;
+        const uint32_t s_addr = lanes + C::kSCol, p_addr = lanes + C::kPCol + 32 * t, o_addr = lanes + C::kOCol + 128 * t;
         const int qi = qi0 + rho / R;
         const bool live = qi < n_q;
-        const int64_t row = (s * n_q + qi) * sh.n_q_heads + hkv * R + rho % R;
         const int64_t pos = live ? pos0 + rho / R : -1;
         const int64_t pos_warp = pos0 + (warp * 32) / R;                   // smallest position among the warp's rows
         {
@@ -431,8 +502,7 @@ prefill_tc_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, 
             for (int half = 0; half < 2; ++half) {
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                    if (live) v = *reinterpret_cast<const uint4*>(q + row * 128 + half * 64 + i * 8);
+                    const uint4 v = *reinterpret_cast<const uint4*>(smem + C::q_offset(rho) + (((8 * half + i) ^ (rho & 7)) << 4));
                     u[4 * i] = (v.x ^ q_sign) & q_keep; u[4 * i + 1] = (v.y ^ q_sign) & q_keep;
                     u[4 * i + 2] = (v.z ^ q_sign) & q_keep; u[4 * i + 3] = (v.w ^ q_sign) & q_keep;
                 }
@@ -441,7 +511,7 @@ prefill_tc_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, 
             pf_st_wait();
             pf_fence_before();
             __syncwarp();
-            if (lane == 0) pf_arrive(&ctl->p_full[t]);
+            if (lane == 0) pf_arrive(&ctl->q_full[t]);
         }
         float m = -INFINITY, l = 0.f;                                       // reference of the weights (log2 domain), their sum
         bool ok = true;
@@ -453,6 +523,9 @@ prefill_tc_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, 
             pf_ld32(b, s_addr + 32);
             pf_ld_wait(a);
             pf_ld_wait(b);
+            pf_fence_before();
+            __syncwarp();
+            if (lane == 0) pf_arrive(&ctl->s_free[t]);
             float* sa = reinterpret_cast<float*>(a);
             float* sb = reinterpret_cast<float*>(b);
             const int64_t j0 = (int64_t)jt * C::kTile;
@@ -482,22 +555,13 @@ prefill_tc_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, 
             // The weights' reference follows the maximum only when it is more than 8 (a factor of 256) behind: the sums
             // rarely have to be rescaled, and fp16 weights up to 256 are as precise as weights up to 1.
             const bool move = m_tile > m + 8.f || (m == -INFINITY && m_tile > -INFINITY);
-            if (__any_sync(0xffffffffu, move)) {
+            const bool rescale = __any_sync(0xffffffffu, move);
+            float f = 1.f;
+            if (rescale) {
                 const float m_new = fmaxf(m, m_tile);
-                const float f = m == -INFINITY ? 0.f : exp2f(m - m_new);
+                f = m == -INFINITY ? 0.f : exp2f(m - m_new);
                 m = m_new;
                 l *= f;
-                if (jt > 0) {                                               // (the sums so far are done: the scores came after them)
-#pragma unroll 1
-                    for (int c0 = 0; c0 < 128; c0 += 32) {
-                        uint32_t o[32];
-                        pf_ld32(o, o_addr + c0);
-                        pf_ld_wait(o);
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f);
-                        pf_st32(o_addr + c0, o);
-                    }
-                }
             }
             const float mm = m == -INFINITY ? 0.f : m;
             uint32_t p[32];
@@ -517,16 +581,33 @@ prefill_tc_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, 
                 p[16 + i] = pack_half2(x0, x1);
             }
             l += l0 + l1;
-            pf_st32(s_addr, p);
+            if (jt > 0) {                                                   // the last sums are done with the weights' columns
+                if (!pf_wait(ctl, &ctl->pv_done[t], (uint32_t)(jt - 1) & 1u)) { ok = false; break; }
+                pf_fence_after();
+                if (rescale) {
+#pragma unroll 1
+                    for (int c0 = 0; c0 < 128; c0 += 32) {
+                        uint32_t o[32];
+                        pf_ld32(o, o_addr + c0);
+                        pf_ld_wait(o);
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f);
+                        pf_st32(o_addr + c0, o);
+                    }
+                }
+            }
+            pf_st32(p_addr, p);
             pf_st_wait();
             pf_fence_before();
             __syncwarp();
             if (lane == 0) pf_arrive(&ctl->p_full[t]);
         }
-        // ---- normalise and write
-        if (n_tiles > 0) ok = ok && pf_wait(ctl, &ctl->o_full, 0u);
+        // ---- normalise and write: through shared memory (the codebooks are done with when the last sums are), so that the
+        // stores take whole lines; a thread per row wrote 32 lines at a time (10.8 thousand cycles per CTA)
+        if (n_tiles > 0) ok = ok && pf_wait(ctl, &ctl->pv_done[t], (uint32_t)(n_tiles - 1) & 1u);
         pf_fence_after();
         const float inv = ok && l > 0.f ? 1.f / l : 0.f;                    // no position: zero row
+        uint8_t* block = smem + warp * 32 * C::kOutStride;
 #pragma unroll 1
         for (int c0 = 0; c0 < 128; c0 += 32) {
             uint32_t o[32];
@@ -534,14 +615,21 @@ prefill_tc_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, 
                 pf_ld32(o, o_addr + c0);
                 pf_ld_wait(o);
             }
-            if (live) {
-                float4* dst = reinterpret_cast<float4*>(out + row * 128 + c0);
 #pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    dst[i] = inv == 0.f ? make_float4(0.f, 0.f, 0.f, 0.f)
-                                        : make_float4(__uint_as_float(o[4 * i]) * inv, __uint_as_float(o[4 * i + 1]) * inv,
-                                                      __uint_as_float(o[4 * i + 2]) * inv, __uint_as_float(o[4 * i + 3]) * inv);
+            for (int i = 0; i < 8; ++i)
+                *reinterpret_cast<float4*>(block + lane * C::kOutStride + 16 * i) =
+                    inv == 0.f ? make_float4(0.f, 0.f, 0.f, 0.f)
+                               : make_float4(__uint_as_float(o[4 * i]) * inv, __uint_as_float(o[4 * i + 1]) * inv,
+                                             __uint_as_float(o[4 * i + 2]) * inv, __uint_as_float(o[4 * i + 3]) * inv);
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int rw = 4 * i + (lane >> 3), rr = warp * 32 + rw, qr = qi0 + rr / R;
+                if (qr < n_q)
+                    *reinterpret_cast<float4*>(out + ((s * n_q + qr) * sh.n_q_heads + hkv * R + rr % R) * 128 + c0 + 4 * (lane & 7)) =
+                        *reinterpret_cast<const float4*>(block + rw * C::kOutStride + 16 * (lane & 7));
             }
+            __syncwarp();
         }
         pf_fence_before();
     }
