@@ -508,7 +508,7 @@ def extra_prefill(cq, dev, reps=5):
     tf = flops / (ms * 1e-3) / 1e12
     res = {"workload": w.name, "ms": ms, "query_tokens_per_s": n_seq * n_q / (ms * 1e-3),
            "roofline": {"bound": "tensor", "achieved": tf, "peak": peak, "unit": "TFLOP/s", "frac": tf / peak, "traffic": None,
-                        "peak_source": "measured bf16 GEMM burst (fp16 has the same nominal rate); mma.sync path"}}
+                        "peak_source": "measured bf16 GEMM burst (fp16 has the same nominal rate); tcgen05 path"}}
     attach_traffic(res["roofline"], w.name)
     return res
 
