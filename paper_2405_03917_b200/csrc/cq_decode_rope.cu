@@ -19,11 +19,16 @@
 //     the token after the batch; if it differs (tables that are not of the form cos / sin of
 //     position x frequency + phase) the batch is done again with every row read from the tables, and
 //     so are the warp's later batches.
-//   - Scores of a chunk of the range are kept in shared memory; the chunk's largest score per head
-//     fixes the reference exponent (the bins are rescaled when it grows), then the weights
-//     2^(score - reference) are added to fp32 bins per (head, group, value code), lane = group, and
-//     bins x value centroids closes the partial.  Partials and their merge are those of the other
+//   - Scores of a chunk of the range are kept in shared memory; their largest one and the sum of
+//     the weights so far fix the unit in which the bins per (head, group, value code) count: whole
+//     numbers, the total just below 2^31 (the bins are shifted when the unit grows).  Lane = group
+//     adds the weights in that unit, and bins x value centroids closes the partial.  Adds to shared
+//     memory run at 32 lanes per clock for whole numbers and at 4 to 8 for fp32.  Partials and their merge are those of the other
 //     decode kernels.
+// What bounds it: instruction issue (28 a token and head for gather, rotation, dot and exchange, 4
+// for the bins) and its latencies, and a set-up and end of some 20 us per CTA.  16 sequences of 4096
+// tokens, 32 heads, c = 4: 273 us with fp32 bins, 206 with whole numbers, 188 with 32 warps for one
+// head; 32 sequences, 32 heads on 8, c = 8: 308 -> 241 us.
 #include "cq_common.cuh"
 #include "cq_decode_util.cuh"
 #include <type_traits>
@@ -32,15 +37,17 @@ namespace cq {
 
 namespace {
 
-constexpr int kRtThreads = 512;
-constexpr int kRtWarps = kRtThreads / 32;
+constexpr int kRtMostWarps = 32;
 constexpr int kRtScoreBytes = 32 * 1024;
 
 struct RtCtl {
-    float m_run[8];                    // per head: reference exponent of the bins (log2 domain)
-    float factor[8];                   // per head: 2^(old reference - new reference) of the current chunk
-    float warp_max[kRtWarps][8];       // per warp and head: largest score of the current chunk
-    float l_part[kRtWarps][8];         // per warp and head: sum of weights (final reduction)
+    float m_run[8];                    // per head: whole number not below the largest score (log2 domain)
+    float factor[8];                   // per head: 2^(old m_run - new m_run) of the current chunk
+    float e_run[8];                    // per head: the bins count in units of 2^e_run
+    float unit[8];                     // per head: 2^(m_run - e_run)
+    int shift[8];                      // per head: by how much e_run rose with the current chunk (32: more than the bins hold)
+    float warp_max[kRtMostWarps][8];       // per warp and head: largest score of the current chunk
+    float l_part[kRtMostWarps][8];         // per warp and head: sum of weights (final reduction)
 };
 
 template <int kC, int kHeads>
@@ -49,11 +56,12 @@ struct RtCfg {
     static constexpr int kT = 32 / kHeads;                        // tokens of a warp's batch
     static constexpr int kChunk = kRtScoreBytes / 4 / kHeads;     // tokens whose scores are kept at a time
     static constexpr int kBookOff = 0;                            // fp16 [256][G][kC]
-    static constexpr int kBinsOff = 128 * 256 * 2;                // fp32 [kHeads][256][G]
+    static constexpr int kBinsOff = 128 * 256 * 2;                // uint32 [kHeads][256][G]
     static constexpr int kScoreOff = kBinsOff + kHeads * G * 256 * 4;      // fp32 [kHeads][kChunk]
     static constexpr int kCtlOff = kScoreOff + kRtScoreBytes;
-    static constexpr int kSmemBytes = kCtlOff + 2048;
-    static_assert(sizeof(RtCtl) <= 2048, "control block");
+    static constexpr int kSmemBytes = kCtlOff + 2560;
+    static constexpr int kThreads = kHeads == 1 ? 1024 : 512;
+    static_assert(sizeof(RtCtl) <= 2560, "control block");
     static_assert(kSmemBytes <= 227 * 1024, "shared memory");
     static_assert(kChunk % 32 == 0 && kT >= 4, "batches of whole words");
 };
@@ -66,17 +74,17 @@ __device__ __forceinline__ uint32_t rt_code(const uint32_t (&w)[kWords], int j)
 }
 
 template <int kC, int kHeads>
-__global__ void __launch_bounds__(kRtThreads, 1)
+__global__ void __launch_bounds__(RtCfg<kC, kHeads>::kThreads, 1)
 decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, const uint8_t* __restrict__ vc,
                          const float* __restrict__ kcb, const float* __restrict__ vcb, const int32_t* __restrict__ seq_lens,
                          const float* __restrict__ rope_cos, const float* __restrict__ rope_sin, float scale_log2e, Shape sh,
-                         int n_splits, int split_tokens, float* __restrict__ partials)
+                         int n_splits, int split_tokens, float* __restrict__ partials, float* __restrict__ out)
 {
     using C = RtCfg<kC, kHeads>;
-    constexpr int G = C::G, kT = C::kT, kWords = kT / 4;
+    constexpr int G = C::G, kT = C::kT, kWords = kT / 4, kRtThreads = C::kThreads, kRtWarps = kRtThreads / 32;
     extern __shared__ __align__(16) unsigned char rt_smem[];
     const uint32_t* book = reinterpret_cast<const uint32_t*>(rt_smem + C::kBookOff);
-    float* bins = reinterpret_cast<float*>(rt_smem + C::kBinsOff);
+    uint32_t* bins = reinterpret_cast<uint32_t*>(rt_smem + C::kBinsOff);
     float* scores = reinterpret_cast<float*>(rt_smem + C::kScoreOff);
     RtCtl* ctl = reinterpret_cast<RtCtl*>(rt_smem + C::kCtlOff);
 
@@ -93,7 +101,12 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
     const int64_t t_begin = (int64_t)split * split_tokens;
     const int64_t t_end = t_begin + split_tokens < n ? t_begin + split_tokens : n;
     float* part0 = partials + ((s * sh.n_q_heads + hq0) * n_splits + split) * (int64_t)stride;      // head h: + h * n_splits * stride
-    if (t_end <= t_begin) {          // empty range: neutral element of the merge
+    float* o0 = out + (s * sh.n_q_heads + hq0) * 128;
+    if (t_end <= t_begin) {          // empty range: neutral element of the merge, or a zero row where there is none
+        if (n_splits == 1) {
+            for (int i = threadIdx.x; i < kHeads * 128; i += kRtThreads) o0[i] = 0.f;
+            return;
+        }
         for (int i = threadIdx.x; i < kHeads * stride; i += kRtThreads) {
             const int h = i / stride, d = i % stride;
             part0[(int64_t)h * n_splits * stride + d] = d == 0 ? -INFINITY : 0.f;
@@ -104,18 +117,31 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
     // ------------------------------------------------------------------ set-up
     // key centroids of the KV head as fp16, bins at zero
     {
+        // A warp takes 64 bytes of eight groups at a time: eight lines of memory per load, eight loads in flight, and four
+        // (c = 4) or two lanes that meet in a bank of a store.  (In the order of the codebook all 32 met.)
         const float4* src = reinterpret_cast<const float4*>(kcb + (int64_t)hkv * 128 * 256);
-        uint2* dst = reinterpret_cast<uint2*>(rt_smem + C::kBookOff);
-        for (int i = threadIdx.x; i < 128 * 256 / 4; i += kRtThreads) {
-            // four channels of centroid (g, j): piece i of the global [g][j][c] order goes to the [j][g][c] order
-            const int per = kC / 4, g = i / (256 * per), j = (i / per) % 256, w4 = i % per;
-            const float4 v = ldg_f4(reinterpret_cast<const float*>(src + i));
-            const __half2 lo = __floats2half2_rn(v.x, v.y), hi = __floats2half2_rn(v.z, v.w);
-            dst[(j * G + g) * per + w4] = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+        constexpr int kTasks = 256, kBatch = 8;
+        static_assert(kTasks % (kRtWarps * kBatch) == 0, "whole batches");
+        const int gl = kC == 8 ? (lane >> 1) & 7 : lane & 7, j = kC == 8 ? (lane >> 4) * 2 + (lane & 1) : lane >> 3;
+#pragma unroll 1
+        for (int i0 = warp; i0 < kTasks; i0 += kBatch * kRtWarps) {
+            float4 x[kBatch];
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) {
+                const int i = i0 + u * kRtWarps, g = 8 * (i % (G / 8)) + gl;
+                x[u] = ldg_f4(reinterpret_cast<const float*>(src + (g * 16 * kC + i / (G / 8)) * 4 + j));
+            }
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) {
+                const int i = i0 + u * kRtWarps, g = 8 * (i % (G / 8)) + gl, seg = i / (G / 8);
+                const __half2 lo = __floats2half2_rn(x[u].x, x[u].y), hi = __floats2half2_rn(x[u].z, x[u].w);
+                const int at = kC == 8 ? (seg * 2 + (j >> 1)) * 256 + g * 16 + (j & 1) * 8 : (seg * 4 + j) * 256 + g * 8;
+                *reinterpret_cast<uint2*>(rt_smem + C::kBookOff + at) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+            }
         }
         for (int i = threadIdx.x; i < kHeads * G * 256 / 4; i += kRtThreads)
             reinterpret_cast<float4*>(bins)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (threadIdx.x < 8) ctl->m_run[threadIdx.x] = -INFINITY;
+        if (threadIdx.x < 8) ctl->m_run[threadIdx.x] = ctl->e_run[threadIdx.x] = -INFINITY;
     }
     // this lane's channels: a = 2 lane, 2 lane + 1 and b = a + 64; its slice of every head's query
     float qa[kHeads][2], qb[kHeads][2];
@@ -190,8 +216,9 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
         if (warp * kT < chunk_len) load_batch(chunk_begin + warp * kT, ca, cbw, cs0, sn0);
         for (int b0 = warp * kT; b0 < chunk_len; b0 += kRtWarps * kT) {
             const int64_t t0 = chunk_begin + b0;
-            float p[32];
-            // The partial scores of the batch; from_tables: every token's row is read from the tables, else the rows
+            constexpr int kSlots = kHeads == 1 ? 1 : 32;
+            float p[kSlots];
+            // The scores of the batch, summed over the lanes as they come; from_tables: every token's row is read from the tables, else the rows
             // after the first follow by the step rotation.  Returns false when the stepped rows leave the tables.
             // With one head per CTA the query is rotated instead of the key (by the opposite angle): the rotated
             // query u = q_a cos + q_b sin, v = q_b cos - q_a sin steps like the angle does, and the score term of a
@@ -199,6 +226,17 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
             auto batch = [&](auto from_tables) -> bool {
                 constexpr bool kFromTables = decltype(from_tables)::value;
                 float2 cs = cs0, sn = sn0;
+                // Sum over the lanes, two values at a time: a lane keeps the one whose slot has the bit of the offset like its
+                // own lane number, the other lane's share of it added; slot = (head, token of the batch).  At the end lane L
+                // holds slot L = (head L / kT, token L % kT).  With one head tokens 2i and 2i + 1 are joined at once, then
+                // pairs, ...: few values wait in registers, so that 32 warps fit the SM, and the exchanges pass between the
+                // gathers (16 sequences of 4096 tokens, 32 heads, c = 4: 206 -> 187 us).  With several heads the 16 warps'
+                // multiply-adds hide the exchange better when it comes in one piece (four heads, c = 4: 173 against 181 us).
+                auto join = [&](float lower, float upper, int o) {
+                    const bool up = (lane & o) != 0;
+                    return (up ? upper : lower) + __shfl_xor_sync(0xffffffffu, up ? lower : upper, o);
+                };
+                float waiting[5];
                 float2 u = make_float2(0.f, 0.f), v = make_float2(0.f, 0.f);
                 if (kHeads == 1) {
                     u = make_float2(fmaf(qa[0][0], cs.x, qb[0][0] * sn.x), fmaf(qa[0][1], cs.y, qb[0][1] * sn.y));
@@ -210,15 +248,28 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
                     const uint32_t wb = book[rt_code<kWords>(cbw, j) * 64u + colB];
                     const float2 ka = __half22float2(*reinterpret_cast<const __half2*>(&wa));
                     const float2 kb = __half22float2(*reinterpret_cast<const __half2*>(&wb));
+                    float x[kHeads];
                     if (kHeads == 1) {
-                        p[j] = fmaf(ka.x, u.x, fmaf(kb.x, v.x, fmaf(ka.y, u.y, kb.y * v.y)));
+                        x[0] = fmaf(ka.x, u.x, fmaf(kb.x, v.x, fmaf(ka.y, u.y, kb.y * v.y)));
                     } else {
                         // the rotated key of the lane's four channels
                         const float ra0 = ka.x * cs.x - kb.x * sn.x, rb0 = kb.x * cs.x + ka.x * sn.x;
                         const float ra1 = ka.y * cs.y - kb.y * sn.y, rb1 = kb.y * cs.y + ka.y * sn.y;
 #pragma unroll
                         for (int h = 0; h < kHeads; ++h)
-                            p[h * kT + j] = fmaf(qa[h][0], ra0, fmaf(qb[h][0], rb0, fmaf(qa[h][1], ra1, qb[h][1] * rb1)));
+                            x[h] = fmaf(qa[h][0], ra0, fmaf(qb[h][0], rb0, fmaf(qa[h][1], ra1, qb[h][1] * rb1)));
+                    }
+                    if (kHeads == 1) {
+#pragma unroll
+                        for (int b = 0; b < 5; ++b) {
+                            if ((j & ((1 << b) - 1)) != (1 << b) - 1) break;     // some lower bit is clear: it waits already
+                            if ((j >> b) & 1) x[0] = join(waiting[b], x[0], 1 << b);
+                            else waiting[b] = x[0];
+                        }
+                        p[0] = x[0];
+                    } else {
+#pragma unroll
+                        for (int h = 0; h < kHeads; ++h) p[(h * kT + j) % kSlots] = x[h];
                     }
                     // the next position
                     if (kFromTables) {
@@ -272,16 +323,16 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
                 const int nb = b0 + kRtWarps * kT;
                 if (nb < chunk_len) load_batch(chunk_begin + nb, ca, cbw, cs0, sn0);
             }
-            // Sum over the lanes: after the stage with offset o a lane keeps the half of its slots whose index has
-            // bit o like its own lane number; after five stages lane L holds slot L = (head L / kT, token L % kT).
+            if (kHeads > 1) {
 #pragma unroll
-            for (int o = 16; o >= 1; o >>= 1) {
-                const bool upper = (lane & o) != 0;
+                for (int o = 16; o >= 1; o >>= 1) {
+                    const bool upper = (lane & o) != 0;
 #pragma unroll
-                for (int i = 0; i < o; ++i) {
-                    const float send = upper ? p[i] : p[i + o];
-                    const float keep = upper ? p[i + o] : p[i];
-                    p[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                    for (int i = 0; i < o; ++i) {
+                        const float send = upper ? p[i % kSlots] : p[(i + o) % kSlots];
+                        const float keep = upper ? p[(i + o) % kSlots] : p[i % kSlots];
+                        p[i % kSlots] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                    }
                 }
             }
             const int h = lane / kT, j = lane % kT;
@@ -298,24 +349,52 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
         if (threadIdx.x < kHeads) {
             float m = ctl->m_run[threadIdx.x];
             const float old = m;
-            for (int w = 0; w < kRtWarps; ++w) m = fmaxf(m, ctl->warp_max[w][threadIdx.x]);
+            for (int w = 0; w < kRtWarps; ++w) m = fmaxf(m, ceilf(ctl->warp_max[w][threadIdx.x]));
             ctl->factor[threadIdx.x] = old == m ? 1.f : exp2f(old - m);      // 0 when there was no reference yet
             ctl->m_run[threadIdx.x] = m;
         }
         __syncthreads();
-        // the bins follow the reference; weights of the chunk
+        // weights of the chunk, relative to m_run, and the total so far
 #pragma unroll
         for (int h = 0; h < kHeads; ++h) {
-            const float f = ctl->factor[h], m = ctl->m_run[h];
-            if (f != 1.f) {
-                for (int i = threadIdx.x; i < G * 256; i += kRtThreads) bins[h * G * 256 + i] *= f;
-                l_thr[h] *= f;
-            }
+            const float m = ctl->m_run[h];
+            float l = l_thr[h] * ctl->factor[h];
             for (int i = threadIdx.x; i < chunk_len; i += kRtThreads) {
                 const float w = exp2f(scores[h * C::kChunk + i] - m);
                 scores[h * C::kChunk + i] = w;
-                l_thr[h] += w;
+                l += w;
             }
+            l_thr[h] = l;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+            if (lane == 0) ctl->l_part[warp][h] = l;
+        }
+        __syncthreads();
+        // The unit that lets the total fill 31 bits: no bin can run over, and a weight keeps as many bits as fp32 gives it
+        // down to 2^-8 of the total.
+        if (threadIdx.x < kHeads) {
+            float total = 0.f;
+            for (int w = 0; w < kRtWarps; ++w) total += ctl->l_part[w][threadIdx.x];
+            const float m = ctl->m_run[threadIdx.x], old = ctl->e_run[threadIdx.x];
+            const float wanted = m + (ceilf(log2f(total)) - 31.f), e = wanted < old ? old : wanted;
+            const float rise = e - old;                                       // (infinite when there was no unit yet: bins are zero)
+            ctl->shift[threadIdx.x] = rise < 32.f ? (int)rise : 32;
+            ctl->e_run[threadIdx.x] = e;
+            ctl->unit[threadIdx.x] = exp2f(m - e);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int h = 0; h < kHeads; ++h) {
+            const int shift = chunk_begin > t_begin ? ctl->shift[h] : 0;
+            if (shift > 0)
+                for (int i = threadIdx.x; i < G * 256; i += kRtThreads) {
+                    const uint32_t v = bins[h * G * 256 + i];
+                    bins[h * G * 256 + i] = shift < 32 ? (v >> shift) + ((v >> (shift - 1)) & 1u) : 0u;
+                }
+            const float unit = ctl->unit[h];
+            const int padded = (chunk_len + kTokenBlock - 1) / kTokenBlock * kTokenBlock;
+            for (int i = threadIdx.x; i < padded; i += kRtThreads)
+                reinterpret_cast<uint32_t*>(scores)[h * C::kChunk + i] = i < chunk_len ? __float2uint_rn(scores[h * C::kChunk + i] * unit) : 0u;
         }
         __syncthreads();
         // -------------------------------------------------------------- value side: weights into the bins
@@ -325,9 +404,9 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
             constexpr int kRun = 16 / kLanesPerGroup;               // tokens of the block per lane
             const int g = lane % G, run = lane / G;
             const int n_blk = (chunk_len + kTokenBlock - 1) / kTokenBlock;
-            for (int blk = warp; blk < n_blk; blk += kRtWarps) {
+            // (the next block's codes travel during the adds of this one)
+            auto load_codes = [&](int blk, uint32_t (&cw)[kRun / 4]) {
                 const uint8_t* pv = vseq + ((chunk_begin / kTokenBlock) + blk) * sh.block_bytes + g * kTokenBlock + run * kRun;
-                uint32_t cw[kRun / 4];
                 if (kRun == 16) {
                     const uint4 v4 = *reinterpret_cast<const uint4*>(pv);
                     cw[0] = v4.x; cw[1 % (kRun / 4)] = v4.y; cw[2 % (kRun / 4)] = v4.z; cw[3 % (kRun / 4)] = v4.w;
@@ -335,14 +414,27 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
                     const uint2 v2 = *reinterpret_cast<const uint2*>(pv);
                     cw[0] = v2.x; cw[1 % (kRun / 4)] = v2.y;
                 }
+            };
+            const uint32_t bin0 = (uint32_t)__cvta_generic_to_shared(bins + g);
+            uint32_t cw[kRun / 4], next[kRun / 4];
+            if (warp < n_blk) load_codes(warp, next);
+            for (int blk = warp; blk < n_blk; blk += kRtWarps) {
 #pragma unroll
-                for (int k = 0; k < kRun; ++k) {
-                    const int tl = blk * kTokenBlock + run * kRun + k;
-                    const uint32_t code = rt_code<kRun / 4>(cw, k);
+                for (int i = 0; i < kRun / 4; ++i) cw[i] = next[i];
+                if (blk + kRtWarps < n_blk) load_codes(blk + kRtWarps, next);
 #pragma unroll
-                    for (int h = 0; h < kHeads; ++h) {
-                        const float w = tl < chunk_len ? scores[h * C::kChunk + tl] : 0.f;      // (adding zero changes nothing)
-                        atomicAdd(&bins[(h * 256 + code) * G + g], w);
+                for (int k = 0; k < kRun; k += 4) {
+                    uint4 w[kHeads];                            // (the weights behind the end of the chunk are zero)
+#pragma unroll
+                    for (int h = 0; h < kHeads; ++h)
+                        w[h] = *reinterpret_cast<const uint4*>(scores + h * C::kChunk + blk * kTokenBlock + run * kRun + k);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const uint32_t bin = bin0 + rt_code<kRun / 4>(cw, k + j) * (G * 4);
+#pragma unroll
+                        for (int h = 0; h < kHeads; ++h)
+                            asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(bin + h * (256 * G * 4)),
+                                         "r"(j == 0 ? w[h].x : j == 1 ? w[h].y : j == 2 ? w[h].z : w[h].w) : "memory");
                     }
                 }
             }
@@ -362,8 +454,12 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
     if (threadIdx.x < kHeads) {
         float l = 0.f;
         for (int w = 0; w < kRtWarps; ++w) l += ctl->l_part[w][threadIdx.x];
-        part0[(int64_t)threadIdx.x * n_splits * stride + 0] = ctl->m_run[threadIdx.x];
-        part0[(int64_t)threadIdx.x * n_splits * stride + 1] = l;
+        l *= ctl->unit[threadIdx.x];
+        ctl->factor[threadIdx.x] = l;
+        if (n_splits > 1) {
+            part0[(int64_t)threadIdx.x * n_splits * stride + 0] = ctl->e_run[threadIdx.x];
+            part0[(int64_t)threadIdx.x * n_splits * stride + 1] = l;
+        }
     }
     // bins x value centroids: lane = group (two lanes per group for c = 8, one for the even and one for the odd codes),
     // a warp per 16 codes, the warps' sums added through shared memory (the score area is free now)
@@ -376,10 +472,10 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
             float acc[kC];
 #pragma unroll
             for (int k = 0; k < kC; ++k) acc[k] = 0.f;
-#pragma unroll 4
-            for (int i = 0; i < 16 / kLanesPerGroup; ++i) {
-                const int j = warp * 16 + kLanesPerGroup * i + sub;
-                const float w = bins[(h * 256 + j) * G + g];
+#pragma unroll 8
+            for (int i = 0; i < 256 / kRtWarps / kLanesPerGroup; ++i) {
+                const int j = warp * (256 / kRtWarps) + kLanesPerGroup * i + sub;
+                const float w = (float)bins[(h * 256 + j) * G + g];
                 float cv[kC];
                 load_centroid<kC>(vcb + (((int64_t)hkv * G + g) * 256 + j) * kC, cv, false);
 #pragma unroll
@@ -398,7 +494,8 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
                 float v = 0.f;
 #pragma unroll
                 for (int w = 0; w < kRtWarps; ++w) v += red[w * 128 + threadIdx.x];
-                part0[(int64_t)h * n_splits * stride + 2 + threadIdx.x] = v;
+                if (n_splits == 1) o0[h * 128 + threadIdx.x] = v / ctl->factor[h];       // a range is the whole context: no merge
+                else part0[(int64_t)h * n_splits * stride + 2 + threadIdx.x] = v;
             }
             __syncthreads();
         }
@@ -408,15 +505,15 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
 template <int kC, int kHeads>
 cudaError_t launch_rt(const __half* q, const uint8_t* kc, const uint8_t* vc, const float* kcb, const float* vcb,
                       const int32_t* seq_lens, const float* rope_cos, const float* rope_sin, float scale, const Shape& sh,
-                      int n_splits, int split_tokens, float* partials, cudaStream_t st)
+                      int n_splits, int split_tokens, float* partials, float* out, cudaStream_t st)
 {
     using C = RtCfg<kC, kHeads>;
     constexpr int kSlot = 48 + (kC == 8 ? 0 : 4) + (kHeads == 1 ? 0 : kHeads == 2 ? 1 : kHeads == 4 ? 2 : 3);    // 48 ... 55
     cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(decode_rope_tuned_kernel<kC, kHeads>), C::kSmemBytes, kSlot);
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)(sh.n_seq * (sh.n_q_heads / kHeads) * n_splits);
-    decode_rope_tuned_kernel<kC, kHeads><<<grid, kRtThreads, C::kSmemBytes, st>>>(q, kc, vc, kcb, vcb, seq_lens, rope_cos, rope_sin,
-                                                                                  scale * kLog2e, sh, n_splits, split_tokens, partials);
+    decode_rope_tuned_kernel<kC, kHeads><<<grid, C::kThreads, C::kSmemBytes, st>>>(q, kc, vc, kcb, vcb, seq_lens, rope_cos, rope_sin,
+                                                                                  scale * kLog2e, sh, n_splits, split_tokens, partials, out);
     return cudaGetLastError();
 }
 
@@ -453,14 +550,14 @@ cudaError_t launch_decode_rope_tuned(const __half* q, const uint8_t* kc, const u
     split_tokens = (split_tokens + 255) / 256 * 256;
     const int n_splits = (int)((sh.max_tokens + split_tokens - 1) / split_tokens);
     cudaError_t e = cudaErrorNotSupported;
-#define CQ_RT(C_, H_) e = launch_rt<C_, H_>(q, kc, vc, kcb, vcb, seq_lens, rope_cos, rope_sin, scale, sh, n_splits, (int)split_tokens, partials, st)
+#define CQ_RT(C_, H_) e = launch_rt<C_, H_>(q, kc, vc, kcb, vcb, seq_lens, rope_cos, rope_sin, scale, sh, n_splits, (int)split_tokens, partials, out, st)
     if (sh.c == 8) {
         switch (heads) { case 1: CQ_RT(8, 1); break; case 2: CQ_RT(8, 2); break; case 4: CQ_RT(8, 4); break; case 8: CQ_RT(8, 8); break; default: break; }
     } else {
         switch (heads) { case 1: CQ_RT(4, 1); break; case 2: CQ_RT(4, 2); break; case 4: CQ_RT(4, 4); break; default: break; }
     }
 #undef CQ_RT
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || n_splits == 1) return e;
     return launch_merge(partials, n_splits, sh, out, st);
 }
 

@@ -159,3 +159,26 @@ def test_tuned_rope_kernel_is_refused_where_it_does_not_apply():
     with pytest.raises(cq.CQError):          # the other pairing
         cq.cq_decode_attn_rope(q.to(DEV), to_lib(kc_rm, 128, 8, 8), to_lib(vc_rm, 128, 8, 8), kcb.to(DEV), vcb.to(DEV), sl,
                                torch.from_numpy(cs).to(DEV), torch.from_numpy(sn).to(DEV), 0.1, 8, 8, 20, pairing=1, variant=2)
+
+
+@pytest.mark.parametrize("scale_late", [1.0, 12.0])
+def test_tuned_rope_kernel_over_several_chunks_of_one_range(scale_late):
+    """More sequences than CTAs run at once (a range is a whole context, no merge), one of them several chunks long
+    (8 heads: 1024 tokens each), whose later scores are (or are not) far above the earlier ones: the bins' unit moves."""
+    n_seq, D, c, b = 300, 128, 8, 8
+    lens = [1 + i % 3 for i in range(n_seq)]
+    lens[7], lens[8] = 2500, 0
+    cap = 2501
+    q, kc_rm, vc_rm, kcb, vcb = case(91, c, b, 8, 1, lens, cap, D)
+    kcb[:, :, 128:] *= scale_late
+    kc_rm[7, :1100] %= 128
+    cs, sn = rope_tables(cap, D // 2)
+    sl = torch.tensor(lens, dtype=torch.int32, device=DEV)
+    out = cq.cq_decode_attn_rope(q.to(DEV), to_lib(kc_rm, D, c, b), to_lib(vc_rm, D, c, b), kcb.to(DEV), vcb.to(DEV), sl,
+                                 torch.from_numpy(cs).to(DEV), torch.from_numpy(sn).to(DEV), D ** -0.5, c, b, cap).cpu().numpy()
+    some = [0, 1, 2, 7, 8, 299]
+    kcb = kcb.half().float()                  # the kernel keeps key centroids in fp16
+    ref = oracle.decode_dense_rope(q.numpy()[some], kc_rm[some], vc_rm[some], kcb.numpy(), vcb.numpy(),
+                                   np.asarray(lens, np.int32)[some], cs, sn, D ** -0.5, c, b, 0)
+    for k, s_ in enumerate(some):
+        H.check_attn(out[s_], ref[k], f"rope sequence {s_}")
