@@ -768,6 +768,13 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
         }
     }
     __syncthreads();
+    // The sums of an item of one part (out != null) stay in the K table's place, 32 words to a row; the last step reads them
+    // again (through global memory that was two trips to L2 at the end of every CTA).
+    auto sum_at = [&](int h, int i) -> float* {
+        const int w = h * (kD + 32) + i;
+        return out ? reinterpret_cast<float*>(smem + (w >> 5) * kRowBytes + (w & 31) * 4) : part_base + (int64_t)h * n_parts * stride + i;
+    };
+    static_assert(R * (kD + 32) <= 256 * 32, "room");
     float acc[R][kC];
     float lsum[R];                            // sum of the bins of group 0 (the normaliser)
 #pragma unroll
@@ -808,12 +815,12 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
                 float v = (up ? acc[h][1] : acc[h][0]) + __shfl_xor_sync(0xffffffffu, up ? acc[h][0] : acc[h][1], 16);
 #pragma unroll
                 for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                if ((lane & 15) == 0) part_base[(int64_t)h * n_parts * stride + 2 + g * kC + (up ? 1 : 0)] = v;
+                if ((lane & 15) == 0) *sum_at(h, 2 + g * kC + (up ? 1 : 0)) = v;
             } else {
                 float v = fold_channels<kC>(acc[h], lane);
                 // lane holds channel fold_channel_of<kC>(lane) summed over the lanes that share it
                 const int ch = fold_channel_of<kC>(lane);
-                if ((lane & (kC == 8 ? 3 : 7)) == 0) part_base[(int64_t)h * n_parts * stride + 2 + g * kC + ch] = v;
+                if ((lane & (kC == 8 ? 3 : 7)) == 0) *sum_at(h, 2 + g * kC + ch) = v;
             }
         }
         if (g == 0) {
@@ -823,8 +830,8 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
                 if (lane == 0) {
-                    part_base[(int64_t)h * n_parts * stride + 0] = (float)ctl->e_cur[h];   // reference exponent (log2 domain)
-                    part_base[(int64_t)h * n_parts * stride + 1] = l;            // normaliser, in the same unit
+                    *sum_at(h, 0) = (float)ctl->e_cur[h];   // reference exponent (log2 domain)
+                    *sum_at(h, 1) = l;            // normaliser, in the same unit
                 }
             }
         }
@@ -840,9 +847,8 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
         __syncthreads();
         for (int i = threadIdx.x; i < R * kD; i += C::kThreads) {
             const int h = i / kD, d = i % kD;
-            const float* ph = part_base + (int64_t)h * n_parts * stride;
-            const float l = ph[1];
-            out[(s * sh.n_q_heads + (int64_t)head_group * R + h) * kD + d] = l > 0.f ? ph[2 + d] / l : 0.f;
+            const float l = *sum_at(h, 1);
+            out[(s * sh.n_q_heads + (int64_t)head_group * R + h) * kD + d] = l > 0.f ? *sum_at(h, 2 + d) / l : 0.f;
         }
     }
 }

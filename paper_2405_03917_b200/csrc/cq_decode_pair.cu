@@ -893,6 +893,10 @@ decode_pair_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc,
             }
         }
         float* red = reinterpret_cast<float*>(smem);                      // [warp][18][32]
+        // an item of one part (out != null): its sums stay in the K table's place behind `red`
+        static_assert(C::kWarps * 18 * 32 * 4 <= 24 * 1024 && 24 * 1024 + R * 132 * 4 <= C::kKBytes, "room");
+        float* sums = out ? reinterpret_cast<float*>(smem + 24 * 1024) : part_base;
+        const int64_t sums_stride = out ? 132 : (int64_t)n_parts * stride;
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             red[(warp * 18 + c) * 32 + lane] = acc0[c];
@@ -911,11 +915,11 @@ decode_pair_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc,
             const int hb2 = ln >> 4, g2 = ln & 15;
             if (slot < 16) {
                 const int h = 2 * (slot >> 3) + hb2;
-                part_base[(int64_t)h * n_parts * stride + 2 + g2 * 8 + (slot & 7)] = v;
+                sums[h * sums_stride + 2 + g2 * 8 + (slot & 7)] = v;
             } else if (g2 == 0) {
                 const int h = 2 * (slot - 16) + hb2;
-                part_base[(int64_t)h * n_parts * stride + 0] = (float)ctl->head[h].e_cur + ctl->offset[h];   // reference exponent (log2 domain)
-                part_base[(int64_t)h * n_parts * stride + 1] = v;                                            // normaliser, in the same unit
+                sums[h * sums_stride + 0] = (float)ctl->head[h].e_cur + ctl->offset[h];   // reference exponent (log2 domain)
+                sums[h * sums_stride + 1] = v;                                            // normaliser, in the same unit
             }
         }
         // One part per item (out != null only then): the partial is the whole sum, so the CTA normalises it itself
@@ -924,7 +928,7 @@ decode_pair_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc,
             __syncthreads();
             for (int i = threadIdx.x; i < R * 128; i += C::kThreads) {
                 const int h = i >> 7, d = i & 127;
-                const float* ph = part_base + (int64_t)h * n_parts * stride;
+                const float* ph = sums + h * sums_stride;
                 const float l = ph[1];
                 out[(s * sh.n_q_heads + (int64_t)head_group * R + h) * 128 + d] = l > 0.f ? ph[2 + d] / l : 0.f;
             }
