@@ -26,9 +26,9 @@
 //     memory run at 32 lanes per clock for whole numbers and at 4 to 8 for fp32.  Partials and their merge are those of the other
 //     decode kernels.
 // What bounds it: instruction issue (28 a token and head for gather, rotation, dot and exchange, 4
-// for the bins) and its latencies, and a set-up and end of some 20 us per CTA.  16 sequences of 4096
-// tokens, 32 heads, c = 4: 273 us with fp32 bins, 206 with whole numbers, 188 with 32 warps for one
-// head; 32 sequences, 32 heads on 8, c = 8: 308 -> 241 us.
+// for the bins; 54 of 75 thousand cycles of a CTA at 4096 tokens).  16 sequences of 4096 tokens, 32
+// heads, c = 4: 273 us with fp32 bins, 206 with whole numbers, 188 with 32 warps for one head, 164 with
+// set-up and end that read the codebooks in whole lines; 32 sequences, 32 heads on 8, c = 8: 308 -> 176.
 #include "cq_common.cuh"
 #include "cq_decode_util.cuh"
 #include <type_traits>
@@ -115,34 +115,6 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
     }
 
     // ------------------------------------------------------------------ set-up
-    // key centroids of the KV head as fp16, bins at zero
-    {
-        // A warp takes 64 bytes of eight groups at a time: eight lines of memory per load, eight loads in flight, and four
-        // (c = 4) or two lanes that meet in a bank of a store.  (In the order of the codebook all 32 met.)
-        const float4* src = reinterpret_cast<const float4*>(kcb + (int64_t)hkv * 128 * 256);
-        constexpr int kTasks = 256, kBatch = 8;
-        static_assert(kTasks % (kRtWarps * kBatch) == 0, "whole batches");
-        const int gl = kC == 8 ? (lane >> 1) & 7 : lane & 7, j = kC == 8 ? (lane >> 4) * 2 + (lane & 1) : lane >> 3;
-#pragma unroll 1
-        for (int i0 = warp; i0 < kTasks; i0 += kBatch * kRtWarps) {
-            float4 x[kBatch];
-#pragma unroll
-            for (int u = 0; u < kBatch; ++u) {
-                const int i = i0 + u * kRtWarps, g = 8 * (i % (G / 8)) + gl;
-                x[u] = ldg_f4(reinterpret_cast<const float*>(src + (g * 16 * kC + i / (G / 8)) * 4 + j));
-            }
-#pragma unroll
-            for (int u = 0; u < kBatch; ++u) {
-                const int i = i0 + u * kRtWarps, g = 8 * (i % (G / 8)) + gl, seg = i / (G / 8);
-                const __half2 lo = __floats2half2_rn(x[u].x, x[u].y), hi = __floats2half2_rn(x[u].z, x[u].w);
-                const int at = kC == 8 ? (seg * 2 + (j >> 1)) * 256 + g * 16 + (j & 1) * 8 : (seg * 4 + j) * 256 + g * 8;
-                *reinterpret_cast<uint2*>(rt_smem + C::kBookOff + at) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
-            }
-        }
-        for (int i = threadIdx.x; i < kHeads * G * 256 / 4; i += kRtThreads)
-            reinterpret_cast<float4*>(bins)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (threadIdx.x < 8) ctl->m_run[threadIdx.x] = ctl->e_run[threadIdx.x] = -INFINITY;
-    }
     // this lane's channels: a = 2 lane, 2 lane + 1 and b = a + 64; its slice of every head's query
     float qa[kHeads][2], qb[kHeads][2];
 #pragma unroll
@@ -166,6 +138,34 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
         st_re.y = (c1.y * c0.y + s1.y * s0.y) / ny;
         st_im.y = (s1.y * c0.y - c1.y * s0.y) / ny;
         exact = __any_sync(0xffffffffu, exact);
+    }
+    // key centroids of the KV head as fp16, bins at zero
+    {
+        // A warp takes 64 bytes of eight groups at a time, a quarter of it two groups: two lines of memory per quarter of a
+        // load, and at most four lanes that meet in a bank of a store.  (In the order of the codebook all 32 met.)
+        const float4* src = reinterpret_cast<const float4*>(kcb + (int64_t)hkv * 128 * 256);
+        constexpr int kTasks = 256, kBatch = 8;
+        static_assert(kTasks % (kRtWarps * kBatch) == 0, "whole batches");
+        const int gl = lane >> 2, j = lane & 3;
+#pragma unroll 1
+        for (int i0 = warp; i0 < kTasks; i0 += kBatch * kRtWarps) {
+            float4 x[kBatch];
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) {
+                const int i = i0 + u * kRtWarps, g = 8 * (i % (G / 8)) + gl;
+                x[u] = ldg_f4(reinterpret_cast<const float*>(src + (g * 16 * kC + i / (G / 8)) * 4 + j));
+            }
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) {
+                const int i = i0 + u * kRtWarps, g = 8 * (i % (G / 8)) + gl, seg = i / (G / 8);
+                const __half2 lo = __floats2half2_rn(x[u].x, x[u].y), hi = __floats2half2_rn(x[u].z, x[u].w);
+                const int at = kC == 8 ? (seg * 2 + (j >> 1)) * 256 + g * 16 + (j & 1) * 8 : (seg * 4 + j) * 256 + g * 8;
+                *reinterpret_cast<uint2*>(rt_smem + C::kBookOff + at) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+            }
+        }
+        for (int i = threadIdx.x; i < kHeads * G * 256 / 4; i += kRtThreads)
+            reinterpret_cast<float4*>(bins)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (threadIdx.x < 8) ctl->m_run[threadIdx.x] = ctl->e_run[threadIdx.x] = -INFINITY;
     }
     // words of the lane's two channels inside a centroid, and its two groups
     const int gA = (2 * lane) / kC, gB = gA + G / 2;
@@ -461,43 +461,58 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
             part0[(int64_t)threadIdx.x * n_splits * stride + 1] = l;
         }
     }
-    // bins x value centroids: lane = group (two lanes per group for c = 8, one for the even and one for the odd codes),
-    // a warp per 16 codes, the warps' sums added through shared memory (the score area is free now)
+    // Bins x value centroids: a warp takes 64 bytes of eight groups at a time, as in the set-up, for all heads together
+    // (one group per lane touched 32 lines of memory per load and read the codebook once per head: 11 thousand cycles per
+    // head); the warps' sums are added through shared memory (the score area is free now).
     {
-        constexpr int kLanesPerGroup = 32 / G;
-        const int g = lane % G, sub = lane / G;
-        float* red = scores;                                     // [warps][128]
+        constexpr int kOct = G / 8, kTasks = 256 / kRtWarps, kBatch = kTasks < 4 ? kTasks : 4;
+        static_assert(kRtWarps % kOct == 0, "a warp stays with its eight groups");
+        const int gl = lane >> 2, j = lane & 3;
+        const int g = 8 * (warp % kOct) + gl;
+        const float4* src = reinterpret_cast<const float4*>(vcb + (int64_t)hkv * 128 * 256) + g * 64 * kC + j;
+        float acc[kHeads][4];
+#pragma unroll
+        for (int h = 0; h < kHeads; ++h) acc[h][0] = acc[h][1] = acc[h][2] = acc[h][3] = 0.f;
 #pragma unroll 1
+        for (int i0 = 0; i0 < kTasks; i0 += kBatch) {
+            float4 x[kBatch];
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) x[u] = ldg_f4(reinterpret_cast<const float*>(src + (warp + (i0 + u) * kRtWarps) / kOct * 4));
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) {
+                const int seg = (warp + (i0 + u) * kRtWarps) / kOct, code = kC == 8 ? seg * 2 + (j >> 1) : seg * 4 + j;
+#pragma unroll
+                for (int h = 0; h < kHeads; ++h) {
+                    const float w = (float)bins[(h * 256 + code) * G + g];
+                    acc[h][0] = fmaf(w, x[u].x, acc[h][0]);
+                    acc[h][1] = fmaf(w, x[u].y, acc[h][1]);
+                    acc[h][2] = fmaf(w, x[u].z, acc[h][2]);
+                    acc[h][3] = fmaf(w, x[u].w, acc[h][3]);
+                }
+            }
+        }
+        float* red = scores;                                     // [heads][warps][8 groups][kC]
+        constexpr int kRow = 8 * kC;
+        static_assert(kHeads * kRtWarps * kRow * 4 <= kRtScoreBytes, "room");
+#pragma unroll
         for (int h = 0; h < kHeads; ++h) {
-            float acc[kC];
 #pragma unroll
-            for (int k = 0; k < kC; ++k) acc[k] = 0.f;
-#pragma unroll 8
-            for (int i = 0; i < 256 / kRtWarps / kLanesPerGroup; ++i) {
-                const int j = warp * (256 / kRtWarps) + kLanesPerGroup * i + sub;
-                const float w = (float)bins[(h * 256 + j) * G + g];
-                float cv[kC];
-                load_centroid<kC>(vcb + (((int64_t)hkv * G + g) * 256 + j) * kC, cv, false);
-#pragma unroll
-                for (int k = 0; k < kC; ++k) acc[k] = fmaf(w, cv[k], acc[k]);
+            for (int k = 0; k < 4; ++k) {
+                acc[h][k] += __shfl_xor_sync(0xffffffffu, acc[h][k], 2);
+                if (kC == 4) acc[h][k] += __shfl_xor_sync(0xffffffffu, acc[h][k], 1);
             }
-            if (kLanesPerGroup == 2) {
+            if (j < kC / 4)
+                *reinterpret_cast<float4*>(red + (h * kRtWarps + warp) * kRow + gl * kC + (kC == 8 ? 4 * (j & 1) : 0)) =
+                    make_float4(acc[h][0], acc[h][1], acc[h][2], acc[h][3]);
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < kHeads * 128; i += kRtThreads) {
+            const int h = i >> 7, d = i & 127;
+            float v = 0.f;
 #pragma unroll
-                for (int k = 0; k < kC; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], 16);
-            }
-            if (sub == 0) {
-#pragma unroll
-                for (int k = 0; k < kC; ++k) red[warp * 128 + g * kC + k] = acc[k];
-            }
-            __syncthreads();
-            if (threadIdx.x < 128) {
-                float v = 0.f;
-#pragma unroll
-                for (int w = 0; w < kRtWarps; ++w) v += red[w * 128 + threadIdx.x];
-                if (n_splits == 1) o0[h * 128 + threadIdx.x] = v / ctl->factor[h];       // a range is the whole context: no merge
-                else part0[(int64_t)h * n_splits * stride + 2 + threadIdx.x] = v;
-            }
-            __syncthreads();
+            for (int w = 0; w < kRtWarps / kOct; ++w) v += red[(h * kRtWarps + w * kOct + d / kRow) * kRow + d % kRow];
+            if (n_splits == 1) o0[h * 128 + d] = v / ctl->factor[h];       // a range is the whole context: no merge
+            else part0[(int64_t)h * n_splits * stride + 2 + d] = v;
         }
     }
 }

@@ -19,7 +19,7 @@
 //     (two per clock and SM quarter); each waits for the other in turn through the two row tiles.
 //     4 x 2048 queries over 8192 tokens, 32 heads on 8, CQ-8c8b: 3.20 ms with m16n8k16 MMAs and the
 //     tiles' fragments in registers, 1.36 ms with one MMA-issuing thread that did scores and sums in
-//     turn, 0.98 ms now, 0.57 ms being the contractions at the measured GEMM rate.
+//     turn, 0.95 ms now, 0.57 ms being the contractions at the measured GEMM rate.
 //   prefill_generic_kernel: any supported shape, one CTA per (sequence, query, head), plain loops.
 #include "cq_common.cuh"
 
@@ -299,12 +299,12 @@ prefill_tc_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, 
     }
     // ---- codebooks as fp16, code-major ([code][group][channel]): the lanes of a gather take different groups, so they
     // meet in no bank whatever the codes are.  For c = 2 (one word per centroid) group g sits in column
-    // 16 (g mod 4) + g / 4.  A warp takes 64 bytes of eight groups at a time: eight lines of memory per load, and at most
-    // 1, 2 or 4 lanes (c = 8, 4, 2) that meet in a bank of a store.  (Straight copies, whose stores met eight at a time,
-    // took 12.7 thousand cycles per CTA; 4 thousand are what the L2 takes to deliver 256 KB.)
+    // 16 (g mod 4) + g / 4.  A warp takes 64 bytes of eight groups at a time, a quarter of it two groups: two lines of
+    // memory per quarter of a load, and at most four lanes that meet in a bank of a store.  (Straight copies, whose stores
+    // met eight at a time, took 12.7 thousand cycles per CTA; 4 thousand are what the L2 takes to deliver 256 KB.)
     {
         constexpr int kTasks = 2 * 256, kBatch = 6, kWarps = C::kThreads / 32;
-        const int gl = kC == 8 ? (lane >> 1) & 7 : lane & 7, j = kC == 8 ? (lane >> 4) * 2 + (lane & 1) : lane >> 3;
+        const int gl = lane >> 2, j = lane & 3;
 #pragma unroll 1
         for (int i0 = warp; i0 < kTasks; i0 += kBatch * kWarps) {
             float4 x[kBatch];
