@@ -864,60 +864,67 @@ decode_pair_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc,
     __syncthreads();
 
     // ---------------------------------------------------------------- epilogue: bins x V centroids
-    // Lane = (hb', g) reads words `lane` of both planes of row j (heads hb' and 2 + hb', group g): a
-    // conflict-free row read; the centroid (g, j) is one 32-byte load.  A warp takes 32 rows; the
-    // eight warps' partial sums meet in shared memory (the K table is no longer needed).
+    // A warp takes four consecutive centroids of eight groups at a time, a lane one of them (32 bytes) for all four heads:
+    // whole lines of the codebook (a group per lane touched 16 lines per load, 12 thousand cycles per CTA).  The eight
+    // warps' partial sums meet in shared memory (the K table is no longer needed).
     {
-        const int g = lane & 15;
-        float acc0[8], acc1[8], l0 = 0.f, l1 = 0.f;
+        const int gl = lane >> 2, jl = lane & 3, g = 8 * (warp & 1) + gl;
+        float acc[R][8], l[R];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) acc0[i] = acc1[i] = 0.f;
-        const float* cg = vcb + (((int64_t)hkv * 16 + g) * kRows + warp * (kRows / C::kWarps)) * 8;
-        const uint8_t* brow = smem + C::kVOffset + warp * (kRows / C::kWarps) * C::kVRowBytes + lane * 4;
+        for (int h = 0; h < R; ++h) {
+            l[h] = 0.f;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) acc[h][c] = 0.f;
+        }
+        const int j0 = 4 * (warp >> 1) + jl;
+        const float* cg = vcb + (((int64_t)hkv * 16 + g) * kRows + j0) * 8;
+        const uint8_t* brow = smem + C::kVOffset + j0 * C::kVRowBytes + g * 4;
+        constexpr int kStep = 4 * (C::kWarps / 2), kEach = kRows / kStep, kBatch = 8;        // codes between a warp's rows
+        static_assert(kEach % kBatch == 0 && C::kWarps % 2 == 0, "whole batches");
 #pragma unroll 1
-        for (int i0 = 0; i0 < kRows / C::kWarps; i0 += 8) {
-            float cv[8][8];                       // eight centroids in flight per lane (the loop's registers are free now)
+        for (int i0 = 0; i0 < kEach; i0 += kBatch) {
+            float cv[kBatch][8];                  // eight centroids in flight per lane (the loop's registers are free now)
 #pragma unroll
-            for (int i = 0; i < 8; ++i) load_centroid<8>(cg + (i0 + i) * 8, cv[i], cb_aligned32 != 0);
+            for (int i = 0; i < kBatch; ++i) load_centroid<8>(cg + (i0 + i) * kStep * 8, cv[i], cb_aligned32 != 0);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const float b0 = (float)*reinterpret_cast<const uint32_t*>(brow + (i0 + i) * C::kVRowBytes);
-                const float b1 = (float)*reinterpret_cast<const uint32_t*>(brow + (i0 + i) * C::kVRowBytes + 128);
-                l0 += b0;
-                l1 += b1;
+            for (int i = 0; i < kBatch; ++i) {
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    acc0[c] = fmaf(b0, cv[i][c], acc0[c]);
-                    acc1[c] = fmaf(b1, cv[i][c], acc1[c]);
+                for (int h = 0; h < R; ++h) {
+                    const float bv = (float)*reinterpret_cast<const uint32_t*>(brow + (i0 + i) * kStep * C::kVRowBytes + (h >> 1) * 128 + (h & 1) * 64);
+                    l[h] += bv;
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) acc[h][c] = fmaf(bv, cv[i][c], acc[h][c]);
                 }
             }
         }
-        float* red = reinterpret_cast<float*>(smem);                      // [warp][18][32]
+        // summed over the four lanes of a group; lane jl keeps head jl
+        const bool up2 = (lane & 2) != 0, up1 = (lane & 1) != 0;
+        auto fold = [&](float h0, float h1, float h2, float h3) {
+            const float x = (up2 ? h2 : h0) + __shfl_xor_sync(0xffffffffu, up2 ? h0 : h2, 2);
+            const float y = (up2 ? h3 : h1) + __shfl_xor_sync(0xffffffffu, up2 ? h1 : h3, 2);
+            return (up1 ? y : x) + __shfl_xor_sync(0xffffffffu, up1 ? x : y, 1);
+        };
+        static_assert(R == 4, "a head per lane of a group");
+        float* red = reinterpret_cast<float*>(smem);                      // [warp][9][32]
+#pragma unroll
+        for (int c = 0; c < 8; ++c) red[(warp * 9 + c) * 32 + lane] = fold(acc[0][c], acc[1][c], acc[2][c], acc[3][c]);
+        red[(warp * 9 + 8) * 32 + lane] = fold(l[0], l[1], l[2], l[3]);
         // an item of one part (out != null): its sums stay in the K table's place behind `red`
-        static_assert(C::kWarps * 18 * 32 * 4 <= 24 * 1024 && 24 * 1024 + R * 132 * 4 <= C::kKBytes, "room");
+        static_assert(C::kWarps * 9 * 32 * 4 <= 24 * 1024 && 24 * 1024 + R * 132 * 4 <= C::kKBytes, "room");
         float* sums = out ? reinterpret_cast<float*>(smem + 24 * 1024) : part_base;
         const int64_t sums_stride = out ? 132 : (int64_t)n_parts * stride;
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            red[(warp * 18 + c) * 32 + lane] = acc0[c];
-            red[(warp * 18 + 8 + c) * 32 + lane] = acc1[c];
-        }
-        red[(warp * 18 + 16) * 32 + lane] = l0;
-        red[(warp * 18 + 17) * 32 + lane] = l1;
         __syncthreads();
-        // 18 x 32 sums of eight terms: slot k < 16 of lane (hb', g) is channel g*8 + k%8 of head 2 (k/8) + hb';
-        // slots 16, 17 of the lanes with g = 0 are the normalisers (sum of the bins of group 0)
-        for (int o = threadIdx.x; o < 18 * 32; o += C::kThreads) {
-            const int slot = o >> 5, ln = o & 31;
+        // sums of four terms: slot c < 8 of lane (gl, h) is channel g * 8 + c of head h, in the warps of g's eight groups;
+        // slot 8 of group 0 is the normaliser (sum of its bins)
+        for (int o = threadIdx.x; o < 2 * 9 * 32; o += C::kThreads) {
+            const int oct = o >= 9 * 32, slot = (o >> 5) - 9 * oct, ln = o & 31;
             float v = 0.f;
 #pragma unroll
-            for (int w = 0; w < C::kWarps; ++w) v += red[(w * 18 + slot) * 32 + ln];
-            const int hb2 = ln >> 4, g2 = ln & 15;
-            if (slot < 16) {
-                const int h = 2 * (slot >> 3) + hb2;
-                sums[h * sums_stride + 2 + g2 * 8 + (slot & 7)] = v;
+            for (int w = 0; w < C::kWarps / 2; ++w) v += red[((2 * w + oct) * 9 + slot) * 32 + ln];
+            const int h = ln & 3, g2 = 8 * oct + (ln >> 2);
+            if (slot < 8) {
+                sums[h * sums_stride + 2 + g2 * 8 + slot] = v;
             } else if (g2 == 0) {
-                const int h = 2 * (slot - 16) + hb2;
                 sums[h * sums_stride + 0] = (float)ctl->head[h].e_cur + ctl->offset[h];   // reference exponent (log2 domain)
                 sums[h * sums_stride + 1] = v;                                            // normaliser, in the same unit
             }
