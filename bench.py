@@ -395,6 +395,12 @@ def extra_encode_cfg3(cq, dev, reps=5):
     res = {"workload": w.name, "ms": ms, "tokens_per_s": tokens / (ms * 1e-3), "vectors_per_s": vectors / (ms * 1e-3),
            "useful_tflops": vectors * 2 * D * (1 << w.b) / (ms * 1e-3) / 1e12,
            "gbs": (vectors * (D * 2 + w.G) + 2 * w.n_kv_heads * D * (1 << w.b) * 4) / (ms * 1e-3) / 1e9}
+    if w.c == 2 and w.b == 8:
+        # two-channel bulk inputs: a few centroids per vector out of per-cell lists, so the memory is the lower ceiling
+        res["roofline"] = {"bound": "hbm", "kernel": "encode_grid_kernel", "achieved": res["gbs"], "peak": measured_peaks()[0], "unit": "GB/s",
+                           "frac": res["gbs"] / measured_peaks()[0], "traffic": None, "peak_source": measured_peaks()[1] + " copy bandwidth"}
+        attach_traffic(res["roofline"], w.name)
+        return res
     # The selection over the 2^b scores of every (vector, group) bounds this kernel: the scores come out of the
     # tensor core into tensor memory, and every one of them has to pass through a min on the ALU pipe, 64 lanes
     # per clock and SM: at least 0.5 operations per score (one 3-input min per two scores).

@@ -304,9 +304,12 @@ int cq_decode_attn_variant(const void *q_fp16, const void *k_codes, const void *
  * warp per (vector, group) with the group's codebook in shared memory, which
  * variant 0 picks for appends of up to 128 vectors per head when the shape has no
  * tuned kernel (CQ_ERR_UNSUPPORTED when 2^b * c * 4 bytes exceed 48 KiB),
- * 4 = the bulk kernel with accumulators in tensor memory (head_dim 128, b = 8,
- * c in {2, 4, 8}, else CQ_ERR_UNSUPPORTED), which variant 0 picks for these shapes
- * once the input fills the device.  Every variant returns the same codes. */
+ * 4 = the kernel with accumulators in tensor memory (head_dim 128, b = 8,
+ * c in {2, 4, 8}, else CQ_ERR_UNSUPPORTED).  Variant 0 picks kernel 4 for these shapes
+ * and for b = 9 and 10, a kernel that looks up the centroids near a point of the plane
+ * for c = 2, b = 8 where the input pays for its tables, and one that reads a codebook
+ * once for all of up to 32 vectors.  Every variant returns the
+ * same codes. */
 int cq_encode_variant(const void *x_fp16, const float *codebooks, const int32_t *seq_offsets,
                       int64_t n_seq, int64_t n_tokens, int64_t token_offset, int64_t max_tokens,
                       int n_heads, int head_dim, int c, int b, void *codes_out, int variant,
