@@ -12,7 +12,9 @@
 // pairs (one 32-bit register each):
 //     A: x words | x words | x words | (1, 1)        | (X_hi, X_lo) | (1, 0)
 //     B: -2C_hi  | -2C_lo  | -2C_lo2 | (N_hi, N_lo)  | (1, 1)       | (N_lo2, 0)
-// (N = ||C_j||^2, X = ||x_g||^2; c = 8 needs two MMAs per tile, c = 4 drops N_lo2).
+// (N = ||C_j||^2, X = ||x_g||^2; c = 8 needs two MMAs per tile, c = 4 drops N_lo2).  fp16 ends at
+// 2^-24: x and C are first scaled by a power of two of their chunk of 256 centroids (EncCtl::scale),
+// so that the terms are as good for small channels as for channels of order one.
 // The accumulator lanes then keep, per vector, the smallest score of four subsets of their
 // columns, with the centroid index packed into the low mantissa byte (one 3-input min per two
 // scores).  The smallest of a quad's 16 subset minima names the winner's subset, whose 16
@@ -43,7 +45,8 @@ struct EncCfg {
 
 struct EncCtl {
     int range_flag[2];     // non-zero: the prepared group holds values fp16 cannot carry
-    float nmax[2];         // largest ||C_j||^2 of the prepared group (float bits, non-negative)
+    float nmax[2];         // largest ||C_j||^2 of the prepared group, scaled (float bits, non-negative)
+    float scale[2];        // its scale
 };
 
 __device__ __forceinline__ uint32_t pack_half2(float lo, float hi)
@@ -100,17 +103,25 @@ __device__ __forceinline__ void prepare_group(const float* __restrict__ cb_g, ui
             cv[4 % kC] = b.x; cv[5 % kC] = b.y; cv[6 % kC] = b.z; cv[7 % kC] = b.w;
         }
     }
-    float nrm = 0.f, amax = 0.f;
+    // The scale: the power of two s >= 1 that brings the largest of 32 channels spread over the centroids to [1, 2), as in
+    // tc_scale of the tensor-memory kernel, where the reasons are.  (Where 2^15 is not enough, nmax stays below 1 and
+    // no row is certain.)
+    const int lane = threadIdx.x & 31;
+    const uint32_t top = __reduce_max_sync(0xffffffffu, __float_as_uint(cb_g[lane * (8 * kC) + lane % kC]) & 0x7fffffffu);
+    const int k = 127 - (int)(top >> 23);
+    const float scale = __uint_as_float((uint32_t)(127 + (k < 0 ? 0 : (k > 15 ? 15 : k))) << 23);
+    if (threadIdx.x == 0) ctl->scale[slot] = scale;
+    float nrm = 0.f;
     float t0[kC], t1[kC], t2[kC];
 #pragma unroll
     for (int i = 0; i < kC; ++i) {
         nrm = fmaf(cv[i], cv[i], nrm);
-        amax = fmaxf(amax, fabsf(cv[i]));
-        split3(-2.f * cv[i], t0[i], t1[i], t2[i]);
+        split3(-2.f * scale * cv[i], t0[i], t1[i], t2[i]);
     }
+    nrm *= scale * scale;
     float n0, n1, n2;
     split3(nrm, n0, n1, n2);
-    if (!(amax < 16000.f) || !(nrm < 60000.f)) atomicOr(&ctl->range_flag[slot], 1);
+    if (!(nrm < 60000.f)) atomicOr(&ctl->range_flag[slot], 1);
     atomicMax(reinterpret_cast<int*>(&ctl->nmax[slot]), __float_as_int(nrm));
     const uint32_t ones = 0x3c003c00u;               // half2(1, 1)
     uint32_t pr[EncCfg<kC>::kSteps][8];
@@ -154,8 +165,8 @@ __device__ __forceinline__ void prepare_group(const float* __restrict__ cb_g, ui
 }
 
 // The A operand of one m-tile for one group, from the x words this lane owns.
-// xw[half] is the 32-bit word (two channels) of row r (half 0) / r + 8 (half 1) that lane p uses,
-// X[half] the squared norm of the row's group.
+// xw[half] is the (scaled) 32-bit word (two channels) of row r (half 0) / r + 8 (half 1) that lane p uses,
+// X[half] the squared norm of the row's group, scaled as well.
 template <int kC>
 __device__ __forceinline__ void build_a(const uint32_t (&xw)[2], const float (&X)[2], int p,
                                         uint32_t (&a)[EncCfg<kC>::kSteps][4])
@@ -279,7 +290,8 @@ encode_tuned_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1
         const int cur = st & 1;
         __syncthreads();                       // bbuf[cur] is complete; bbuf[cur ^ 1] is no longer read
         const bool out_of_range = ctl->range_flag[cur] != 0;
-        const float nmax = ctl->nmax[cur];
+        const float nmax = ctl->nmax[cur], scale = ctl->scale[cur];
+        const __half2 scale2 = __float2half2_rn(scale);
         __syncthreads();                       // everyone has read the control words of `cur`
         if (threadIdx.x == 0) { ctl->range_flag[cur ^ 1] = 0; ctl->nmax[cur ^ 1] = 0.f; }
         __syncthreads();
@@ -294,25 +306,29 @@ encode_tuned_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1
         for (int mt = 0; mt < kMT; ++mt) {
             uint32_t xw[2];
             float X[2];
+            auto scaled = [&](uint32_t w) {    // exact, or infinite: the row's scores are NaN then, and it is not certain
+                const __half2 f = __hmul2(*reinterpret_cast<const __half2*>(&w), scale2);
+                return *reinterpret_cast<const uint32_t*>(&f);
+            };
 #pragma unroll
             for (int hf = 0; hf < 2; ++hf) {
                 const int64_t v = v0 + mt * 16 + r + 8 * hf;
-                xw[hf] = 0u;
+                xwreg[mt][hf] = 0u;
                 X[hf] = 0.f;
                 if (v < n_vec) {
                     const uint32_t* gp = reinterpret_cast<const uint32_t*>(xrow0 + (mt * 16 + r + 8 * hf) * row_stride + g * kC);
-                    xw[hf] = gp[wsel];
+                    xwreg[mt][hf] = gp[wsel];
                     // squared norm of the whole group (every lane of the quad computes the same value)
 #pragma unroll
                     for (int w = 0; w < kC / 2; ++w) {
-                        const uint32_t ww = (kC == 2) ? xw[hf] : gp[w];
+                        const uint32_t ww = scaled((kC == 2) ? xwreg[mt][hf] : gp[w]);
                         const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&ww));
                         X[hf] = fmaf(f.x, f.x, X[hf]);
                         X[hf] = fmaf(f.y, f.y, X[hf]);
                     }
                 }
+                xw[hf] = scaled(xwreg[mt][hf]);
                 Xrow[mt][hf] = X[hf];
-                xwreg[mt][hf] = xw[hf];
             }
             build_a<kC>(xw, X, p, a[mt]);
         }
@@ -422,10 +438,11 @@ encode_tuned_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1
                 }
                 const int64_t v = v0 + mt * 16 + r + 8 * hf;
                 const float ss = __uint_as_float(__float_as_uint(s2) & keep);
-                // Evaluation error of a score: fp32 accumulation of up to ~20 terms bounded by
-                // 2 (X + N) in magnitude, plus the mantissa byte given to the index.  dbest is exact.
+                // Evaluation error of a score (of the scaled values): fp32 accumulation of up to ~20 terms bounded by
+                // 2 (X + N) in magnitude, what the fp16 terms leave of them, and the mantissa byte given to the index.
+                // dbest is exact, and its scaling too.
                 const float tau = 1.6e-5f * (Xrow[mt][hf] + nmax) + 6.2e-5f * fabsf(ss);
-                const bool certain = !out_of_range && (ss - dbest > tau);
+                const bool certain = !out_of_range && nmax >= 1.f && (ss - dbest * scale * scale > tau);
                 // exact recomputation of the uncertain rows, one row at a time by the whole warp
                 unsigned pending = __ballot_sync(0xffffffffu, !certain && p == 0 && v < n_vec);
                 while (pending) {

@@ -9,7 +9,9 @@
 // tcgen05.mma (M = 128, N = 128, K = 16; two of them, accumulating, for c = 8) evaluates
 //     d_j ~ ||x_g||^2 - 2 <x_g, C_j> + ||C_j||^2
 // with the fp32 centroids and norms carried as sums of three fp16 terms, so that every product is
-// exact and only the fp32 accumulation rounds.  K slots, in pairs:
+// exact and only the fp32 accumulation rounds.  fp16 ends at 2^-24: vectors and centroids of a group
+// are first scaled by a power of two (tc_scale), so that the terms are as good for channels of
+// standard deviation 0.001 as for channels of standard deviation 1.  K slots, in pairs:
 //     c = 2   A: x | x | x | (1,1) | (X_hi,X_lo) | (1,0) | 0 | 0
 //             B: t0 | t1 | t2 | (N_hi,N_lo) | (1,1) | (N_lo2,0) | 0 | 0        (-2C = t0 + t1 + t2)
 //     c = 4   A: x x | x x | x x | (1,1) | (X_hi,X_lo)      B: t0 t0 | t1 t1 | t2 t2 | (N_hi,N_lo) | (1,1)
@@ -205,22 +207,39 @@ __device__ __noinline__ int tc_exact_code(const float* __restrict__ cb_g, int n_
     return arg;
 }
 
-// B operand of one chunk, one centroid: K slots as in the header comment; every warp leaves its largest squared norm and its range flag of this pass in the control block.
+// The scale of a group: the power of two s >= 1 that brings the largest of 32 channels spread over the centroids of a
+// chunk (the same ones in every warp: no exchange between warps, and no load that waits for another) to [1, 2).  Larger
+// ones stay: fp16 carries them, and a vector's channels would lose their last bits to a scale below one.  Whatever the
+// other channels are, the largest squared norm N of the scaled centroids is then at least 1, and what three fp16 terms
+// leave of a channel or a norm is 2^-25 at most.  Where s would have to exceed 2^15, N stays below 1 and no row is
+// certain; where another centroid is so much larger (a hundred times) that fp16 does not carry its norm, neither.
+// (The largest norm of all centroids instead took a barrier more: 8192 vectors x 32 heads, c = 8, 227 against 215 us,
+// 211 without any scale and with wrong codes below a standard deviation of 0.03.)
 template <int kC>
-__device__ __forceinline__ void tc_prepare_b(const float (&cv)[kC], int j, unsigned char* bbuf, TcCtl* ctl, int slot, int pass)
+__device__ __forceinline__ float tc_scale(const float* __restrict__ cb_g)
+{
+    const int lane = threadIdx.x & 31;
+    const uint32_t top = __reduce_max_sync(0xffffffffu, __float_as_uint(cb_g[lane * (8 * kC) + lane % kC]) & 0x7fffffffu);
+    const int k = 127 - (int)(top >> 23);
+    return __uint_as_float((uint32_t)(127 + (k < 0 ? 0 : (k > 15 ? 15 : k))) << 23);
+}
+
+// B operand of one chunk, one centroid (scaled): K slots as in the header comment; every warp leaves its largest squared norm and its range flag of this pass in the control block.
+template <int kC>
+__device__ __forceinline__ void tc_prepare_b(const float (&cv)[kC], float scale, int j, unsigned char* bbuf, TcCtl* ctl, int slot, int pass)
 {
     using C = TcCfg<kC, 1>;
-    float nrm = 0.f, amax = 0.f;
+    float nrm = 0.f;
     float t0[kC], t1[kC], t2[kC];
 #pragma unroll
     for (int i = 0; i < kC; ++i) {
         nrm = fmaf(cv[i], cv[i], nrm);
-        amax = fmaxf(amax, fabsf(cv[i]));
-        tc_split3(-2.f * cv[i], t0[i], t1[i], t2[i]);
+        tc_split3(-2.f * scale * cv[i], t0[i], t1[i], t2[i]);
     }
+    nrm *= scale * scale;
     float n0, n1, n2;
     tc_split3(nrm, n0, n1, n2);
-    const bool bad = !(amax < 16000.f) || !(nrm < 60000.f);
+    const bool bad = !(nrm < 60000.f);
     const unsigned any_bad = __ballot_sync(0xffffffffu, bad);
     const float wmax = __uint_as_float(__reduce_max_sync(0xffffffffu, bad ? 0u : __float_as_uint(nrm)));   // nrm >= 0: bits order as values
     if ((threadIdx.x & 31) == 0) {
@@ -391,29 +410,35 @@ encode_tc_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, c
         if (v < n_vec) tc_fetch_x<kC>(x + (v * n_heads + h) * 128 + (g_begin + (rs >> log_rt)) * kC, xw_pf);
     };
     uint32_t xw_nxt[kC / 2];
-    float X_nxt = 0.f;
+    float X_nxt = 0.f, scale = 1.f;                      // squared norm of the scaled vector; scale of the group built last
     // what step st needs and its predecessor has not left: the chunk's centroids (first row tile of a group), the row
     // tile's vectors (first chunk)
     auto build = [&](int st) {
         const int rs = st / kChunks, ch = st % kChunks, slot = slot_of(st);
         if ((rs & rt_mask) == 0) {                       // centroids threadIdx.x and threadIdx.x + 128 of the chunk
             const float* cb_g = cb + (((int64_t)h * G + g_begin + (rs >> log_rt)) * kChunks + ch) * 256 * kC;
+            if (ch == 0) scale = tc_scale<kC>(cb_g);
             float cv[2][kC];
             tc_fetch_centroid<kC>(cb_g, threadIdx.x, cv[0]);
             tc_fetch_centroid<kC>(cb_g, threadIdx.x + 128, cv[1]);
-            tc_prepare_b<kC>(cv[0], threadIdx.x, b_buf(slot), ctl, slot, 0);
-            tc_prepare_b<kC>(cv[1], threadIdx.x + 128, b_buf(slot), ctl, slot, 1);
+            tc_prepare_b<kC>(cv[0], scale, threadIdx.x, b_buf(slot), ctl, slot, 0);
+            tc_prepare_b<kC>(cv[1], scale, threadIdx.x + 128, b_buf(slot), ctl, slot, 1);
         }
         if (ch != 0) return;
+        // (the scaled channels are exact, or infinite: the row's scores are NaN then, and it is not certain)
         X_nxt = 0.f;
+        uint32_t xs[kC / 2];
+        const __half2 scale2 = __float2half2_rn(scale);
 #pragma unroll
         for (int w = 0; w < kC / 2; ++w) {
             xw_nxt[w] = xw_pf[w];
-            const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&xw_pf[w]));
+            const __half2 v = __hmul2(*reinterpret_cast<const __half2*>(&xw_pf[w]), scale2);
+            xs[w] = *reinterpret_cast<const uint32_t*>(&v);
+            const float2 f = __half22float2(v);
             X_nxt = fmaf(f.x, f.x, X_nxt);
             X_nxt = fmaf(f.y, f.y, X_nxt);
         }
-        tc_build_a<kC>(xw_pf, X_nxt, a_buf(rs), row);
+        tc_build_a<kC>(xs, X_nxt, a_buf(rs), row);
     };
     // the MMA of one half of step st (half 1 = centroids 128 ... 255), then the commit that arrives on that half's
     // barrier when it is done
@@ -553,12 +578,15 @@ encode_tc_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, c
         }
         int code = (int)((__float_as_uint(m1) & kRowBits) << 4) | (int)(__float_as_uint(c1) & 15u);
         // Every centroid but the named one lies in another row or another column of the grid, so its score is at least
-        // the smaller of the two second minima.  tau bounds the evaluation error of two scores: an MMA adds 17 exact
-        // terms of at most X + N each, aligned to the largest and cut below its last fp32 bit (17 x 2^-23 (X + N); two
-        // MMAs for c = 8), plus the mantissa bits given to the indexes.
+        // the smaller of the two second minima.  tau bounds, for two scores and in units of X + N (of the scaled values,
+        // N = nmax): the sums of an MMA, exact terms of at most X + N each, aligned to the largest and cut below its last
+        // fp32 bit (11, 16 and, in two MMAs, 30 of them: 2.7e-6, 3.9e-6, 7.2e-6 for c = 2, 4, 8); the rounding of the exact
+        // distances that decide elsewhere, (c + 2) 2^-24 of at most 2 (X + N) each, and of the norms, c 2^-24 (1.3e-6,
+        // 2.0e-6, 3.4e-6); what the fp16 terms leave (0.2e-6; 0.4e-6 for c = 4, whose norms have two); and, on top, the
+        // mantissa bits given to the indexes.
         const float gap = fminf(m2, c2) - fmaxf(m1, c1);
-        const float tau = (kC == 8 ? 1.2e-5f : 6e-6f) * (X + nmax) + (kRowBits == 15u ? 2.1e-6f : 8e-6f) * (fabsf(m2) + fabsf(m1));
-        const bool certain = scores_valid && !out_of_range && gap > tau;
+        const float tau = (kC == 8 ? 1.2e-5f : kC == 4 ? 6.5e-6f : 4.5e-6f) * (X + nmax) + (kRowBits == 15u ? 2.1e-6f : 8e-6f) * (fabsf(m2) + fabsf(m1));
+        const bool certain = scores_valid && !out_of_range && nmax >= 1.f && gap > tau;
         const int64_t off = offsets[(rs & rt_mask) * kTcThreads];
         // exact recomputation of the uncertain rows, one row at a time by the whole warp
         unsigned pending = __ballot_sync(0xffffffffu, !certain && off != -2);
