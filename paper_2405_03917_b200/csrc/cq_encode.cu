@@ -511,6 +511,8 @@ encode_few_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, 
     __shared__ unsigned long long near[kFewVecs][8];          // per vector and warp: (distance, centroid)
     const int g = blockIdx.x % G, h = blockIdx.x / G, n_heads = sh.n_kv_heads;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // launched ahead of the end of whatever lies before it in the stream, which may well write the codebooks (a k-means update)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     float cv[kPer][kC];
 #pragma unroll
     for (int u = 0; u < kPer; ++u) {
@@ -526,7 +528,6 @@ encode_few_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, 
             }
         }
     }
-    asm volatile("griddepcontrol.wait;" ::: "memory");       // (the codebooks are never written by the kernel ahead)
     for (int v0 = 0; v0 < n_vec; v0 += kFewVecs) {
         const int nv = n_vec - v0 < kFewVecs ? n_vec - v0 : kFewVecs;
         if (threadIdx.x < kFewVecs * kC) {
