@@ -267,7 +267,8 @@ int cq_decode_attn_rope_variant(const void *q_fp16, const void *k_codes, const v
  *
  * A query whose position is negative (seq_lens[s] < n_q_tokens) has nothing to attend and
  * gets a zero row.  No workspace.  head_dim 128 with one byte per code and c = 2, 4 or 8
- * (and a number of query heads per KV head that divides 64) runs on tensor cores: the
+ * (and a number of query heads per KV head that divides 64) runs on tensor cores (every
+ * wait inside that kernel is bounded; should one ever give up, the rows it held up are NaN): the
  * codes are turned back into fp16 vectors tile by tile, so results carry fp16 rounding of
  * the centroids and of the softmax weights (within the library's attention tolerance);
  * every other supported shape runs on a plain kernel.  CQ_ERR_SHAPE for n_q_tokens < 1 or

@@ -142,6 +142,7 @@ struct PfCtl {
     uint64_t q_full[2];                   // queries of the row tile are in tensor memory (one arrival per warp)
     uint64_t p_full[2];                   // its weights are (one arrival per warp)
     uint64_t pv_done[2];                  // the sums with those weights are done
+    uint64_t drained[2];                  // every MMA of the warp that issues the scores / the sums is done
     uint32_t tmem_base;
     int failed;                           // a wait gave up
 };
@@ -177,10 +178,14 @@ __device__ __forceinline__ void pf_arrive(uint64_t* bar)
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 // Waits for the phase with the given parity; gives up after a bounded number of polls, or when another wait has, and then
-// returns false: every role leaves its loop and the CTA ends.
+// returns false: the other roles leave their loops (by a vote: the lanes of a warp can come out of it with different
+// answers), the softmax warps run through theirs, in step and for nothing, and their rows become NaN.
+#ifndef CQ_PREFILL_POLLS
+#define CQ_PREFILL_POLLS (1 << 17)
+#endif
 __device__ __forceinline__ bool pf_wait(PfCtl* ctl, uint64_t* bar, uint32_t parity)
 {
-    for (int poll = 0; poll < (1 << 17); ++poll) {
+    for (int poll = 0; poll < CQ_PREFILL_POLLS; ++poll) {
         uint32_t done;
         asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
                      : "=r"(done) : "r"(smem_u32(bar)), "r"(parity) : "memory");
@@ -215,6 +220,19 @@ __device__ __forceinline__ bool pf_elect()
 __device__ __forceinline__ void pf_commit(uint64_t* bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+// Waits, also after another wait has given up, until the MMAs that this warp has issued are done with shared memory and
+// tensor memory: the CTA gives both back next.
+__device__ __forceinline__ void pf_drain(uint64_t* bar)
+{
+    if (pf_elect()) pf_commit(bar);
+    for (int poll = 0; poll < (1 << 20); ++poll) {
+        uint32_t done;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(done) : "r"(smem_u32(bar)) : "memory");
+        if (done) break;
+    }
+    __syncwarp();
 }
 
 #define CQ_R32(u) "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]), "=r"(u[8]), "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15]), "=r"(u[16]), "=r"(u[17]), "=r"(u[18]), "=r"(u[19]), "=r"(u[20]), "=r"(u[21]), "=r"(u[22]), "=r"(u[23]), "=r"(u[24]), "=r"(u[25]), "=r"(u[26]), "=r"(u[27]), "=r"(u[28]), "=r"(u[29]), "=r"(u[30]), "=r"(u[31])
@@ -280,6 +298,7 @@ prefill_tc_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, 
             pf_init(&ctl->q_full[t], 4);
             pf_init(&ctl->p_full[t], 4);
             pf_init(&ctl->pv_done[t], 1);
+            pf_init(&ctl->drained[t], 1);
         }
         ctl->failed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -454,6 +473,8 @@ prefill_tc_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, 
         if (n_work > 0) {
             if (n_halves == 2) go(std::integral_constant<int, 2>());
             else go(std::integral_constant<int, 1>());
+            __syncwarp();
+            pf_drain(&ctl->drained[0]);
         }
     } else if (warp == C::kSumWarp) {
         // ---------------------------------------------------------------- sums: P Vhat, in the same order
@@ -486,6 +507,8 @@ prefill_tc_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, 
         if (n_work > 0) {
             if (n_halves == 2) go(std::integral_constant<int, 2>());
             else go(std::integral_constant<int, 1>());
+            __syncwarp();
+            pf_drain(&ctl->drained[1]);
         }
     } else if (warp < 4 * n_halves) {
         // ---------------------------------------------------------------- softmax: a thread per row
@@ -516,7 +539,7 @@ prefill_tc_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, 
         float m = -INFINITY, l = 0.f;                                       // reference of the weights (log2 domain), their sum
         bool ok = true;
         for (int jt = 0; jt < n_tiles; ++jt) {
-            if (!pf_wait(ctl, &ctl->s_full[t], (uint32_t)jt & 1u)) { ok = false; break; }
+            ok &= pf_wait(ctl, &ctl->s_full[t], (uint32_t)jt & 1u);
             pf_fence_after();
             uint32_t a[32], b[32];
             pf_ld32(a, s_addr);
@@ -582,7 +605,7 @@ prefill_tc_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, 
             }
             l += l0 + l1;
             if (jt > 0) {                                                   // the last sums are done with the weights' columns
-                if (!pf_wait(ctl, &ctl->pv_done[t], (uint32_t)(jt - 1) & 1u)) { ok = false; break; }
+                ok &= pf_wait(ctl, &ctl->pv_done[t], (uint32_t)(jt - 1) & 1u);
                 pf_fence_after();
                 if (rescale) {
 #pragma unroll 1
@@ -604,9 +627,11 @@ prefill_tc_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, 
         }
         // ---- normalise and write: through shared memory (the codebooks are done with when the last sums are), so that the
         // stores take whole lines; a thread per row wrote 32 lines at a time (10.8 thousand cycles per CTA)
-        if (n_tiles > 0) ok = ok && pf_wait(ctl, &ctl->pv_done[t], (uint32_t)(n_tiles - 1) & 1u);
+        if (n_tiles > 0) ok &= pf_wait(ctl, &ctl->pv_done[t], (uint32_t)(n_tiles - 1) & 1u);
+        ok = __all_sync(0xffffffffu, ok);
         pf_fence_after();
-        const float inv = ok && l > 0.f ? 1.f / l : 0.f;                    // no position: zero row
+        // no position: zero row; a wait gave up: NaN rows, so that nothing takes them for a result
+        const float inv = !ok ? __int_as_float(0x7fffffff) : l > 0.f ? 1.f / l : 0.f;
         uint8_t* block = smem + warp * 32 * C::kOutStride;
 #pragma unroll 1
         for (int c0 = 0; c0 < 128; c0 += 32) {
@@ -633,7 +658,7 @@ prefill_tc_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, 
         }
         pf_fence_before();
     }
-    // every MMA that was issued has been waited for (or a wait gave up); hand the tensor memory back
+    // every MMA that was issued has been waited for; hand the tensor memory back
     __syncthreads();
     if (warp == C::kMmaWarp) {
         pf_fence_after();
