@@ -69,7 +69,23 @@ bool hold_codes(const at::Tensor& k, const at::Tensor& v, int64_t n_seq, int64_t
     return k.numel() >= need && v.numel() >= need;
 }
 
-PyObject* status(int st) { return PyLong_FromLong(st); }
+// The status of a library call, which runs without the interpreter's lock: a launch waits where the launch queue is full
+// (and the host step for the GPU), and other Python threads go on meanwhile.  (The arguments are taken under the lock; the
+// tensors live on in the caller's frame.)
+struct Unlocked {
+    PyThreadState* state = PyEval_SaveThread();
+    ~Unlocked() { PyEval_RestoreThread(state); }
+};
+template <typename... Params, typename... A>
+PyObject* call(int (*function)(Params...), A... a)
+{
+    int st;
+    {
+        Unlocked unlocked;
+        st = function(a...);
+    }
+    return PyLong_FromLong(st);
+}
 
 constexpr auto kHalf = c10::ScalarType::Half;
 constexpr auto kFloat = c10::ScalarType::Float;
@@ -91,9 +107,9 @@ PyObject* decode_step(PyObject*, PyObject* const* argv, Py_ssize_t n)
     const int64_t ns = q->size(0), hq = q->size(1), D = q->size(2), hkv = kb->size(0);
     if (!is_shape(*kn, {ns, hkv, D}) || !is_shape(*vn, {ns, hkv, D}) || sl->numel() != ns || !hold_codes(*kc, *vc, ns, cap, hkv, D, c, b))
         Py_RETURN_NONE;
-    return status(cq_decode_step(q->data_ptr(), kn->data_ptr(), vn->data_ptr(), (const int32_t*)sl->data_ptr(), kc->data_ptr(), vc->data_ptr(),
-                                 (const float*)kb->data_ptr(), (const float*)vb->data_ptr(), scale, (int)ns, (int)hq, (int)hkv, (int)D, c, b,
-                                 cap, (float*)out->data_ptr(), ws->data_ptr(), (size_t)ws->numel(), current_stream()));
+    return call(cq_decode_step, q->data_ptr(), kn->data_ptr(), vn->data_ptr(), (const int32_t*)sl->data_ptr(), kc->data_ptr(), vc->data_ptr(),
+                (const float*)kb->data_ptr(), (const float*)vb->data_ptr(), scale, (int)ns, (int)hq, (int)hkv, (int)D, c, b,
+                cap, (float*)out->data_ptr(), ws->data_ptr(), (size_t)ws->numel(), current_stream());
 }
 
 // q, k_new, v_new, seq_lens (host), k_codes, v_codes, k_cb, v_cb, scale, c, b, max_tokens, out (host), workspace
@@ -109,14 +125,9 @@ PyObject* decode_step_host(PyObject*, PyObject* const* argv, Py_ssize_t n)
     const at::Tensor *out = a.host(12, kFloat), *ws = a.device(13, kByte);
     if (!a.ok || q->dim() != 3 || kb->dim() < 1) Py_RETURN_NONE;
     const int64_t ns = q->size(0), hq = q->size(1), D = q->size(2), hkv = kb->size(0);
-    int st;
-    void* stream = current_stream();
-    Py_BEGIN_ALLOW_THREADS                                  // this call waits for the GPU
-    st = cq_decode_step_host(q->data_ptr(), kn->data_ptr(), vn->data_ptr(), (const int32_t*)sl->data_ptr(), kc->data_ptr(), vc->data_ptr(),
-                             (const float*)kb->data_ptr(), (const float*)vb->data_ptr(), scale, (int)ns, (int)hq, (int)hkv, (int)D, c, b, cap,
-                             (float*)out->data_ptr(), ws->data_ptr(), (size_t)ws->numel(), stream);
-    Py_END_ALLOW_THREADS
-    return status(st);
+    return call(cq_decode_step_host, q->data_ptr(), kn->data_ptr(), vn->data_ptr(), (const int32_t*)sl->data_ptr(), kc->data_ptr(), vc->data_ptr(),
+                (const float*)kb->data_ptr(), (const float*)vb->data_ptr(), scale, (int)ns, (int)hq, (int)hkv, (int)D, c, b, cap,
+                (float*)out->data_ptr(), ws->data_ptr(), (size_t)ws->numel(), current_stream());
 }
 
 // q, k_codes, v_codes, k_cb, v_cb, seq_lens, scale, c, b, max_tokens, out, workspace, variant
@@ -134,9 +145,9 @@ PyObject* decode_attn(PyObject*, PyObject* const* argv, Py_ssize_t n)
     if (!a.ok || q->dim() != 3 || kb->dim() != 4) Py_RETURN_NONE;
     const int64_t ns = q->size(0), hq = q->size(1), D = q->size(2), hkv = kb->size(0);
     if (!is_book(*kb, hkv, D, c, b) || !is_book(*vb, hkv, D, c, b) || sl->numel() != ns || !hold_codes(*kc, *vc, ns, cap, hkv, D, c, b)) Py_RETURN_NONE;
-    return status(cq_decode_attn_variant(q->data_ptr(), kc->data_ptr(), vc->data_ptr(), (const float*)kb->data_ptr(), (const float*)vb->data_ptr(),
-                                         (const int32_t*)sl->data_ptr(), scale, (int)ns, (int)hq, (int)hkv, (int)D, c, b, cap,
-                                         (float*)out->data_ptr(), ws->data_ptr(), (size_t)ws->numel(), variant, current_stream()));
+    return call(cq_decode_attn_variant, q->data_ptr(), kc->data_ptr(), vc->data_ptr(), (const float*)kb->data_ptr(), (const float*)vb->data_ptr(),
+                (const int32_t*)sl->data_ptr(), scale, (int)ns, (int)hq, (int)hkv, (int)D, c, b, cap,
+                (float*)out->data_ptr(), ws->data_ptr(), (size_t)ws->numel(), variant, current_stream());
 }
 
 // q, k_codes, v_codes, k_cb, v_cb, seq_lens, rope_cos, rope_sin, scale, c, b, max_tokens, pairing, out, workspace, variant
@@ -155,10 +166,10 @@ PyObject* decode_attn_rope(PyObject*, PyObject* const* argv, Py_ssize_t n)
     if (!a.ok || q->dim() != 3 || kb->dim() < 1) Py_RETURN_NONE;
     const int64_t ns = q->size(0), hq = q->size(1), D = q->size(2), hkv = kb->size(0);
     if (!is_shape(*cs, {cap, D / 2}) || !is_shape(*sn, {cap, D / 2}) || !hold_codes(*kc, *vc, ns, cap, hkv, D, c, b)) Py_RETURN_NONE;
-    return status(cq_decode_attn_rope_variant(q->data_ptr(), kc->data_ptr(), vc->data_ptr(), (const float*)kb->data_ptr(), (const float*)vb->data_ptr(),
-                                              (const int32_t*)sl->data_ptr(), (const float*)cs->data_ptr(), (const float*)sn->data_ptr(), pairing,
-                                              scale, (int)ns, (int)hq, (int)hkv, (int)D, c, b, cap, (float*)out->data_ptr(), ws->data_ptr(),
-                                              (size_t)ws->numel(), variant, current_stream()));
+    return call(cq_decode_attn_rope_variant, q->data_ptr(), kc->data_ptr(), vc->data_ptr(), (const float*)kb->data_ptr(), (const float*)vb->data_ptr(),
+                (const int32_t*)sl->data_ptr(), (const float*)cs->data_ptr(), (const float*)sn->data_ptr(), pairing,
+                scale, (int)ns, (int)hq, (int)hkv, (int)D, c, b, cap, (float*)out->data_ptr(), ws->data_ptr(),
+                (size_t)ws->numel(), variant, current_stream());
 }
 
 // q, k_codes, v_codes, k_cb, v_cb, seq_lens, scale, c, b, max_tokens, out, variant
@@ -177,9 +188,9 @@ PyObject* prefill_attn(PyObject*, PyObject* const* argv, Py_ssize_t n)
     const int64_t ns = q->size(0), nq = q->size(1), hq = q->size(2), D = q->size(3), hkv = kb->size(0);
     if (nq > INT_MAX || !is_book(*kb, hkv, D, c, b) || !is_book(*vb, hkv, D, c, b) || sl->numel() != ns || !hold_codes(*kc, *vc, ns, cap, hkv, D, c, b))
         Py_RETURN_NONE;
-    return status(cq_prefill_attn_variant(q->data_ptr(), kc->data_ptr(), vc->data_ptr(), (const float*)kb->data_ptr(), (const float*)vb->data_ptr(),
-                                          (const int32_t*)sl->data_ptr(), scale, (int)ns, (int)nq, (int)hq, (int)hkv, (int)D, c, b, cap,
-                                          (float*)out->data_ptr(), variant, current_stream()));
+    return call(cq_prefill_attn_variant, q->data_ptr(), kc->data_ptr(), vc->data_ptr(), (const float*)kb->data_ptr(), (const float*)vb->data_ptr(),
+                (const int32_t*)sl->data_ptr(), scale, (int)ns, (int)nq, (int)hq, (int)hkv, (int)D, c, b, cap,
+                (float*)out->data_ptr(), variant, current_stream());
 }
 
 // x, codebooks, seq_offsets | None, c, b, codes_out, max_tokens, token_offset, variant
@@ -195,8 +206,8 @@ PyObject* encode(PyObject*, PyObject* const* argv, Py_ssize_t n)
     if (!a.ok || x->dim() != 4) Py_RETURN_NONE;
     const int64_t ns = x->size(0), nt = x->size(1), h = x->size(2), D = x->size(3);
     if (!is_book(*cb, h, D, c, b) || (so && so->numel() != ns) || !hold_codes(*codes, *codes, ns, cap, h, D, c, b)) Py_RETURN_NONE;
-    return status(cq_encode_variant(x->data_ptr(), (const float*)cb->data_ptr(), so ? (const int32_t*)so->data_ptr() : nullptr, ns, nt, offset, cap,
-                                    (int)h, (int)D, c, b, codes->data_ptr(), variant, current_stream()));
+    return call(cq_encode_variant, x->data_ptr(), (const float*)cb->data_ptr(), so ? (const int32_t*)so->data_ptr() : nullptr, ns, nt, offset, cap,
+                (int)h, (int)D, c, b, codes->data_ptr(), variant, current_stream());
 }
 
 // k, v, k_cb, v_cb, seq_offsets | None, c, b, k_codes, v_codes, max_tokens, token_offset
@@ -210,9 +221,9 @@ PyObject* encode_kv(PyObject*, PyObject* const* argv, Py_ssize_t n)
     const int64_t cap = a.integer(9), offset = a.integer(10);
     if (!a.ok || k->dim() != 4 || k->sizes() != v->sizes()) Py_RETURN_NONE;
     const int64_t ns = k->size(0), nt = k->size(1), h = k->size(2), D = k->size(3);
-    return status(cq_encode_kv(k->data_ptr(), v->data_ptr(), (const float*)kb->data_ptr(), (const float*)vb->data_ptr(),
-                               so ? (const int32_t*)so->data_ptr() : nullptr, ns, nt, offset, cap, (int)h, (int)D, c, b, kc->data_ptr(),
-                               vc->data_ptr(), current_stream()));
+    return call(cq_encode_kv, k->data_ptr(), v->data_ptr(), (const float*)kb->data_ptr(), (const float*)vb->data_ptr(),
+                so ? (const int32_t*)so->data_ptr() : nullptr, ns, nt, offset, cap, (int)h, (int)D, c, b, kc->data_ptr(),
+                vc->data_ptr(), current_stream());
 }
 
 #define CQ_METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&name)), METH_FASTCALL, nullptr}
