@@ -226,7 +226,19 @@ PyObject* encode_kv(PyObject*, PyObject* const* argv, Py_ssize_t n)
                 vc->data_ptr(), current_stream());
 }
 
-#define CQ_METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&name)), METH_FASTCALL, nullptr}
+// torch throws where a tensor has no memory (under tracing or vmap) or no current stream: no exception may leave for the
+// interpreter.  Nothing has been called then, and the wrapper's own checks meet the same error as a Python exception.
+template <PyObject* (*function)(PyObject*, PyObject* const*, Py_ssize_t)>
+PyObject* guarded(PyObject* self, PyObject* const* argv, Py_ssize_t n)
+{
+    try {
+        return function(self, argv, n);
+    } catch (...) {
+        Py_RETURN_NONE;
+    }
+}
+
+#define CQ_METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&guarded<&name>)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {CQ_METHOD(decode_step), CQ_METHOD(decode_step_host), CQ_METHOD(decode_attn), CQ_METHOD(decode_attn_rope),
                          CQ_METHOD(prefill_attn), CQ_METHOD(encode), CQ_METHOD(encode_kv), {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_cq_native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
