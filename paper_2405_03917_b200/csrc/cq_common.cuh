@@ -68,7 +68,7 @@ __host__ __device__ inline int partial_stride(int head_dim) { return head_dim + 
 // SM count of the current device (queried once per device and process).
 int device_sm_count();
 // cudaFuncAttributeMaxDynamicSharedMemorySize for `func`, set once per device and (func, bytes);
-// `slot` is a small integer unique to the call site (0 <= slot < 64).
+// `slot` is a small integer unique to the call site (0 <= slot < 96).
 cudaError_t ensure_dynamic_smem(const void* func, int bytes, int slot);
 
 // Launch plan of one tuned decode call: context chunk per CTA, partial slots per (sequence, query

@@ -1,4 +1,6 @@
-// Tuned encode kernels for head_dim 128, b = 8, c in {2, 4, 8} (CQ-2c8b, -4c8b, -8c8b).
+// Encode for head_dim 128, c in {2, 4, 8}, b in {8, 9, 10, 12}: which kernel takes an input (launch_encode_tuned), the
+// kernel of few vectors (encode_few_kernel, b <= 10) and the one on warp-level tensor-core instructions
+// (encode_tuned_kernel, described here), which takes b = 12 and, when it is asked for, the others.
 //
 // CQ encode (Section 3.2 of the paper, the map CQ(.) of Eq. 5): every group of c contiguous
 // channels of a vector is replaced by the index of its nearest centroid in L2 distance,
@@ -235,10 +237,9 @@ __device__ __forceinline__ int exact_code(const float (&xg)[kC], const float* __
 // kMT: 16-vector m-tiles per warp (4 for bulk encode, 1 when there are few vectors).
 // A launch covers one tensor, or two of the same shape (the key and the value of an append):
 // blockIdx.y picks (x, cb, codes) or (x2, cb2, codes2).
-// kWide: 2^b > 256 centroids per group (b = 9, 10, 12): the group's codebook is taken in chunks of
-// 256 centroids, each chunk exactly as a codebook of b = 8, and the chunk winners are compared by
-// their exact distances (the earlier chunk wins ties, so the lowest index still does).
-template <int kC, int kMT, bool kWide>
+// The group's codebook is taken in chunks of 256 centroids (one for b = 8), and the chunk winners are
+// compared by their exact distances (the earlier chunk wins ties, so the lowest index still does).
+template <int kC, int kMT>
 __global__ void __launch_bounds__(kEncThreads, 2)
 encode_tuned_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, const int32_t* __restrict__ seq_offsets,
                     Shape sh, int64_t n_tokens, int64_t token_offset, uint8_t* __restrict__ codes1, int groups_per_cta,
@@ -275,15 +276,15 @@ encode_tuned_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1
 
     if (threadIdx.x < 2) { ctl->range_flag[threadIdx.x] = 0; ctl->nmax[threadIdx.x] = 0.f; }
     __syncthreads();
-    const int n_chunks = kWide ? sh.K / 256 : 1;
+    const int n_chunks = sh.K / 256;
     const int n_steps = (g_end - g_begin) * n_chunks;
     // centroids of step st: chunk st % n_chunks of group g_begin + st / n_chunks
     auto chunk_ptr = [&](int st) {
         return cb + (((int64_t)h * G + g_begin + st / n_chunks) * n_chunks + st % n_chunks) * 256 * kC;
     };
     prepare_group<kC>(chunk_ptr(0), bbuf[0], ctl, 0);
-    float dkeep[kWide ? kMT : 1][2];           // best exact distance and code over the chunks seen so far
-    int ckeep[kWide ? kMT : 1][2];
+    float dkeep[kMT][2];                       // best exact distance and code over the chunks seen so far
+    int ckeep[kMT][2];
 
     for (int st = 0; st < n_steps; ++st) {
         const int g = g_begin + st / n_chunks, ch = st % n_chunks;
@@ -461,20 +462,17 @@ encode_tuned_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1
                     const int ec = exact_code<kC>(xg, cb_g, lane, &ed);
                     if ((lane & ~3) == src) { code = ec; dbest = ed; }
                 }
-                if (kWide) {
-                    // dbest is the exact distance of `code` within this chunk: keep the best chunk so far
-                    const int m = kWide ? mt : 0;
-                    if (ch == 0 || dbest < dkeep[m][hf]) { dkeep[m][hf] = dbest; ckeep[m][hf] = code + 256 * ch; }
-                    if (ch + 1 < n_chunks) continue;
-                    code = ckeep[m][hf];
-                }
+                // dbest is the exact distance of `code` within this chunk: keep the best chunk so far
+                if (ch == 0 || dbest < dkeep[mt][hf]) { dkeep[mt][hf] = dbest; ckeep[mt][hf] = code + 256 * ch; }
+                if (ch + 1 < n_chunks) continue;
+                code = ckeep[mt][hf];
                 if (p == 0 && v < n_vec) {
                     const int64_t s = v / n_tokens, i = v % n_tokens;
                     const int64_t pos = token_offset + (seq_offsets ? seq_offsets[s] : 0) + i;
                     if (pos >= 0 && pos < sh.max_tokens) {
                         const int k = (int)(pos % kTokenBlock);
                         codes[code_word_offset(sh, n_heads, s, h, pos / kTokenBlock, g) + k] = (uint8_t)code;
-                        if (kWide) {        // upper bits: replaced in the 32-bit word that other tokens share
+                        if (sh.hb) {        // upper bits: replaced in the 32-bit word that other tokens share
                             const int bit = k * sh.hb;
                             const uintptr_t a = reinterpret_cast<uintptr_t>(codes) +
                                                 (uintptr_t)code_high_offset(sh, n_heads, s, h, pos / kTokenBlock, g) + (bit >> 3);
@@ -597,7 +595,7 @@ cudaError_t launch_few(const __half* x, const float* cb, const int32_t* seq_offs
     return sh.b == 8 ? go(encode_few_kernel<kC, 1>) : sh.b == 9 ? go(encode_few_kernel<kC, 2>) : go(encode_few_kernel<kC, 4>);
 }
 
-template <int kC, int kMT, bool kWide = false>
+template <int kC, int kMT>
 cudaError_t launch_enc(const __half* x, const float* cb, const int32_t* seq_offsets, const Shape& sh, int64_t n_tokens,
                        int64_t token_offset, uint8_t* codes, cudaStream_t st, const __half* x2 = nullptr,
                        const float* cb2 = nullptr, uint8_t* codes2 = nullptr)
@@ -615,11 +613,11 @@ cudaError_t launch_enc(const __half* x, const float* cb, const int32_t* seq_offs
     const int64_t grid = tiles * sh.n_kv_heads * n_gsplit;
     if (grid > 0x7fffffff) return cudaErrorInvalidConfiguration;
     const size_t smem = (size_t)2 * C::kBufWords * 4 + sizeof(EncCtl);
-    // call-site slots of ensure_dynamic_smem: 16 ... 27, one per template instance
-    constexpr int kSlot = 16 + 4 * (kC == 2 ? 0 : kC == 4 ? 1 : 2) + 2 * (kMT == 1 ? 0 : 1) + (kWide ? 1 : 0);
-    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(encode_tuned_kernel<kC, kMT, kWide>), (int)smem, kSlot);
+    // call-site slots of ensure_dynamic_smem: 16 ... 21, one per template instance
+    constexpr int kSlot = 16 + 2 * (kC == 2 ? 0 : kC == 4 ? 1 : 2) + (kMT == 1 ? 0 : 1);
+    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(encode_tuned_kernel<kC, kMT>), (int)smem, kSlot);
     if (e != cudaSuccess) return e;
-    encode_tuned_kernel<kC, kMT, kWide><<<dim3((unsigned)grid, x2 ? 2u : 1u), kEncThreads, smem, st>>>(
+    encode_tuned_kernel<kC, kMT><<<dim3((unsigned)grid, x2 ? 2u : 1u), kEncThreads, smem, st>>>(
         x, cb, seq_offsets, sh, n_tokens, token_offset, codes, groups_per_cta, x2, cb2, codes2);
     return cudaGetLastError();
 }
@@ -652,17 +650,6 @@ cudaError_t launch_encode_tuned(const __half* x, const float* cb, const int32_t*
     if (allow_tc && encode_tc_supported(sh))
         return launch_encode_tc(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2);
     const bool few = n_vec * sh.n_kv_heads < (int64_t)device_sm_count() * 512 * 2;    // not enough vectors for 64 per warp
-    if (sh.b > 8) {
-        switch (sh.c) {
-            case 2: return few ? launch_enc<2, 1, true>(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2)
-                               : launch_enc<2, 4, true>(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2);
-            case 4: return few ? launch_enc<4, 1, true>(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2)
-                               : launch_enc<4, 4, true>(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2);
-            case 8: return few ? launch_enc<8, 1, true>(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2)
-                               : launch_enc<8, 4, true>(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2);
-            default: return cudaErrorNotSupported;
-        }
-    }
     switch (sh.c) {
         case 2: return few ? launch_enc<2, 1>(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2)
                            : launch_enc<2, 4>(x, cb, seq_offsets, sh, n_tokens, token_offset, codes, st, x2, cb2, codes2);
