@@ -15,7 +15,7 @@
 //     A: x words | x words | x words | (1, 1)        | (X_hi, X_lo) | (1, 0)
 //     B: -2C_hi  | -2C_lo  | -2C_lo2 | (N_hi, N_lo)  | (1, 1)       | (N_lo2, 0)
 // (N = ||C_j||^2, X = ||x_g||^2; c = 8 needs two MMAs per tile, c = 4 drops N_lo2).  fp16 ends at
-// 2^-24: x and C are first scaled by a power of two of their chunk of 256 centroids (EncCtl::scale),
+// 2^-24: x and C are first scaled by a power of two of their group (EncCtl::scale),
 // so that the terms are as good for small channels as for channels of order one.
 // The accumulator lanes then keep, per vector, the smallest score of four subsets of their
 // columns, with the centroid index packed into the low mantissa byte (one 3-input min per two
@@ -90,7 +90,7 @@ __device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], u
 // Layout: word (j * 8 + p * 2 + q) of a k-step holds slot pair p + 4 q of centroid j, so that
 // lane (n, p) of the MMA reads its (b0, b1) for centroid nt * 8 + n as one 8-byte word.
 template <int kC>
-__device__ __forceinline__ void prepare_group(const float* __restrict__ cb_g, uint32_t* buf, EncCtl* ctl, int slot)
+__device__ __forceinline__ void prepare_group(const float* __restrict__ cb_g, uint32_t* buf, EncCtl* ctl, int slot, bool first)
 {
     const int j = threadIdx.x;
     float cv[kC];
@@ -105,13 +105,16 @@ __device__ __forceinline__ void prepare_group(const float* __restrict__ cb_g, ui
             cv[4 % kC] = b.x; cv[5 % kC] = b.y; cv[6 % kC] = b.z; cv[7 % kC] = b.w;
         }
     }
-    // The scale: the power of two s >= 1 that brings the largest of 32 channels spread over the centroids to [1, 2), as in
-    // tc_scale of the tensor-memory kernel, where the reasons are.  (Where 2^15 is not enough, nmax stays below 1 and
-    // no row is certain.)
-    const int lane = threadIdx.x & 31;
-    const uint32_t top = __reduce_max_sync(0xffffffffu, __float_as_uint(cb_g[lane * (8 * kC) + lane % kC]) & 0x7fffffffu);
-    const int k = 127 - (int)(top >> 23);
-    const float scale = __uint_as_float((uint32_t)(127 + (k < 0 ? 0 : (k > 15 ? 15 : k))) << 23);
+    // The scale: the power of two s >= 1 that brings the largest of 32 channels spread over the centroids of the group's
+    // first chunk to [1, 2), as in tc_scale of the tensor-memory kernel, where the reasons are.  (Where 2^15 is not
+    // enough, nmax stays below 1 and no row is certain.)
+    float scale = ctl->scale[slot ^ 1];
+    if (first) {
+        const int lane = threadIdx.x & 31;
+        const uint32_t top = __reduce_max_sync(0xffffffffu, __float_as_uint(cb_g[lane * (8 * kC) + lane % kC]) & 0x7fffffffu);
+        const int k = 127 - (int)(top >> 23);
+        scale = __uint_as_float((uint32_t)(127 + (k < 0 ? 0 : (k > 15 ? 15 : k))) << 23);
+    }
     if (threadIdx.x == 0) ctl->scale[slot] = scale;
     float nrm = 0.f;
     float t0[kC], t1[kC], t2[kC];
@@ -282,7 +285,7 @@ encode_tuned_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1
     auto chunk_ptr = [&](int st) {
         return cb + (((int64_t)h * G + g_begin + st / n_chunks) * n_chunks + st % n_chunks) * 256 * kC;
     };
-    prepare_group<kC>(chunk_ptr(0), bbuf[0], ctl, 0);
+    prepare_group<kC>(chunk_ptr(0), bbuf[0], ctl, 0, true);
     float dkeep[kMT][2];                       // best exact distance and code over the chunks seen so far
     int ckeep[kMT][2];
 
@@ -296,7 +299,7 @@ encode_tuned_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1
         __syncthreads();                       // everyone has read the control words of `cur`
         if (threadIdx.x == 0) { ctl->range_flag[cur ^ 1] = 0; ctl->nmax[cur ^ 1] = 0.f; }
         __syncthreads();
-        if (st + 1 < n_steps) prepare_group<kC>(chunk_ptr(st + 1), bbuf[cur ^ 1], ctl, cur ^ 1);
+        if (st + 1 < n_steps) prepare_group<kC>(chunk_ptr(st + 1), bbuf[cur ^ 1], ctl, cur ^ 1, ch + 1 == n_chunks);
         const float* cb_g = chunk_ptr(st);
 
         // A operands of this warp's m-tiles
