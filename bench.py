@@ -395,23 +395,17 @@ def extra_encode_cfg3(cq, dev, reps=5):
     res = {"workload": w.name, "ms": ms, "tokens_per_s": tokens / (ms * 1e-3), "vectors_per_s": vectors / (ms * 1e-3),
            "useful_tflops": vectors * 2 * D * (1 << w.b) / (ms * 1e-3) / 1e12,
            "gbs": (vectors * (D * 2 + w.G) + 2 * w.n_kv_heads * D * (1 << w.b) * 4) / (ms * 1e-3) / 1e9}
-    if w.c == 2 and w.b == 8:
-        # two-channel bulk inputs: a few centroids per vector out of per-cell lists, so the memory is the lower ceiling
-        res["roofline"] = {"bound": "hbm", "kernel": "encode_grid_kernel", "achieved": res["gbs"], "peak": measured_peaks()[0], "unit": "GB/s",
-                           "frac": res["gbs"] / measured_peaks()[0], "traffic": None, "peak_source": measured_peaks()[1] + " copy bandwidth"}
-        attach_traffic(res["roofline"], w.name)
-        return res
-    # The selection over the 2^b scores of every (vector, group) bounds this kernel: the scores come out of the
-    # tensor core into tensor memory, and every one of them has to pass through a min on the ALU pipe, 64 lanes
-    # per clock and SM: at least 0.5 operations per score (one 3-input min per two scores).
-    pairs = vectors * w.G * (1 << w.b)
+    # Two-channel bulk inputs: a few centroids per vector out of per-box lists.  The issue slots bound the kernel: 142 warp
+    # instructions per 32 vectors of a group (counted with ncu as the difference of two input sizes; making the lists
+    # comes on top), four per clock and SM.  The memory is the other ceiling.
     props = torch.cuda.get_device_properties(dev)
     n_sm, mhz = props.multi_processor_count, props.clock_rate / 1e3
-    alu_peak = n_sm * 64 * mhz * 1e6
-    res["roofline"] = {"bound": "alu", "kernel": "encode_tc_kernel", "achieved": 0.5 * pairs / (ms * 1e-3), "peak": alu_peak,
-                       "unit": "lane-ops/s", "frac": 0.5 * pairs / (ms * 1e-3) / alu_peak, "traffic": None,
-                       "lane_ops_per_score": 0.5,
-                       "peak_source": f"64 ALU lanes/clk/SM x {n_sm} SMs x {mhz:.0f} MHz (device maximum)"}
+    issued, slots = 142.0 * vectors / 32 * w.G / (ms * 1e-3), 4.0 * n_sm * mhz * 1e6
+    hbm, which = measured_peaks()
+    res["roofline"] = {"bound": "issue", "kernel": "encode_grid_kernel", "achieved": issued, "peak": slots, "unit": "warp instructions/s",
+                       "frac": issued / slots, "instructions_per_32_vectors_of_a_group": 142, "traffic": None,
+                       "peak_source": f"4 warp instructions/clk/SM x {n_sm} SMs x {mhz:.0f} MHz (device maximum)",
+                       "hbm": {"achieved": res["gbs"], "peak": hbm, "unit": "GB/s", "frac": res["gbs"] / hbm, "peak_source": which + " copy bandwidth"}}
     attach_traffic(res["roofline"], w.name)
     return res
 

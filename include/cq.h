@@ -37,7 +37,8 @@
  *     exist for head_dim 128: encode for c = 2, 4, 8 with b = 8, 9, 10, 12 (codebooks
  *     of more than 256 centroids are taken in chunks of 256); for b = 8 decode attention
  *     for c = 8, 4 and 2 with any number of query heads per KV head (a CTA serves up to 4, 2, 1 of them);
- *     and for decode attention of CQ-8c10b (head_dim 128, c = 8, b = 10).
+ *     and for decode attention of CQ-8c10b (head_dim 128, c = 8, b = 10); for head_dim 64,
+ *     decode attention with b = 8 and c = 4 or 8.
  *     Every other supported shape runs on generic sm_100a kernels (never on the CPU).
  *   - Inputs must be finite.
  *
@@ -338,6 +339,9 @@ int cq_encode_variant(const void *x_fp16, const float *codebooks, const int32_t 
  * (assignment = cq_encode, then every centroid moves to the weighted mean of its members; a
  * centroid without members stays; codebooks_in and codebooks_out must differ);
  * cq_learn_centroids runs the initialisation and n_iters iterations.
+ *
+ * Up to 32768 vectors with c = 2, 4 or 8 a problem stays on chip for all of its draws; more vectors
+ * (and other c) take two launches per draw, several times longer for the initialisation.
  */
 size_t cq_learn_workspace_bytes(int64_t n_vec, int n_heads, int head_dim, int c, int b);
 int cq_kmeanspp_init(const void *x_fp16, const float *weights, const double *uniforms, int64_t n_vec,

@@ -150,7 +150,7 @@ int cq_encode_variant(const void* x_fp16, const float* codebooks, const int32_t*
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     // An append (a few vectors per head) is latency-bound.  Shapes without a tuned kernel take the
     // few-vector kernel for it (13 us against 300 us of the generic kernel for 64 vectors x 8 heads of
-    // CQ-8c8b); the tuned kernel's single-tile form is still faster where it exists (9 us).
+    // CQ-8c8b); the others have a kernel of their own for it (launch_encode_tuned).
     if (variant == 3 || (variant == 0 && !tuned_ok && small_ok && n_seq * n_tokens <= kSmallEncodeVectors)) {
         cudaError_t es = launch_encode_small(static_cast<const __half*>(x_fp16), codebooks, seq_offsets, sh, n_tokens,
                                              token_offset, static_cast<uint8_t*>(codes_out), cs);

@@ -95,7 +95,7 @@ cudaError_t launch_encode_generic(const __half* x, const float* cb, const int32_
 bool encode_small_supported(const Shape& sh);       // few-vector kernel: the group's codebook fits 48 KiB
 cudaError_t launch_encode_small(const __half* x, const float* cb, const int32_t* seq_offsets, const Shape& sh,
                                 int64_t n_tokens, int64_t token_offset, uint8_t* codes, cudaStream_t st);
-// tcgen05 / tensor-memory encode kernel (head_dim 128, b = 8, c in {2, 4, 8}); same arguments as launch_encode_tuned
+// tcgen05 / tensor-memory encode kernel (head_dim 128, b in {8, 9, 10}, c in {2, 4, 8}); same arguments as launch_encode_tuned
 bool encode_tc_supported(const Shape& sh);
 cudaError_t launch_encode_tc(const __half* x, const float* cb, const int32_t* seq_offsets, const Shape& sh, int64_t n_tokens,
                              int64_t token_offset, uint8_t* codes, cudaStream_t st, const __half* x2, const float* cb2,
@@ -107,7 +107,8 @@ cudaError_t launch_encode_grid(const __half* x, const float* cb, const int32_t* 
                                uint8_t* codes2);
 bool encode_tuned_supported(const Shape& sh);
 // (x2, cb2, codes2): an optional second tensor of the same shape, encoded by the same launch.
-// allow_tc: bulk inputs of byte codes go to the tensor-memory kernel (false: always the mma.sync kernels).
+// allow_tc: the kernel of few vectors, the plane kernel (c = 2) or the tensor-memory kernel where they apply, mma.sync for
+// b = 12 only (false: always mma.sync).
 cudaError_t launch_encode_tuned(const __half* x, const float* cb, const int32_t* seq_offsets, const Shape& sh,
                                 int64_t n_tokens, int64_t token_offset, uint8_t* codes, cudaStream_t st,
                                 const __half* x2 = nullptr, const float* cb2 = nullptr, uint8_t* codes2 = nullptr,

@@ -26,8 +26,8 @@
 // across subsets, out-of-range codebooks) the warp recomputes that (vector, group) over all 256
 // centroids exactly, lowest index on ties -- the arithmetic of the generic kernel.
 //
-// The selection, not the tensor pipe, is what bounds this kernel: the ALU pipe (min / logic,
-// 64 lanes per clock and SM) is about 77 % busy, the tensor pipe about 14 %.
+// No pipe bounds this kernel at b = 12 (2048 vectors x 8 heads, c = 8, 1.2 ms): issue slots and ALU pipe are 38 % busy,
+// warps wait for the chunk's centroids and for each other (a chunk of 256 is one step).
 #include "cq_common.cuh"
 
 namespace cq {

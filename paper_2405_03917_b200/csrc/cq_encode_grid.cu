@@ -18,9 +18,11 @@
 // all (tensor, head, set of eight groups, vector); a thread takes a vector through the eight groups.
 //
 // Measured (8 x 8192 tokens, 32 heads, key and value): 8.25 ms on the tensor-memory kernel before, 2.33 ms here, of
-// which the tables take 0.6 ms.  Bound: the issue slots (142 warp instructions per 32 vectors of a group: 28 find the
-// box, 40 evaluate a word's four centroids) at 70 %; the shared-memory pipe, where words and centroids are gathered
-// (six wavefronts per centroid and warp), at 40 %.
+// which the tables take 0.8 to 0.9 ms (what is left when the time is carried back to no vectors).  Bound: the issue
+// slots, 69 to 72 % busy (142 warp instructions per 32 vectors of a group: the difference of two inputs' counts; 28 find
+// the box, 40 evaluate a word's four centroids); the shared-memory pipe, where words and centroids are gathered (six
+// wavefronts per centroid and warp), is 60 % busy.  A vector's row is fetched from DRAM once per set of eight groups and
+// not once in all: a set reads 32 bytes of it, DRAM delivers more (4.3 GB read where the vectors are 1.07).
 #include "cq_common.cuh"
 
 namespace cq {
@@ -444,7 +446,8 @@ encode_grid_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1,
 
 // Making the tables of eight groups takes a CTA about 140 us, and a CTA makes those of its share of the units and of
 // one cut unit more; after that a vector of a head costs 1.8 ns less than on the tensor-memory kernel.  (32 heads, one
-// tensor: 4096 vectors 585 against 387 us, 8192 629 against 727, 65536 1298 against 4968.)
+// tensor: 6636 vectors, the first that come here, 567 against 557 us, 7000 573 against 580, 8192 585 against 674, 65536
+// 1212 against 4672.)
 bool encode_grid_pays(const Shape& sh, int64_t n_tokens, int n_tensors)
 {
     const int64_t n_vec = sh.n_seq * n_tokens;

@@ -28,9 +28,9 @@
 // recomputes that row over all centroids exactly: sum (x - C)^2 in fp32, lowest index on ties.
 // (Before, the winning column's 16 centroids were evaluated exactly from shared memory: at c = 8 the bank
 // conflicts of those reads kept the shared-memory pipe 74 % busy.  8192 vectors x 32 heads: c = 8
-// 350 -> 217 us.)  More than 256 centroids (b = 9, 10) come in chunks of 256 whose operands all
+// 350 -> 215 us.)  More than 256 centroids (b = 9, 10) come in chunks of 256 whose operands all
 // stay in shared memory while a row tile passes them; the grid then has 32 or 64 rows.  (CQ-8c10b,
-// 32768 vectors x 8 heads: 3.1 -> 1.2 ms against the mma.sync kernel.)
+// 32768 vectors x 8 heads: 3.1 -> 1.13 ms against the mma.sync kernel.)
 //
 // A CTA is one tile of 128 vectors of one head: 4 warps, warp w owning the tensor memory lanes
 // 32 w ... 32 w + 31, and 128 tensor-memory columns, so that four CTAs (fewer for wide codes, whose
@@ -76,7 +76,7 @@ constexpr int kTcColumns = 128;            // tensor-memory columns of a CTA
 
 struct TcCtl {
     int range_flag[4][8];      // per slot, warp and pass, non-zero: those centroids of the prepared chunk hold values fp16 cannot carry
-    float nmax[4][8];          // per slot, warp and pass, the largest ||C_j||^2 among those centroids
+    float nmax[4][8];          // per slot, warp and pass, the largest ||C_j||^2 among those centroids (scaled)
     uint32_t tmem_base;
     int wait_failed;           // a wait on an MMA barrier gave up
     uint64_t bar[2];           // completion of the MMA of the low / high half of a step
@@ -224,7 +224,8 @@ __device__ __forceinline__ float tc_scale(const float* __restrict__ cb_g)
     return __uint_as_float((uint32_t)(127 + (k < 0 ? 0 : (k > 15 ? 15 : k))) << 23);
 }
 
-// B operand of one chunk, one centroid (scaled): K slots as in the header comment; every warp leaves its largest squared norm and its range flag of this pass in the control block.
+// B operand of one chunk, one centroid (scaled): K slots as in the header comment; every warp leaves its largest squared
+// norm and its range flag of this pass in the control block.
 template <int kC>
 __device__ __forceinline__ void tc_prepare_b(const float (&cv)[kC], float scale, int j, unsigned char* bbuf, TcCtl* ctl, int slot, int pass)
 {

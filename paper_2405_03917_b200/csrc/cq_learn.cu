@@ -803,7 +803,8 @@ cudaLaunchConfig_t cluster_config(int grid, int threads, size_t smem, int cluste
 }
 
 // Cluster size of pp_cluster_kernel: what the vectors need, and more CTAs per problem while the device has room for
-// all of them at once (few problems: a draw is then shorter).  0: more vectors than a cluster holds.
+// all of them at once (few problems: a draw is then shorter).  0: more vectors than a cluster of portable size holds
+// (kPpMaxCluster * kPpSlice = 32768); the draws then take two launches each.
 int pp_cluster_size(int64_t n_vec, int n_prob)
 {
     int c = 1;
