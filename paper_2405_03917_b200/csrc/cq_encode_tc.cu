@@ -80,6 +80,7 @@ struct TcCtl {
     uint32_t tmem_base;
     int wait_failed;           // a wait on an MMA barrier gave up
     uint64_t bar[2];           // completion of the MMA of the low / high half of a step
+    uint64_t drained;          // completion of everything issued, after a wait gave up
 };
 
 __device__ __forceinline__ uint32_t tc_smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -375,6 +376,7 @@ encode_tc_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, c
     if (threadIdx.x == 32) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc_smem_u32(&ctl->bar[0])) : "memory");
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc_smem_u32(&ctl->bar[1])) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc_smem_u32(&ctl->drained)) : "memory");
         ctl->wait_failed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -636,7 +638,12 @@ encode_tc_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, c
         }
     }
 
-    // every MMA that was issued has been waited for (or the wait gave up); hand the tensor memory back
+    // Every MMA that was issued has been waited for; where a wait gave up (the rows since went the exact way), this is
+    // done now, with a limit again, by the thread that issues them.  Then the tensor memory goes back.
+    if (threadIdx.x == 0 && *reinterpret_cast<volatile int*>(&ctl->wait_failed) != 0) {
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(tc_smem_u32(&ctl->drained)) : "memory");
+        tc_wait(&ctl->drained, 0u);
+    }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0) {
