@@ -179,7 +179,7 @@ class DecodeState:
         self.ws = torch.empty(max(256, cq.cq_decode_step_workspace_bytes(w.n_seq, w.n_q_heads, w.n_kv_heads, D, c, b,
                                                                         self.cap)), dtype=torch.uint8, device=dev)
         self.scale = D ** -0.5
-        # launches of one cq_decode_step call: 1 or 2 where the attention kernel appends the token itself
+        # launches of one cq_decode_step call: up to 3 ([append,] attention [, merge]); 4: append and attention are calls of their own
         self.fused_launches = cq.cq_decode_step_launches(w.n_seq, w.n_q_heads, w.n_kv_heads, D, c, b, self.cap)
 
     def kv_tokens(self) -> int:
@@ -209,7 +209,7 @@ class DecodeState:
         """Append-encode the new token (K, V) at the last position, then attend: one cq_decode_step call where the
         kernel appends inside the attention launch, else cq_encode_kv followed by cq_decode_attn."""
         w = self.w
-        if self.fused_launches <= 2:
+        if self.fused_launches < 4:
             if ev is not None:
                 ev[0].record()
             cq.cq_decode_step(self.q, self.k_new, self.v_new, self.append_pos, self.k_codes, self.v_codes, self.k_cb,
@@ -268,7 +268,8 @@ def decode_roofline(w, st, ms, dev, sm_mhz=None):
     nbytes = st.algorithmic_bytes()
     t_hbm, t_smem = nbytes / (hbm * 1e9), lane_ops / smem_peak
     a_hbm, a_smem = nbytes / (ms * 1e-3) / 1e9, lane_ops / (ms * 1e-3)
-    merged = w.b == 10 or st.fused_launches != 1         # a merge launch follows unless the kernel writes the output itself
+    # a merge launch follows unless the kernel writes the output itself
+    merged = w.b == 10 or st.fused_launches != (1 if shared_word_kernel(w) else 2)
     o = {"kernel": ("decode_pair_kernel" if shared_word_kernel(w) else
                     "decode_wide_kernel" if w.b == 10 else "decode_tuned_kernel") +
                    (" + merge_kernel (one attention call)" if merged else " (one attention call; the kernel writes the output itself)"),
@@ -657,7 +658,7 @@ def main():
             "e2e": {"value": kv_tokens / (e2e_ms * 1e-3), "unit": UNIT, "h2d_bytes_per_step": h2d,
                     "d2h_bytes_per_step": d2h, "ms_per_step": e2e_ms},
             # per layer: attention (which appends the new token where the kernel can) and merge, else also the append-encode
-            "gpu_launches": args.steps * len(states) * (st.fused_launches if st.fused_launches <= 2 else 3),
+            "gpu_launches": args.steps * len(states) * (st.fused_launches if st.fused_launches < 4 else 3),
             "roofline": roofline}
 
     if args.extras != "none" and world == 1:

@@ -358,13 +358,14 @@ int cq_learn_centroids(const void *x_fp16, const float *weights, const double *u
  * One decode step of one layer on DEVICE buffers: the new token's key and value
  * vectors are encoded (CQ encode, Section 3.2, as cq_encode does) and appended at
  * position seq_lens[s] of every sequence, and the step's query attends over
- * seq_lens[s] + 1 tokens (Eq. 1, as cq_decode_attn does).  For head_dim 128 with
- * b = 8 and c in {2, 4, 8} (the shapes with tuned decode kernels) the append
- * happens INSIDE the attention launch: the CTAs whose part of the context holds
- * the new position work the codes out, use them, and one of them writes them to
- * the cache; the step is then one attention launch, plus the merge of the partials
- * where contexts are split over CTAs (cq_decode_step_launches tells).  Every other
- * shape runs cq_encode_kv and cq_decode_attn one after the other.
+ * seq_lens[s] + 1 tokens (Eq. 1, as cq_decode_attn does).  CQ-8c8b at head_dim 128
+ * with a multiple of four query heads per KV head appends INSIDE the attention launch:
+ * the CTAs whose part of the context holds the new position work the codes out, use
+ * them, and one of them writes them to the cache.  The other shapes of head_dim 128
+ * with b = 8 and c in {2, 4, 8} take a kernel ahead of the attention, which appends and,
+ * for few queries, builds the attention's tables.  The merge of the partials follows
+ * where contexts are split over CTAs.  Every other shape runs cq_encode_kv and
+ * cq_decode_attn one after the other.
  *
  *   q_fp16       [n_seq][n_q_heads][head_dim] fp16, device
  *   k_new_fp16, v_new_fp16   [n_seq][n_kv_heads][head_dim] fp16, device, 16-byte aligned
@@ -374,14 +375,17 @@ int cq_learn_centroids(const void *x_fp16, const float *weights, const double *u
  *   k_codes, v_codes   device, layout of cq_encode; one byte per group is written per sequence
  *                and KV head.  Must not alias each other.
  *   out          [n_seq][n_q_heads][head_dim] fp32, device
- *   workspace    device, 16-byte aligned, at least cq_decode_step_workspace_bytes(...) bytes
+ *   workspace    device, 16-byte aligned, cq_decode_step_workspace_bytes(...) bytes (for few queries
+ *                they count in the tables, at most 1 MiB; with less than that, but room for the
+ *                partials and the lengths, the attention builds its tables itself)
  * Errors: as cq_decode_attn.  Asynchronous on `stream`.
  */
 size_t cq_decode_step_workspace_bytes(int n_seq, int n_q_heads, int n_kv_heads, int head_dim,
                                       int c, int b, int64_t max_tokens);
 /* Kernel launches of one cq_decode_step call on this shape (1: the attention kernel appends the
- * token and, with one part of the context per CTA, also writes the output; 2: plus the merge of
- * the partials; 4: lengths plus one, append, attention, merge); 0 for an unsupported shape. */
+ * token and, with one part of the context per CTA, also writes the output; one more for the append
+ * ahead of it, and one for the merge of the partials; 4: lengths plus one, append, attention,
+ * merge); 0 for an unsupported shape. */
 int cq_decode_step_launches(int n_seq, int n_q_heads, int n_kv_heads, int head_dim, int c, int b,
                             int64_t max_tokens);
 int cq_decode_step(const void *q_fp16, const void *k_new_fp16, const void *v_new_fp16,

@@ -8,10 +8,10 @@ using namespace cq;
 namespace cq {
 
 namespace {
-constexpr int kDeviceSlots = 64;
+constexpr int kDeviceSlots = 64, kSmemSlots = 128;
 std::mutex g_device_mutex;
 int g_sm_count[kDeviceSlots] = {};                   // 0: not queried yet
-int g_smem_set[kDeviceSlots][96] = {};               // per device and call site: dynamic shared memory size already set
+int g_smem_set[kDeviceSlots][kSmemSlots] = {};               // per device and call site: dynamic shared memory size already set
 }  // namespace
 
 int device_sm_count()
@@ -38,7 +38,7 @@ cudaError_t ensure_dynamic_smem(const void* func, int bytes, int slot)
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kDeviceSlots || slot < 0 || slot >= 96)
+    if (dev < 0 || dev >= kDeviceSlots || slot < 0 || slot >= kSmemSlots)
         return cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     std::lock_guard<std::mutex> lock(g_device_mutex);
     if (g_smem_set[dev][slot] >= bytes && bytes > 0) return cudaSuccess;
@@ -476,22 +476,36 @@ int cq_learn_centroids(const void* x_fp16, const float* weights, const double* u
     return e == cudaSuccess ? CQ_OK : CQ_ERR_CUDA;
 }
 
+namespace {
+// Workspace that cq_decode_step cannot do without: the partials, and the lengths after the append where they are needed.
+// Behind them, where they pay (decode_tables_pay) and the caller gives that much (cq_decode_step_workspace_bytes), the tables.
+size_t step_least_bytes(const Shape& sh) { return round_up(partial_bytes(sh), 256) + round_up((size_t)sh.n_seq * 4, 256); }
+// The device copies of cq_decode_step_host's inputs and output.
+size_t host_staging_bytes(const Shape& sh)
+{
+    const size_t q = (size_t)sh.n_seq * sh.n_q_heads * sh.head_dim, kv = (size_t)sh.n_seq * sh.n_kv_heads * sh.head_dim;
+    return round_up(q * 2, 256) + 2 * round_up(kv * 2, 256) + round_up((size_t)sh.n_seq * 4, 256) + round_up(q * 4, 256);
+}
+// Shapes whose new tokens the kernel ahead of the attention encodes (cq_decode_tables.cu); the others take cq_encode_kv.
+bool step_append_ahead(const Shape& sh) { return decode_tuned_supported(sh) && sh.head_dim == 128 && sh.b == 8; }
+}  // namespace
+
 // Staging area of cq_decode_step_host inside the caller's workspace (all 256-byte aligned):
-//   [q fp16][k_new fp16][v_new fp16][seq_lens int32][seq_lens+1 int32][out fp32][attention workspace]
+//   [q fp16][k_new fp16][v_new fp16][seq_lens int32][out fp32][workspace of cq_decode_step]
 size_t cq_decode_step_workspace_bytes(int n_seq, int n_q_heads, int n_kv_heads, int head_dim, int c, int b,
                                       int64_t max_tokens)
 {
-    const size_t attn = cq_decode_attn_workspace_bytes(n_seq, n_q_heads, n_kv_heads, head_dim, c, b, max_tokens);
-    if (attn == 0) return 0;
-    return attn + round_up((size_t)n_seq * 4, 256);          // the lengths after the append, where they are needed
+    Shape sh;
+    if (make_shape(n_seq, max_tokens, n_q_heads, n_kv_heads, head_dim, c, b, &sh) != CQ_OK) return 0;
+    return step_least_bytes(sh) + (decode_tables_pay(sh) ? decode_tables_bytes(sh) : 0);
 }
 
 int cq_decode_step_launches(int n_seq, int n_q_heads, int n_kv_heads, int head_dim, int c, int b, int64_t max_tokens)
 {
     Shape sh;
     if (make_shape(n_seq, max_tokens, n_q_heads, n_kv_heads, head_dim, c, b, &sh) != CQ_OK) return 0;
-    if (decode_tuned_supported(sh) && decode_fused_append_supported(sh))
-        return decode_step_fused_launches(sh);                   // attention (with the append inside) [+ merge]
+    if (step_append_ahead(sh) || (decode_tuned_supported(sh) && decode_appends_inside(sh)))
+        return decode_tuned_launches(sh) + (decode_appends_inside(sh) ? 0 : 1);      // [append,] attention [, merge]
     return 4;                                                      // lengths plus one, append, attention, merge
 }
 
@@ -510,17 +524,37 @@ int cq_decode_step(const void* q_fp16, const void* k_new_fp16, const void* v_new
         (reinterpret_cast<uintptr_t>(out) & 3u))
         return CQ_ERR_ALIGN;
     if (k_codes == v_codes) return CQ_ERR_SHAPE;
-    const size_t attn_bytes = round_up(partial_bytes(sh), 256);
-    if (workspace_bytes < attn_bytes + round_up((size_t)n_seq * 4, 256)) return CQ_ERR_WORKSPACE;
+    const size_t attn_bytes = round_up(partial_bytes(sh), 256), least = step_least_bytes(sh);
+    if (workspace_bytes < least) return CQ_ERR_WORKSPACE;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
-    if (decode_tuned_supported(sh) && decode_fused_append_supported(sh)) {
-        AppendArgs app;
-        app.k_new = static_cast<const __half*>(k_new_fp16);
-        app.v_new = static_cast<const __half*>(v_new_fp16);
-        app.kc_w = static_cast<uint8_t*>(k_codes);
-        app.vc_w = static_cast<uint8_t*>(v_codes);
-        cudaError_t e = launch_decode_step_fused(static_cast<const __half*>(q_fp16), app.kc_w, app.vc_w, k_cb, v_cb, seq_lens,
-                                                 scale, sh, out, static_cast<float*>(workspace), app, cs);
+    const __half* q = static_cast<const __half*>(q_fp16);
+    const uint8_t *kc = static_cast<const uint8_t*>(k_codes), *vc = static_cast<const uint8_t*>(v_codes);
+    float* partials = static_cast<float*>(workspace);
+    AppendArgs app;
+    app.k_new = static_cast<const __half*>(k_new_fp16);
+    app.v_new = static_cast<const __half*>(v_new_fp16);
+    app.kc_w = static_cast<uint8_t*>(k_codes);
+    app.vc_w = static_cast<uint8_t*>(v_codes);
+    AheadArgs ahead;
+    ahead.appended = 1;
+    float* tables = decode_tables_pay(sh) && workspace_bytes >= least + decode_tables_bytes(sh)
+                        ? reinterpret_cast<float*>(static_cast<char*>(workspace) + least) : nullptr;
+    cudaError_t e = cudaSuccess;
+    if (decode_tuned_supported(sh) && decode_appends_inside(sh)) {
+        e = launch_decode_tuned(q, kc, vc, k_cb, v_cb, seq_lens, scale, sh, out, partials, cs, false, app);
+        return e == cudaSuccess ? CQ_OK : CQ_ERR_CUDA;
+    }
+    if (step_append_ahead(sh) || tables) {
+        if (!step_append_ahead(sh)) {                          // tables with an append of its own (CQ-8c10b)
+            st = cq_encode_kv(k_new_fp16, v_new_fp16, k_cb, v_cb, seq_lens, n_seq, 1, 0, max_tokens, n_kv_heads, head_dim, c, b, k_codes,
+                              v_codes, stream);
+            if (st != CQ_OK) return st;
+            app = AppendArgs();
+        }
+        e = launch_decode_ahead(q, k_cb, v_cb, seq_lens, scale, sh, tables, app, cs);
+        if (e != cudaSuccess) return CQ_ERR_CUDA;
+        ahead.tables = tables;
+        e = launch_decode_tuned(q, kc, vc, k_cb, v_cb, seq_lens, scale, sh, out, partials, cs, false, AppendArgs(), ahead);
         return e == cudaSuccess ? CQ_OK : CQ_ERR_CUDA;
     }
     // every other shape: the append is a launch of its own, the attention reads the lengths plus one
@@ -536,13 +570,9 @@ int cq_decode_step(const void* q_fp16, const void* k_new_fp16, const void* v_new
 size_t cq_decode_step_host_workspace_bytes(int n_seq, int n_q_heads, int n_kv_heads, int head_dim, int c, int b,
                                            int64_t max_tokens)
 {
-    const size_t attn = cq_decode_attn_workspace_bytes(n_seq, n_q_heads, n_kv_heads, head_dim, c, b, max_tokens);
-    if (attn == 0) return 0;
-    const size_t q = round_up((size_t)n_seq * n_q_heads * head_dim * 2, 256);
-    const size_t kv = round_up((size_t)n_seq * n_kv_heads * head_dim * 2, 256);
-    const size_t sl = round_up((size_t)n_seq * 4, 256);
-    const size_t o = round_up((size_t)n_seq * n_q_heads * head_dim * 4, 256);
-    return q + 2 * kv + 2 * sl + o + attn;
+    Shape sh;
+    if (make_shape(n_seq, max_tokens, n_q_heads, n_kv_heads, head_dim, c, b, &sh) != CQ_OK) return 0;
+    return host_staging_bytes(sh) + cq_decode_step_workspace_bytes(n_seq, n_q_heads, n_kv_heads, head_dim, c, b, max_tokens);
 }
 
 int cq_decode_step_host(const void* q_host, const void* k_new_host, const void* v_new_host,
@@ -554,12 +584,10 @@ int cq_decode_step_host(const void* q_host, const void* k_new_host, const void* 
     if (!q_host || !k_new_host || !v_new_host || !seq_lens_host || !k_codes || !v_codes || !k_cb || !v_cb ||
         !out_host || !workspace)
         return CQ_ERR_NULL;
-    const size_t need = cq_decode_step_host_workspace_bytes(n_seq, n_q_heads, n_kv_heads, head_dim, c, b, max_tokens);
-    if (need == 0) {
-        Shape sh;
-        return make_shape(n_seq, max_tokens, n_q_heads, n_kv_heads, head_dim, c, b, &sh);
-    }
-    if (workspace_bytes < need) return CQ_ERR_WORKSPACE;
+    Shape sh;
+    const int shape_ok = make_shape(n_seq, max_tokens, n_q_heads, n_kv_heads, head_dim, c, b, &sh);
+    if (shape_ok != CQ_OK) return shape_ok;
+    if (workspace_bytes < host_staging_bytes(sh) + step_least_bytes(sh)) return CQ_ERR_WORKSPACE;
     if (!aligned16(workspace)) return CQ_ERR_ALIGN;
     for (int s = 0; s < n_seq; ++s)
         if (seq_lens_host[s] < 0 || seq_lens_host[s] >= max_tokens) return CQ_ERR_SHAPE;

@@ -68,7 +68,7 @@ __host__ __device__ inline int partial_stride(int head_dim) { return head_dim + 
 // SM count of the current device (queried once per device and process).
 int device_sm_count();
 // cudaFuncAttributeMaxDynamicSharedMemorySize for `func`, set once per device and (func, bytes);
-// `slot` is a small integer unique to the call site (0 <= slot < 96).
+// `slot` is a small integer unique to the call site (0 <= slot < 128).
 cudaError_t ensure_dynamic_smem(const void* func, int bytes, int slot);
 
 // Launch plan of one tuned decode call: context chunk per CTA, partial slots per (sequence, query
@@ -87,6 +87,14 @@ struct AppendArgs {
     const __half* v_new = nullptr;
     uint8_t* kc_w = nullptr;
     uint8_t* vc_w = nullptr;
+};
+
+// What a kernel ahead of the attention has done (cq_decode_tables.cu).  tables[sequence][query head][code value][group]:
+// scale * log2(e) * <q_g, C_j>, fp32 (null: every CTA builds its own).  appended: the new token's codes are in the caches, the
+// attention covers seq_lens[s] + 1 tokens.
+struct AheadArgs {
+    const float* tables = nullptr;
+    int appended = 0;
 };
 
 // ---- launchers implemented in the .cu files (return cudaGetLastError()) ----
@@ -139,15 +147,17 @@ int decode_tuned_parts(const Shape& sh);      // partial slots per (sequence, qu
 cudaError_t launch_decode_tuned(const __half* q, const uint8_t* kc, const uint8_t* vc, const float* kcb,
                                 const float* vcb, const int32_t* seq_lens, float scale, const Shape& sh,
                                 float* out, float* partials, cudaStream_t st, bool per_head_tables = false,
-                                const AppendArgs& app = AppendArgs());
-// True when launch_decode_tuned would take a kernel that can append a token inside the attention launch.
-bool decode_fused_append_supported(const Shape& sh);
-int decode_step_fused_launches(const Shape& sh);      // 1: the attention kernel also writes the output; 2: plus the merge
-// One decode step: the token (app) is encoded and appended at position seq_lens[s] and the attention covers
-// seq_lens[s] + 1 tokens, in one attention launch (plus the merge).  Only where decode_fused_append_supported.
-cudaError_t launch_decode_step_fused(const __half* q, const uint8_t* kc, const uint8_t* vc, const float* kcb,
-                                     const float* vcb, const int32_t* seq_lens, float scale, const Shape& sh,
-                                     float* out, float* partials, const AppendArgs& app, cudaStream_t st);
+                                const AppendArgs& app = AppendArgs(), const AheadArgs& ahead = AheadArgs());
+// (app: only where decode_appends_inside; the launch then encodes the token as well and covers seq_lens[s] + 1 tokens)
+bool decode_appends_inside(const Shape& sh);
+int decode_tuned_launches(const Shape& sh);           // 1: the attention kernel also writes the output; 2: plus the merge
+
+// The kernel ahead of the attention of a decode step (cq_decode_tables.cu; b = 8, and for the tables CQ-8c10b): encodes and
+// appends the new tokens (app, may be empty) and, where that pays, builds the tables (tables, may be null).
+bool decode_tables_pay(const Shape& sh);
+size_t decode_tables_bytes(const Shape& sh);
+cudaError_t launch_decode_ahead(const __half* q, const float* kcb, const float* vcb, const int32_t* seq_lens, float scale,
+                                const Shape& sh, float* tables, const AppendArgs& app, cudaStream_t st);
 
 // CQ-8c8b with a multiple of four query heads per KV head: two query heads per table word (cq_decode_pair.cu).
 bool decode_pair_supported(const Shape& sh);

@@ -65,8 +65,7 @@ struct Cfg {
     // One plane: K and V planes share a row (K at +0, V at +128).  Two planes: separate tables.
     static constexpr int kVOffset = (kPlanes == 1) ? 128 : kRows * kRowBytes;
     static constexpr int kTableBytes = (kPlanes == 1) ? kRows * kRowBytes : 2 * kRows * kRowBytes;
-    static constexpr int kNewOffset = 128 + R * kD * 4;                  // codes of an appended token: [key | value][64 groups]
-    static constexpr int kCtlBytes = kNewOffset + 128;                   // control words + scaled query + those codes
+    static constexpr int kCtlBytes = 128 + R * kD * 4;                   // control words + scaled query
     static constexpr int kSmemBytes = kTableBytes + kCtlBytes;
 
     // word inside a plane that lane (r, p) uses for its m-th code word: run r / (8 / kRuns), a bijection lanes -> banks
@@ -190,72 +189,15 @@ __device__ __forceinline__ float fold_channels(const float (&a)[kC], int lane)
 }
 
 
-// byte k (0..15) of a 16-byte code word replaced
-__device__ __forceinline__ void put_code(uint4& w, int k, uint32_t code)
-{
-    const uint32_t keep = ~(0xffu << (8 * (k & 3))), put = code << (8 * (k & 3));
-    if ((k >> 2) == 0) w.x = (w.x & keep) | put;
-    else if ((k >> 2) == 1) w.y = (w.y & keep) | put;
-    else if ((k >> 2) == 2) w.z = (w.z & keep) | put;
-    else w.w = (w.w & keep) | put;
-}
-
-// The value codes of the token that the launch appends (CQ encode, Section 3.2), by the whole CTA: a warp takes
-// the groups it owns, its lanes walk the centroids; d_j = sum_i (x_i - C_ji)^2 in fp32 in the order of the encode
-// kernels, lowest index on ties.  The codes go to newcode[g] and, from the CTA that `writer` names, to position
-// `pos` of the cache.  (The key codes come out of the table build, which reads the key centroids anyway.)
-template <int kC, int kGroupsPerWarp>
-__device__ __noinline__ void encode_new_value_tuned(uint8_t* newcode, const __half* __restrict__ v_new, uint8_t* vc_w,
-                                                    const float* __restrict__ vcb, Shape sh, int64_t s, int hkv, int64_t pos,
-                                                    bool writer)
-{
-    constexpr int G = 128 / kC;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll 1
-    for (int e = 0; e < kGroupsPerWarp; ++e) {
-        const int g = warp * kGroupsPerWarp + e;
-        const __half* xp = v_new + (s * sh.n_kv_heads + hkv) * 128 + g * kC;
-        const float* cg = vcb + ((int64_t)hkv * G + g) * kRows * kC;
-        float xg[kC];
-#pragma unroll
-        for (int i = 0; i < kC; ++i) xg[i] = __half2float(xp[i]);
-        float cv[kRows / 32][kC];                     // all loads in flight at once
-#pragma unroll
-        for (int t = 0; t < kRows / 32; ++t) load_centroid<kC>(cg + (int64_t)(t * 32 + lane) * kC, cv[t], false);
-        float best = INFINITY;
-        int arg = 0;
-#pragma unroll
-        for (int t = 0; t < kRows / 32; ++t) {
-            float d = 0.f;
-#pragma unroll
-            for (int i = 0; i < kC; ++i) {
-                const float diff = xg[i] - cv[t][i];
-                d = fmaf(diff, diff, d);
-            }
-            if (d < best) { best = d; arg = t * 32 + lane; }        // ascending: strict < keeps the lowest index
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float ob = __shfl_xor_sync(0xffffffffu, best, o);
-            const int oa = __shfl_xor_sync(0xffffffffu, arg, o);
-            if (ob < best || (ob == best && oa < arg)) { best = ob; arg = oa; }
-        }
-        if (lane == 0) {
-            newcode[g] = (uint8_t)arg;
-            if (writer) vc_w[code_word_offset(sh, sh.n_kv_heads, s, hkv, pos / kTokenBlock, g) + pos % kTokenBlock] = (uint8_t)arg;
-        }
-    }
-}
-
-// kAppend: the launch also encodes and appends one token per sequence (a second instance, so that the plain attention
-// carries none of that code)
-template <int kD, int G, int R, bool kShared, bool kAppend>
+// kTables: the tables come from the kernel ahead (cq_decode_tables.cu); an instance of its own, so that neither carries the
+// other's code.
+template <int kD, int G, int R, bool kShared, bool kTables>
 __global__ void __launch_bounds__(Cfg<kD, G, R>::kThreads, Cfg<kD, G, R>::kMinBlocks)
 decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, const uint8_t* __restrict__ vc,
                     const float* __restrict__ kcb, const float* __restrict__ vcb,
                     const int32_t* __restrict__ seq_lens, float scale_log2e, Shape sh, int chunk_tokens, int n_parts,
                     int tail_first, int cb_aligned32, int kv_share, float* __restrict__ partials, float* __restrict__ out,
-                    AppendArgs app)
+                    AheadArgs ahead)
 {
     // out: non-null only when every item is one part; the CTA then normalises its partial itself (no merge launch).
     // R is the number of query heads one CTA serves.  A KV head with more query heads than that
@@ -268,6 +210,17 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int r = lane >> 2, p = lane & 3;
+
+    // bins start at zero (16-byte stores over the V planes)
+    auto clear_bins = [&]() {
+        for (int i = threadIdx.x; i < kRows * 8 * C::kPlanes; i += C::kThreads)
+            *reinterpret_cast<uint4*>(smem + C::kVOffset + (i / (8 * C::kPlanes)) * kRowBytes + (i % (8 * C::kPlanes)) * 16) =
+                make_uint4(0u, 0u, 0u, 0u);
+    };
+    clear_bins();
+    // launched ahead of the end of the kernel before it (the append, for one); the merge, or the call behind, may be from here on
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     // Work item: (context part, sequence, KV head); parts are the slowest index so that the
     // always-populated first parts start first.  With a tail (tail_first >= 0) the items before
@@ -290,10 +243,7 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
 
     int64_t n = seq_lens[s];
     n = n < 0 ? 0 : (n > sh.max_tokens ? sh.max_tokens : n);
-    // With an append, seq_lens counts the tokens cached before this launch: the new token takes position n and
-    // the attention covers n + 1 tokens (a sequence at capacity gets no new token).
-    const bool has_new = kAppend && app.k_new != nullptr && n < sh.max_tokens;
-    if (has_new) ++n;
+    if (ahead.appended && n < sh.max_tokens) ++n;         // (a sequence at capacity got no new token)
     if (tail_first == kEvenShares) chunk_tokens = share_of_context(n, n_parts, chunk_tokens);
     const int64_t t_begin = (int64_t)part * chunk_tokens;
     const int64_t t_end = (whole || t_begin + chunk_tokens >= n) ? n : t_begin + chunk_tokens;
@@ -320,14 +270,6 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
     const int64_t blk_lim = (t_end + kTokenBlock - 1) / kTokenBlock;       // blocks holding a valid token
     const int n_iters = (int)((t_end - t_begin + C::kRoundTokens - 1) / C::kRoundTokens);
     const int qb = r % C::kBlocksPerIter;                 // block of this quad inside the warp's iteration
-    // The new token, when its position is in this CTA's range: the CTA works its codes out itself (so do the CTAs of
-    // the other query heads that share the KV head) and puts them into the code words it loads of that block; one
-    // CTA per KV head also writes them to the cache.
-    const bool new_here = kAppend && has_new && t_begin <= n - 1 && n - 1 < t_end;
-    const int64_t new_blk = (n - 1) / kTokenBlock;
-    const int new_tok = (int)((n - 1) % kTokenBlock);
-    const bool new_writer = !kShared || head_group % kv_share == 0;
-    uint8_t* newcode = smem + C::kTableBytes + C::kNewOffset;               // [key | value][64]
     uint32_t lane_off[C::kSlots];      // byte offset of this lane's word inside a plane, per code word
 #pragma unroll
     for (int m = 0; m < C::kSlots; ++m) lane_off[m] = 4u * C::word(r, p, m) + C::lane_plane_bytes(r);
@@ -342,11 +284,6 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
 #pragma unroll
             for (int m = 0; m < C::kSlots; ++m)
                 dst[m] = ldg_codes(reinterpret_cast<const uint4*>(bp + C::group_of(lane_off[m] >> 2) * kTokenBlock));
-            if (kAppend && new_here && blk == new_blk) {
-                const uint8_t* nc = newcode + (base == vbase ? 64 : 0);
-#pragma unroll
-                for (int m = 0; m < C::kSlots; ++m) put_code(dst[m], new_tok, nc[C::group_of(lane_off[m] >> 2)]);
-            }
         } else {
 #pragma unroll
             for (int m = 0; m < C::kSlots; ++m) dst[m] = make_uint4(0u, 0u, 0u, 0u);
@@ -366,7 +303,7 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
         for (int jb = 0; jb < kJb; ++jb) load_centroid<kC>(cg + jb * 32 * kC, cv[jb], cb_aligned32 != 0);
     };
     float cva[kJb][kC], cvb[kJb][kC];
-    load_unit(cva, kcb, 0);
+    if (!kTables) load_unit(cva, kcb, 0);
 
     // ---------------------------------------------------------------- set-up: query, LUT, bins
     if (threadIdx.x < 4) {
@@ -376,12 +313,8 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
         ctl->req_need[threadIdx.x] = kUnset;
     }
     if (threadIdx.x == 4) { ctl->want = 0; ctl->lut_absmax = 0.f; }
-    for (int i = threadIdx.x; i < R * kD; i += C::kThreads)
+    for (int i = threadIdx.x; !kTables && i < R * kD; i += C::kThreads)
         qs[i] = __half2float(q[(s * sh.n_q_heads + (int64_t)head_group * R) * kD + i]) * scale_log2e;
-    // bins start at zero (16-byte stores over the V planes)
-    for (int i = threadIdx.x; i < kRows * 8 * C::kPlanes; i += C::kThreads)
-        *reinterpret_cast<uint4*>(smem + C::kVOffset + (i / (8 * C::kPlanes)) * kRowBytes + (i % (8 * C::kPlanes)) * 16) =
-            make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
 
     // Table build.  A warp owns whole groups and its lanes walk the code values j, so the
@@ -389,26 +322,49 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
     // rows) would fall into one bank, so the build writes row j rotated by j words and a second
     // pass un-rotates every row.  Entries are half2 (hi, lo) of LUT * 2^-kexp; kexp = 0 unless an
     // entry reaches 2^15 (then the build is repeated once with the exponent that fits).
-    if (kAppend && new_here)
-        encode_new_value_tuned<kC, C::kGroupsPerWarp>(newcode + 64, app.v_new, app.vc_w, vcb, sh, s, hkv, n - 1, new_writer);
-    // the new token's key, when this CTA appends it: its code of group g is the centroid nearest to it, found on the
-    // way (d_j = sum_i (x_i - C_ji)^2 in fp32 in the order of the encode kernels, lowest index on ties)
-    float xnew[kC], dnew = INFINITY;
-    int jnew = 0;
+    constexpr int kOwnRowPlanes = kRows / C::kWarps * C::kPlanes;
+    static_assert(kOwnRowPlanes % 8 == 0, "row batches");
     float lut_scale = 1.f;           // scores in table units * lut_scale = log2-domain scores
+    if constexpr (kTables) {
+        // the rows (code value, G groups) of the CTA's heads, four groups per load
+        constexpr int kPieces = G / 4, kEach = R * kRows * kPieces / C::kThreads;
+        static_assert(R * kRows * kPieces % C::kThreads == 0 && kRows * kPieces % C::kThreads == 0, "whole rounds per head");
+        const float4* src = reinterpret_cast<const float4*>(ahead.tables + (s * sh.n_q_heads + (int64_t)head_group * R) * kRows * G);
+        float4 v[kEach];
+#pragma unroll
+        for (int i = 0; i < kEach; ++i) v[i] = __ldcg(src + i * C::kThreads + threadIdx.x);
+        float absmax = 0.f;
+#pragma unroll
+        for (int i = 0; i < kEach; ++i)
+            absmax = fmaxf(absmax, fmaxf(fmaxf(fabsf(v[i].x), fabsf(v[i].y)), fmaxf(fabsf(v[i].z), fabsf(v[i].w))));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) absmax = fmaxf(absmax, __shfl_xor_sync(0xffffffffu, absmax, o));
+        if (lane == 0) atomicMax(reinterpret_cast<int*>(&ctl->lut_absmax), __float_as_int(absmax));
+        __syncthreads();
+        const float amax = ctl->lut_absmax;
+        if (amax >= 32768.f) {
+            int ex;
+            frexpf(amax, &ex);                            // amax < 2^ex
+            lut_scale = exp2f((float)(ex - 15));
+        }
+        const float inv = 1.f / lut_scale;
+#pragma unroll
+        for (int i = 0; i < kEach; ++i) {
+            const int e = i * C::kThreads + threadIdx.x;
+            const int h = i / (kEach / R), j = e / kPieces % kRows, g = e % kPieces * 4;
+            const uint4 w = make_uint4(pack_hi_lo(v[i].x * inv), pack_hi_lo(v[i].y * inv), pack_hi_lo(v[i].z * inv), pack_hi_lo(v[i].w * inv));
+            uint8_t* row = smem + j * kRowBytes + C::plane_of(g, h) * 128;
+            // (neighbouring rows start with different copies: they would meet in the same banks)
+#pragma unroll
+            for (int copy = 0; copy < C::kCopies; ++copy)
+                *reinterpret_cast<uint4*>(row + (((copy + j) % C::kCopies) * G + C::word_of(g, h)) * 4) = w;
+        }
+    } else {
     for (int attempt = 0; attempt < 2; ++attempt) {
         const float inv = 1.f / lut_scale;
         float absmax = 0.f;
-        const bool find_key = kAppend && new_here && attempt == 0;
         auto build_unit = [&](const float (&cv)[kJb][kC], int u) {
             const int g = warp * C::kGroupsPerWarp + u / kUnitsPerGroup;
-            if (kAppend && find_key && u % kUnitsPerGroup == 0) {
-                const __half* xp = app.k_new + (s * sh.n_kv_heads + hkv) * 128 + g * kC;
-#pragma unroll
-                for (int i = 0; i < kC; ++i) xnew[i] = __half2float(xp[i]);
-                dnew = INFINITY;
-                jnew = 0;
-            }
             float qreg[R][kC];
 #pragma unroll
             for (int h = 0; h < R; ++h)
@@ -429,28 +385,6 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
                     #pragma unroll
                     for (int copy = 1; copy < C::kCopies; ++copy)
                         *reinterpret_cast<uint32_t*>(row + ((copy * G + C::word_of(g, h) + j) & 31) * 4) = e;
-                }
-                if (kAppend && find_key) {
-                    float d = 0.f;
-#pragma unroll
-                    for (int i = 0; i < kC; ++i) {
-                        const float diff = xnew[i] - cv[jb][i];
-                        d = fmaf(diff, diff, d);
-                    }
-                    if (d < dnew) { dnew = d; jnew = j; }        // a lane's j ascend: strict < keeps the lowest index
-                }
-            }
-            if (kAppend && find_key && u % kUnitsPerGroup == kUnitsPerGroup - 1) {
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    const float ob = __shfl_xor_sync(0xffffffffu, dnew, o);
-                    const int oa = __shfl_xor_sync(0xffffffffu, jnew, o);
-                    if (ob < dnew || (ob == dnew && oa < jnew)) { dnew = ob; jnew = oa; }
-                }
-                if (lane == 0) {
-                    newcode[g] = (uint8_t)jnew;
-                    if (new_writer)
-                        app.kc_w[code_word_offset(sh, sh.n_kv_heads, s, hkv, (n - 1) / kTokenBlock, g) + (n - 1) % kTokenBlock] = (uint8_t)jnew;
                 }
             }
         };
@@ -479,8 +413,6 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
         __syncthreads();
     }
     // un-rotate: a warp owns rows warp, warp + kWarps, ...; eight (row, plane) pairs per step
-    constexpr int kOwnRowPlanes = kRows / C::kWarps * C::kPlanes;
-    static_assert(kOwnRowPlanes % 8 == 0, "row batches");
 #pragma unroll 1
     for (int i0 = 0; i0 < kOwnRowPlanes; i0 += 8) {
         uint32_t e[8];
@@ -497,6 +429,7 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
             uint8_t* row = smem + j * kRowBytes + (i0 + k) % C::kPlanes * 128;
             *reinterpret_cast<uint32_t*>(row + lane * 4) = e[k];
         }
+    }
     }
     __syncthreads();
 
@@ -897,11 +830,12 @@ __device__ __forceinline__ uint32_t wide_index(const uint4& w, uint32_t hw, int 
     return (low << row_shift) + (hi << (row_shift + 8)) + lane_off;
 }
 
+template <bool kTables>
 __global__ void __launch_bounds__(WideCfg::kThreads, 1)
 decode_wide_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, const uint8_t* __restrict__ vc,
                    const float* __restrict__ kcb, const float* __restrict__ vcb,
                    const int32_t* __restrict__ seq_lens, float scale_log2e, Shape sh, int chunk_tokens, int n_parts,
-                   int tail_first, int cb_aligned32, float* __restrict__ partials)
+                   int tail_first, int cb_aligned32, float* __restrict__ partials, AheadArgs ahead)
 {
     using C = WideCfg;
     constexpr int kC = C::kC;
@@ -912,7 +846,13 @@ decode_wide_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc,
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int r = lane >> 2, p = lane & 3;
 
-    asm volatile("griddepcontrol.wait;" ::: "memory");      // launched ahead of the end of the append that writes the codes
+    auto clear_bins = [&]() {
+        for (int i = threadIdx.x; i < C::kRows * C::kVRowBytes / 16; i += C::kThreads)
+            *reinterpret_cast<uint4*>(smem + C::kVOffset + i * 16) = make_uint4(0u, 0u, 0u, 0u);
+    };
+    clear_bins();
+    asm volatile("griddepcontrol.wait;" ::: "memory");      // (as in decode_tuned_kernel)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // work item: (context part, sequence, query head), with the same tail rule as decode_tuned_kernel
     const int n_items = (int)(sh.n_q_heads * sh.n_seq);
     int item = blockIdx.x % n_items;
@@ -929,6 +869,7 @@ decode_wide_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc,
 
     int64_t n = seq_lens[s];
     n = n < 0 ? 0 : (n > sh.max_tokens ? sh.max_tokens : n);
+    if (ahead.appended && n < sh.max_tokens) ++n;
     if (tail_first == kEvenShares) chunk_tokens = share_of_context(n, n_parts, chunk_tokens);
     const int64_t t_begin = (int64_t)part * chunk_tokens;
     const int64_t t_end = (whole || t_begin + chunk_tokens >= n) ? n : t_begin + chunk_tokens;
@@ -983,7 +924,7 @@ decode_wide_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc,
         for (int jb = 0; jb < kJb; ++jb) load_centroid<kC>(cg + jb * 32 * kC, cv[jb], cb_aligned32 != 0);
     };
     float cva[kJb][kC], cvb[kJb][kC];
-    load_unit(cva, kcb, 0);
+    if (!kTables) load_unit(cva, kcb, 0);
 
     // ---------------------------------------------------------------- set-up: query, LUT, bins
     if (threadIdx.x < 4) {
@@ -993,15 +934,43 @@ decode_wide_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc,
         ctl->req_need[threadIdx.x] = kUnset;
     }
     if (threadIdx.x == 4) { ctl->want = 0; ctl->lut_absmax = 0.f; }
-    if (threadIdx.x < 128)
+    if (!kTables && threadIdx.x < 128)
         qs[threadIdx.x] = __half2float(q[(s * sh.n_q_heads + hq) * 128 + threadIdx.x]) * scale_log2e;
-    for (int i = threadIdx.x; i < C::kRows * C::kVRowBytes / 16; i += C::kThreads)
-        *reinterpret_cast<uint4*>(smem + C::kVOffset + i * 16) = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
 
     // K table: row j is written rotated by j words (a column would fall into one bank), both copies,
     // then every row is un-rotated.  Entries are half2 (hi, lo) of LUT * 2^-kexp as in decode_tuned_kernel.
     float lut_scale = 1.f;
+    if constexpr (kTables) {            // as in decode_tuned_kernel
+        constexpr int kPieces = C::kG / 4, kEach = C::kRows * kPieces / C::kThreads;
+        const float4* src = reinterpret_cast<const float4*>(ahead.tables + (s * sh.n_q_heads + hq) * C::kRows * C::kG);
+        float4 v[kEach];
+#pragma unroll
+        for (int i = 0; i < kEach; ++i) v[i] = __ldcg(src + i * C::kThreads + threadIdx.x);
+        float absmax = 0.f;
+#pragma unroll
+        for (int i = 0; i < kEach; ++i)
+            absmax = fmaxf(absmax, fmaxf(fmaxf(fabsf(v[i].x), fabsf(v[i].y)), fmaxf(fabsf(v[i].z), fabsf(v[i].w))));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) absmax = fmaxf(absmax, __shfl_xor_sync(0xffffffffu, absmax, o));
+        if (lane == 0) atomicMax(reinterpret_cast<int*>(&ctl->lut_absmax), __float_as_int(absmax));
+        __syncthreads();
+        const float amax = ctl->lut_absmax;
+        if (amax >= 32768.f) {
+            int ex;
+            frexpf(amax, &ex);
+            lut_scale = exp2f((float)(ex - 15));
+        }
+        const float inv = 1.f / lut_scale;
+#pragma unroll
+        for (int i = 0; i < kEach; ++i) {
+            const int e = i * C::kThreads + threadIdx.x, j = e / kPieces, gp = e % kPieces * 4;
+            const uint4 w = make_uint4(pack_hi_lo(v[i].x * inv), pack_hi_lo(v[i].y * inv), pack_hi_lo(v[i].z * inv), pack_hi_lo(v[i].w * inv));
+#pragma unroll
+            for (int copy = 0; copy < 2; ++copy)
+                *reinterpret_cast<uint4*>(smem + j * C::kKRowBytes + (((copy + j) & 1) * 16 + gp) * 4) = w;
+        }
+    } else {
     for (int attempt = 0; attempt < 2; ++attempt) {
         const float inv = 1.f / lut_scale;
         float absmax = 0.f;
@@ -1057,6 +1026,7 @@ decode_wide_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc,
             const int j = warp + (i0 + k) * C::kWarps;
             *reinterpret_cast<uint32_t*>(smem + j * C::kKRowBytes + lane * 4) = e[k];
         }
+    }
     }
     __syncthreads();
 
@@ -1325,38 +1295,27 @@ Plan plan_for(const Shape& sh)
 template <int kD, int G, int R>
 cudaError_t launch_cfg(const __half* q, const uint8_t* kc, const uint8_t* vc, const float* kcb, const float* vcb,
                        const int32_t* seq_lens, float scale, const Shape& sh, const Plan& pl, float* partials,
-                       cudaStream_t st, float* out, const AppendArgs& app)
+                       cudaStream_t st, float* out, const AheadArgs& ahead)
 {
     using C = Cfg<kD, G, R>;
     const int kv_share = sh.R / R;
-    // call-site slots of ensure_dynamic_smem: 1 is the wide kernel, 2 ... 13 the template instances of head_dim 128,
-    // 78 ... 89 those of head_dim 64
+    // call-site slots of ensure_dynamic_smem: 1 and 95 are the wide kernel; 2 ... 13 the instances of head_dim 128, 78 ... 89 those
+    // of head_dim 64; 96 ... 119 those with tables
     constexpr int kSlot = (kD == 128 ? 2 : 78) + 2 * ((G == 16 ? 0 : G == 64 ? 5 : 3) + (R == 1 ? 0 : R == 2 ? 1 : 2));
-    const bool append = app.k_new != nullptr;
-    if (append && kD != 128) return cudaErrorNotSupported;
-    // one launch per (shared KV head or not, appending or not) instance; smem call-site slots kSlot, kSlot + 1 and 64 + those
-#define CQ_LAUNCH_TUNED(SHARED, APPEND, SLOT)                                                                                   \
-    do {                                                                                                                        \
-        cudaError_t e_ = ensure_dynamic_smem(reinterpret_cast<const void*>(decode_tuned_kernel<kD, G, R, SHARED, APPEND>),           \
-                                             C::kSmemBytes, SLOT);                                                              \
-        if (e_ != cudaSuccess) return e_;                                                                                       \
-        decode_tuned_kernel<kD, G, R, SHARED, APPEND><<<pl.grid, C::kThreads, C::kSmemBytes, st>>>(                                  \
-            q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, pl.chunk, pl.n_parts, pl.tail_first, aligned32(kcb, vcb),         \
-            kv_share, partials, pl.n_parts == 1 ? out : nullptr, app);                                                          \
-    } while (0)
-    if (kv_share > 1) {
-        if constexpr (kD == 128) {
-            if (append) CQ_LAUNCH_TUNED(true, true, 62 + kSlot);
-        }
-        if (!append) CQ_LAUNCH_TUNED(true, false, kSlot);
-    } else {
-        if constexpr (kD == 128) {
-            if (append) CQ_LAUNCH_TUNED(false, true, 62 + kSlot + 1);
-        }
-        if (!append) CQ_LAUNCH_TUNED(false, false, kSlot + 1);
+    constexpr int kTabSlot = 96 + (kD == 128 ? kSlot - 2 : kSlot - 66);
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = overlapped_config(pl.grid, C::kThreads, C::kSmemBytes, st, &attr);
+    auto go = [&](auto kernel, int slot) {
+        const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), C::kSmemBytes, slot);
+        if (e != cudaSuccess) return e;
+        return cudaLaunchKernelEx(&cfg, kernel, q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, pl.chunk, pl.n_parts, pl.tail_first,
+                                  aligned32(kcb, vcb), kv_share, partials, pl.n_parts == 1 ? out : nullptr, ahead);
+    };
+    if constexpr (kD == 128) {
+        if (ahead.tables) return kv_share > 1 ? go(decode_tuned_kernel<kD, G, R, true, true>, kTabSlot) : go(decode_tuned_kernel<kD, G, R, false, true>, kTabSlot + 1);
     }
-#undef CQ_LAUNCH_TUNED
-    return cudaGetLastError();
+    if (ahead.tables) return cudaErrorNotSupported;
+    return kv_share > 1 ? go(decode_tuned_kernel<kD, G, R, true, false>, kSlot) : go(decode_tuned_kernel<kD, G, R, false, false>, kSlot + 1);
 }
 
 bool wide_shape(const Shape& sh) { return sh.head_dim == 128 && sh.c == 8 && sh.b == 10; }
@@ -1415,25 +1374,21 @@ int decode_tuned_parts(const Shape& sh)
     return pair > own ? pair : own;
 }
 
-bool decode_fused_append_supported(const Shape& sh) { return decode_tuned_supported(sh) && !wide_shape(sh) && sh.head_dim == 128; }
+// decode_pair_kernel reads a codebook once for four heads, so an append inside it costs less than a kernel ahead: 48 sequences of
+// 301 to 889 tokens, 32 heads on 8, 49.6 against 54.2 us; 64 x 16384 248.7 against 249.8.  With one or two heads per CTA the
+// kernel ahead is the better one (16 x 4096 tokens, 32 heads of CQ-4c8b: 73.3 -> 68.7 us; 10 x 147: 31.3 -> 25.7; 32 sequences of 8
+// to 32 k tokens, 40 heads of CQ-8c8b: 279 -> 265): inside, every CTA took the value centroids once more for it.
+bool decode_appends_inside(const Shape& sh) { return decode_pair_supported(sh); }
 
-int decode_step_fused_launches(const Shape& sh)
+int decode_tuned_launches(const Shape& sh)
 {
-    if (decode_pair_supported(sh)) return decode_pair_plan(sh).n_parts == 1 ? 1 : 2;
-    return plan_dispatch(sh).n_parts == 1 ? 1 : 2;
-}
-
-cudaError_t launch_decode_step_fused(const __half* q, const uint8_t* kc, const uint8_t* vc, const float* kcb,
-                                     const float* vcb, const int32_t* seq_lens, float scale, const Shape& sh,
-                                     float* out, float* partials, const AppendArgs& app, cudaStream_t st)
-{
-    if (!decode_fused_append_supported(sh)) return cudaErrorNotSupported;
-    return launch_decode_tuned(q, kc, vc, kcb, vcb, seq_lens, scale, sh, out, partials, st, false, app);
+    const bool one = (decode_pair_supported(sh) ? decode_pair_plan(sh).n_parts : plan_dispatch(sh).n_parts) == 1;
+    return one && !wide_shape(sh) ? 1 : 2;
 }
 
 cudaError_t launch_decode_tuned(const __half* q, const uint8_t* kc, const uint8_t* vc, const float* kcb,
                                 const float* vcb, const int32_t* seq_lens, float scale, const Shape& sh, float* out,
-                                float* partials, cudaStream_t st, bool per_head_tables, const AppendArgs& app)
+                                float* partials, cudaStream_t st, bool per_head_tables, const AppendArgs& app, const AheadArgs& ahead)
 {
     if (!per_head_tables && decode_pair_supported(sh)) {
         const DecodePlan pp = decode_pair_plan(sh);
@@ -1442,20 +1397,22 @@ cudaError_t launch_decode_tuned(const __half* q, const uint8_t* kc, const uint8_
         return launch_merge(partials, pp.n_parts, sh, out, st);
     }
     const Plan pl = plan_dispatch(sh);
-    if (pl.chunk <= 0) return cudaErrorNotSupported;
+    if (app.k_new || pl.chunk <= 0) return cudaErrorNotSupported;
     cudaError_t e = cudaErrorNotSupported;
     if (wide_shape(sh)) {
-        if (app.k_new) return cudaErrorNotSupported;          // this kernel does not append
-        e = ensure_dynamic_smem(reinterpret_cast<const void*>(decode_wide_kernel), WideCfg::kSmemBytes, 1);
-        if (e != cudaSuccess) return e;
         cudaLaunchAttribute attr;
         const cudaLaunchConfig_t cfg = overlapped_config(pl.grid, WideCfg::kThreads, WideCfg::kSmemBytes, st, &attr);
-        e = cudaLaunchKernelEx(&cfg, decode_wide_kernel, q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, pl.chunk, pl.n_parts, pl.tail_first,
-                               aligned32(kcb, vcb), partials);
+        auto go = [&](auto kernel, int slot) {
+            const cudaError_t es = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), WideCfg::kSmemBytes, slot);
+            if (es != cudaSuccess) return es;
+            return cudaLaunchKernelEx(&cfg, kernel, q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, pl.chunk, pl.n_parts, pl.tail_first,
+                                      aligned32(kcb, vcb), partials, ahead);
+        };
+        e = ahead.tables ? go(decode_wide_kernel<true>, 95) : go(decode_wide_kernel<false>, 1);
     }
     else {
         e = with_instance(sh, [&](auto i) {
-            return launch_cfg<i.D, i.groups, i.heads>(q, kc, vc, kcb, vcb, seq_lens, scale, sh, pl, partials, st, out, app);
+            return launch_cfg<i.D, i.groups, i.heads>(q, kc, vc, kcb, vcb, seq_lens, scale, sh, pl, partials, st, out, ahead);
         });
     }
     if (e != cudaSuccess) return e;

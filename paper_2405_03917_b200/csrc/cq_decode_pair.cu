@@ -376,6 +376,12 @@ decode_pair_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc,
     const int p = lane & 3, r = lane >> 2;
     const int hb = p & 1, pu = p >> 1;
 
+    // launched ahead of the end of the kernel before it (which may write codes: they are read by bulk copies, hence the proxy
+    // fence); the merge, or the call behind, may be launched from here on
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("fence.proxy.async;" ::: "memory");
+
     // Work item: (context part, sequence, group of four query heads).  Items before tail_first take
     // their whole context in one CTA; each later item is spread over n_parts CTAs of chunk_tokens
     // (see the launch plan).
@@ -1004,13 +1010,13 @@ cudaError_t launch_decode_pair(const __half* q, const uint8_t* kc, const uint8_t
                                float* partials, cudaStream_t st, const AppendArgs& app, float* out)
 {
     using C = PairCfg;
-    const cudaError_t attr = ensure_dynamic_smem(reinterpret_cast<const void*>(decode_pair_kernel), C::kSmemBytes, 0);
-    if (attr != cudaSuccess) return attr;
+    const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(decode_pair_kernel), C::kSmemBytes, 0);
+    if (e != cudaSuccess) return e;
     const int aligned = ((reinterpret_cast<uintptr_t>(kcb) | reinterpret_cast<uintptr_t>(vcb)) & 31u) == 0 ? 1 : 0;
-    decode_pair_kernel<<<pl.grid, C::kThreads, C::kSmemBytes, st>>>(q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, pl.chunk,
-                                                                    pl.n_parts, pl.tail_first, aligned, partials, app,
-                                                                    pl.n_parts == 1 ? out : nullptr);
-    return cudaGetLastError();
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = overlapped_config(pl.grid, C::kThreads, C::kSmemBytes, st, &attr);
+    return cudaLaunchKernelEx(&cfg, decode_pair_kernel, q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, pl.chunk, pl.n_parts,
+                              pl.tail_first, aligned, partials, app, pl.n_parts == 1 ? out : nullptr);
 }
 
 }  // namespace cq

@@ -28,7 +28,7 @@
 //
 // No pipe bounds this kernel at b = 12 (2048 vectors x 8 heads, c = 8, 1.2 ms): issue slots and ALU pipe are 38 % busy,
 // warps wait for the chunk's centroids and for each other (a chunk of 256 is one step).
-#include "cq_common.cuh"
+#include "cq_encode_few.cuh"
 
 namespace cq {
 
@@ -490,17 +490,31 @@ encode_tuned_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1
     }
 }
 
-// Few vectors per head (the append of a decode step): one CTA per (head, group) reads the group's codebook once, a thread
-// holding kPer of its 256 * kPer centroids in registers, and takes the vectors past them sixteen at a time.
-// Distances are the direct form sum (x - C)^2 in fp32 in the order of the generic kernel, lowest index on ties.  What
-// it takes is one pass over the codebooks (16 vectors x 32 heads of CQ-8c10b, key and value: 33 MB; 52 us on the
-// tensor-memory kernel, which walks its steps one after the other with 16 of 128 rows in use, 17 us here; one vector of
-// CQ-8c8b, 8 heads: 5.6 -> 1.9 us).
-constexpr int kFewVecs = 16;
 constexpr int kFewMost = 32;          // vectors per head up to which it is the faster one (32 heads, key and value of CQ-8c10b: 31 against 45 us; 64: 59 against 46)
+
+// 256 centroids (the device code is the append of a decode step's as well)
+template <int kC>
+__global__ void __launch_bounds__(kFewThreads)
+encode_few_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, const int32_t* __restrict__ seq_offsets, Shape sh,
+                  int n_vec, int n_tokens, int64_t token_offset, uint8_t* __restrict__ codes1, const __half* __restrict__ x2,
+                  const float* __restrict__ cb2, uint8_t* __restrict__ codes2, int share)
+{
+    // launched ahead of the end of whatever lies before it in the stream, which may well write the codebooks (a k-means update)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const bool second = blockIdx.y != 0;
+    encode_few<kC>(second ? x2 : x1, second ? cb2 : cb1, seq_offsets, sh, blockIdx.x, n_vec, share, n_tokens,
+                         token_offset, second ? codes2 : codes1, false);
+}
+
+// 512 and 1024 centroids: one CTA per (head, group) reads the group's codebook once, a thread holding kPer of its 256 * kPer
+// centroids in registers, and takes the vectors past them sixteen at a time.  Distances and ties as in encode_few.  What it
+// takes is one pass over the codebooks (16 vectors x 32 heads of CQ-8c10b, key and value: 33 MB; 52 us on the tensor-memory
+// kernel, which walks its steps one after the other with 16 of 128 rows in use, 17 us here).  A warp per 256 centroids
+// (encode_few) has too few warps for this many (27 us; two vectors, 40 heads 12.6 against 9.9 us).
+constexpr int kFewWideVecs = 16;
 template <int kC, int kPer>
 __global__ void __launch_bounds__(256)
-encode_few_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, const int32_t* __restrict__ seq_offsets, Shape sh,
+encode_few_wide_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, const int32_t* __restrict__ seq_offsets, Shape sh,
                   int n_vec, int n_tokens, int64_t token_offset, uint8_t* __restrict__ codes1, const __half* __restrict__ x2,
                   const float* __restrict__ cb2, uint8_t* __restrict__ codes2)
 {
@@ -508,8 +522,8 @@ encode_few_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, 
     const float* cb = blockIdx.y ? cb2 : cb1;
     uint8_t* codes = blockIdx.y ? codes2 : codes1;
     constexpr int G = 128 / kC;
-    __shared__ float xs[kFewVecs][kC];
-    __shared__ unsigned long long near[kFewVecs][8];          // per vector and warp: (distance, centroid)
+    __shared__ float xs[kFewWideVecs][kC];
+    __shared__ unsigned long long near[kFewWideVecs][8];          // per vector and warp: (distance, centroid)
     const int g = blockIdx.x % G, h = blockIdx.x / G, n_heads = sh.n_kv_heads;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // launched ahead of the end of whatever lies before it in the stream, which may well write the codebooks (a k-means update)
@@ -529,9 +543,9 @@ encode_few_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, 
             }
         }
     }
-    for (int v0 = 0; v0 < n_vec; v0 += kFewVecs) {
-        const int nv = n_vec - v0 < kFewVecs ? n_vec - v0 : kFewVecs;
-        if (threadIdx.x < kFewVecs * kC) {
+    for (int v0 = 0; v0 < n_vec; v0 += kFewWideVecs) {
+        const int nv = n_vec - v0 < kFewWideVecs ? n_vec - v0 : kFewWideVecs;
+        if (threadIdx.x < kFewWideVecs * kC) {
             const int v = threadIdx.x / kC, e = threadIdx.x % kC;
             xs[v][e] = v < nv ? __half2float(x[((int64_t)(v0 + v) * n_heads + h) * 128 + g * kC + e]) : 0.f;
         }
@@ -588,14 +602,16 @@ template <int kC>
 cudaError_t launch_few(const __half* x, const float* cb, const int32_t* seq_offsets, const Shape& sh, int64_t n_tokens, int64_t token_offset,
                        uint8_t* codes, cudaStream_t st, const __half* x2, const float* cb2, uint8_t* codes2)
 {
-    cudaLaunchAttribute attr;
-    cudaLaunchConfig_t cfg = overlapped_config((unsigned)(sh.n_kv_heads * EncCfg<kC>::G), 256, 0, st, &attr);
-    cfg.gridDim.y = x2 ? 2 : 1;
     const int n_vec = (int)(sh.n_seq * n_tokens);
-    auto go = [&](auto kernel) {
-        return cudaLaunchKernelEx(&cfg, kernel, x, cb, seq_offsets, sh, n_vec, (int)n_tokens, token_offset, codes, x2, cb2, codes2);
+    cudaLaunchAttribute attr;
+    cudaLaunchConfig_t cfg = overlapped_config((unsigned)(sh.b == 8 ? few_ctas(sh, n_vec) : sh.n_kv_heads * EncCfg<kC>::G), kFewThreads, 0, st, &attr);
+    cfg.gridDim.y = x2 ? 2 : 1;
+    auto go = [&](auto kernel, auto... share) {
+        return cudaLaunchKernelEx(&cfg, kernel, x, cb, seq_offsets, sh, n_vec, (int)n_tokens, token_offset, codes, x2, cb2, codes2, share...);
     };
-    return sh.b == 8 ? go(encode_few_kernel<kC, 1>) : sh.b == 9 ? go(encode_few_kernel<kC, 2>) : go(encode_few_kernel<kC, 4>);
+    if (sh.b == 8) return go(encode_few_kernel<kC>, few_share(sh, n_vec));
+    if (sh.b == 9) return go(encode_few_wide_kernel<kC, 2>);
+    return go(encode_few_wide_kernel<kC, 4>);
 }
 
 template <int kC, int kMT>

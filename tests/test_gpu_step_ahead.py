@@ -1,0 +1,109 @@
+"""Decode steps whose kernel ahead of the attention appends the tokens and, for few queries, builds the tables of all sequences
+(cq_decode_tables.cu), against cq_encode_kv and cq_decode_attn, whose CTAs build their tables: the entries are the same sums in
+the same order, so the results agree as two calls do."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2405_03917_b200 as cq
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+SPREAD = 2e-6          # two calls of one kernel differ by no more (the weight unit depends on warp timing)
+
+
+def make(c, b, n_seq, n_q, n_kv, D, cap, seed):
+    g = torch.Generator().manual_seed(seed)
+    books = [torch.randn(n_kv, D // c, 1 << b, c, generator=g).to(DEV) for _ in range(2)]
+    x = [torch.randn(n_seq, cap, n_kv, D, generator=g).half().to(DEV) for _ in range(2)]
+    codes = [torch.zeros(cq.cq_codes_bytes(n_seq, cap, n_kv, D, c, b), dtype=torch.uint8, device=DEV) for _ in range(2)]
+    for i in range(2):
+        cq.cq_encode(x[i], books[i], c, b, codes[i], cap)
+    q = torch.randn(n_seq, n_q, D, generator=g).half().to(DEV)
+    new = [torch.randn(n_seq, n_kv, D, generator=g).half().to(DEV) for _ in range(2)]
+    return q, codes, books, new
+
+
+def lengths(n_seq, cap):
+    # empty, one token, both sides of a block's end, a warp's share, one below capacity, capacity
+    edge = [0, 1, 15, 16, 17, min(cap, 129), cap - 1, cap]
+    return torch.tensor([edge[(i * 5) % 8] if i % 3 else (i * 37) % (cap + 1) for i in range(n_seq)], dtype=torch.int32, device=DEV)
+
+
+def close(got, want):
+    got, want = got.double().cpu().numpy(), want.double().cpu().numpy()
+    assert np.abs(got - want).max() <= SPREAD * max(1.0, np.abs(want).max())
+
+
+# (c, b, n_seq, query heads, KV heads): tables ahead (at most 2^18 entries) and not, every width of a CTA, one vector per warp
+# of the append up to more than one warp's share (16), more queries of a KV head than a CTA of the tables takes (32)
+SHAPES = [(2, 8, 4, 3, 3), (2, 8, 33, 4, 2), (4, 8, 1, 1, 1), (4, 8, 5, 3, 3), (4, 8, 7, 8, 2), (4, 8, 37, 2, 2), (8, 8, 1, 1, 1), (8, 8, 9, 6, 1),
+          (8, 8, 34, 1, 1), (8, 8, 34, 4, 2), (8, 8, 17, 8, 2), (8, 10, 4, 2, 2), (8, 10, 6, 8, 2), (8, 10, 15, 1, 1)]
+
+
+@pytest.mark.parametrize("scale", [None, 40.0])          # 40: entries beyond what a half holds, the tables are scaled
+@pytest.mark.parametrize("c,b,n_seq,n_q,n_kv", SHAPES)
+def test_step(c, b, n_seq, n_q, n_kv, scale):
+    cap, D = 700, 128
+    q, codes, books, new = make(c, b, n_seq, n_q, n_kv, D, cap, 3 * c + b + n_seq)
+    if scale:
+        q = q * 64
+    scale = scale or D ** -0.5
+    lens = lengths(n_seq, cap)
+    ref = [x.clone() for x in codes]
+    cq.cq_encode_kv(new[0][:, None].contiguous(), new[1][:, None].contiguous(), *books, c, b, *ref, cap, seq_offsets=lens)
+    want = cq.cq_decode_attn(q, *ref, *books, torch.clamp(lens + 1, max=cap), scale, c, b, cap)
+    got = cq.cq_decode_step(q, *new, lens, *codes, *books, scale, c, b, cap)
+    assert torch.equal(codes[0], ref[0]) and torch.equal(codes[1], ref[1])
+    close(got, want)
+
+
+@pytest.mark.parametrize("n_q", [1, 4])
+def test_contexts_split_over_ctas(n_q):
+    c, b, n_seq, D, cap = 8, 8, 4, 128, 9000
+    q, codes, books, new = make(c, b, n_seq, n_q, 1, D, cap, 1)
+    lens = torch.tensor([9000, 0, 4096, 2047], dtype=torch.int32, device=DEV)
+    ref = [x.clone() for x in codes]
+    cq.cq_encode_kv(new[0][:, None].contiguous(), new[1][:, None].contiguous(), *books, c, b, *ref, cap, seq_offsets=lens)
+    want = cq.cq_decode_attn(q, *ref, *books, torch.clamp(lens + 1, max=cap), D ** -0.5, c, b, cap)
+    got = cq.cq_decode_step(q, *new, lens, *codes, *books, D ** -0.5, c, b, cap)
+    assert torch.equal(codes[0], ref[0]) and torch.equal(codes[1], ref[1])
+    close(got, want)
+
+
+@pytest.mark.parametrize("c,b", [(4, 8), (8, 10)])
+def test_a_workspace_without_room_for_tables(c, b):
+    n_seq, D, cap = 6, 128, 300
+    q, codes, books, new = make(c, b, n_seq, 2, 2, D, cap, 2)
+    lens = lengths(n_seq, cap)
+    full = cq.cq_decode_step_workspace_bytes(n_seq, 2, 2, D, c, b, cap)
+    assert full > n_seq * 2 * (D // c) * (1 << b) * 4
+    ws = torch.empty(full - 256, dtype=torch.uint8, device=DEV)
+    other = [x.clone() for x in codes]
+    want = cq.cq_decode_step(q, *new, lens, *other, *books, D ** -0.5, c, b, cap)
+    got = cq.cq_decode_step(q, *new, lens, *codes, *books, D ** -0.5, c, b, cap, workspace=ws)
+    assert torch.equal(codes[0], other[0]) and torch.equal(codes[1], other[1])
+    close(got, want)
+
+
+def test_steps_right_behind_one_another():
+    # every kernel is launched ahead of the end of the one before: 12 steps without a wait between them against the same steps
+    # with one, the lengths and the caches carried on
+    c, b, n_seq, D, cap = 4, 8, 3, 128, 64
+    q, codes, books, new = make(c, b, n_seq, 2, 2, D, cap, 4)
+    ws = torch.empty(cq.cq_decode_step_workspace_bytes(n_seq, 2, 2, D, c, b, cap), dtype=torch.uint8, device=DEV)
+
+    def run(wait):
+        kv = [x.clone() for x in codes]
+        lens = torch.tensor([0, 15, 40], dtype=torch.int32, device=DEV)
+        outs = []
+        for _ in range(12):
+            outs.append(cq.cq_decode_step(q, *new, lens, *kv, *books, D ** -0.5, c, b, cap, workspace=ws).clone())
+            lens.add_(1)
+            if wait:
+                torch.cuda.synchronize()
+        return outs, kv
+    (a, ka), (w, kw) = run(False), run(True)
+    assert torch.equal(ka[0], kw[0]) and torch.equal(ka[1], kw[1])
+    for x, y in zip(a, w):
+        close(x, y)
