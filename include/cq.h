@@ -376,7 +376,7 @@ int cq_learn_centroids(const void *x_fp16, const float *weights, const double *u
  *                and KV head.  Must not alias each other.
  *   out          [n_seq][n_q_heads][head_dim] fp32, device
  *   workspace    device, 16-byte aligned, cq_decode_step_workspace_bytes(...) bytes (for few queries
- *                they count in the tables, at most 1 MiB; with less than that, but room for the
+ *                they count in the tables, at most 512 KiB; with less than that, but room for the
  *                partials and the lengths, the attention builds its tables itself)
  * Errors: as cq_decode_attn.  Asynchronous on `stream`.
  */

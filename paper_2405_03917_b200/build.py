@@ -10,7 +10,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libcq.so")
 NATIVE = os.path.join(HERE, "_cq_native.so")
-SOURCES = ["cq_api.cu", "cq_generic.cu", "cq_encode.cu", "cq_encode_tc.cu", "cq_encode_grid.cu", "cq_decode.cu", "cq_decode_pair.cu", "cq_decode_rope.cu", "cq_decode_tables.cu", "cq_prefill.cu", "cq_learn.cu"]
+SOURCES = ["cq_api.cu", "cq_generic.cu", "cq_encode.cu", "cq_encode_tc.cu", "cq_encode_grid.cu", "cq_decode.cu", "cq_decode_pair.cu", "cq_decode_rope.cu", "cq_decode_tables.cu", "cq_prefill.cu", "cq_learn.cu", "cq_learn_assign.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "--cudart", "shared", "-Xlinker", "-rpath=/usr/local/cuda/lib64"]
 

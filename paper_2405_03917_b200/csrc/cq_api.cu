@@ -437,7 +437,7 @@ int cq_kmeanspp_init(const void* x_fp16, const float* weights, const double* uni
     int st = learn_shape(n_vec, n_heads, head_dim, c, b, &sh);
     if (st != CQ_OK) return st;
     if (!aligned16(x_fp16) || !aligned16(codebooks_out) || !aligned16(workspace)) return CQ_ERR_ALIGN;
-    if (workspace_bytes < learn_workspace_bytes(sh, n_vec)) return CQ_ERR_WORKSPACE;
+    if (workspace_bytes < learn_least_bytes(sh, n_vec)) return CQ_ERR_WORKSPACE;
     cudaError_t e = launch_kmeanspp_init(static_cast<const __half*>(x_fp16), weights, uniforms, sh, n_vec, codebooks_out,
                                          workspace, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? CQ_OK : CQ_ERR_CUDA;
@@ -454,7 +454,7 @@ int cq_lloyd_step(const void* x_fp16, const float* weights, const float* codeboo
     if (st != CQ_OK) return st;
     if (!aligned16(x_fp16) || !aligned16(codebooks_in) || !aligned16(codebooks_out) || !aligned16(workspace))
         return CQ_ERR_ALIGN;
-    if (workspace_bytes < learn_workspace_bytes(sh, n_vec)) return CQ_ERR_WORKSPACE;
+    if (workspace_bytes < learn_least_bytes(sh, n_vec)) return CQ_ERR_WORKSPACE;
     cudaError_t e = launch_lloyd_step(static_cast<const __half*>(x_fp16), weights, codebooks_in, sh, n_vec, codebooks_out,
                                       objective_out, workspace, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? CQ_OK : CQ_ERR_CUDA;
@@ -470,9 +470,9 @@ int cq_learn_centroids(const void* x_fp16, const float* weights, const double* u
     int st = learn_shape(n_vec, n_heads, head_dim, c, b, &sh);
     if (st != CQ_OK) return st;
     if (!aligned16(x_fp16) || !aligned16(codebooks_out) || !aligned16(workspace)) return CQ_ERR_ALIGN;
-    if (workspace_bytes < learn_workspace_bytes(sh, n_vec)) return CQ_ERR_WORKSPACE;
+    if (workspace_bytes < learn_least_bytes(sh, n_vec)) return CQ_ERR_WORKSPACE;
     cudaError_t e = launch_learn(static_cast<const __half*>(x_fp16), weights, uniforms, sh, n_vec, n_iters, codebooks_out,
-                                 objective_out, workspace, static_cast<cudaStream_t>(stream));
+                                 objective_out, workspace, workspace_bytes, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? CQ_OK : CQ_ERR_CUDA;
 }
 

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <functional>
+
 #include "../../include/cq.h"
 
 namespace cq {
@@ -178,13 +180,23 @@ cudaError_t launch_prefill(const __half* q, const uint8_t* kc, const uint8_t* vc
 cudaError_t launch_add_one(const int32_t* src, int32_t* dst, int n, cudaStream_t st);
 
 // Centroid learning (cq_learn.cu): the vectors are [n_vec][n_heads][head_dim], weights [n_vec][n_heads][G] or null.
-size_t learn_workspace_bytes(const Shape& sh, int64_t n_vec);
+size_t learn_workspace_bytes(const Shape& sh, int64_t n_vec);        // what a call makes use of
+size_t learn_least_bytes(const Shape& sh, int64_t n_vec);            // what it cannot do without
 cudaError_t launch_kmeanspp_init(const __half* x, const float* weights, const double* uniforms, const Shape& sh,
                                  int64_t n_vec, float* codebooks, void* workspace, cudaStream_t st);
 cudaError_t launch_lloyd_step(const __half* x, const float* weights, const float* cb_in, const Shape& sh, int64_t n_vec,
                               float* cb_out, double* objective, void* workspace, cudaStream_t st);
 cudaError_t launch_learn(const __half* x, const float* weights, const double* uniforms, const Shape& sh, int64_t n_vec,
-                         int n_iters, float* codebooks, double* objective, void* workspace, cudaStream_t st);
+                         int n_iters, float* codebooks, double* objective, void* workspace, size_t workspace_bytes, cudaStream_t st);
+
+// k-means iterations that skip what cannot change (cq_learn_assign.cu), in place on `codebooks`.  codes: the layout of one
+// sequence of n_vec tokens; thr: n_vec (rounded up to 16) floats per problem; state: learn_bounds_bytes.  objective(codes,
+// codebooks) launches what forms the objective of the last assignment.
+using LearnObjective = std::function<cudaError_t(const uint8_t*, const float*)>;
+bool learn_bounds_supported(const Shape& sh, int64_t n_vec);
+size_t learn_bounds_bytes(const Shape& sh);
+cudaError_t launch_learn_bounds(const __half* x, const float* weights, const Shape& sh, int64_t n_vec, int n_iters, float* codebooks,
+                                uint8_t* codes, float* thr, void* state, cudaStream_t st, const LearnObjective& objective);
 
 // Configuration of a launch that may start before the kernel ahead of it in the stream has ended (its kernel executes
 // griddepcontrol.wait before it touches memory); `attr` is the caller's and outlives the launch.

@@ -19,10 +19,11 @@ constexpr int kTabThreads = 256;
 constexpr int kTabRows = 32;              // queries of a KV head that a CTA takes at most
 // Entries up to which tables ahead pay (step, us, tables by the attention's CTAs before this kernel appended > tables ahead; the
 // append ahead alone takes attention + 3): 32 heads of CQ-8c8b, 128 tokens, 1 sequence (2^17 entries) 14.5 > 10.7, 2 (2^18)
-// 14.5 > 13.3, 4 (2^19) 14.5 > 14.2; CQ-4c8b, 8 heads on 1, 4 sequences (2^18) 18.6 > 15.9, 32 heads on 8, 4 (2^20) 18.6 > 19.8.
+// 14.5 > 13.3, 4 (2^19) 14.5 > 14.2; 32 heads of CQ-4c8b, 1 sequence of 1063 tokens (2^18) 18.4 > 19.0; 32 heads on 8, 4
+// sequences (2^20) 18.6 > 19.8.
 // With many queries the attention's CTAs overlap their builds with each other's loops, and the tables only cost a
 // trip through L2: 64 sequences of 1024 tokens, 32 heads on 8, CQ-2c8b: attention 180 > 216.
-constexpr int64_t kMostEntries = 1 << 18;
+constexpr int64_t kMostEntries = 1 << 17;
 
 // A warp: eight neighbouring groups x four neighbouring code values at a time (whole sectors of the codebook and of the
 // tables), kU such steps of centroids in registers.

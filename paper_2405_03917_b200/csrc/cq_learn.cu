@@ -849,6 +849,19 @@ cudaError_t launch_update(const __half* x, const float* weights, const uint8_t* 
                               cb_out, objective);
 }
 
+cudaError_t update_dispatch(const __half* x, const float* weights, const uint8_t* codes, const float* cb_in, const Shape& sh,
+                            int64_t n_vec, float* cb_out, double* objective, cudaStream_t st)
+{
+#define CQ_UPD(C_) return sh.G % 2 == 0 ? launch_update<C_, 2>(x, weights, codes, cb_in, sh, n_vec, cb_out, objective, st)   \
+                                        : launch_update<C_, 1>(x, weights, codes, cb_in, sh, n_vec, cb_out, objective, st)
+    switch (sh.c) {
+        case 2: CQ_UPD(2);
+        case 4: CQ_UPD(4);
+        default: CQ_UPD(8);
+    }
+#undef CQ_UPD
+}
+
 size_t round256(size_t v) { return (v + 255) / 256 * 256; }
 
 struct LearnLayout {
@@ -868,7 +881,11 @@ LearnLayout learn_layout(const Shape& sh, int64_t n_vec)
 
 }  // namespace
 
-size_t learn_workspace_bytes(const Shape& sh, int64_t n_vec) { return learn_layout(sh, n_vec).total; }
+size_t learn_least_bytes(const Shape& sh, int64_t n_vec) { return learn_layout(sh, n_vec).total; }
+size_t learn_workspace_bytes(const Shape& sh, int64_t n_vec)
+{
+    return learn_least_bytes(sh, n_vec) + (learn_bounds_supported(sh, n_vec) ? learn_bounds_bytes(sh) : 0);
+}
 
 cudaError_t launch_kmeanspp_init(const __half* x, const float* weights, const double* uniforms, const Shape& sh,
                                  int64_t n_vec, float* codebooks, void* workspace, cudaStream_t st)
@@ -908,17 +925,7 @@ cudaError_t launch_lloyd_step(const __half* x, const float* weights, const float
     cudaError_t e = encode_tuned_supported(es) ? launch_encode_tuned(x, cb_in, nullptr, es, n_vec, 0, codes, st)
                                                : launch_encode_generic(x, cb_in, nullptr, es, n_vec, 0, codes, st);
     if (e != cudaSuccess) return e;
-    if (sh.K <= kUpdMaxK && (sh.c == 2 || sh.c == 4 || sh.c == 8)) {
-#define CQ_UPD(C_) e = sh.G % 2 == 0 ? launch_update<C_, 2>(x, weights, codes, cb_in, es, n_vec, cb_out, objective, st)   \
-                                     : launch_update<C_, 1>(x, weights, codes, cb_in, es, n_vec, cb_out, objective, st)
-        switch (sh.c) {
-            case 2: CQ_UPD(2); break;
-            case 4: CQ_UPD(4); break;
-            default: CQ_UPD(8); break;
-        }
-#undef CQ_UPD
-        return e;
-    }
+    if (sh.K <= kUpdMaxK && (sh.c == 2 || sh.c == 4 || sh.c == 8)) return update_dispatch(x, weights, codes, cb_in, es, n_vec, cb_out, objective, st);
     const size_t smem = (size_t)(2 * sh.K * sh.c + sh.K) * sizeof(float);
     e = ensure_dynamic_smem(reinterpret_cast<const void*>(lloyd_update_generic_kernel), (int)smem, 34);
     if (e != cudaSuccess) return e;
@@ -928,12 +935,24 @@ cudaError_t launch_lloyd_step(const __half* x, const float* weights, const float
 }
 
 cudaError_t launch_learn(const __half* x, const float* weights, const double* uniforms, const Shape& sh, int64_t n_vec,
-                         int n_iters, float* codebooks, double* objective, void* workspace, cudaStream_t st)
+                         int n_iters, float* codebooks, double* objective, void* workspace, size_t workspace_bytes, cudaStream_t st)
 {
     const LearnLayout l = learn_layout(sh, n_vec);
     float* tmp = reinterpret_cast<float*>(static_cast<char*>(workspace) + l.codes + 2 * l.dist);
     cudaError_t e = launch_kmeanspp_init(x, weights, uniforms, sh, n_vec, codebooks, workspace, st);
     if (e != cudaSuccess) return e;
+    if (n_iters > 0 && learn_bounds_supported(sh, n_vec) && workspace_bytes >= l.total + learn_bounds_bytes(sh)) {
+        Shape es = sh;                                      // the vectors are one sequence of n_vec tokens
+        es.n_seq = 1;
+        es.max_tokens = n_vec;
+        es.n_blocks = (n_vec + kTokenBlock - 1) / kTokenBlock;
+        // (the thresholds take the place of the distances of the initialisation: 4 bytes for 8)
+        return launch_learn_bounds(x, weights, es, n_vec, n_iters, codebooks, static_cast<uint8_t*>(workspace),
+                                   reinterpret_cast<float*>(static_cast<char*>(workspace) + l.codes), static_cast<char*>(workspace) + l.total, st,
+                                   [&](const uint8_t* codes, const float* cb) {
+                                       return objective ? update_dispatch(x, weights, codes, cb, es, n_vec, tmp, objective, st) : cudaSuccess;
+                                   });
+    }
     float* cur = codebooks;
     float* nxt = tmp;
     for (int it = 0; it < n_iters; ++it) {

@@ -1,0 +1,95 @@
+"""Iterations of cq_learn_centroids that skip vectors whose nearest centroid cannot have changed (cq_learn_assign.cu) against
+iterations that evaluate every vector (cq_lloyd_step)."""
+import pytest
+import torch
+
+import paper_2405_03917_b200 as cq
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+D = 128
+
+
+def vectors(n, heads, seed, scale=1.0):
+    g = torch.Generator().manual_seed(seed)
+    A = torch.randn(heads, 32, D, generator=g) / 32 ** 0.5
+    x = torch.einsum("nhr,hrd->nhd", torch.randn(n, heads, 32, generator=g), A) + 0.1 * torch.randn(n, heads, D, generator=g)
+    x = x + 0.5 * torch.randn(heads, D, generator=g)
+    x[..., ::31] = 8 + 5 * x[..., ::31]
+    return (scale * x).half().contiguous().to(DEV), g
+
+
+def learn(x, w, u, c, iters):
+    return cq.cq_learn_centroids(x, w, u, c, 8, iters)
+
+
+def plain(x, w, u, c, iters):
+    cb, obj = cq.cq_kmeanspp_init(x, w, u, c, 8), None
+    for _ in range(iters):
+        cb, obj = cq.cq_lloyd_step(x, w, cb, c, 8)
+    return cb, obj
+
+
+# one tile and less, a tile's end, several CTAs to a problem (more than 4096 vectors), blocks of 16 that are not whole
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("c,n,heads", [(8, 300, 2), (8, 1024, 1), (8, 4097, 1), (4, 333, 2), (4, 2047, 1), (4, 9001, 1)])
+def test_the_first_iterations_are_those_of_full_evaluation(c, n, heads, weighted):
+    x, g = vectors(n, heads, c + n)
+    w = torch.randn(n, heads, D // c, generator=g).square().to(DEV) if weighted else None
+    u = torch.rand(heads, D // c, 256, generator=g, dtype=torch.float64).to(DEV)
+    for iters in (1, 2, 5):
+        a, oa = learn(x, w, u, c, iters)
+        b, ob = plain(x, w, u, c, iters)
+        # fp32 sums of up to n / 256 members on one side: 1e-5 of the largest channel.  A vector whose two nearest centroids
+        # are that close may part the two runs: of five iterations' 5 n evaluations fewer than one in 10^5 is.
+        off = (a - b).abs().amax(dim=(2, 3)) > 1e-5 * b.abs().amax()
+        assert off.float().mean() <= 5 * n * iters * 1e-5 / 5, (iters, off.sum())
+        assert torch.allclose(oa, ob, rtol=1e-3)
+
+
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** -9])
+@pytest.mark.parametrize("c,n,heads,weighted", [(8, 700, 2, True), (8, 1500, 1, False), (4, 900, 1, True), (4, 600, 2, False)])
+def test_what_has_converged_is_a_fixed_point_of_full_evaluation(c, n, heads, weighted, scale):
+    # few vectors to a centroid converge within some twenty iterations; a vector wrongly skipped would move a centroid now
+    x, g = vectors(n, heads, 7 * c + n, scale)
+    w = torch.rand(n, heads, D // c, generator=g).add(0.1).to(DEV) if weighted else None
+    u = torch.rand(heads, D // c, 256, generator=g, dtype=torch.float64).to(DEV)
+    a, _ = learn(x, w, u, c, 80)
+    b, _ = cq.cq_lloyd_step(x, w, a, c, 8)
+    assert (a - b).abs().amax() <= 1e-5 * a.abs().amax()
+    again, _ = learn(x, w, u, c, 80)
+    assert torch.equal(a, again)                       # whole-number sums: no order of additions shows
+
+
+@pytest.mark.parametrize("c", [4, 8])
+def test_weights_over_many_orders_of_magnitude(c):
+    n = 1000
+    x, g = vectors(n, 1, c)
+    w = torch.pow(10.0, -12 * torch.rand(n, 1, D // c, generator=g)).to(DEV)
+    w[::7] = 0
+    u = torch.rand(1, D // c, 256, generator=g, dtype=torch.float64).to(DEV)
+    a, oa = learn(x, w, u, c, 3)
+    b, ob = plain(x, w, u, c, 3)
+    off = (a - b).abs().amax(dim=(2, 3)) > 1e-5 * b.abs().amax()
+    assert off.float().mean() <= 0.1 and torch.allclose(oa, ob, rtol=1e-3)
+
+
+@pytest.mark.parametrize("what", ["inf", "nan", "negative weight", "infinite weight"])
+def test_problems_without_bounds(what):
+    # the problem that holds the value is evaluated in full; the others keep their result
+    n, c, heads = 500, 8, 2
+    x, g = vectors(n, heads, 3)
+    w = torch.rand(n, heads, D // c, generator=g).add(0.1).to(DEV)
+    u = torch.rand(heads, D // c, 256, generator=g, dtype=torch.float64).to(DEV)
+    good, _ = learn(x, w, u, c, 4)
+    if what in ("inf", "nan"):
+        x[17, 1, 8 * 3 + 2] = float(what)
+    else:
+        w[17, 1, 3] = -0.5 if what == "negative weight" else float("inf")
+    got, _ = learn(x, w, u, c, 4)
+    keep = torch.ones(heads, D // c, dtype=torch.bool)
+    keep[1, 3] = False
+    assert torch.equal(got[keep.to(DEV)], good[keep.to(DEV)])
+    if what == "negative weight":
+        want, _ = plain(x, w, u, c, 4)
+        assert torch.allclose(got[1, 3], want[1, 3], rtol=1e-4, atol=1e-4)

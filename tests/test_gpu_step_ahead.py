@@ -35,7 +35,7 @@ def close(got, want):
     assert np.abs(got - want).max() <= SPREAD * max(1.0, np.abs(want).max())
 
 
-# (c, b, n_seq, query heads, KV heads): tables ahead (at most 2^18 entries) and not, every width of a CTA, one vector per warp
+# (c, b, n_seq, query heads, KV heads): tables ahead (at most 2^17 entries) and not, every width of a CTA, one vector per warp
 # of the append up to more than one warp's share (16), more queries of a KV head than a CTA of the tables takes (32)
 SHAPES = [(2, 8, 4, 3, 3), (2, 8, 33, 4, 2), (4, 8, 1, 1, 1), (4, 8, 5, 3, 3), (4, 8, 7, 8, 2), (4, 8, 37, 2, 2), (8, 8, 1, 1, 1), (8, 8, 9, 6, 1),
           (8, 8, 34, 1, 1), (8, 8, 34, 4, 2), (8, 8, 17, 8, 2), (8, 10, 4, 2, 2), (8, 10, 6, 8, 2), (8, 10, 15, 1, 1)]
