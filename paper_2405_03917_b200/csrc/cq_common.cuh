@@ -200,7 +200,19 @@ cudaError_t launch_learn_bounds(const __half* x, const float* weights, const Sha
 
 // Configuration of a launch that may start before the kernel ahead of it in the stream has ended (its kernel executes
 // griddepcontrol.wait before it touches memory); `attr` is the caller's and outlives the launch.
-cudaLaunchConfig_t overlapped_config(unsigned grid, unsigned threads, size_t smem, cudaStream_t st, cudaLaunchAttribute* attr);
+inline cudaLaunchConfig_t overlapped_config(unsigned grid, unsigned threads, size_t smem, cudaStream_t st, cudaLaunchAttribute* attr)
+{
+    attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr->val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
 
 // Merge of split-K partials into out (shared by the decode kernels).
 cudaError_t launch_merge(const float* partials, int n_parts, const Shape& sh, float* out, cudaStream_t st);

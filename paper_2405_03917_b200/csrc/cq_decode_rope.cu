@@ -80,6 +80,8 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
                          const float* __restrict__ rope_cos, const float* __restrict__ rope_sin, float scale_log2e, Shape sh,
                          int n_splits, int split_tokens, float* __restrict__ partials, float* __restrict__ out)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory");      // launched ahead of the end of the kernel before it, and
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");       // the kernel behind it ahead of its own
     using C = RtCfg<kC, kHeads>;
     constexpr int G = C::G, kT = C::kT, kWords = kT / 4, kRtThreads = C::kThreads, kRtWarps = kRtThreads / 32;
     extern __shared__ __align__(16) unsigned char rt_smem[];
@@ -527,9 +529,10 @@ cudaError_t launch_rt(const __half* q, const uint8_t* kc, const uint8_t* vc, con
     cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(decode_rope_tuned_kernel<kC, kHeads>), C::kSmemBytes, kSlot);
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)(sh.n_seq * (sh.n_q_heads / kHeads) * n_splits);
-    decode_rope_tuned_kernel<kC, kHeads><<<grid, C::kThreads, C::kSmemBytes, st>>>(q, kc, vc, kcb, vcb, seq_lens, rope_cos, rope_sin,
-                                                                                  scale * kLog2e, sh, n_splits, split_tokens, partials, out);
-    return cudaGetLastError();
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = overlapped_config(grid, C::kThreads, C::kSmemBytes, st, &attr);
+    return cudaLaunchKernelEx(&cfg, decode_rope_tuned_kernel<kC, kHeads>, q, kc, vc, kcb, vcb, seq_lens, rope_cos, rope_sin,
+                              scale * kLog2e, sh, n_splits, split_tokens, partials, out);
 }
 
 int rope_heads_per_cta(const Shape& sh)

@@ -501,6 +501,7 @@ encode_few_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, 
 {
     // launched ahead of the end of whatever lies before it in the stream, which may well write the codebooks (a k-means update)
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const bool second = blockIdx.y != 0;
     encode_few<kC>(second ? x2 : x1, second ? cb2 : cb1, seq_offsets, sh, blockIdx.x, n_vec, share, n_tokens,
                          token_offset, second ? codes2 : codes1, false);
@@ -528,6 +529,7 @@ encode_few_wide_kernel(const __half* __restrict__ x1, const float* __restrict__ 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // launched ahead of the end of whatever lies before it in the stream, which may well write the codebooks (a k-means update)
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     float cv[kPer][kC];
 #pragma unroll
     for (int u = 0; u < kPer; ++u) {

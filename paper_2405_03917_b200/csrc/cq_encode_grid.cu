@@ -126,6 +126,8 @@ encode_grid_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1,
                    uint32_t n_tokens, int64_t token_offset, uint8_t* __restrict__ codes1, const __half* __restrict__ x2,
                    const float* __restrict__ cb2, uint8_t* __restrict__ codes2, int n_units, uint32_t warps_per_unit)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory");      // launched ahead of the end of the kernel before it, and
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");       // the kernel behind it ahead of its own
     constexpr int G = 64, kSets = G / kGrGroups;
     extern __shared__ __align__(16) unsigned char gr_smem[];
     uint32_t* cells = reinterpret_cast<uint32_t*>(gr_smem + GrSmem::kCellOff);
@@ -463,9 +465,10 @@ cudaError_t launch_encode_grid(const __half* x, const float* cb, const int32_t* 
     if (e != cudaSuccess) return e;
     const int n_units = (x2 ? 2 : 1) * sh.n_kv_heads * (64 / kGrGroups);
     const uint32_t per_unit = (uint32_t)((sh.n_seq * n_tokens + 31) / 32);
-    encode_grid_kernel<<<(unsigned)device_sm_count(), kGrThreads, GrSmem::kBytes, st>>>(
-        x, cb, seq_offsets, sh, (uint32_t)n_tokens, token_offset, codes, x2, cb2, codes2, n_units, per_unit);
-    return cudaGetLastError();
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = overlapped_config((unsigned)device_sm_count(), kGrThreads, GrSmem::kBytes, st, &attr);
+    return cudaLaunchKernelEx(&cfg, encode_grid_kernel, x, cb, seq_offsets, sh, (uint32_t)n_tokens, token_offset, codes, x2, cb2, codes2,
+                              n_units, per_unit);
 }
 
 }  // namespace cq

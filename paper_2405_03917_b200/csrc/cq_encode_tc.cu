@@ -53,6 +53,8 @@ encode_tc_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, c
                  Shape sh, int64_t n_tokens, int64_t token_offset, uint8_t* __restrict__ codes1, int groups_per_cta, int log_rt,
                  const __half* __restrict__ x2, const float* __restrict__ cb2, uint8_t* __restrict__ codes2)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory");      // launched ahead of the end of the kernel before it, and
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");       // the kernel behind it ahead of its own
     const __half* x = blockIdx.y ? x2 : x1;
     const float* cb = blockIdx.y ? cb2 : cb1;
     uint8_t* codes = blockIdx.y ? codes2 : codes1;
@@ -335,9 +337,11 @@ cudaError_t launch_enc_tc(const __half* x, const float* cb, const int32_t* seq_o
     constexpr int kSlot = kSlots[3 * (kC == 2 ? 0 : kC == 4 ? 1 : 2) + (kChunks == 1 ? 0 : kChunks == 2 ? 1 : 2)];
     cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(encode_tc_kernel<kC, kChunks>), C::kSmemBytes, kSlot);
     if (e != cudaSuccess) return e;
-    encode_tc_kernel<kC, kChunks><<<dim3((unsigned)grid, x2 ? 2u : 1u), kTcThreads, C::kSmemBytes, st>>>(
-        x, cb, seq_offsets, sh, n_tokens, token_offset, codes, groups_per_cta, log_rt, x2, cb2, codes2);
-    return cudaGetLastError();
+    cudaLaunchAttribute attr;
+    cudaLaunchConfig_t cfg = overlapped_config((unsigned)grid, kTcThreads, C::kSmemBytes, st, &attr);
+    cfg.gridDim.y = x2 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, encode_tc_kernel<kC, kChunks>, x, cb, seq_offsets, sh, n_tokens, token_offset, codes, groups_per_cta,
+                              log_rt, x2, cb2, codes2);
 }
 
 }  // namespace

@@ -581,6 +581,7 @@ merge_kernel(const float* __restrict__ partials, int n_parts, Shape sh, float* _
     const float* base = partials + (s * sh.n_q_heads + hq) * (int64_t)n_parts * stride;
     float* o = out + (s * sh.n_q_heads + hq) * (int64_t)sh.head_dim;
     asm volatile("griddepcontrol.wait;" ::: "memory");      // launched ahead of the end of the kernel that writes the partials
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     float M = -INFINITY;
     for (int p = lane; p < n_parts; p += 32) M = fmaxf(M, base[p * stride]);
     for (int d = 16; d > 0; d >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, d));
@@ -617,22 +618,6 @@ merge_kernel(const float* __restrict__ partials, int n_parts, Shape sh, float* _
     for (int d = 16; d > 0; d >>= 1) L += __shfl_xor_sync(0xffffffffu, L, d);
     if (d0 < sh.head_dim) o[d0] = a[0] / L;
     if (d1 < sh.head_dim) o[d1] = a[1] / L;
-}
-
-// A launch that may start before the kernel ahead of it in the stream has ended (its kernel waits for that end itself,
-// with griddepcontrol.wait, before it touches memory): the launch's own latency passes behind that kernel.
-cudaLaunchConfig_t overlapped_config(unsigned grid, unsigned threads, size_t smem, cudaStream_t st, cudaLaunchAttribute* attr)
-{
-    attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr->val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cfg;
 }
 
 cudaError_t launch_merge(const float* partials, int n_parts, const Shape& sh, float* out, cudaStream_t st)

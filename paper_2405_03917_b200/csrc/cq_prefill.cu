@@ -261,6 +261,8 @@ prefill_tc_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, 
                   const int32_t* __restrict__ seq_lens, float scale_log2e, Shape sh, int n_q, int row_tiles,
                   float* __restrict__ out)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory");      // launched ahead of the end of the kernel before it, and
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");       // the kernel behind it ahead of its own
     using C = PfCfg;
     constexpr int G = 128 / kC;
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -683,25 +685,14 @@ cudaError_t launch_prefill(const __half* q, const uint8_t* kc, const uint8_t* vc
         const int row_tiles = (n_q + q_per_tile - 1) / q_per_tile;
         const int64_t grid = sh.n_seq * sh.n_kv_heads * row_tiles;
         if (grid > 0x7fffffff) return cudaErrorInvalidConfiguration;
-        cudaError_t e = cudaSuccess;
-        switch (sh.c) {
-            case 8:
-                e = ensure_dynamic_smem(reinterpret_cast<const void*>(prefill_tc_kernel<8>), C::kSmemBytes, 40);
-                if (e != cudaSuccess) return e;
-                prefill_tc_kernel<8><<<(unsigned)grid, C::kThreads, C::kSmemBytes, st>>>(q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, n_q, row_tiles, out);
-                break;
-            case 4:
-                e = ensure_dynamic_smem(reinterpret_cast<const void*>(prefill_tc_kernel<4>), C::kSmemBytes, 41);
-                if (e != cudaSuccess) return e;
-                prefill_tc_kernel<4><<<(unsigned)grid, C::kThreads, C::kSmemBytes, st>>>(q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, n_q, row_tiles, out);
-                break;
-            default:
-                e = ensure_dynamic_smem(reinterpret_cast<const void*>(prefill_tc_kernel<2>), C::kSmemBytes, 42);
-                if (e != cudaSuccess) return e;
-                prefill_tc_kernel<2><<<(unsigned)grid, C::kThreads, C::kSmemBytes, st>>>(q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, n_q, row_tiles, out);
-                break;
-        }
-        return cudaGetLastError();
+        cudaLaunchAttribute attr;
+        const cudaLaunchConfig_t cfg = overlapped_config((unsigned)grid, C::kThreads, C::kSmemBytes, st, &attr);
+        auto go = [&](auto kernel, int slot) {
+            const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), C::kSmemBytes, slot);
+            if (e != cudaSuccess) return e;
+            return cudaLaunchKernelEx(&cfg, kernel, q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, n_q, row_tiles, out);
+        };
+        return sh.c == 8 ? go(prefill_tc_kernel<8>, 40) : sh.c == 4 ? go(prefill_tc_kernel<4>, 41) : go(prefill_tc_kernel<2>, 42);
     }
     const int64_t grid = sh.n_seq * (int64_t)n_q * sh.n_q_heads;
     if (grid > 0x7fffffff) return cudaErrorInvalidConfiguration;

@@ -73,7 +73,7 @@ def test_contexts_split_over_ctas(n_q):
 
 @pytest.mark.parametrize("c,b", [(4, 8), (8, 10)])
 def test_a_workspace_without_room_for_tables(c, b):
-    n_seq, D, cap = 6, 128, 300
+    n_seq, D, cap = 4, 128, 300
     q, codes, books, new = make(c, b, n_seq, 2, 2, D, cap, 2)
     lens = lengths(n_seq, cap)
     full = cq.cq_decode_step_workspace_bytes(n_seq, 2, 2, D, c, b, cap)
