@@ -161,6 +161,14 @@ size_t decode_tables_bytes(const Shape& sh);
 cudaError_t launch_decode_ahead(const __half* q, const float* kcb, const float* vcb, const int32_t* seq_lens, float scale,
                                 const Shape& sh, float* tables, const AppendArgs& app, cudaStream_t st);
 
+// Copies up to four pieces of pinned host memory (device addresses) to the device with a kernel (cq_decode_tables.cu).
+struct HostPieces {
+    const void* src[4];
+    void* dst[4];
+    size_t bytes[4];
+};
+cudaError_t launch_fetch_host(const HostPieces& pieces, cudaStream_t st);
+
 // CQ-8c8b with a multiple of four query heads per KV head: two query heads per table word (cq_decode_pair.cu).
 bool decode_pair_supported(const Shape& sh);
 DecodePlan decode_pair_plan(const Shape& sh);

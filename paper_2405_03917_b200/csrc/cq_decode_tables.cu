@@ -114,7 +114,38 @@ cudaError_t launch_ahead(const __half* q, const float* kcb, const float* vcb, co
     return go(decode_ahead_kernel<kC, kPer>);
 }
 
+// A step's inputs from pinned host memory: reads over the bus, a thread 16 bytes at a time, and no hand-over between the copy
+// engine and the kernels behind.
+constexpr int kFetchThreads = 256;
+__global__ void __launch_bounds__(kFetchThreads) fetch_host_kernel(HostPieces p)
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");      // whatever lies ahead may still read the staging area
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const size_t t = (size_t)blockIdx.x * kFetchThreads + threadIdx.x, step = (size_t)gridDim.x * kFetchThreads;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const char* src = static_cast<const char*>(p.src[i]);
+        char* dst = static_cast<char*>(p.dst[i]);
+        if (((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15u) == 0) {
+            const size_t n = p.bytes[i] / 16;
+            for (size_t k = t; k < n; k += step) reinterpret_cast<uint4*>(dst)[k] = reinterpret_cast<const uint4*>(src)[k];
+            if (t < p.bytes[i] % 16) dst[n * 16 + t] = src[n * 16 + t];
+        } else {
+            for (size_t k = t; k < p.bytes[i]; k += step) dst[k] = src[k];
+        }
+    }
+}
+
 }  // namespace
+
+cudaError_t launch_fetch_host(const HostPieces& pieces, cudaStream_t st)
+{
+    const size_t total = pieces.bytes[0] + pieces.bytes[1] + pieces.bytes[2] + pieces.bytes[3];
+    const size_t ctas = (total + 16 * kFetchThreads - 1) / (16 * kFetchThreads), most = 2 * (size_t)device_sm_count();
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = overlapped_config((unsigned)(ctas < most ? ctas : most), kFetchThreads, 0, st, &attr);
+    return cudaLaunchKernelEx(&cfg, fetch_host_kernel, pieces);
+}
 
 bool decode_tables_pay(const Shape& sh)
 {

@@ -107,3 +107,30 @@ def test_steps_right_behind_one_another():
     assert torch.equal(ka[0], kw[0]) and torch.equal(ka[1], kw[1])
     for x, y in zip(a, w):
         close(x, y)
+
+
+@pytest.mark.parametrize("c,b,n_seq,n_q,n_kv", [(8, 8, 3, 8, 2), (4, 8, 2, 3, 3), (8, 10, 2, 2, 1), (4, 4, 2, 2, 2)])
+@pytest.mark.parametrize("how", ["pinned", "one block", "off by two bytes", "pageable", "pageable result"])
+def test_host_buffers(c, b, n_seq, n_q, n_kv, how):
+    # pinned buffers are read and written by kernels (16 bytes at a time where they are aligned), others are copied
+    D, cap = 128, 200
+    q, codes, books, new = make(c, b, n_seq, n_q, n_kv, D, cap, 9 + c)
+    lens = torch.arange(5, 5 + 60 * n_seq, 60, dtype=torch.int32)
+    other = [x.clone() for x in codes]
+    want = cq.cq_decode_step(q, *new, lens.to(DEV), *other, *books, D ** -0.5, c, b, cap)
+    parts = [q, *new]
+    skip = 1 if how == "off by two bytes" else 0
+    pin = (lambda t: t) if how == "pageable" else (lambda t: t.pin_memory())
+    if how == "pinned":
+        host = [pin(p.cpu()) for p in parts]
+    else:
+        block = pin(torch.empty(sum(p.numel() for p in parts) + skip, dtype=torch.float16))
+        host, at = [], skip
+        for p in parts:
+            host.append(block[at:at + p.numel()].view(p.shape).copy_(p.cpu()))
+            at += p.numel()
+    out = torch.empty(n_seq, n_q, D) if "pageable" in how else torch.empty(n_seq, n_q, D).pin_memory()
+    ws = torch.empty(cq.cq_decode_step_host_workspace_bytes(n_seq, n_q, n_kv, D, c, b, cap), dtype=torch.uint8, device=DEV)
+    got = cq.cq_decode_step_host(*host, pin(lens), *codes, *books, D ** -0.5, c, b, cap, out, ws)
+    assert torch.equal(codes[0], other[0]) and torch.equal(codes[1], other[1])
+    close(got, want)
