@@ -8,6 +8,7 @@
 // pp_cluster_kernel draws the same vectors from sums in another order, with a proof per draw that the
 // order does not matter (and the ordered sum where it might); pp_pick_kernel and pp_dist_kernel are
 // the plain form for shapes it does not take.
+#include "cq_bulk_copy.cuh"
 #include "cq_common.cuh"
 
 namespace cq {
@@ -115,7 +116,7 @@ pp_pick_kernel(const __half* __restrict__ x, const double* __restrict__ uniforms
 
 // k-means++ of a whole problem by one thread-block cluster.  The vectors of the problem are split over the CTAs of
 // the cluster (kPpSlice each at most) and stay on chip for all the draws: the vectors and weights in shared memory,
-// distances and contributions in registers.  One draw is two cluster barriers:
+// distances and contributions in registers.  One draw is two exchanges:
 //   1. every thread brings the distances of its vectors up to date with the last centre (an fp32 bound with its
 //      rounding error taken off rules out nearly all of them, the others are evaluated in fp64 as defined), the warps
 //      sum their contributions and hand the sums to every CTA of the cluster;
@@ -126,18 +127,59 @@ pp_pick_kernel(const __half* __restrict__ x, const double* __restrict__ uniforms
 // n 2^-53 of the total T, so where the target is farther than that from both ends of the vector's interval the two
 // orders draw the same vector.  Otherwise (about one draw in a million) the cluster writes its contributions out and
 // one thread adds them up in index order.  Measured (32768 vectors, 512 problems, 256 centres, c = 8, weighted):
-// 213 -> 21.7 ms, 5.3 us a draw and cluster; what is left is the latency of the two exchanges and of the fp64 shuffles.
+// 213 -> 21.7 ms with a cluster barrier after each exchange and the drawn vector read from memory again, 19.9 as it is now.
+// A draw takes 12.8 thousand cycles with two CTAs on an SM: 3.9 the distances (mostly those that go to fp64, where the
+// conversions take the time; exact differences built from the bits instead of conversions: 28.8 ms), 2.8 the wait for the
+// slowest warp's sum, 1.5 finding the warp, 1.6 the wait for the vector.
 constexpr int kPpThreads = 512;
 constexpr int kPpWarps = kPpThreads / 32;
 constexpr int kPpPer = 8;                          // vectors per thread
 constexpr int kPpSlice = kPpThreads * kPpPer;      // vectors per CTA
+constexpr int kPpUniforms = 256;                   // of a problem, kept on chip
 constexpr int kPpMaxCluster = 8;                   // portable cluster size
 
+// Draw k uses the buffers k & 1.  A CTA sends what belongs to draw k + 2 only when it knows the centre of draw k + 1, which
+// takes the sums of every warp of the cluster, so whatever belongs to draw k has been read by then.
 struct PpCtl {
-    double sums[kPpMaxCluster * kPpWarps];         // contributions per (CTA of the cluster, warp), in index order
-    long long pick;                                // the drawn vector; -1: too close to call
-    uint32_t centre[4];                            // its channels, fp16
+    double sums[2][kPpMaxCluster * kPpWarps];      // contributions per (CTA of the cluster, warp), in index order
+    alignas(16) uint32_t centre[2][4];             // the drawn vector's channels, fp16
+    long long pick[2];                             // the drawn vector; -1: too close to call
+    uint64_t sums_here[2], pick_here[2];           // mbarriers: all of that has arrived
 };
+
+// Stores to another CTA's shared memory that count themselves at an mbarrier there.
+__device__ __forceinline__ void pp_send64(uint32_t to, unsigned long long v, uint32_t bar)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(to), "l"(v), "r"(bar) : "memory");
+}
+template <int kWords>
+__device__ __forceinline__ void pp_send32(uint32_t to, const uint32_t (&w)[kWords], uint32_t bar)
+{
+    if (kWords == 4)
+        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                     ::"r"(to), "r"(w[0]), "r"(w[1 % kWords]), "r"(w[2 % kWords]), "r"(w[3 % kWords]), "r"(bar) : "memory");
+    else if (kWords == 2)
+        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];"
+                     ::"r"(to), "r"(w[0]), "r"(w[1 % kWords]), "r"(bar) : "memory");
+    else
+        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(to), "r"(w[0]), "r"(bar) : "memory");
+}
+// The next phase of an mbarrier (nothing is ordered by it: what it counts is sent later).
+__device__ __forceinline__ void pp_arm(uint64_t* bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.relaxed.cta.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
+}
+// Waits for the phase with the given parity; gives up after a bounded number of polls (returns false).
+__device__ __forceinline__ bool pp_wait(uint64_t* bar, uint32_t parity)
+{
+    for (int poll = 0; poll < (1 << 22); ++poll) {
+        uint32_t done;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(done) : "r"(smem_addr(bar)), "r"(parity) : "memory");
+        if (done) return true;
+    }
+    return false;
+}
 
 __device__ __forceinline__ uint32_t pp_map_shared(const void* p, int rank)
 {
@@ -212,6 +254,7 @@ pp_cluster_kernel(const __half* __restrict__ x, const float* __restrict__ weight
 {
     extern __shared__ __align__(16) unsigned char pp_smem[];        // [slice][kC] fp16, then [slice] weights
     __shared__ PpCtl ctl;
+    __shared__ double us[kPpUniforms];
     unsigned char* xs = pp_smem;
     float* ws = reinterpret_cast<float*>(pp_smem + (size_t)slice * kC * 2);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -236,19 +279,40 @@ pp_cluster_kernel(const __half* __restrict__ x, const float* __restrict__ weight
         part[j] = 0.0;
     }
     const double* up = uniforms + (int64_t)p * K;
-    for (int i = threadIdx.x; i < kPpMaxCluster * kPpWarps; i += kPpThreads) ctl.sums[i] = 0.0;
+    for (int i = threadIdx.x; i < kPpMaxCluster * kPpWarps; i += kPpThreads) ctl.sums[0][i] = ctl.sums[1][i] = 0.0;
+    constexpr uint32_t kPickBytes = kC * 2 + 8;
+    const uint32_t sums_bytes = (uint32_t)cluster * kPpWarps * 8;
+    if (threadIdx.x == 0) {
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&ctl.sums_here[b], 1);
+            mbar_init(&ctl.pick_here[b], 1);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        for (int b = 0; b < 2; ++b) {
+            pp_arm(&ctl.sums_here[b], sums_bytes);
+            pp_arm(&ctl.pick_here[b], kPickBytes);
+        }
+    }
+    __syncthreads();
     pp_cluster_sync();                                              // every CTA of the cluster has started: its memory may be written
 
-    // The vector `pick` (index within the problem) becomes centre k: one whole warp hands it to every CTA.
-    auto publish = [&](int64_t pick, int k) {
-        uint32_t w[kC / 2];
-        pp_words<kC>(reinterpret_cast<const unsigned char*>(x + (pick * n_prob + p) * kC), w);
+    // The vector `pick` (index within the problem, its words w) becomes centre k: one whole warp hands it to every CTA.  plain:
+    // between two cluster barriers, for a draw that was undecided; otherwise counted at the CTAs' mbarriers.
+    auto publish = [&](int64_t pick, int k, const uint32_t (&w)[kC / 2], bool plain) {
+        const int b = k & 1;
         if (lane < cluster) {
+            if (plain) {
 #pragma unroll
-            for (int q = 0; q < kC / 2; ++q)
-                asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(pp_map_shared(&ctl.centre[q], lane)), "r"(w[q]) : "memory");
-            asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(pp_map_shared(&ctl.pick, lane)), "l"((long long)pick) : "memory");
+                for (int q = 0; q < kC / 2; ++q)
+                    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(pp_map_shared(&ctl.centre[b][q], lane)), "r"(w[q]) : "memory");
+                asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(pp_map_shared(&ctl.pick[b], lane)), "l"((long long)pick) : "memory");
+            } else {
+                const uint32_t bar = pp_map_shared(&ctl.pick_here[b], lane);
+                pp_send32<kC / 2>(pp_map_shared(&ctl.centre[b][0], lane), w, bar);
+                pp_send64(pp_map_shared(&ctl.pick[b], lane), (unsigned long long)pick, bar);
+            }
         }
+        if (pick < 0) return;
         if (lane == 0) {
             float* cb = codebooks + ((int64_t)p * K + k) * kC;
 #pragma unroll
@@ -259,9 +323,10 @@ pp_cluster_kernel(const __half* __restrict__ x, const float* __restrict__ weight
             }
         }
     };
-    auto undecided = [&]() {
-        if (lane < cluster)
-            asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(pp_map_shared(&ctl.pick, lane)), "l"(-1ll) : "memory");
+    auto publish_any = [&](int64_t pick, int k, bool plain) {        // (a vector that may lie in another CTA's slice)
+        uint32_t w[kC / 2];
+        pp_words<kC>(reinterpret_cast<const unsigned char*>(x + (pick * n_prob + p) * kC), w);
+        publish(pick, k, w, plain);
     };
     // no running sum decides: the first centre, or every vector already is a centre
     auto plain_pick = [&](double u) {
@@ -269,19 +334,27 @@ pp_cluster_kernel(const __half* __restrict__ x, const float* __restrict__ weight
         return pick >= n_vec ? n_vec - 1 : pick;
     };
 
+    bool ok = true;                      // false: a wait gave up (never expected); the problem's centroids become NaN
     for (int k = 0; k < K; ++k) {
-        const double u = up[k];
+        if (k % kPpUniforms == 0) {      // (from memory, each would be a trip of a tenth of a draw)
+            __syncthreads();
+            if (threadIdx.x < kPpUniforms && k + (int)threadIdx.x < K) us[threadIdx.x] = up[k + threadIdx.x];
+            __syncthreads();
+        }
+        const double u = us[k % kPpUniforms];
         if (k == 0) {
-            if (rank == 0 && warp == 0) publish(plain_pick(u), 0);
-            pp_cluster_sync();
+            if (rank == 0 && warp == 0) publish_any(plain_pick(u), 0, false);
+            if (!(ok = pp_wait(&ctl.pick_here[0], 0u))) break;
+            if (threadIdx.x == 0) pp_arm(&ctl.pick_here[0], kPickBytes);
             continue;
         }
+        const int b = k & 1;
         // ---- distances to the centre drawn last; sum of the contributions of this warp's vectors
         uint32_t cw[kC / 2];
         float cf[kC];
 #pragma unroll
         for (int q = 0; q < kC / 2; ++q) {
-            cw[q] = ctl.centre[q];
+            cw[q] = ctl.centre[b ^ 1][q];
             const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&cw[q]));
             cf[2 * q] = f.x;
             cf[2 * q + 1] = f.y;
@@ -301,8 +374,10 @@ pp_cluster_kernel(const __half* __restrict__ x, const float* __restrict__ weight
                     d32 = fmaf(dx, dx, d32);
                     d32 = fmaf(dy, dy, d32);
                 }
-                // d32 is within 2e-6 of the distance (differences of fp16 values rounded once, sums of squares)
-                if (d32 * 0.999996f <= __double2float_ru(dist[j])) {
+                // d32 is within 2e-6 of the distance (differences of fp16 values rounded once, sums of squares).  The comparison
+                // is one of the upper words of doubles, which a float's bits give without a conversion (d32 is zero, normal
+                // or not finite: squares of fp16 differences are 2^-48 at least): never false for a smaller distance.
+                if ((int)((__float_as_uint(d32 * 0.999996f) >> 3) + (896u << 20)) <= __double2hiint(dist[j])) {
                     const double d = pp_exact<kC>(xw, cw);
                     if (d < dist[j]) {
                         dist[j] = d;
@@ -315,15 +390,17 @@ pp_cluster_kernel(const __half* __restrict__ x, const float* __restrict__ weight
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         if (lane < cluster)
-            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(pp_map_shared(&ctl.sums[rank * kPpWarps + warp], lane)), "d"(sum) : "memory");
-        pp_cluster_sync();
+            pp_send64(pp_map_shared(&ctl.sums[b][rank * kPpWarps + warp], lane), (unsigned long long)__double_as_longlong(sum),
+                      pp_map_shared(&ctl.sums_here[b], lane));
+        if (!(ok = pp_wait(&ctl.sums_here[b], (uint32_t)((k - 1) >> 1) & 1u))) break;
+        if (threadIdx.x == 0) pp_arm(&ctl.sums_here[b], sums_bytes);         // for draw k + 2
 
         // ---- which warp's range holds the target (the same answer in every warp of the cluster)
         constexpr int kPerLane = kPpMaxCluster * kPpWarps / 32;
         double s[kPerLane], run = 0.0;
 #pragma unroll
         for (int e = 0; e < kPerLane; ++e) {
-            s[e] = ctl.sums[lane * kPerLane + e];
+            s[e] = ctl.sums[b][lane * kPerLane + e];
             run += s[e];
         }
         double upto = run;                                          // inclusive over the lanes
@@ -334,7 +411,7 @@ pp_cluster_kernel(const __half* __restrict__ x, const float* __restrict__ weight
         }
         const double total = __shfl_sync(0xffffffffu, upto, 31);
         if (!(total > 0.0)) {
-            if (rank == 0 && warp == 0) publish(plain_pick(u), k);
+            if (rank == 0 && warp == 0) publish_any(plain_pick(u), k, false);
         } else {
             const double target = __dmul_rn(u, total);
             const double slack = total * ((double)n_vec + 64.0) * 4.5e-16;
@@ -397,13 +474,16 @@ pp_cluster_kernel(const __half* __restrict__ x, const float* __restrict__ weight
                     const bool clear = target - (before + (inc - v)) > slack && (before + inc) - target > slack;
                     if (__shfl_sync(0xffffffffu, clear ? 1 : 0, l) && hit_in) pick = base + warp * (32 * per) + 32 * j + l;
                 }
-                if (pick >= 0 && pick < n_vec) publish(pick, k);
-                else undecided();
+                if (pick < 0 || pick >= n_vec) pick = -1;
+                uint32_t w[kC / 2];                                  // (this CTA's slice holds it)
+                pp_words<kC>(xs + (size_t)(pick < 0 ? 0 : pick - base) * kC * 2, w);
+                publish(pick, k, w, false);
             }
         }
-        pp_cluster_sync();
+        if (!(ok = pp_wait(&ctl.pick_here[b], (uint32_t)(k >> 1) & 1u))) break;
+        if (threadIdx.x == 0) pp_arm(&ctl.pick_here[b], kPickBytes);
 
-        if (ctl.pick < 0) {                                         // the same value in every CTA of the cluster
+        if (*reinterpret_cast<volatile long long*>(&ctl.pick[b]) < 0) {         // the same value in every CTA of the cluster
             double* cp = contrib + (int64_t)p * n_vec;
 #pragma unroll
             for (int j = 0; j < kPpPer; ++j)
@@ -414,11 +494,14 @@ pp_cluster_kernel(const __half* __restrict__ x, const float* __restrict__ weight
                 long long pick = 0;
                 if (lane == 0) pick = pp_serial_pick(cp, n_vec, u);
                 pick = __shfl_sync(0xffffffffu, pick, 0);
-                publish(pick, k);
+                publish_any(pick, k, true);
             }
             pp_cluster_sync();
         }
     }
+    pp_cluster_sync();                                              // no CTA leaves while another may write to its memory
+    if (!ok && lane == 0)
+        for (int i = 0; i < K * kC; ++i) codebooks[(int64_t)p * K * kC + i] = __int_as_float(0x7fc00000);
 }
 
 // Distances to the nearest chosen centre and the contributions w * D, for tiles of 32 vectors x 32 problems.
