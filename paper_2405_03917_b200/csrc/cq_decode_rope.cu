@@ -25,8 +25,9 @@
 //     adds the weights in that unit, and bins x value centroids closes the partial.  Adds to shared
 //     memory run at 32 lanes per clock for whole numbers and at 4 to 8 for fp32.  Partials and their merge are those of the other
 //     decode kernels.
-// What bounds it: instruction issue (28 a token and head for gather, rotation, dot and exchange, 4
-// for the bins; 54 of 75 thousand cycles of a CTA at 4096 tokens).  16 sequences of 4096 tokens, 32
+// What bounds it: scores (42 of a CTA's 75 thousand cycles at 4096 tokens, one head) and values (16); neither the issue slots nor
+// a pipe is full.  Rotation, dot and address in packed and permuting instructions (28 -> 21 a token and head) took 153.4 to
+// 151.7 us only; four blocks of value codes in flight instead of one, or their prefetch to L2, nothing or less (spills).  16 sequences of 4096 tokens, 32
 // heads, c = 4: 273 us with fp32 bins, 206 with whole numbers, 188 with 32 warps for one head, 164 with
 // set-up and end that read the codebooks in whole lines; 32 sequences, 32 heads on 8, c = 8: 308 -> 176.
 #include "cq_common.cuh"
@@ -73,6 +74,33 @@ __device__ __forceinline__ uint32_t rt_code(const uint32_t (&w)[kWords], int j)
     return (w[j >> 2] >> (8 * (j & 3))) & 0xffu;
 }
 
+// Two fp32 values in a register pair: one instruction multiplies and adds both.
+typedef unsigned long long rt_pair;
+__device__ __forceinline__ rt_pair rt_pack(float x, float y)
+{
+    rt_pair d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+    return d;
+}
+__device__ __forceinline__ float2 rt_unpack(rt_pair a)
+{
+    float2 d;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(a));
+    return d;
+}
+__device__ __forceinline__ rt_pair rt_mul(rt_pair a, rt_pair b)
+{
+    rt_pair d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ rt_pair rt_fma(rt_pair a, rt_pair b, rt_pair c)
+{
+    rt_pair d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
 template <int kC, int kHeads>
 __global__ void __launch_bounds__(RtCfg<kC, kHeads>::kThreads, 1)
 decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, const uint8_t* __restrict__ vc,
@@ -85,7 +113,6 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
     using C = RtCfg<kC, kHeads>;
     constexpr int G = C::G, kT = C::kT, kWords = kT / 4, kRtThreads = C::kThreads, kRtWarps = kRtThreads / 32;
     extern __shared__ __align__(16) unsigned char rt_smem[];
-    const uint32_t* book = reinterpret_cast<const uint32_t*>(rt_smem + C::kBookOff);
     uint32_t* bins = reinterpret_cast<uint32_t*>(rt_smem + C::kBinsOff);
     float* scores = reinterpret_cast<float*>(rt_smem + C::kScoreOff);
     RtCtl* ctl = reinterpret_cast<RtCtl*>(rt_smem + C::kCtlOff);
@@ -172,8 +199,10 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
     // words of the lane's two channels inside a centroid, and its two groups
     const int gA = (2 * lane) / kC, gB = gA + G / 2;
     // word of the lane's channels a in the centroid row of a code: code * (64 words) + colA; channels b: + 32 words
-    const uint32_t colA = (uint32_t)(gA * kC + (2 * lane) % kC) / 2u, colB = colA + 32u;
-    static_assert(128 / 2 == 64, "64 words of fp16 pairs per code");
+    // (in bytes: a row is 256 of them, so that one byte permutation puts a code byte and a column together)
+    const uint32_t colA = (uint32_t)(gA * kC + (2 * lane) % kC) * 2u, colB = colA + 128u;
+    static_assert(128 * 2 == 256, "bytes of a code's row");
+    const rt_pair re2 = rt_pack(st_re.x, st_re.y), im2 = rt_pack(st_im.x, st_im.y), nim2 = rt_pack(-st_im.x, -st_im.y);
     const uint8_t* kseq = kc + code_word_offset(sh, sh.n_kv_heads, s, hkv, 0, 0);
     const uint8_t* vseq = vc + code_word_offset(sh, sh.n_kv_heads, s, hkv, 0, 0);
     float l_thr[kHeads];
@@ -239,27 +268,32 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
                     return (up ? upper : lower) + __shfl_xor_sync(0xffffffffu, up ? lower : upper, o);
                 };
                 float waiting[5];
-                float2 u = make_float2(0.f, 0.f), v = make_float2(0.f, 0.f);
-                if (kHeads == 1) {
-                    u = make_float2(fmaf(qa[0][0], cs.x, qb[0][0] * sn.x), fmaf(qa[0][1], cs.y, qb[0][1] * sn.y));
-                    v = make_float2(fmaf(qb[0][0], cs.x, -qa[0][0] * sn.x), fmaf(qb[0][1], cs.y, -qa[0][1] * sn.y));
-                }
+                // (one head: the rotated query; several: cosines and sines)
+                rt_pair u2 = rt_pack(cs.x, cs.y), v2 = rt_pack(sn.x, sn.y);
+                auto rotated_query = [&]() {
+                    u2 = rt_pack(fmaf(qa[0][0], cs.x, qb[0][0] * sn.x), fmaf(qa[0][1], cs.y, qb[0][1] * sn.y));
+                    v2 = rt_pack(fmaf(qb[0][0], cs.x, -qa[0][0] * sn.x), fmaf(qb[0][1], cs.y, -qa[0][1] * sn.y));
+                };
+                if (kHeads == 1) rotated_query();
 #pragma unroll
                 for (int j = 0; j < kT; ++j) {
-                    const uint32_t wa = book[rt_code<kWords>(ca, j) * 64u + colA];
-                    const uint32_t wb = book[rt_code<kWords>(cbw, j) * 64u + colB];
-                    const float2 ka = __half22float2(*reinterpret_cast<const __half2*>(&wa));
-                    const float2 kb = __half22float2(*reinterpret_cast<const __half2*>(&wb));
+                    const uint32_t wa = *reinterpret_cast<const uint32_t*>(rt_smem + C::kBookOff + __byte_perm(ca[j >> 2], colA, 0x5504u | (j & 3) << 4));
+                    const uint32_t wb = *reinterpret_cast<const uint32_t*>(rt_smem + C::kBookOff + __byte_perm(cbw[j >> 2], colB, 0x5504u | (j & 3) << 4));
+                    const float2 fa = __half22float2(*reinterpret_cast<const __half2*>(&wa));
+                    const float2 fb = __half22float2(*reinterpret_cast<const __half2*>(&wb));
+                    const rt_pair ka = rt_pack(fa.x, fa.y), kb = rt_pack(fb.x, fb.y);
                     float x[kHeads];
                     if (kHeads == 1) {
-                        x[0] = fmaf(ka.x, u.x, fmaf(kb.x, v.x, fmaf(ka.y, u.y, kb.y * v.y)));
+                        const float2 t = rt_unpack(rt_fma(ka, u2, rt_mul(kb, v2)));
+                        x[0] = t.x + t.y;
                     } else {
                         // the rotated key of the lane's four channels
-                        const float ra0 = ka.x * cs.x - kb.x * sn.x, rb0 = kb.x * cs.x + ka.x * sn.x;
-                        const float ra1 = ka.y * cs.y - kb.y * sn.y, rb1 = kb.y * cs.y + ka.y * sn.y;
+                        const rt_pair ra = rt_fma(ka, u2, rt_mul(kb, v2 ^ 0x8000000080000000ull)), rb = rt_fma(kb, u2, rt_mul(ka, v2));
 #pragma unroll
-                        for (int h = 0; h < kHeads; ++h)
-                            x[h] = fmaf(qa[h][0], ra0, fmaf(qb[h][0], rb0, fmaf(qa[h][1], ra1, qb[h][1] * rb1)));
+                        for (int h = 0; h < kHeads; ++h) {
+                            const float2 t = rt_unpack(rt_fma(rt_pack(qa[h][0], qa[h][1]), ra, rt_mul(rt_pack(qb[h][0], qb[h][1]), rb)));
+                            x[h] = t.x + t.y;
+                        }
                     }
                     if (kHeads == 1) {
 #pragma unroll
@@ -279,24 +313,21 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
                             const int64_t tn = t0 + j + 1 < sh.max_tokens ? t0 + j + 1 : t0 + j;
                             cs = *reinterpret_cast<const float2*>(rope_cos + tn * 64 + 2 * lane);
                             sn = *reinterpret_cast<const float2*>(rope_sin + tn * 64 + 2 * lane);
-                            if (kHeads == 1) {
-                                u = make_float2(fmaf(qa[0][0], cs.x, qb[0][0] * sn.x), fmaf(qa[0][1], cs.y, qb[0][1] * sn.y));
-                                v = make_float2(fmaf(qb[0][0], cs.x, -qa[0][0] * sn.x), fmaf(qb[0][1], cs.y, -qa[0][1] * sn.y));
-                            }
+                            if (kHeads == 1) rotated_query();
+                            else { u2 = rt_pack(cs.x, cs.y); v2 = rt_pack(sn.x, sn.y); }
                         }
                     } else if (kHeads == 1) {
-                        const float ux = fmaf(u.x, st_re.x, v.x * st_im.x), vx = fmaf(v.x, st_re.x, -u.x * st_im.x);
-                        const float uy = fmaf(u.y, st_re.y, v.y * st_im.y), vy = fmaf(v.y, st_re.y, -u.y * st_im.y);
-                        u = make_float2(ux, uy);
-                        v = make_float2(vx, vy);
+                        const rt_pair un = rt_fma(u2, re2, rt_mul(v2, im2)), vn = rt_fma(v2, re2, rt_mul(u2, nim2));
+                        u2 = un;
+                        v2 = vn;
                     } else {
-                        const float cx = cs.x * st_re.x - sn.x * st_im.x, sx = sn.x * st_re.x + cs.x * st_im.x;
-                        const float cy = cs.y * st_re.y - sn.y * st_im.y, sy = sn.y * st_re.y + cs.y * st_im.y;
-                        cs = make_float2(cx, cy);
-                        sn = make_float2(sx, sy);
+                        const rt_pair cn = rt_fma(u2, re2, rt_mul(v2, nim2)), sn2 = rt_fma(v2, re2, rt_mul(u2, im2));
+                        u2 = cn;
+                        v2 = sn2;
                     }
                 }
                 if (kFromTables) return true;
+                const float2 u = rt_unpack(u2), v = rt_unpack(v2);
                 // what was stepped to is the prediction for position t0 + kT: it must be what the tables hold there
                 bool off = false;
                 if (t0 + kT < sh.max_tokens) {
@@ -310,8 +341,8 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
                         const float by = tol * (fabsf(qa[0][1]) + fabsf(qb[0][1])) * (1.f + fabsf(ct.y) + fabsf(stt.y));
                         off = !(fabsf(ux - u.x) <= bx) || !(fabsf(vx - v.x) <= bx) || !(fabsf(uy - u.y) <= by) || !(fabsf(vy - v.y) <= by);
                     } else {
-                        off = !(fabsf(ct.x - cs.x) <= tol * (1.f + fabsf(ct.x))) || !(fabsf(ct.y - cs.y) <= tol * (1.f + fabsf(ct.y))) ||
-                              !(fabsf(stt.x - sn.x) <= tol * (1.f + fabsf(stt.x))) || !(fabsf(stt.y - sn.y) <= tol * (1.f + fabsf(stt.y)));
+                        off = !(fabsf(ct.x - u.x) <= tol * (1.f + fabsf(ct.x))) || !(fabsf(ct.y - u.y) <= tol * (1.f + fabsf(ct.y))) ||
+                              !(fabsf(stt.x - v.x) <= tol * (1.f + fabsf(stt.x))) || !(fabsf(stt.y - v.y) <= tol * (1.f + fabsf(stt.y)));
                     }
                 }
                 return !__any_sync(0xffffffffu, off);
@@ -348,12 +379,17 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
         for (int o = 1; o < kT; o <<= 1) lane_max = fmaxf(lane_max, __shfl_xor_sync(0xffffffffu, lane_max, o));
         if (lane % kT == 0) ctl->warp_max[warp][lane / kT] = lane_max;
         __syncthreads();
-        if (threadIdx.x < kHeads) {
-            float m = ctl->m_run[threadIdx.x];
-            const float old = m;
-            for (int w = 0; w < kRtWarps; ++w) m = fmaxf(m, ceilf(ctl->warp_max[w][threadIdx.x]));
-            ctl->factor[threadIdx.x] = old == m ? 1.f : exp2f(old - m);      // 0 when there was no reference yet
-            ctl->m_run[threadIdx.x] = m;
+        // (warp h takes head h, a lane per warp: one thread that walked the warps' values cost a thousand cycles each time)
+        if (warp < kHeads) {
+            float m = lane < kRtWarps ? ceilf(ctl->warp_max[lane][warp]) : -INFINITY;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if (lane == 0) {
+                const float old = ctl->m_run[warp];
+                m = fmaxf(m, old);
+                ctl->factor[warp] = old == m ? 1.f : exp2f(old - m);      // 0 when there was no reference yet
+                ctl->m_run[warp] = m;
+            }
         }
         __syncthreads();
         // weights of the chunk, relative to m_run, and the total so far
@@ -374,15 +410,18 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
         __syncthreads();
         // The unit that lets the total fill 31 bits: no bin can run over, and a weight keeps as many bits as fp32 gives it
         // down to 2^-8 of the total.
-        if (threadIdx.x < kHeads) {
-            float total = 0.f;
-            for (int w = 0; w < kRtWarps; ++w) total += ctl->l_part[w][threadIdx.x];
-            const float m = ctl->m_run[threadIdx.x], old = ctl->e_run[threadIdx.x];
-            const float wanted = m + (ceilf(log2f(total)) - 31.f), e = wanted < old ? old : wanted;
-            const float rise = e - old;                                       // (infinite when there was no unit yet: bins are zero)
-            ctl->shift[threadIdx.x] = rise < 32.f ? (int)rise : 32;
-            ctl->e_run[threadIdx.x] = e;
-            ctl->unit[threadIdx.x] = exp2f(m - e);
+        if (warp < kHeads) {
+            float total = lane < kRtWarps ? ctl->l_part[lane][warp] : 0.f;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+            if (lane == 0) {
+                const float m = ctl->m_run[warp], old = ctl->e_run[warp];
+                const float wanted = m + (ceilf(log2f(total)) - 31.f), e = wanted < old ? old : wanted;
+                const float rise = e - old;                                   // (infinite when there was no unit yet: bins are zero)
+                ctl->shift[warp] = rise < 32.f ? (int)rise : 32;
+                ctl->e_run[warp] = e;
+                ctl->unit[warp] = exp2f(m - e);
+            }
         }
         __syncthreads();
 #pragma unroll
@@ -453,14 +492,17 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
         if (lane == 0) ctl->l_part[warp][h] = l;
     }
     __syncthreads();
-    if (threadIdx.x < kHeads) {
-        float l = 0.f;
-        for (int w = 0; w < kRtWarps; ++w) l += ctl->l_part[w][threadIdx.x];
-        l *= ctl->unit[threadIdx.x];
-        ctl->factor[threadIdx.x] = l;
-        if (n_splits > 1) {
-            part0[(int64_t)threadIdx.x * n_splits * stride + 0] = ctl->e_run[threadIdx.x];
-            part0[(int64_t)threadIdx.x * n_splits * stride + 1] = l;
+    if (warp < kHeads) {
+        float l = lane < kRtWarps ? ctl->l_part[lane][warp] : 0.f;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (lane == 0) {
+            l *= ctl->unit[warp];
+            ctl->factor[warp] = l;
+            if (n_splits > 1) {
+                part0[(int64_t)warp * n_splits * stride + 0] = ctl->e_run[warp];
+                part0[(int64_t)warp * n_splits * stride + 1] = l;
+            }
         }
     }
     // Bins x value centroids: a warp takes 64 bytes of eight groups at a time, as in the set-up, for all heads together

@@ -371,7 +371,9 @@ learn_move_kernel(const __half* __restrict__ x, const float* __restrict__ weight
                   const int* __restrict__ last_moved, const uint32_t* __restrict__ top, float* __restrict__ cb)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");      // launched ahead of the end of the assignment
-    __shared__ float acc[kAsK * (kC + 1)];
+    // the problem's sums, read in whole lines (a row of 8 (c + 1) 2 bytes per thread touched 32 lines a load); or fp32 sums
+    __shared__ __align__(16) unsigned long long rows[kAsK * 2 * (kC + 1)];
+    float* acc = reinterpret_cast<float*>(rows);
     __shared__ float best[2][kAsK / 32];
     __shared__ int arg[kAsK / 32];
     const int p = blockIdx.x, j = threadIdx.x, lane = j & 31, warp = j >> 5;
@@ -394,20 +396,28 @@ learn_move_kernel(const __half* __restrict__ x, const float* __restrict__ weight
             for (int q = 0; q < kC; ++q) cj[q] = acc[j * (kC + 1) + q] / ws;
         return;
     }
+    {
+        const ulonglong2* src = reinterpret_cast<const ulonglong2*>(sums + (int64_t)p * kAsK * 2 * (kC + 1));
+#pragma unroll
+        for (int i = 0; i <= kC; ++i) reinterpret_cast<ulonglong2*>(rows)[i * kAsK + j] = __ldcg(src + i * kAsK + j);
+    }
+    __syncthreads();
     int ex, ew;
     as_scales(top, p, weights != nullptr, ex, ew);
     const double limb = ldexp(1.0, -limb_bits), back = ldexp(1.0, ex);
-    const unsigned long long* row = sums + ((int64_t)p * kAsK + j) * 2 * (kC + 1);
+    const unsigned long long* row = rows + j * 2 * (kC + 1);
     auto value = [&](int ch) { return (double)(long long)row[ch] + (double)(long long)row[kC + 1 + ch] * limb; };
     const double ws = value(kC);
     float d2 = 0.f;
-    if (ws > 0.0)                                            // (a centroid without members stays)
+    if (ws > 0.0) {                                          // (a centroid without members stays)
+        const double share = back / ws;
 #pragma unroll
         for (int q = 0; q < kC; ++q) {
-            const float was = cj[q], now = (float)(value(q) / ws * back), d = now - was;
+            const float was = cj[q], now = (float)(value(q) * share), d = now - was;
             cj[q] = now;
             d2 = fmaf(d, d, d2);
         }
+    }
     // the largest move of any other centroid: the two largest of the problem
     const float move = __fsqrt_ru(d2) * 1.000002f;
     float m1 = move, m2 = -1.f;
