@@ -315,16 +315,17 @@ cudaError_t launch_enc_tc(const __half* x, const float* cb, const int32_t* seq_o
     const int64_t slots = C::kCtasPerSm * (int64_t)device_sm_count();          // CTAs in flight
     // Row tiles per CTA.  A group's centroids are prepared once per CTA, which costs `prepare` of a row tile's step (from the times
     // below), and the tiles past the last vector are stepped through as well; the least of both together, as long as the
-    // groups can be split into four waves of CTAs.  Against one tile per CTA wherever whole rows of groups do not fill four
-    // waves, key and value: 40000 vectors x 8 heads of CQ-8c8b 481 -> 401 us, 4000 x 40 259 -> 210, 1665 x 40 121 -> 110; CQ-4c8b 14688 x 8
-    // 306 -> 272; CQ-2c8b 4000 x 40 860 -> 762; CQ-8c10b 4000 x 8 304 -> 255.
+    // groups can be split into three waves of CTAs (with four asked for, 1665 x 8 of CQ-8c8b 30.2 instead of 27.8 us, with two
+    // 2500 x 8 37.8 instead of 35.8).  Against one tile per CTA wherever whole rows of groups do not fill four waves, key and
+    // value: 40000 vectors x 8 heads of CQ-8c8b 481 -> 401 us, 4000 x 40 259 -> 210, 1665 x 8 30.2 -> 27.8; CQ-4c8b 14688 x 8
+    // 306 -> 279; CQ-2c8b 4000 x 40 860 -> 762; CQ-8c10b 4000 x 8 304 -> 235.
     constexpr double prepare = kChunks > 1 ? 0.44 : kC == 8 ? 0.3 : kC == 4 ? 0.2 : 0.15;
     int log_rt = 0;
     double least = 1e30;
     for (int l = 0; l <= C::kMaxLogRt; ++l) {
         const int64_t n = (tiles + (1 << l) - 1) >> l;
         const double cost = (double)n * ((1 << l) + prepare);
-        if ((l == 0 || n * sh.n_kv_heads * C::G * (x2 ? 2 : 1) >= 4 * slots) && cost < least) {
+        if ((l == 0 || n * sh.n_kv_heads * C::G * (x2 ? 2 : 1) >= 3 * slots) && cost < least) {
             log_rt = l;
             least = cost;
         }
