@@ -482,9 +482,13 @@ namespace {
 size_t step_least_bytes(const Shape& sh) { return round_up(partial_bytes(sh), 256) + round_up((size_t)sh.n_seq * 4, 256); }
 // Bytes of inputs and output of a cq_decode_step_host call up to which its pinned buffers are read and written by kernels: no
 // hand-over between copy engine and kernels, and the result leaves as the CTAs end.  Over what was measured (1 KB to 3.3 MB)
-// it is the faster way or level: 64 sequences of 500 tokens, 32 heads on 8, CQ-8c8b (1.8 MB) 109 -> 84 us, 16 sequences 60 -> 46, one
-// of 128 tokens 52 -> 38, one of 20000 50.0 -> 50.8; 64 sequences, 32 heads of CQ-4c8b (2.6 MB) 191 -> 146.
+// it is the faster way: 64 sequences of 500 tokens, 32 heads on 8, CQ-8c8b (1.8 MB) 109 -> 82 us, 16 sequences 57 -> 44, one of 128
+// tokens 46 -> 36; 64 sequences, 32 heads of CQ-4c8b (2.6 MB) 191 -> 146.
 constexpr size_t kDirectHostBytes = (size_t)4 << 20;
+// Inputs from which the fetching kernel is faster than two copies (back to back in host memory) under a result written in
+// place: one sequence of 20000 tokens, 32 heads on 8 (12 KB) 51.5 against 48.2 us, 32 heads of CQ-4c8b, 2000 tokens (25 KB) 38.9 against
+// 34.5; four sequences of 500 (49 KB) 37.6 against 39.8, 16 of 500 (197 KB) 44 against 52.
+constexpr size_t kFetchHostBytes = (size_t)40 << 10;
 // The address under which kernels of the current device reach pinned host memory; false for any other memory.
 bool pinned_on_device(const void* host, const void** dev)
 {
@@ -622,38 +626,37 @@ int cq_decode_step_host(const void* q_host, const void* k_new_host, const void* 
     const size_t step_bytes = workspace_bytes - (size_t)(w - static_cast<char*>(workspace));
 
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
-    // Pinned buffers of a small step: a kernel fetches the inputs and the attention writes the result to host memory.
-    const void *q_dev = nullptr, *k_dev = nullptr, *v_dev = nullptr, *sl_dev = nullptr, *out_dev = nullptr;
-    if (qb + 2 * kvb + slb + ob <= kDirectHostBytes && pinned_on_device(q_host, &q_dev) && pinned_on_device(k_new_host, &k_dev) &&
-        pinned_on_device(v_new_host, &v_dev) && pinned_on_device(seq_lens_host, &sl_dev) && pinned_on_device(out_host, &out_dev) &&
-        (reinterpret_cast<uintptr_t>(out_dev) & 3u) == 0) {
-        const HostPieces pieces = {{q_dev, k_dev, v_dev, sl_dev}, {d_q, d_k, d_v, d_sl}, {qb, kvb, kvb, slb}};
-        if (launch_fetch_host(pieces, cs) != cudaSuccess) return CQ_ERR_CUDA;
-        const int st = cq_decode_step(d_q, d_k, d_v, d_sl, k_codes, v_codes, k_cb, v_cb, scale, n_seq, n_q_heads, n_kv_heads, head_dim, c, b,
-                                      max_tokens, static_cast<float*>(const_cast<void*>(out_dev)), step_ws, step_bytes, stream);
-        if (st != CQ_OK) return st;
-        return cudaStreamSynchronize(cs) == cudaSuccess ? CQ_OK : CQ_ERR_CUDA;
-    }
     // Few, large copies: query, key and value travel in one copy when the caller keeps them back to back
     // in host memory (the staging areas are then packed the same way).
     const bool packed = static_cast<const char*>(k_new_host) == static_cast<const char*>(q_host) + qb &&
                         static_cast<const char*>(v_new_host) == static_cast<const char*>(k_new_host) + kvb &&
                         qb % 16 == 0 && kvb % 16 == 0;
-    if (packed) {
+    // Pinned buffers of a small step: a kernel fetches the inputs (where they are more than a copy has done at once), and
+    // the attention writes the result to host memory.
+    const void *q_dev = nullptr, *k_dev = nullptr, *v_dev = nullptr, *sl_dev = nullptr, *out_dev = nullptr;
+    const bool direct = qb + 2 * kvb + slb + ob <= kDirectHostBytes && pinned_on_device(q_host, &q_dev) && pinned_on_device(k_new_host, &k_dev) &&
+                        pinned_on_device(v_new_host, &v_dev) && pinned_on_device(seq_lens_host, &sl_dev) &&
+                        pinned_on_device(out_host, &out_dev) && (reinterpret_cast<uintptr_t>(out_dev) & 3u) == 0;
+    const bool fetch = direct && (!packed || qb + 2 * kvb + slb >= kFetchHostBytes);
+    if (fetch) {
+        const HostPieces pieces = {{q_dev, k_dev, v_dev, sl_dev}, {d_q, d_k, d_v, d_sl}, {qb, kvb, kvb, slb}};
+        if (launch_fetch_host(pieces, cs) != cudaSuccess) return CQ_ERR_CUDA;
+    } else if (packed && cudaMemcpyAsync(d_q, q_host, qb + 2 * kvb, cudaMemcpyHostToDevice, cs) == cudaSuccess) {
         d_k = d_q + qb;
         d_v = d_k + kvb;            // (fits: the three areas were sized with their paddings)
-        if (cudaMemcpyAsync(d_q, q_host, qb + 2 * kvb, cudaMemcpyHostToDevice, cs) != cudaSuccess) return CQ_ERR_CUDA;
     } else {
+        cudaGetLastError();         // (pinned allocations that lie side by side by chance are refused as one copy)
         if (cudaMemcpyAsync(d_q, q_host, qb, cudaMemcpyHostToDevice, cs) != cudaSuccess) return CQ_ERR_CUDA;
         if (cudaMemcpyAsync(d_k, k_new_host, kvb, cudaMemcpyHostToDevice, cs) != cudaSuccess) return CQ_ERR_CUDA;
         if (cudaMemcpyAsync(d_v, v_new_host, kvb, cudaMemcpyHostToDevice, cs) != cudaSuccess) return CQ_ERR_CUDA;
     }
-    if (cudaMemcpyAsync(d_sl, seq_lens_host, slb, cudaMemcpyHostToDevice, cs) != cudaSuccess) return CQ_ERR_CUDA;
+    if (!fetch && cudaMemcpyAsync(d_sl, seq_lens_host, slb, cudaMemcpyHostToDevice, cs) != cudaSuccess) return CQ_ERR_CUDA;
+    if (direct) d_out = static_cast<float*>(const_cast<void*>(out_dev));
     // The new token is appended at position seq_lens[s]; the attention then reads seq_lens[s] + 1 tokens.
     const int st = cq_decode_step(d_q, d_k, d_v, d_sl, k_codes, v_codes, k_cb, v_cb, scale, n_seq, n_q_heads, n_kv_heads,
                                   head_dim, c, b, max_tokens, d_out, step_ws, step_bytes, stream);
     if (st != CQ_OK) return st;
-    if (cudaMemcpyAsync(out_host, d_out, ob, cudaMemcpyDeviceToHost, cs) != cudaSuccess) return CQ_ERR_CUDA;
+    if (!direct && cudaMemcpyAsync(out_host, d_out, ob, cudaMemcpyDeviceToHost, cs) != cudaSuccess) return CQ_ERR_CUDA;
     if (cudaStreamSynchronize(cs) != cudaSuccess) return CQ_ERR_CUDA;
     return CQ_OK;
 }

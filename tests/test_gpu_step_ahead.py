@@ -109,8 +109,8 @@ def test_steps_right_behind_one_another():
         close(x, y)
 
 
-@pytest.mark.parametrize("c,b,n_seq,n_q,n_kv", [(8, 8, 3, 8, 2), (4, 8, 2, 3, 3), (8, 10, 2, 2, 1), (4, 4, 2, 2, 2)])
-@pytest.mark.parametrize("how", ["pinned", "one block", "off by two bytes", "pageable", "pageable result"])
+@pytest.mark.parametrize("c,b,n_seq,n_q,n_kv", [(8, 8, 3, 8, 2), (4, 8, 2, 3, 3), (4, 8, 3, 24, 24), (8, 10, 2, 2, 1), (4, 4, 2, 2, 2)])
+@pytest.mark.parametrize("how", ["pinned", "side by side", "one block", "off by two bytes", "pageable", "pageable result"])
 def test_host_buffers(c, b, n_seq, n_q, n_kv, how):
     # pinned buffers are read and written by kernels (16 bytes at a time where they are aligned), others are copied
     D, cap = 128, 200
@@ -123,6 +123,12 @@ def test_host_buffers(c, b, n_seq, n_q, n_kv, how):
     pin = (lambda t: t) if how == "pageable" else (lambda t: t.pin_memory())
     if how == "pinned":
         host = [pin(p.cpu()) for p in parts]
+    elif how == "side by side":                        # allocations of their own that happen to lie back to back: not one copy
+        pool = sorted((torch.empty(parts[0].numel(), dtype=torch.float16).pin_memory() for _ in range(40)), key=lambda t: t.data_ptr())
+        run = [i for i in range(38) if pool[i + 1].data_ptr() - pool[i].data_ptr() == pool[i + 2].data_ptr() - pool[i + 1].data_ptr() == 2 * parts[0].numel()]
+        if n_q != n_kv or not run:
+            pytest.skip("no such allocations here")
+        host = [pool[run[0] + i].view(p.shape).copy_(p.cpu()) for i, p in enumerate(parts)]
     else:
         block = pin(torch.empty(sum(p.numel() for p in parts) + skip, dtype=torch.float16))
         host, at = [], skip
