@@ -510,10 +510,19 @@ encode_few_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, 
 // 512 and 1024 centroids: one CTA per (head, group) reads the group's codebook once, a thread holding kPer of its 256 * kPer
 // centroids in registers, and takes the vectors past them sixteen at a time.  Distances and ties as in encode_few.  What it
 // takes is one pass over the codebooks (16 vectors x 32 heads of CQ-8c10b, key and value: 33 MB; 52 us on the tensor-memory
-// kernel, which walks its steps one after the other with 16 of 128 rows in use, 17 us here).  A warp per 256 centroids
+// kernel, which walks its steps one after the other with 16 of 128 rows in use, 17 us here with single instructions).  A warp per 256 centroids
 // (encode_few) has too few warps for this many (27 us; two vectors, 40 heads 12.6 against 9.9 us).
+// Many vectors are bound by the issue of the subtractions and multiply-adds: kPacked takes two centroids per instruction
+// (packed fp32, each half rounded as the single ones are; (c - x)^2 for (x - c)^2).  For few vectors the packing costs as
+// much as it saves (wide_packed_pays).
 constexpr int kFewWideVecs = 16;
-template <int kC, int kPer>
+__device__ __forceinline__ unsigned long long few_pack(float x, float y)
+{
+    unsigned long long d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+    return d;
+}
+template <int kC, int kPer, bool kPacked>
 __global__ void __launch_bounds__(256)
 encode_few_wide_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, const int32_t* __restrict__ seq_offsets, Shape sh,
                   int n_vec, int n_tokens, int64_t token_offset, uint8_t* __restrict__ codes1, const __half* __restrict__ x2,
@@ -545,6 +554,11 @@ encode_few_wide_kernel(const __half* __restrict__ x1, const float* __restrict__ 
             }
         }
     }
+    unsigned long long c2[kPer / 2][kC];                          // (kPacked only)
+#pragma unroll
+    for (int u = 0; u < kPer / 2; ++u)
+#pragma unroll
+        for (int e = 0; e < kC; ++e) c2[u][e] = few_pack(cv[2 * u][e], cv[2 * u + 1][e]);
     for (int v0 = 0; v0 < n_vec; v0 += kFewWideVecs) {
         const int nv = n_vec - v0 < kFewWideVecs ? n_vec - v0 : kFewWideVecs;
         if (threadIdx.x < kFewWideVecs * kC) {
@@ -559,16 +573,33 @@ encode_few_wide_kernel(const __half* __restrict__ x1, const float* __restrict__ 
             for (int e = 0; e < kC; ++e) xv[e] = xs[v][e];
             float best = kInfBits;
             int arg = 0;
+            float dist[kPer];
+            if (kPacked) {
 #pragma unroll
-            for (int u = 0; u < kPer; ++u) {
-                float d = 0.f;
+                for (int u = 0; u < kPer / 2; ++u) {
+                    unsigned long long d2 = 0ull;
 #pragma unroll
-                for (int e = 0; e < kC; ++e) {
-                    const float diff = xv[e] - cv[u][e];
-                    d = fmaf(diff, diff, d);
+                    for (int e = 0; e < kC; ++e) {
+                        unsigned long long diff;
+                        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(diff) : "l"(c2[u][e]), "l"(few_pack(-xv[e], -xv[e])));
+                        asm("fma.rn.f32x2 %0, %1, %1, %2;" : "=l"(d2) : "l"(diff), "l"(d2));
+                    }
+                    asm("mov.b64 {%0, %1}, %2;" : "=f"(dist[2 * u]), "=f"(dist[2 * u + 1]) : "l"(d2));
                 }
-                if (d < best) { best = d; arg = u * 256 + (int)threadIdx.x; }      // ascending: strict < keeps the lowest index
+            } else {
+#pragma unroll
+                for (int u = 0; u < kPer; ++u) {
+                    dist[u] = 0.f;
+#pragma unroll
+                    for (int e = 0; e < kC; ++e) {
+                        const float diff = xv[e] - cv[u][e];
+                        dist[u] = fmaf(diff, diff, dist[u]);
+                    }
+                }
             }
+#pragma unroll
+            for (int u = 0; u < kPer; ++u)
+                if (dist[u] < best) { best = dist[u]; arg = u * 256 + (int)threadIdx.x; }      // ascending: strict < keeps the lowest index
             // (distances are not negative: their bits order as they do)
             const unsigned db = __float_as_uint(best), dm = __reduce_min_sync(0xffffffffu, db);
             const unsigned jm = __reduce_min_sync(0xffffffffu, db == dm ? (unsigned)arg : 0xffffffffu);
@@ -600,6 +631,11 @@ encode_few_wide_kernel(const __half* __restrict__ x1, const float* __restrict__ 
     }
 }
 
+// From four vectors, and only with more CTAs than SMs (a CTA alone on its SM waits for its reductions, not for issue slots).  Key and
+// value, single against packed: 40 heads of CQ-8c10b, 1 / 4 / 16 / 30 vectors 6.2 / 8.8 / 20.9 / 37.2 against 6.7 / 8.4 / 17.7 / 30.4 us, of
+// CQ-8c9b 4.6 / 5.9 / 12.6 / 21.5 against 4.8 / 5.9 / 11.5 / 19.0; one head of CQ-4c10b, 30 vectors 6.4 against 6.6.
+bool wide_packed_pays(int n_vec, int64_t ctas) { return n_vec >= 4 && ctas > device_sm_count(); }
+
 template <int kC>
 cudaError_t launch_few(const __half* x, const float* cb, const int32_t* seq_offsets, const Shape& sh, int64_t n_tokens, int64_t token_offset,
                        uint8_t* codes, cudaStream_t st, const __half* x2, const float* cb2, uint8_t* codes2)
@@ -612,8 +648,9 @@ cudaError_t launch_few(const __half* x, const float* cb, const int32_t* seq_offs
         return cudaLaunchKernelEx(&cfg, kernel, x, cb, seq_offsets, sh, n_vec, (int)n_tokens, token_offset, codes, x2, cb2, codes2, share...);
     };
     if (sh.b == 8) return go(encode_few_kernel<kC>, few_share(sh, n_vec));
-    if (sh.b == 9) return go(encode_few_wide_kernel<kC, 2>);
-    return go(encode_few_wide_kernel<kC, 4>);
+    const bool packed = wide_packed_pays(n_vec, (int64_t)cfg.gridDim.x * cfg.gridDim.y);
+    if (sh.b == 9) return packed ? go(encode_few_wide_kernel<kC, 2, true>) : go(encode_few_wide_kernel<kC, 2, false>);
+    return packed ? go(encode_few_wide_kernel<kC, 4, true>) : go(encode_few_wide_kernel<kC, 4, false>);
 }
 
 template <int kC, int kMT>

@@ -226,3 +226,26 @@ def test_few_vectors_equal_the_generic_kernel(c, b, n_seq):
     want = start.clone()
     cq.cq_encode(xv.to(DEV), vcb.to(DEV), c, b, want, cap, seq_offsets=offs, variant=1)
     assert torch.equal(got_v, want)
+
+
+@pytest.mark.parametrize("c,b", [(2, 9), (4, 9), (8, 9), (2, 10), (8, 10)])
+@pytest.mark.parametrize("n_vec,n_heads", [(3, 10), (4, 1), (4, 10), (5, 10), (17, 10)])
+def test_few_vectors_two_centroids_at_a_time(c, b, n_vec, n_heads):
+    # both sides of the rule (four vectors, more CTAs than SMs); centroids that occur twice (in one thread's pair, two pairs apart, in another
+    # thread) tie and the lowest index wins; a vector and a centroid with infinities
+    g = torch.Generator().manual_seed(c * b + n_vec)
+    cb = torch.randn(2, n_heads, 128 // c, 1 << b, c, generator=g)
+    cb[..., 256:300, :] = cb[..., :44, :]
+    cb[..., (1 << b) - 30:, :] = cb[..., 20:50, :]
+    cb[:, 0, 0, 7, 0] = float("inf")
+    x = torch.randn(2, n_vec, 1, n_heads, 128, generator=g).half()
+    x[:, :, :, :, :c] = cb[:, None, None, :, 0, 20:21].squeeze(4).half()
+    x[:, 0, 0, 0, c] = float("inf")
+    x, cb = x.to(DEV), cb.to(DEV)
+    start = torch.zeros(cq.cq_codes_bytes(n_vec, 16, n_heads, 128, c, b), dtype=torch.uint8, device=DEV)
+    got = [start.clone(), start.clone()]
+    cq.cq_encode_kv(x[0], x[1], cb[0], cb[1], c, b, *got, 16)
+    for i in range(2):
+        want = start.clone()
+        cq.cq_encode(x[i], cb[i], c, b, want, 16, variant=1)
+        assert torch.equal(got[i], want)
