@@ -218,9 +218,8 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
                 make_uint4(0u, 0u, 0u, 0u);
     };
     clear_bins();
-    // launched ahead of the end of the kernel before it (the append, for one); the merge, or the call behind, may be from here on
+    // launched ahead of the end of the kernel before it (the append, for one)
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     // Work item: (context part, sequence, KV head); parts are the slowest index so that the
     // always-populated first parts start first.  With a tail (tail_first >= 0) the items before
@@ -679,6 +678,12 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
         coarsen();
     }
     __syncthreads();
+
+    // The merge, or the call behind, may be launched from here on: its launch passes behind the epilogue, and its CTAs do not wait on the
+    // SMs beside the last wave's loops.  Step of 16 x 4096 tokens, 32 heads of CQ-4c8b, triggered behind the wait above / here: 68.2 / 66.2 us,
+    // 9 x 0.9-3 k, 40 heads 40.0 / 39.9, attention at head_dim 64 21.6 / 21.1.  (decode_pair_kernel and decode_wide_kernel lose by
+    // it: steps of one sequence of 20011 tokens 29.9 / 37.2, 16 x 8192 tokens of CQ-8c10b without any trigger 137.7 / 139.4.)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     // ---------------------------------------------------------------- epilogue: bins x V centroids
     // Same ownership as the table build: a warp owns whole groups, lanes walk the code values.
