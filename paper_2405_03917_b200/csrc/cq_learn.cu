@@ -410,10 +410,11 @@ pp_cluster_kernel(const __half* __restrict__ x, const float* __restrict__ weight
             if (lane >= o) upto += t;
         }
         const double total = __shfl_sync(0xffffffffu, upto, 31);
-        if (!(total > 0.0)) {
-            if (rank == 0 && warp == 0) publish_any(plain_pick(u), k, false);
+        const double target = __dmul_rn(u, total);
+        if (!(total > 0.0) || target != target) {
+            // (zero times an infinite total is not a number: no running sum reaches it, and as defined the last vector is drawn)
+            if (rank == 0 && warp == 0) publish_any(total > 0.0 ? n_vec - 1 : plain_pick(u), k, false);
         } else {
-            const double target = __dmul_rn(u, total);
             const double slack = total * ((double)n_vec + 64.0) * 4.5e-16;
             const unsigned hit = __ballot_sync(0xffffffffu, upto >= target);
             // (the lanes' order of the sums is the vectors' order; no hit: the target is within rounding of the total)

@@ -149,3 +149,20 @@ def test_kmeanspp_and_one_iteration_at_the_edges_of_the_split(c, n_vec, weighted
     got_new, got_obj = cq.cq_lloyd_step(x.to(DEV), wd, got, c, b)
     assert np.allclose(got_new.cpu().numpy(), new, rtol=0, atol=2e-5 * max(1.0, np.abs(new).max()))
     assert np.allclose(got_obj.cpu().numpy(), obj, rtol=1e-5, atol=1e-9)
+
+
+@pytest.mark.parametrize("c,n_vec", [(8, 300), (4, 1000), (2, 2000), (8, 3000), (8, 32769)])
+def test_a_draw_of_zero_times_an_infinite_total(c, n_vec):
+    # one infinite weight and a uniform of exactly 0: the target is not a number, no running sum reaches it and the last vector
+    # is drawn; the draws after it have an infinite target.  One, two, four and eight CTAs per problem, and the plain kernels
+    b, G = 3, 128 // c
+    x = calib(380 + c, n_vec, 1, False, c)
+    w = fisher_like_weights(c + b, n_vec, 1, G)
+    w[n_vec // 3] = float("inf")
+    u = torch.rand(1, G, 1 << b, dtype=torch.float64, generator=torch.Generator().manual_seed(n_vec))
+    u[0, :, 0] = 0.9                                                     # (not the vector with the infinite weight)
+    u[0, :, 1:3] = 0.0
+    want, chosen = oracle.kmeanspp_init(x.numpy(), w.numpy(), u.numpy(), c, b)
+    assert (chosen[0, :, 1:3] == n_vec - 1).all() and (chosen[0, :, 3] == n_vec // 3).all()
+    got = cq.cq_kmeanspp_init(x.to(DEV), w.to(DEV), u.to(DEV), c, b).cpu().numpy()
+    assert np.array_equal(got, want)
