@@ -108,8 +108,10 @@ decode_rope_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict
                          const float* __restrict__ rope_cos, const float* __restrict__ rope_sin, float scale_log2e, Shape sh,
                          int n_splits, int split_tokens, float* __restrict__ partials, float* __restrict__ out)
 {
-    asm volatile("griddepcontrol.wait;" ::: "memory");      // launched ahead of the end of the kernel before it, and
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");       // the kernel behind it ahead of its own
+    // Launched ahead of the end of the kernel before it.  It lets nothing go ahead itself: a CTA fills an SM, so that what follows finds
+    // room only where a CTA has ended, and its CTAs then share SMs while others idle.  Calls back to back, us, let ahead at the
+    // start / not: 2 x 10183 tokens, 32 heads on 8 of CQ-4c8b 39.5 / 37.6, 8 x 2480 of CQ-8c8b 47.1 / 46.0, 16 x 4096, 32 heads of CQ-4c8b 150.1 / 150.1.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     using C = RtCfg<kC, kHeads>;
     constexpr int G = C::G, kT = C::kT, kWords = kT / 4, kRtThreads = C::kThreads, kRtWarps = kRtThreads / 32;
     extern __shared__ __align__(16) unsigned char rt_smem[];
