@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(PairCfg::kThreads, 2)
 decode_pair_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc, const uint8_t* __restrict__ vc,
                    const float* __restrict__ kcb, const float* __restrict__ vcb,
                    const int32_t* __restrict__ seq_lens, float scale_log2e, Shape sh, int chunk_tokens, int n_parts,
-                   int tail_first, int cb_aligned32, float* __restrict__ partials, AppendArgs app, float* __restrict__ out)
+                   int tail_first, int cb_aligned32, int next_at_start, float* __restrict__ partials, AppendArgs app, float* __restrict__ out)
 {
     using C = PairCfg;
     constexpr int R = C::kHeads;
@@ -377,9 +377,9 @@ decode_pair_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc,
     const int hb = p & 1, pu = p >> 1;
 
     // launched ahead of the end of the kernel before it (which may write codes: they are read by bulk copies, hence the proxy
-    // fence); the merge, or the call behind, may be launched from here on
+    // fence); next_at_start: the merge, or the call behind, may be launched from here on (see the launch)
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (next_at_start) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("fence.proxy.async;" ::: "memory");
 
     // Work item: (context part, sequence, group of four query heads).  Items before tail_first take
@@ -869,6 +869,7 @@ decode_pair_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc,
     }
     __syncthreads();
 
+    if (!next_at_start) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // ---------------------------------------------------------------- epilogue: bins x V centroids
     // A warp takes four consecutive centroids of eight groups at a time, a lane one of them (32 bytes) for all four heads:
     // whole lines of the codebook (a group per lane touched 16 lines per load, 12 thousand cycles per CTA).  The eight
@@ -1013,10 +1014,16 @@ cudaError_t launch_decode_pair(const __half* q, const uint8_t* kc, const uint8_t
     const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(decode_pair_kernel), C::kSmemBytes, 0);
     if (e != cudaSuccess) return e;
     const int aligned = ((reinterpret_cast<uintptr_t>(kcb) | reinterpret_cast<uintptr_t>(vcb)) & 31u) == 0 ? 1 : 0;
+    // What follows may be launched at the CTAs' start where each of them has an SM to itself: its CTAs then wait on the other half of
+    // the SMs.  With more CTAs it goes ahead at their epilogue; CTAs launched earlier are placed two to an SM while other SMs
+    // have one.  Steps of CQ-8c8b back to back, us, at the start / at the epilogue: 104 CTAs (13 x 962 tokens, 32 heads on 8) 25.0 / 27.6,
+    // 128 (20011) 29.7 / 37.3; 232 (29 x 171 tokens) 25.6 / 25.3, 248 (31 x 8-23 k) 161 / 147, 256 (32 x 6.6-12 k) 99.2 / 91.6, 368
+    // (23 x 1-1.3 k) 39.6 / 38.9, 416 (13 x 18-27 k) 108.5 / 107.8.
+    const int next_at_start = (int64_t)pl.grid <= device_sm_count() ? 1 : 0;
     cudaLaunchAttribute attr;
     const cudaLaunchConfig_t cfg = overlapped_config(pl.grid, C::kThreads, C::kSmemBytes, st, &attr);
     return cudaLaunchKernelEx(&cfg, decode_pair_kernel, q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, pl.chunk, pl.n_parts,
-                              pl.tail_first, aligned, partials, app, pl.n_parts == 1 ? out : nullptr);
+                              pl.tail_first, aligned, next_at_start, partials, app, pl.n_parts == 1 ? out : nullptr);
 }
 
 }  // namespace cq

@@ -140,3 +140,27 @@ def test_host_buffers(c, b, n_seq, n_q, n_kv, how):
     got = cq.cq_decode_step_host(*host, pin(lens), *codes, *books, D ** -0.5, c, b, cap, out, ws)
     assert torch.equal(codes[0], other[0]) and torch.equal(codes[1], other[1])
     close(got, want)
+
+
+@pytest.mark.parametrize("n_seq,cap", [(2, 64), (20, 64), (3, 9000), (14, 9000)])
+def test_steps_with_the_append_inside_right_behind_one_another(n_seq, cap):
+    # decode_pair_kernel lets the next kernel go ahead at its start or at its epilogue, by its CTAs (16, 160; 96 and 448 of split
+    # contexts): 8 steps without a wait between them against the same steps with one
+    c, b, D = 8, 8, 128
+    q, codes, books, new = make(c, b, n_seq, 32, 8, D, cap, n_seq)
+    ws = torch.empty(cq.cq_decode_step_workspace_bytes(n_seq, 32, 8, D, c, b, cap), dtype=torch.uint8, device=DEV)
+
+    def run(wait):
+        kv = [x.clone() for x in codes]
+        lens = torch.clamp(lengths(n_seq, cap), max=cap - 8)
+        outs = []
+        for _ in range(8):
+            outs.append(cq.cq_decode_step(q, *new, lens, *kv, *books, D ** -0.5, c, b, cap, workspace=ws).clone())
+            lens.add_(1)
+            if wait:
+                torch.cuda.synchronize()
+        return outs, kv
+    (a, ka), (w, kw) = run(False), run(True)
+    assert torch.equal(ka[0], kw[0]) and torch.equal(ka[1], kw[1])
+    for x, y in zip(a, w):
+        close(x, y)
