@@ -324,12 +324,14 @@ int cq_encode_variant(const void *x_fp16, const float *codebooks, const int32_t 
  * initialisation and a fixed number of k-means iterations (Section 4.3).
  *
  *   x_fp16     [n_vec][n_heads][head_dim] fp16, 16-byte aligned
- *   weights    NULL (Eq. 5), or [n_vec][n_heads][G] fp32, non-negative (Eq. 6)
+ *   weights    NULL (Eq. 5), or [n_vec][n_heads][G] fp32, non-negative (Eq. 6); of any magnitudes: a
+ *              centroid whose members all weigh next to nothing moves to their mean like any other
  *   uniforms   [n_heads][G][2^b] fp64 in [0, 1): the random draws of k-means++, supplied by the
  *              caller (the library draws nothing).  Centre 0 of a problem is vector
  *              floor(u_0 n_vec); centre k is the first vector whose running sum of w_i D_i, in
  *              index order and in fp64, reaches u_k times the total (D_i: squared distance to
- *              the nearest centre chosen so far)
+ *              the nearest centre chosen so far), and the last vector where none does (an
+ *              infinite total times a u_k of 0)
  *   codebooks  [n_heads][G][2^b][c] fp32, 16-byte aligned
  *   objective_out  NULL, or [n_heads][G] fp64: sum_i w_i ||x_i - CQ(x_i)||^2 of the last
  *              assignment (measured against the codebooks that assignment used)

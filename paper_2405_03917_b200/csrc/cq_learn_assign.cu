@@ -15,7 +15,8 @@
 //     is left behind by that, the sums are whole numbers: w x in units of 2^-L of the largest |x| and w of the problem, and
 //     the rest below that in a second word of L bits (L = 62 - log2 n: 94 bits for 32768 vectors; products of a
 //     24-bit weight and an 11-bit channel are exact down to 2^-59 of the largest).  They do not depend on the order of the
-//     additions either.
+//     additions either.  A centroid whose members all weigh so little beside the problem's largest weight that these words hold
+//     less of their sums than fp32 sums would (ThinRule) is summed up anew, in fp64.
 //   - A problem in which nothing moved in an iteration has converged: the iterations after it return at once.
 // The codes are those of the full evaluation bit for bit: thr is lowered by a bound on every rounding (below), and a row that
 // was not certain is evaluated again each time.  Problems with infinities, NaNs or negative weights (found by
@@ -46,27 +47,53 @@ struct AsCfg {
     static_assert(4 * (kSmemBytes + 1024) <= 228 * 1024 && 5 * (kSmemBytes + 1024) > 228 * 1024, "four CTAs per SM");
 };
 
-// Is the problem one for the fixed-point sums and the bounds: largest |x| (fp16 bits) and weight (fp32 bits) finite, no
-// weight negative (its bits would be larger than those of infinity).
-__device__ __forceinline__ bool as_plain(const uint32_t* top, int p) { return top[2 * p] < 0x7c00u && top[2 * p + 1] < 0x7f800000u; }
+// What learn_range_kernel notes of a problem: the largest |x| (fp16 bits), the largest weight (fp32 bits) and the complement of the
+// smallest weight's bits that is not zero (0: every weight is).  All zero before it.
+struct AsRange {
+    uint32_t x, w, w_least;
+};
+
+// Is the problem one for the fixed-point sums and the bounds: largest |x| and weight finite, no weight negative (its bits
+// would be larger than those of infinity).
+__device__ __forceinline__ bool as_plain(const AsRange* top, int p) { return top[p].x < 0x7c00u && top[p].w < 0x7f800000u; }
 
 // exponents: |x| < 2^ex, w < 2^ew
-__device__ __forceinline__ void as_scales(const uint32_t* top, int p, bool weighted, int& ex, int& ew)
+__device__ __forceinline__ void as_scales(const AsRange* top, int p, bool weighted, int& ex, int& ew)
 {
-    frexpf(__half2float(__ushort_as_half((unsigned short)top[2 * p])), &ex);
+    frexpf(__half2float(__ushort_as_half((unsigned short)top[p].x)), &ex);
     ew = 1;
-    if (weighted) frexpf(__uint_as_float(top[2 * p + 1]), &ew);
+    if (weighted) frexpf(__uint_as_float(top[p].w), &ew);
 }
 
-// top[2 p], top[2 p + 1]: the largest |x| of problem p (fp16 bits) and the largest weight (fp32 bits); zero on entry.
+// Weight sums (in units of 2^(ew - L), the first word's) with which a centroid's sums are formed anew.  Each member's terms are
+// rounded by 2^-L / 2 of the first word's unit at most, so that the mean of m members with weight sum ws is off by no more than
+// m 2^-L 2^ex / ws.  That is within 2^-48, 2^-24 of the smallest fp16 channel, for ws >= m 2^(48 + ex - L): for every centroid
+// whose ws reaches n 2^(48 + ex - L) (32768 vectors below 32: 2^-26 of the largest weight), and, because ws >= m w_least, for every
+// one of the problem if w_least >= 2^(48 + ex + ew - 2 L) (2^-41 of it); then there is no floor.  A sum of zero is exact, no member
+// weighs anything, where w_least is not lost in the rounding.
+struct ThinRule {
+    double floor;
+    bool zero_is_exact;
+    __device__ __forceinline__ bool thin(double ws) const { return ws < floor && !(zero_is_exact && ws == 0.0); }
+};
+__device__ __forceinline__ ThinRule thin_rule(const AsRange* top, int p, bool weighted, int ex, int ew, int limb_bits, int64_t n_vec)
+{
+    ThinRule r = {0.0, true};
+    if (!weighted || top[p].w_least == 0u) return r;
+    const int field = (int)(~top[p].w_least >> 23), least = (field ? field - 127 : -149) + 2 * limb_bits - ew;       // w_least >= 2^(least + ew - 2 L)
+    if (least < 48 + ex) r.floor = (double)n_vec * __hiloint2double((1023 + 48 + ex - limb_bits) << 20, 0);
+    r.zero_is_exact = least >= 0;
+    return r;
+}
+
 constexpr int kRangeThreads = 256, kRangeVecs = 256;
 template <int kC>
 __global__ void __launch_bounds__(kRangeThreads)
-learn_range_kernel(const __half* __restrict__ x, const float* __restrict__ weights, Shape sh, int64_t n_vec, uint32_t* __restrict__ top)
+learn_range_kernel(const __half* __restrict__ x, const float* __restrict__ weights, Shape sh, int64_t n_vec, AsRange* __restrict__ top)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, h = blockIdx.y, n_prob = sh.n_kv_heads * sh.G;
     const int64_t v0 = (int64_t)blockIdx.x * kRangeVecs, v1 = v0 + kRangeVecs < n_vec ? v0 + kRangeVecs : n_vec;
-    uint32_t tx = 0, tw = 0;
+    uint32_t tx = 0, tw = 0, tl = 0;
 #pragma unroll 4
     for (int64_t v = v0 + warp; v < v1; v += kRangeThreads / 32) {
         const uint2 xw = *reinterpret_cast<const uint2*>(x + (v * sh.n_kv_heads + h) * 128 + 4 * lane);
@@ -75,11 +102,15 @@ learn_range_kernel(const __half* __restrict__ x, const float* __restrict__ weigh
         if (weights && lane < sh.G) {
             const uint32_t w = __float_as_uint(weights[v * n_prob + h * sh.G + lane]);
             tw = max(tw, w == 0x80000000u ? 0u : w);
+            if (w << 1) tl = max(tl, ~w);
         }
     }
     if (kC == 8) tx = max(tx, __shfl_xor_sync(0xffffffffu, tx, 1));
-    if (lane % (kC / 4) == 0) atomicMax(&top[2 * (h * sh.G + 4 * lane / kC)], tx);
-    if (weights && lane < sh.G) atomicMax(&top[2 * (h * sh.G + lane) + 1], tw);
+    if (lane % (kC / 4) == 0) atomicMax(&top[h * sh.G + 4 * lane / kC].x, tx);
+    if (weights && lane < sh.G) {
+        atomicMax(&top[h * sh.G + lane].w, tw);
+        atomicMax(&top[h * sh.G + lane].w_least, tl);
+    }
 }
 
 // One CTA: the vectors [range * i, range * (i + 1)) of one problem; blockIdx.x = (i, head, group), the groups of a head
@@ -89,7 +120,7 @@ __global__ void __launch_bounds__(kTcThreads, 4)
 assign_kernel(const __half* __restrict__ x, const float* __restrict__ weights, const float* __restrict__ cb, Shape sh, int64_t n_vec,
               int64_t n_pad, int range, int it, int limb_bits, uint8_t* __restrict__ codes, float* __restrict__ thr,
               unsigned long long* __restrict__ sums, const float* __restrict__ cum_all, int* __restrict__ last_moved,
-              const uint32_t* __restrict__ top)
+              const AsRange* __restrict__ top)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");      // launched ahead of the end of the kernel that moves the centroids
     using C = AsCfg<kC>;
@@ -362,13 +393,36 @@ assign_kernel(const __half* __restrict__ x, const float* __restrict__ weights, c
     }
 }
 
+// The rows of the centroids with thin[code] become their members' weighted channels and weights, summed in fp64, in place of the words
+// of the fixed-point sums.  By a whole CTA, between two barriers.  (Out of line, for the registers of the kernel around it.)
+template <int kC>
+__device__ __noinline__ void as_sum_thin(double* rows, const uint8_t* thin, const __half* __restrict__ x, const float* __restrict__ weights,
+                                         const uint8_t* __restrict__ codes, const Shape& sh, int64_t n_vec, int p)
+{
+    const int h = p / sh.G, g = p % sh.G, n_prob = sh.n_kv_heads * sh.G;
+    for (int64_t blk = threadIdx.x; blk < (n_vec + kTokenBlock - 1) / kTokenBlock; blk += kAsK) {
+        const uint4 cw = *reinterpret_cast<const uint4*>(codes + code_word_offset(sh, sh.n_kv_heads, 0, h, blk, g));
+#pragma unroll 1
+        for (int k = 0; k < 16; ++k) {
+            const int code = (int)((k < 4 ? cw.x : k < 8 ? cw.y : k < 12 ? cw.z : cw.w) >> (8 * (k & 3)) & 0xffu);
+            const int64_t v = blk * kTokenBlock + k;
+            if (!thin[code] || v >= n_vec) continue;
+            double* row = rows + code * 2 * (kC + 1);
+            const double w = (double)weights[v * n_prob + p];
+#pragma unroll 1
+            for (int q = 0; q < kC; ++q) atomicAdd(row + q, w * (double)__half2float(x[(v * n_prob + p) * kC + q]));
+            atomicAdd(row + kC, w);
+        }
+    }
+}
+
 // The centroids of one problem from its sums, and the sums of moves that the thresholds are compared with.  A thread per
 // centroid.
 template <int kC>
 __global__ void __launch_bounds__(kAsK)
 learn_move_kernel(const __half* __restrict__ x, const float* __restrict__ weights, const uint8_t* __restrict__ codes, Shape sh,
                   int64_t n_vec, int it, int limb_bits, const unsigned long long* __restrict__ sums, float* __restrict__ cum,
-                  const int* __restrict__ last_moved, const uint32_t* __restrict__ top, float* __restrict__ cb)
+                  const int* __restrict__ last_moved, const AsRange* __restrict__ top, float* __restrict__ cb)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");      // launched ahead of the end of the assignment
     // the problem's sums, read in whole lines (a row of 8 (c + 1) 2 bytes per thread touched 32 lines a load); or fp32 sums
@@ -376,6 +430,7 @@ learn_move_kernel(const __half* __restrict__ x, const float* __restrict__ weight
     float* acc = reinterpret_cast<float*>(rows);
     __shared__ float best[2][kAsK / 32];
     __shared__ int arg[kAsK / 32];
+    __shared__ uint8_t thin_s[kAsK];
     const int p = blockIdx.x, j = threadIdx.x, lane = j & 31, warp = j >> 5;
     if (last_moved[p] < it + 1) return;
     float* cj = cb + ((int64_t)p * kAsK + j) * kC;
@@ -405,15 +460,27 @@ learn_move_kernel(const __half* __restrict__ x, const float* __restrict__ weight
     int ex, ew;
     as_scales(top, p, weights != nullptr, ex, ew);
     const double limb = ldexp(1.0, -limb_bits), back = ldexp(1.0, ex);
-    const unsigned long long* row = rows + j * 2 * (kC + 1);
+    unsigned long long* row = rows + j * 2 * (kC + 1);
     auto value = [&](int ch) { return (double)(long long)row[ch] + (double)(long long)row[kC + 1 + ch] * limb; };
-    const double ws = value(kC);
+    double ws = value(kC);
+    const ThinRule rule = thin_rule(top, p, weights != nullptr, ex, ew, limb_bits, n_vec);
+    const bool thin = rule.thin(ws);
+    if (rule.floor > 0.0) {
+        thin_s[j] = thin ? 1 : 0;
+        if (thin)
+            for (int ch = 0; ch <= kC; ++ch) row[ch] = 0ull;
+        if (__syncthreads_or(thin)) {
+            as_sum_thin<kC>(reinterpret_cast<double*>(rows), thin_s, x, weights, codes, sh, n_vec, p);
+            __syncthreads();
+        }
+        if (thin) ws = __longlong_as_double((long long)row[kC]);
+    }
     float d2 = 0.f;
     if (ws > 0.0) {                                          // (a centroid without members stays)
-        const double share = back / ws;
+        const double share = (thin ? 1.0 : back) / ws;
 #pragma unroll
         for (int q = 0; q < kC; ++q) {
-            const float was = cj[q], now = (float)(value(q) * share), d = now - was;
+            const float was = cj[q], now = (float)((thin ? __longlong_as_double((long long)row[q]) : value(q)) * share), d = now - was;
             cj[q] = now;
             d2 = fmaf(d, d, d2);
         }
@@ -453,11 +520,11 @@ bool learn_bounds_supported(const Shape& sh, int64_t n_vec)
     return sh.head_dim == 128 && sh.b == 8 && (sh.c == 4 || sh.c == 8) && n_vec >= 16 && n_vec <= (1 << 23);
 }
 
-// sums, sums of moves, last iteration with a move, largest |x| and weight (the thresholds lie in the distances' place)
+// sums, sums of moves, last iteration with a move, ranges of |x| and weights (the thresholds lie in the distances' place)
 size_t learn_bounds_bytes(const Shape& sh)
 {
     const size_t n_prob = (size_t)sh.n_kv_heads * sh.G;
-    return as_round(n_prob * kAsK * 2 * (sh.c + 1) * 8) + as_round(n_prob * kAsK * 4) + as_round(n_prob * 4) + as_round(n_prob * 8);
+    return as_round(n_prob * kAsK * 2 * (sh.c + 1) * 8) + as_round(n_prob * kAsK * 4) + as_round(n_prob * 4) + as_round(n_prob * sizeof(AsRange));
 }
 
 template <int kC>
@@ -470,7 +537,7 @@ static cudaError_t run_bounds(const __half* x, const float* weights, const Shape
     unsigned long long* sums = reinterpret_cast<unsigned long long*>(w);      w += as_round((size_t)n_prob * kAsK * 2 * (kC + 1) * 8);
     float* cum = reinterpret_cast<float*>(w);                                 w += as_round((size_t)n_prob * kAsK * 4);
     int* last_moved = reinterpret_cast<int*>(w);                              w += as_round((size_t)n_prob * 4);
-    uint32_t* top = reinterpret_cast<uint32_t*>(w);
+    AsRange* top = reinterpret_cast<AsRange*>(w);
     cudaError_t e = cudaMemsetAsync(state, 0, learn_bounds_bytes(sh), st);
     if (e != cudaSuccess) return e;
     learn_range_kernel<kC><<<dim3((unsigned)((n_vec + kRangeVecs - 1) / kRangeVecs), (unsigned)sh.n_kv_heads), kRangeThreads, 0, st>>>(

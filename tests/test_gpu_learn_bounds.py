@@ -74,6 +74,30 @@ def test_weights_over_many_orders_of_magnitude(c):
     assert off.float().mean() <= 0.1 and torch.allclose(oa, ob, rtol=1e-3)
 
 
+# Some vectors weigh up to 2^-120 of the others.  The heavy ones are drawn first and are fewer than the centroids, so that light
+# ones become centres too and centroids have light members only.  2^-40: ruled out by the smallest weight; 2^-60 and less: sums
+# formed anew, 2^-95 and less: the fixed-point sums would hold less than fp32 ones, or nothing.  (200 vectors: fewer than
+# centroids, whose rest stays empty; 5000: two CTAs to a problem)
+@pytest.mark.parametrize("light", [2.0 ** -40, 2.0 ** -60, 2.0 ** -95, 2.0 ** -120])
+@pytest.mark.parametrize("c,n", [(8, 900), (4, 900), (8, 200), (4, 5000)])
+def test_centroids_with_light_members_only(c, n, light):
+    x, g = vectors(n, 1, 5 * c + n)
+    w = torch.rand(n, 1, D // c, generator=g).add(0.5)
+    w *= torch.where(torch.arange(n) % (n // 100) == 0, 1.0, light)[:, None, None]
+    w[3] = 0
+    w = w.to(DEV)
+    u = torch.rand(1, D // c, 256, generator=g, dtype=torch.float64).to(DEV)
+    start = cq.cq_kmeanspp_init(x, w, u, c, 8)
+    for iters in (1, 3):
+        a, oa = learn(x, w, u, c, iters)
+        b, ob = plain(x, w, u, c, iters)
+        # as for the first iterations above: fp32 sums on one side, and vectors with two centroids equally near
+        off = (a - b).abs().amax(dim=(2, 3)) > 1e-5 * b.abs().amax()
+        assert off.float().mean() <= 0.1 and torch.allclose(oa, ob, rtol=1e-3)
+        if n > 256:
+            assert (b != start).any(-1).float().mean() > 0.2       # centroids of light vectors have moved, not only heavy ones
+
+
 @pytest.mark.parametrize("what", ["inf", "nan", "negative weight", "infinite weight"])
 def test_problems_without_bounds(what):
     # the problem that holds the value is evaluated in full; the others keep their result
