@@ -499,16 +499,16 @@ encode_few_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, 
                   int n_vec, int n_tokens, int64_t token_offset, uint8_t* __restrict__ codes1, const __half* __restrict__ x2,
                   const float* __restrict__ cb2, uint8_t* __restrict__ codes2, int share)
 {
-    // launched ahead of the end of whatever lies before it in the stream, which may well write the codebooks (a k-means update)
+    // Launched ahead of the end of whatever lies before it in the stream, which may well write the codebooks (a k-means update).  It
+    // lets nothing go ahead itself: calls back to back, let ahead / not: 12 vectors x 8 heads of CQ-4c8b 3.9 / 3.2 us, 30 x 8 of 2c8b 6.4 / 5.3.
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const bool second = blockIdx.y != 0;
     encode_few<kC>(second ? x2 : x1, second ? cb2 : cb1, seq_offsets, sh, blockIdx.x, n_vec, share, n_tokens,
                          token_offset, second ? codes2 : codes1, false);
 }
 
-// 512 and 1024 centroids: one CTA per (head, group) reads the group's codebook once, a thread holding kPer of its 256 * kPer
-// centroids in registers, and takes the vectors past them sixteen at a time.  Distances and ties as in encode_few.  What it
+// 512 and 1024 centroids, and 256 where few_by_cta: one CTA per (head, group) reads the group's codebook once, a thread holding kPer of
+// its 256 * kPer centroids in registers, and takes the vectors past them sixteen at a time.  Distances and ties as in encode_few.  What it
 // takes is one pass over the codebooks (16 vectors x 32 heads of CQ-8c10b, key and value: 33 MB; 52 us on the tensor-memory
 // kernel, which walks its steps one after the other with 16 of 128 rows in use, 17 us here with single instructions).  A warp per 256 centroids
 // (encode_few) has too few warps for this many (27 us; two vectors, 40 heads 12.6 against 9.9 us).
@@ -554,7 +554,7 @@ encode_few_wide_kernel(const __half* __restrict__ x1, const float* __restrict__ 
             }
         }
     }
-    unsigned long long c2[kPer / 2][kC];                          // (kPacked only)
+    unsigned long long c2[kPer > 1 ? kPer / 2 : 1][kC];           // (kPacked only)
 #pragma unroll
     for (int u = 0; u < kPer / 2; ++u)
 #pragma unroll
@@ -636,18 +636,35 @@ encode_few_wide_kernel(const __half* __restrict__ x1, const float* __restrict__ 
 // CQ-8c9b 4.6 / 5.9 / 12.6 / 21.5 against 4.8 / 5.9 / 11.5 / 19.0; one head of CQ-4c10b, 30 vectors 6.4 against 6.6.
 bool wide_packed_pays(int n_vec, int64_t ctas) { return n_vec >= 4 && ctas > device_sm_count(); }
 
+// 256 centroids: a CTA per (head, group) (encode_few_wide_kernel) or warps with shares of the vectors (encode_few_kernel).  The warps
+// each read the whole 32 c bytes x 32 of a group and sit eight to a CTA on few SMs; where the CTAs are at most four to an SM and the
+// vectors few, reading once and reducing over eight warps is the shorter way.  us, by CTAs / by warps, key and value, of CQ-8c8b: 1 vector x 8
+// heads 1.7 / 2.5, 8 x 8 2.3 / 3.3, 16 x 8 3.0 / 3.7, 20 x 8 4.0 / 4.1, 16 x 24 6.9 / 5.4; of CQ-4c8b: 1 x 8 1.9 / 2.2, 8 x 8 2.5 / 2.7, 16 x 8 3.5 / 3.4, 8 x 24
+// 4.4 / 4.7, 24 x 12 7.8 / 4.6.  With more CTAs of CQ-8c8b: up to eight vectors (8 x 32 4.5 / 4.6), and where a warp would take
+// all vectors (16 x 40 heads 7.8 / 9.7) or the warps would not run at once (20 x 40 10.5 / 12.2).
+bool few_by_cta(const Shape& sh, int n_vec, int64_t ctas)
+{
+    if (ctas <= 4 * (int64_t)device_sm_count()) return n_vec <= (sh.c == 8 ? kFewWideVecs : kFewWideVecs / 2);
+    if (sh.c != 8) return false;
+    const int share = few_share(sh, n_vec), shares = (n_vec + share - 1) / share;
+    return n_vec <= kFewWideVecs / 2 || shares == 1 || ctas * shares > 16 * (int64_t)device_sm_count();
+}
+
 template <int kC>
 cudaError_t launch_few(const __half* x, const float* cb, const int32_t* seq_offsets, const Shape& sh, int64_t n_tokens, int64_t token_offset,
                        uint8_t* codes, cudaStream_t st, const __half* x2, const float* cb2, uint8_t* codes2)
 {
     const int n_vec = (int)(sh.n_seq * n_tokens);
     cudaLaunchAttribute attr;
-    cudaLaunchConfig_t cfg = overlapped_config((unsigned)(sh.b == 8 ? few_ctas(sh, n_vec) : sh.n_kv_heads * EncCfg<kC>::G), kFewThreads, 0, st, &attr);
-    cfg.gridDim.y = x2 ? 2 : 1;
+    const int tensors = x2 ? 2 : 1;
+    const bool by_cta = sh.b != 8 || few_by_cta(sh, n_vec, (int64_t)tensors * sh.n_kv_heads * EncCfg<kC>::G);
+    cudaLaunchConfig_t cfg = overlapped_config((unsigned)(by_cta ? sh.n_kv_heads * EncCfg<kC>::G : few_ctas(sh, n_vec)), kFewThreads, 0, st, &attr);
+    cfg.gridDim.y = (unsigned)tensors;
     auto go = [&](auto kernel, auto... share) {
         return cudaLaunchKernelEx(&cfg, kernel, x, cb, seq_offsets, sh, n_vec, (int)n_tokens, token_offset, codes, x2, cb2, codes2, share...);
     };
-    if (sh.b == 8) return go(encode_few_kernel<kC>, few_share(sh, n_vec));
+    if (!by_cta) return go(encode_few_kernel<kC>, few_share(sh, n_vec));
+    if (sh.b == 8) return go(encode_few_wide_kernel<kC, 1, false>);
     const bool packed = wide_packed_pays(n_vec, (int64_t)cfg.gridDim.x * cfg.gridDim.y);
     if (sh.b == 9) return packed ? go(encode_few_wide_kernel<kC, 2, true>) : go(encode_few_wide_kernel<kC, 2, false>);
     return packed ? go(encode_few_wide_kernel<kC, 4, true>) : go(encode_few_wide_kernel<kC, 4, false>);

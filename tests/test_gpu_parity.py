@@ -559,3 +559,23 @@ def test_attention_head_dim_64_tuned(c, n_q, n_kv, lens):
         out, ref = attn_both(q, kc_rm, vc_rm, kcb, vcb, lens, 64 ** -0.5, c, 8, variant)
         err, rel = H.check_attn(out, ref, f"head_dim 64 c={c} R={n_q // n_kv} variant={variant}")
         assert rel < 2e-6
+
+
+# both forms of the encode of few vectors at the sizes where one takes over from the other: eight and sixteen vectors, four CTAs per
+# (head, group) and SM (18 heads at c = 8, 9 at c = 4, key and value), a warp with all vectors (40 heads)
+@pytest.mark.parametrize("n_vec", [1, 8, 9, 16, 17, 32])
+@pytest.mark.parametrize("c,n_heads", [(8, 1), (8, 18), (8, 19), (8, 40), (4, 9), (4, 10), (2, 4), (2, 5)])
+def test_encode_of_few_vectors_equals_the_generic_kernel(c, n_heads, n_vec):
+    g = torch.Generator().manual_seed(c * n_heads + n_vec)
+    x = torch.randn(2, n_vec, 1, n_heads, 128, generator=g).half()
+    cb = torch.randn(2, n_heads, 128 // c, 256, c, generator=g)
+    cb[:, :, :, 200] = cb[:, :, :, 7]                                # equal centroids: the lower index
+    x[0, 0, 0, 0, :c], x[1, n_vec // 2, 0, n_heads - 1, -1] = cb[0, 0, 0, 200].half(), float("nan")
+    x, cb = x.to(DEV), cb.to(DEV)
+    size = cq.cq_codes_bytes(n_vec, 20, n_heads, 128, c, 8)
+    got, want = (torch.zeros(2, size, dtype=torch.uint8, device=DEV) for _ in range(2))
+    off = torch.arange(n_vec, dtype=torch.int32, device=DEV) % 21    # 20: no room, the vector is dropped
+    cq.cq_encode_kv(x[0], x[1], cb[0], cb[1], c, 8, got[0], got[1], 20, seq_offsets=off)
+    for i in range(2):
+        cq.cq_encode(x[i], cb[i], c, 8, want[i], 20, seq_offsets=off, variant=1)
+    assert torch.equal(got, want)

@@ -60,7 +60,7 @@ def test_nothing_is_read_before_the_wait(file, name, text):
         assert not re.search(rf"\b{p}\s*\[", ahead), f"{file}: {name} reads {p} ahead of its wait"
 
 
-@pytest.mark.parametrize("name", ["merge_kernel", "decode_rope_tuned_kernel", "encode_tc_kernel"])
+@pytest.mark.parametrize("name", ["merge_kernel", "decode_rope_tuned_kernel", "encode_tc_kernel", "encode_few_kernel"])
 def test_lets_nothing_go_ahead(name):
     # the CTAs of a kernel launched beside these kernels' are placed unevenly over the SMs, and stay there
     (body,) = [text.split("__global__")[0] for _, kernel, text in kernels() if kernel == name]
