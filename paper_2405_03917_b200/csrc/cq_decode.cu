@@ -1305,9 +1305,10 @@ cudaError_t launch_cfg(const __half* q, const uint8_t* kc, const uint8_t* vc, co
     using C = Cfg<kD, G, R>;
     const int kv_share = sh.R / R;
     // call-site slots of ensure_dynamic_smem: 1 and 95 are the wide kernel; 2 ... 13 the instances of head_dim 128, 78 ... 89 those
-    // of head_dim 64; 96 ... 119 those with tables
+    // of head_dim 64; 96 ... 107 those of head_dim 128 with tables
     constexpr int kSlot = (kD == 128 ? 2 : 78) + 2 * ((G == 16 ? 0 : G == 64 ? 5 : 3) + (R == 1 ? 0 : R == 2 ? 1 : 2));
-    constexpr int kTabSlot = 96 + (kD == 128 ? kSlot - 2 : kSlot - 66);
+    // (four heads per CTA at 16 groups are decode_pair_supported: their steps append inside and take no tables)
+    constexpr bool kTakesTables = kD == 128 && !(G == 16 && R == 4);
     cudaLaunchAttribute attr;
     const cudaLaunchConfig_t cfg = overlapped_config(pl.grid, C::kThreads, C::kSmemBytes, st, &attr);
     auto go = [&](auto kernel, int slot) {
@@ -1316,8 +1317,8 @@ cudaError_t launch_cfg(const __half* q, const uint8_t* kc, const uint8_t* vc, co
         return cudaLaunchKernelEx(&cfg, kernel, q, kc, vc, kcb, vcb, seq_lens, scale * kLog2e, sh, pl.chunk, pl.n_parts, pl.tail_first,
                                   aligned32(kcb, vcb), kv_share, partials, pl.n_parts == 1 ? out : nullptr, ahead);
     };
-    if constexpr (kD == 128) {
-        if (ahead.tables) return kv_share > 1 ? go(decode_tuned_kernel<kD, G, R, true, true>, kTabSlot) : go(decode_tuned_kernel<kD, G, R, false, true>, kTabSlot + 1);
+    if constexpr (kTakesTables) {
+        if (ahead.tables) return kv_share > 1 ? go(decode_tuned_kernel<kD, G, R, true, true>, 94 + kSlot) : go(decode_tuned_kernel<kD, G, R, false, true>, 95 + kSlot);
     }
     if (ahead.tables) return cudaErrorNotSupported;
     return kv_share > 1 ? go(decode_tuned_kernel<kD, G, R, true, false>, kSlot) : go(decode_tuned_kernel<kD, G, R, false, false>, kSlot + 1);

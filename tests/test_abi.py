@@ -178,3 +178,13 @@ def test_new_entry_points_validate_on_the_host(L):
     assert encv(b=10) == -3
     assert encv(D=64) == -3
     assert encv(variant=5) == -2
+
+
+@pytest.mark.parametrize("n_q,n_kv,tables", [(1, 1, True), (2, 1, True), (6, 1, True), (4, 1, False), (8, 2, False), (12, 1, False)])
+def test_which_steps_have_tables_ahead(L, n_q, n_kv, tables):
+    # four query heads per CTA of CQ-8c8b append inside the attention and build their own tables: decode_tuned_kernel has no
+    # instance for them with tables from the kernel ahead
+    entries = n_q * 16 * 256 * 4
+    attn = cq.cq_decode_attn_workspace_bytes(1, n_q, n_kv, 128, 8, 8, 1000)
+    step = cq.cq_decode_step_workspace_bytes(1, n_q, n_kv, 128, 8, 8, 1000)
+    assert (step - attn >= entries) == tables
