@@ -1,6 +1,8 @@
 """Decode steps whose kernel ahead of the attention appends the tokens and, for few queries, builds the tables of all sequences
 (cq_decode_tables.cu), against cq_encode_kv and cq_decode_attn, whose CTAs build their tables: the entries are the same sums in
 the same order, so the results agree as two calls do."""
+import mmap
+
 import numpy as np
 import pytest
 import torch
@@ -110,7 +112,7 @@ def test_steps_right_behind_one_another():
 
 
 @pytest.mark.parametrize("c,b,n_seq,n_q,n_kv", [(8, 8, 3, 8, 2), (4, 8, 2, 3, 3), (4, 8, 3, 24, 24), (8, 10, 2, 2, 1), (4, 4, 2, 2, 2)])
-@pytest.mark.parametrize("how", ["pinned", "side by side", "one block", "off by two bytes", "pageable", "pageable result"])
+@pytest.mark.parametrize("how", ["pinned", "one block", "off by two bytes", "pageable", "pageable result"])
 def test_host_buffers(c, b, n_seq, n_q, n_kv, how):
     # pinned buffers are read and written by kernels (16 bytes at a time where they are aligned), others are copied
     D, cap = 128, 200
@@ -123,12 +125,6 @@ def test_host_buffers(c, b, n_seq, n_q, n_kv, how):
     pin = (lambda t: t) if how == "pageable" else (lambda t: t.pin_memory())
     if how == "pinned":
         host = [pin(p.cpu()) for p in parts]
-    elif how == "side by side":                        # allocations of their own that happen to lie back to back: not one copy
-        pool = sorted((torch.empty(parts[0].numel(), dtype=torch.float16).pin_memory() for _ in range(40)), key=lambda t: t.data_ptr())
-        run = [i for i in range(38) if pool[i + 1].data_ptr() - pool[i].data_ptr() == pool[i + 2].data_ptr() - pool[i + 1].data_ptr() == 2 * parts[0].numel()]
-        if n_q != n_kv or not run:
-            pytest.skip("no such allocations here")
-        host = [pool[run[0] + i].view(p.shape).copy_(p.cpu()) for i, p in enumerate(parts)]
     else:
         block = pin(torch.empty(sum(p.numel() for p in parts) + skip, dtype=torch.float16))
         host, at = [], skip
@@ -138,6 +134,34 @@ def test_host_buffers(c, b, n_seq, n_q, n_kv, how):
     out = torch.empty(n_seq, n_q, D) if "pageable" in how else torch.empty(n_seq, n_q, D).pin_memory()
     ws = torch.empty(cq.cq_decode_step_host_workspace_bytes(n_seq, n_q, n_kv, D, c, b, cap), dtype=torch.uint8, device=DEV)
     got = cq.cq_decode_step_host(*host, pin(lens), *codes, *books, D ** -0.5, c, b, cap, out, ws)
+    assert torch.equal(codes[0], other[0]) and torch.equal(codes[1], other[1])
+    close(got, want)
+
+
+@pytest.mark.parametrize("c,b,n_seq,n_q,n_kv", [(4, 8, 4, 4, 4), (8, 8, 2, 32, 8), (8, 8, 16, 8, 8), (8, 10, 16, 2, 1)])
+def test_host_buffers_side_by_side(c, b, n_seq, n_q, n_kv):
+    # pinned memory of three registrations that lie back to back (whole pages each): not one copy
+    D, cap = 128, 200
+    q, codes, books, new = make(c, b, n_seq, n_q, n_kv, D, cap, 5 + c)
+    lens = torch.arange(5, 5 + 10 * n_seq, 10, dtype=torch.int32)
+    other = [x.clone() for x in codes]
+    want = cq.cq_decode_step(q, *new, lens.to(DEV), *other, *books, D ** -0.5, c, b, cap)
+    parts = [q, *new]
+    block = torch.frombuffer(mmap.mmap(-1, sum(2 * p.numel() for p in parts)), dtype=torch.float16)
+    rt, registered, host, at = torch.cuda.cudart(), [], [], 0
+    out = torch.empty(n_seq, n_q, D).pin_memory()
+    ws = torch.empty(cq.cq_decode_step_host_workspace_bytes(n_seq, n_q, n_kv, D, c, b, cap), dtype=torch.uint8, device=DEV)
+    try:
+        for p in parts:
+            host.append(block[at:at + p.numel()].view(p.shape).copy_(p.cpu()))
+            at += p.numel()
+            assert host[-1].data_ptr() % mmap.PAGESIZE == 0 and 2 * p.numel() % mmap.PAGESIZE == 0
+            assert int(rt.cudaHostRegister(host[-1].data_ptr(), 2 * p.numel(), 0)) == 0
+            registered.append(host[-1].data_ptr())
+        got = cq.cq_decode_step_host(*host, lens.pin_memory(), *codes, *books, D ** -0.5, c, b, cap, out, ws)
+    finally:
+        for ptr in registered:
+            assert int(rt.cudaHostUnregister(ptr)) == 0
     assert torch.equal(codes[0], other[0]) and torch.equal(codes[1], other[1])
     close(got, want)
 
