@@ -482,8 +482,8 @@ namespace {
 size_t step_least_bytes(const Shape& sh) { return round_up(partial_bytes(sh), 256) + round_up((size_t)sh.n_seq * 4, 256); }
 // Bytes of inputs and output of a cq_decode_step_host call up to which its pinned buffers are read and written by kernels: no
 // hand-over between copy engine and kernels, and the result leaves as the CTAs end.  Over what was measured (1 KB to 3.3 MB)
-// it is the faster way: 64 sequences of 500 tokens, 32 heads on 8, CQ-8c8b (1.8 MB) 109 -> 82 us, 16 sequences 57 -> 44, one of 128
-// tokens 46 -> 36; 64 sequences, 32 heads of CQ-4c8b (2.6 MB) 191 -> 146.
+// it is the faster way: 64 sequences of 500 tokens, 32 heads on 8, CQ-8c8b (1.8 MB) 103 -> 86 us, 16 sequences 57 -> 48, one of 128
+// tokens 44 -> 35; 64 sequences, 32 heads of CQ-4c8b (2.6 MB) 192 -> 146 (with the steps' launches overlapped).
 constexpr size_t kDirectHostBytes = (size_t)4 << 20;
 // Inputs from which the fetching kernel is faster than two copies (back to back in host memory) under a result written in
 // place: one sequence of 20000 tokens, 32 heads on 8 (12 KB) 51.5 against 48.2 us, 32 heads of CQ-4c8b, 2000 tokens (25 KB) 38.9 against

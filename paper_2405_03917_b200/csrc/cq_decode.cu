@@ -681,8 +681,8 @@ decode_tuned_kernel(const __half* __restrict__ q, const uint8_t* __restrict__ kc
 
     // The merge, or the call behind, may be launched from here on: its launch passes behind the epilogue, and its CTAs do not wait on the
     // SMs beside the last wave's loops.  Step of 16 x 4096 tokens, 32 heads of CQ-4c8b, triggered behind the wait above / here: 68.2 / 66.2 us,
-    // 9 x 0.9-3 k, 40 heads 40.0 / 39.9, attention at head_dim 64 21.6 / 21.1.  (decode_pair_kernel and decode_wide_kernel lose by
-    // it: steps of one sequence of 20011 tokens 29.9 / 37.2, 16 x 8192 tokens of CQ-8c10b without any trigger 137.7 / 139.4.)
+    // 9 x 0.9-3 k, 40 heads 40.0 / 39.9, attention at head_dim 64 21.6 / 21.1.  (decode_pair_kernel
+    // goes by its CTAs, see its launch; decode_wide_kernel has no trigger: step of 16 x 8192 tokens of CQ-8c10b 137.7, 139.4 with this one.)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     // ---------------------------------------------------------------- epilogue: bins x V centroids
@@ -1382,7 +1382,7 @@ int decode_tuned_parts(const Shape& sh)
 
 // decode_pair_kernel reads a codebook once for four heads, so an append inside it costs less than a kernel ahead: 48 sequences of
 // 301 to 889 tokens, 32 heads on 8, 49.6 against 54.2 us; 64 x 16384 248.7 against 249.8.  With one or two heads per CTA the
-// kernel ahead is the better one (16 x 4096 tokens, 32 heads of CQ-4c8b: 73.3 -> 68.7 us; 10 x 147: 31.3 -> 25.7; 32 sequences of 8
+// kernel ahead is the better one (16 x 4096 tokens, 32 heads of CQ-4c8b: 72.9 -> 66.2 us; 10 x 147: 31.3 -> 25.7; 32 sequences of 8
 // to 32 k tokens, 40 heads of CQ-8c8b: 279 -> 265): inside, every CTA took the value centroids once more for it.
 bool decode_appends_inside(const Shape& sh) { return decode_pair_supported(sh); }
 

@@ -3,12 +3,13 @@
 //
 // Append.  A CTA of the attention that works the new token's codes out itself reads the value centroids (128 KiB) once more
 // than it otherwise would, per sequence; here they are read once per 16 sequences (encode_few).  16 x 4096 tokens, 32 heads
-// of CQ-4c8b: step 73.3 -> 68.7 us (attention alone 61.5); 15 x 10 k, 40 heads of CQ-2c8b: 306 -> 289.
+// of CQ-4c8b: step 72.9 -> 66.2 us (attention alone 59.4); 15 x 10 k, 40 heads of CQ-2c8b: 281 -> 264.
 //
 // Tables.  The attention (cq_decode.cu) looks the scores up in scale * log2(e) * <q_g, C_j> per (query head, group, code value).
 // With few queries its few CTAs read the key centroids one after the other while most SMs idle; here a warp takes 4 kU code
 // values of eight groups past all queries, so that the table is ready in the time of one load.  One sequence of 1024
-// tokens, one head of CQ-8c8b: 14.3 -> 9.3 us (append alone: 11).
+// tokens, one head of CQ-8c8b, calls back to back on the same buffers: 14.3 -> 9.3 to 9.8 us (append alone: 11); a first call on
+// buffers that the GPU has not seen 24.
 #include "cq_encode_few.cuh"
 
 namespace cq {

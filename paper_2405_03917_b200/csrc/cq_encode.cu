@@ -637,9 +637,9 @@ encode_few_wide_kernel(const __half* __restrict__ x1, const float* __restrict__ 
 bool wide_packed_pays(int n_vec, int64_t ctas) { return n_vec >= 4 && ctas > device_sm_count(); }
 
 // 256 centroids: a CTA per (head, group) (encode_few_wide_kernel) or warps with shares of the vectors (encode_few_kernel).  The warps
-// each read the whole 32 c bytes x 32 of a group and sit eight to a CTA on few SMs; where the CTAs are at most four to an SM and the
-// vectors few, reading once and reducing over eight warps is the shorter way.  us, by CTAs / by warps, key and value, of CQ-8c8b: 1 vector x 8
-// heads 1.7 / 2.5, 8 x 8 2.3 / 3.3, 16 x 8 3.0 / 3.7, 20 x 8 4.0 / 4.1, 16 x 24 6.9 / 5.4; of CQ-4c8b: 1 x 8 1.9 / 2.2, 8 x 8 2.5 / 2.7, 16 x 8 3.5 / 3.4, 8 x 24
+// each read the whole codebook of a group and sit eight to a CTA on few SMs; where the CTAs are at most four to an SM and the
+// vectors few, reading once and reducing over eight warps is the shorter way.  us, by CTAs / by warps, key and value, calls replayed from
+// a graph, of CQ-8c8b: 1 vector x 8 heads 1.7 / 2.5, 8 x 8 2.3 / 3.3, 16 x 8 3.0 / 3.7, 20 x 8 4.0 / 4.1, 16 x 24 6.9 / 5.4; of CQ-4c8b: 1 x 8 1.9 / 2.2, 8 x 8 2.5 / 2.7, 16 x 8 3.5 / 3.4, 8 x 24
 // 4.4 / 4.7, 24 x 12 7.8 / 4.6.  With more CTAs of CQ-8c8b: up to eight vectors (8 x 32 4.5 / 4.6), and where a warp would take
 // all vectors (16 x 40 heads 7.8 / 9.7) or the warps would not run at once (20 x 40 10.5 / 12.2).
 bool few_by_cta(const Shape& sh, int n_vec, int64_t ctas)

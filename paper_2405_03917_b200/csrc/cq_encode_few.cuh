@@ -11,7 +11,7 @@ namespace {
 // takes its share of the vectors past them.  Distances are the direct form sum (x - C)^2 in fp32 in the order of the
 // generic kernel, lowest index on ties.  Issue slots are what it takes (c multiply-adds and subtractions per centroid);
 // with a centroid per thread and the argmin over the eight warps of a CTA the reductions were a third of them: 30 vectors x
-// 40 heads of CQ-4c8b, key and value, 18.3 -> 12.6 us.
+// 40 heads of CQ-4c8b, key and value, 18.1 -> 14.2 us (where the CTA is the better form all the same: few_by_cta).
 constexpr int kFewThreads = 256;
 constexpr int kFewVecs = 16;              // vectors a warp takes at most
 
