@@ -394,23 +394,23 @@ assign_kernel(const __half* __restrict__ x, const float* __restrict__ weights, c
 }
 
 // The rows of the centroids with thin[code] become their members' weighted channels and weights, summed in fp64, in place of the words
-// of the fixed-point sums.  By a whole CTA, between two barriers.  (Out of line, for the registers of the kernel around it.)
+// of the fixed-point sums.  By a whole CTA, between two barriers; x, weights and codes are the problem's.  (Out of line and without
+// a stack, for the kernel around it.)
 template <int kC>
 __device__ __noinline__ void as_sum_thin(double* rows, const uint8_t* thin, const __half* __restrict__ x, const float* __restrict__ weights,
-                                         const uint8_t* __restrict__ codes, const Shape& sh, int64_t n_vec, int p)
+                                         const uint8_t* __restrict__ codes, int block_bytes, int n_prob, int64_t n_vec)
 {
-    const int h = p / sh.G, g = p % sh.G, n_prob = sh.n_kv_heads * sh.G;
     for (int64_t blk = threadIdx.x; blk < (n_vec + kTokenBlock - 1) / kTokenBlock; blk += kAsK) {
-        const uint4 cw = *reinterpret_cast<const uint4*>(codes + code_word_offset(sh, sh.n_kv_heads, 0, h, blk, g));
+        const uint4 cw = *reinterpret_cast<const uint4*>(codes + blk * block_bytes);
 #pragma unroll 1
         for (int k = 0; k < 16; ++k) {
             const int code = (int)((k < 4 ? cw.x : k < 8 ? cw.y : k < 12 ? cw.z : cw.w) >> (8 * (k & 3)) & 0xffu);
             const int64_t v = blk * kTokenBlock + k;
             if (!thin[code] || v >= n_vec) continue;
             double* row = rows + code * 2 * (kC + 1);
-            const double w = (double)weights[v * n_prob + p];
+            const double w = (double)weights[v * n_prob];
 #pragma unroll 1
-            for (int q = 0; q < kC; ++q) atomicAdd(row + q, w * (double)__half2float(x[(v * n_prob + p) * kC + q]));
+            for (int q = 0; q < kC; ++q) atomicAdd(row + q, w * (double)__half2float(x[v * n_prob * kC + q]));
             atomicAdd(row + kC, w);
         }
     }
@@ -470,7 +470,9 @@ learn_move_kernel(const __half* __restrict__ x, const float* __restrict__ weight
         if (thin)
             for (int ch = 0; ch <= kC; ++ch) row[ch] = 0ull;
         if (__syncthreads_or(thin)) {
-            as_sum_thin<kC>(reinterpret_cast<double*>(rows), thin_s, x, weights, codes, sh, n_vec, p);
+            const int n_prob = sh.n_kv_heads * sh.G;
+            as_sum_thin<kC>(reinterpret_cast<double*>(rows), thin_s, x + p * kC, weights + p,
+                            codes + code_word_offset(sh, sh.n_kv_heads, 0, p / sh.G, 0, p % sh.G), (int)sh.block_bytes, n_prob, n_vec);
             __syncthreads();
         }
         if (thin) ws = __longlong_as_double((long long)row[kC]);
