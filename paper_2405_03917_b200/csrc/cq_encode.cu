@@ -526,7 +526,7 @@ template <int kC, int kPer, bool kPacked>
 __global__ void __launch_bounds__(256)
 encode_few_wide_kernel(const __half* __restrict__ x1, const float* __restrict__ cb1, const int32_t* __restrict__ seq_offsets, Shape sh,
                   int n_vec, int n_tokens, int64_t token_offset, uint8_t* __restrict__ codes1, const __half* __restrict__ x2,
-                  const float* __restrict__ cb2, uint8_t* __restrict__ codes2)
+                  const float* __restrict__ cb2, uint8_t* __restrict__ codes2, int next_ahead)
 {
     const __half* x = blockIdx.y ? x2 : x1;
     const float* cb = blockIdx.y ? cb2 : cb1;
@@ -538,7 +538,7 @@ encode_few_wide_kernel(const __half* __restrict__ x1, const float* __restrict__ 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // launched ahead of the end of whatever lies before it in the stream, which may well write the codebooks (a k-means update)
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (next_ahead) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     float cv[kPer][kC];
 #pragma unroll
     for (int u = 0; u < kPer; ++u) {
@@ -631,15 +631,16 @@ encode_few_wide_kernel(const __half* __restrict__ x1, const float* __restrict__ 
     }
 }
 
-// From four vectors, and only with more CTAs than SMs (a CTA alone on its SM waits for its reductions, not for issue slots).  Key and
-// value, single against packed: 40 heads of CQ-8c10b, 1 / 4 / 16 / 30 vectors 6.2 / 8.8 / 20.9 / 37.2 against 6.7 / 8.4 / 17.7 / 30.4 us, of
-// CQ-8c9b 4.6 / 5.9 / 12.6 / 21.5 against 4.8 / 5.9 / 11.5 / 19.0; one head of CQ-4c10b, 30 vectors 6.4 against 6.6.
-bool wide_packed_pays(int n_vec, int64_t ctas) { return n_vec >= 4 && ctas > device_sm_count(); }
+// From so many vectors that a thread's sums (n_vec x centroids x channels) take longer than the packing of its centroids, and only with
+// more CTAs than SMs (a CTA alone on its SM waits for its reductions, not for issue slots).  Key and value, single / packed, calls
+// replayed from a graph: CQ-8c10b, 2 x 40 heads 7.2 / 7.4, 4 x 40 8.8 / 8.3, 4 x 12 4.1 / 4.0, 16 x 40 20.7 / 17.3, 32 x 40 38.9 / 31.8; CQ-8c9b, 4 x 24
+// 4.5 / 4.9, 8 x 24 5.8 / 5.7, 32 x 40 22.4 / 19.6; CQ-4c10b, 4 x 24 6.8 / 7.0, 8 x 24 9.7 / 8.9, 32 x 40 46.5 / 38.2; 16 x 4 heads of CQ-8c9b 3.6 / 3.8.
+bool wide_packed_pays(int n_vec, int per_thread, int64_t ctas) { return n_vec * per_thread >= 128 && ctas > device_sm_count(); }
 
 // 256 centroids: a CTA per (head, group) (encode_few_wide_kernel) or warps with shares of the vectors (encode_few_kernel).  The warps
 // each read the whole codebook of a group and sit eight to a CTA on few SMs; where the CTAs are at most four to an SM and the
 // vectors few, reading once and reducing over eight warps is the shorter way.  us, by CTAs / by warps, key and value, calls replayed from
-// a graph, of CQ-8c8b: 1 vector x 8 heads 1.7 / 2.5, 8 x 8 2.3 / 3.3, 16 x 8 3.0 / 3.7, 20 x 8 4.0 / 4.1, 16 x 24 6.9 / 5.4; of CQ-4c8b: 1 x 8 1.9 / 2.2, 8 x 8 2.5 / 2.7, 16 x 8 3.5 / 3.4, 8 x 24
+// a graph, of CQ-8c8b: 1 vector x 8 heads 1.7 / 2.5, 8 x 8 2.3 / 3.3, 16 x 8 3.0 / 3.7, 20 x 8 4.0 / 4.1, 16 x 24 5.7 / 5.4; of CQ-4c8b: 1 x 8 1.9 / 2.2, 8 x 8 2.5 / 2.7, 16 x 8 3.5 / 3.4, 8 x 24
 // 4.4 / 4.7, 24 x 12 7.8 / 4.6.  With more CTAs of CQ-8c8b: up to eight vectors (8 x 32 4.5 / 4.6), and where a warp would take
 // all vectors (16 x 40 heads 7.8 / 9.7) or the warps would not run at once (20 x 40 10.5 / 12.2).
 bool few_by_cta(const Shape& sh, int n_vec, int64_t ctas)
@@ -664,10 +665,15 @@ cudaError_t launch_few(const __half* x, const float* cb, const int32_t* seq_offs
         return cudaLaunchKernelEx(&cfg, kernel, x, cb, seq_offsets, sh, n_vec, (int)n_tokens, token_offset, codes, x2, cb2, codes2, share...);
     };
     if (!by_cta) return go(encode_few_kernel<kC>, few_share(sh, n_vec));
-    if (sh.b == 8) return go(encode_few_wide_kernel<kC, 1, false>);
-    const bool packed = wide_packed_pays(n_vec, (int64_t)cfg.gridDim.x * cfg.gridDim.y);
-    if (sh.b == 9) return packed ? go(encode_few_wide_kernel<kC, 2, true>) : go(encode_few_wide_kernel<kC, 2, false>);
-    return packed ? go(encode_few_wide_kernel<kC, 4, true>) : go(encode_few_wide_kernel<kC, 4, false>);
+    const int64_t ctas = (int64_t)cfg.gridDim.x * cfg.gridDim.y;
+    // What follows may go ahead where the CTAs do not all run at once: beside CTAs that do, its own are placed unevenly.  Back to back, us,
+    // ahead / not: 16 x 12 heads of CQ-8c10b (384 CTAs) 9.2 / 7.7, of CQ-8c9b 6.9 / 5.4, 6 x 24 of CQ-8c8b (768, eight to an SM) 4.1 / 3.4; step of
+    // 16 x 8192 tokens, 32 heads of CQ-8c10b (1024) 138.4 / 139.0.
+    const int next_ahead = ctas > (sh.b == 8 ? 8 : 4) * (int64_t)device_sm_count() ? 1 : 0;
+    if (sh.b == 8) return go(encode_few_wide_kernel<kC, 1, false>, next_ahead);
+    const bool packed = wide_packed_pays(n_vec, kC << (sh.b - 8), ctas);
+    if (sh.b == 9) return packed ? go(encode_few_wide_kernel<kC, 2, true>, next_ahead) : go(encode_few_wide_kernel<kC, 2, false>, next_ahead);
+    return packed ? go(encode_few_wide_kernel<kC, 4, true>, next_ahead) : go(encode_few_wide_kernel<kC, 4, false>, next_ahead);
 }
 
 template <int kC, int kMT>

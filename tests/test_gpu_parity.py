@@ -565,17 +565,25 @@ def test_attention_head_dim_64_tuned(c, n_q, n_kv, lens):
 # (head, group) and SM (18 heads at c = 8, 9 at c = 4, key and value), a warp with all vectors (40 heads)
 @pytest.mark.parametrize("n_vec", [1, 8, 9, 16, 17, 32])
 @pytest.mark.parametrize("c,n_heads", [(8, 1), (8, 18), (8, 19), (8, 40), (4, 9), (4, 10), (2, 4), (2, 5)])
-def test_encode_of_few_vectors_equals_the_generic_kernel(c, n_heads, n_vec):
+def test_encode_of_few_vectors_equals_the_generic_kernel(c, n_heads, n_vec, b=8):
     g = torch.Generator().manual_seed(c * n_heads + n_vec)
     x = torch.randn(2, n_vec, 1, n_heads, 128, generator=g).half()
-    cb = torch.randn(2, n_heads, 128 // c, 256, c, generator=g)
+    cb = torch.randn(2, n_heads, 128 // c, 1 << b, c, generator=g)
     cb[:, :, :, 200] = cb[:, :, :, 7]                                # equal centroids: the lower index
     x[0, 0, 0, 0, :c], x[1, n_vec // 2, 0, n_heads - 1, -1] = cb[0, 0, 0, 200].half(), float("nan")
     x, cb = x.to(DEV), cb.to(DEV)
-    size = cq.cq_codes_bytes(n_vec, 20, n_heads, 128, c, 8)
+    size = cq.cq_codes_bytes(n_vec, 20, n_heads, 128, c, b)
     got, want = (torch.zeros(2, size, dtype=torch.uint8, device=DEV) for _ in range(2))
     off = torch.arange(n_vec, dtype=torch.int32, device=DEV) % 21    # 20: no room, the vector is dropped
-    cq.cq_encode_kv(x[0], x[1], cb[0], cb[1], c, 8, got[0], got[1], 20, seq_offsets=off)
+    cq.cq_encode_kv(x[0], x[1], cb[0], cb[1], c, b, got[0], got[1], 20, seq_offsets=off)
     for i in range(2):
-        cq.cq_encode(x[i], cb[i], c, 8, want[i], 20, seq_offsets=off, variant=1)
+        cq.cq_encode(x[i], cb[i], c, b, want[i], 20, seq_offsets=off, variant=1)
     assert torch.equal(got, want)
+
+
+# 512 and 1024 centroids: one centroid per instruction and two, from 128 channels of centroids a thread and vector, with more CTAs than SMs;
+# with and without the next launch ahead (more than four CTAs to an SM)
+@pytest.mark.parametrize("c,b,n_heads,n_vec", [(8, 10, 4, 4), (8, 10, 5, 3), (8, 10, 5, 4), (8, 10, 19, 17), (8, 9, 5, 7), (8, 9, 5, 8), (8, 9, 19, 32),
+                                               (4, 10, 3, 7), (4, 10, 3, 8), (4, 10, 10, 16), (2, 9, 2, 31), (2, 9, 2, 32), (2, 10, 5, 16)])
+def test_encode_of_few_vectors_with_wide_codes_equals_the_generic_kernel(c, b, n_heads, n_vec):
+    test_encode_of_few_vectors_equals_the_generic_kernel(c, n_heads, n_vec, b)
