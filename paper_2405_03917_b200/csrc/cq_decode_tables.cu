@@ -24,9 +24,6 @@ constexpr int kTabRows = 32;              // queries of a KV head that a CTA tak
 // sequences (2^20) 18.6 > 19.8.
 // With many queries the attention's CTAs overlap their builds with each other's loops, and the tables only cost a
 // trip through L2: 64 sequences of 1024 tokens, 32 heads on 8, CQ-2c8b: attention 180 > 216.
-// CQ-8c8b with three or more queries to a codebook up to twice as many (append alone / tables ahead, calls back to back): 8 x 500 tokens,
-// 8 heads 14.7 / 12.5, 2000 17.7 / 14.2; 64 x 2000, one head 17.5 / 14.0; 3 x 500, 20 heads 14.5 / 12.4; two queries, 2 x 500, 32 heads
-// 14.6 / 15.2.  At 2^19: 12 x 500, 8 heads 15.0 / 15.8; CQ-4c8b at 2^18: 32 x 200, one head 11.6 / 12.5.
 constexpr int64_t kMostEntries = 1 << 17;
 
 // A warp: eight neighbouring groups x four neighbouring code values at a time (whole sectors of the codebook and of the
@@ -153,9 +150,8 @@ cudaError_t launch_fetch_host(const HostPieces& pieces, cudaStream_t st)
 
 bool decode_tables_pay(const Shape& sh)
 {
-    const bool twice = sh.c == 8 && sh.K == 256 && sh.n_seq * sh.R >= 3;
     return decode_tuned_supported(sh) && sh.head_dim == 128 && !decode_pair_supported(sh) &&
-           sh.n_seq * sh.n_q_heads * sh.G * sh.K <= (twice ? 2 * kMostEntries : kMostEntries);
+           sh.n_seq * sh.n_q_heads * sh.G * sh.K <= kMostEntries;
 }
 
 size_t decode_tables_bytes(const Shape& sh) { return (size_t)sh.n_seq * sh.n_q_heads * sh.G * sh.K * sizeof(float); }

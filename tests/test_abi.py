@@ -180,15 +180,11 @@ def test_new_entry_points_validate_on_the_host(L):
     assert encv(variant=5) == -2
 
 
-@pytest.mark.parametrize("c,n_seq,n_q,n_kv,tables", [
+@pytest.mark.parametrize("n_q,n_kv,tables", [(1, 1, True), (2, 1, True), (6, 1, True), (4, 1, False), (8, 2, False), (12, 1, False)])
+def test_which_steps_have_tables_ahead(L, n_q, n_kv, tables):
     # four query heads per CTA of CQ-8c8b append inside the attention and build their own tables: decode_tuned_kernel has no
     # instance for them with tables from the kernel ahead
-    (8, 1, 1, 1, True), (8, 1, 2, 1, True), (8, 1, 6, 1, True), (8, 1, 4, 1, False), (8, 1, 8, 2, False), (8, 1, 12, 1, False),
-    # 2^17 entries; twice as many for CQ-8c8b with three queries to a codebook
-    (8, 1, 32, 32, True), (8, 2, 17, 17, False), (8, 3, 21, 21, True), (8, 3, 22, 22, False), (8, 64, 1, 1, True), (8, 65, 1, 1, False),
-    (8, 10, 6, 1, True), (8, 11, 6, 1, False), (4, 16, 1, 1, True), (4, 17, 1, 1, False), (2, 8, 1, 1, True), (2, 9, 1, 1, False)])
-def test_which_steps_have_tables_ahead(L, c, n_seq, n_q, n_kv, tables):
-    size = n_seq * n_q * (128 // c) * 256 * 4
-    attn = cq.cq_decode_attn_workspace_bytes(n_seq, n_q, n_kv, 128, c, 8, 1000)
-    step = cq.cq_decode_step_workspace_bytes(n_seq, n_q, n_kv, 128, c, 8, 1000)
-    assert (step - attn >= size) == tables
+    entries = n_q * 16 * 256 * 4
+    attn = cq.cq_decode_attn_workspace_bytes(1, n_q, n_kv, 128, 8, 8, 1000)
+    step = cq.cq_decode_step_workspace_bytes(1, n_q, n_kv, 128, 8, 8, 1000)
+    assert (step - attn >= entries) == tables

@@ -60,12 +60,6 @@ def test_step(c, b, n_seq, n_q, n_kv, scale):
     close(got, want)
 
 
-# at and past 2^18 table entries, and with two queries to a codebook, where 2^17 is the most
-@pytest.mark.parametrize("n_seq,n_q,n_kv", [(8, 8, 8), (9, 8, 8), (64, 1, 1), (65, 1, 1), (2, 17, 17), (10, 6, 1)])
-def test_step_at_the_most_entries(n_seq, n_q, n_kv):
-    test_step(8, 8, n_seq, n_q, n_kv, None)
-
-
 @pytest.mark.parametrize("n_q", [1, 4])
 def test_contexts_split_over_ctas(n_q):
     c, b, n_seq, D, cap = 8, 8, 4, 128, 9000
