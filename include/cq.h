@@ -407,8 +407,9 @@ int cq_decode_step(const void *q_fp16, const void *k_new_fp16, const void *v_new
  *   k_new_host, v_new_host   [n_seq][n_kv_heads][head_dim] fp16
  *                (when q_host, k_new_host and v_new_host lie back to back in host memory, in
  *                this order, the three travel in one copy instead of three.  Where all five host
- *                buffers are pinned and hold 4 MiB at most, kernels write the result in place and
- *                read the inputs in place where these hold 40 KiB or are not back to back)
+ *                buffers are pinned, each by one allocation or registration from its first byte to its
+ *                last, and hold 4 MiB at most, kernels write the result in place and read the inputs
+ *                in place where these hold 40 KiB or are not back to back)
  *   seq_lens_host [n_seq] int32: tokens already cached, each < max_tokens
  *   k_codes, v_codes, k_cb, v_cb   device, as in cq_decode_attn (codes are updated)
  *   out_host     [n_seq][n_q_heads][head_dim] fp32

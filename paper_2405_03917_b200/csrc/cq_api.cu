@@ -1,4 +1,6 @@
 // extern "C" entry points of the CQ library: host-side validation and dispatch only.
+#include <cuda.h>
+
 #include <mutex>
 
 #include "cq_common.cuh"
@@ -489,16 +491,34 @@ constexpr size_t kDirectHostBytes = (size_t)4 << 20;
 // place: one sequence of 20000 tokens, 32 heads on 8 (12 KB) 51.5 against 48.2 us, 32 heads of CQ-4c8b, 2000 tokens (25 KB) 38.9 against
 // 34.5; four sequences of 500 (49 KB) 37.6 against 39.8, 16 of 500 (197 KB) 44 against 52.
 constexpr size_t kFetchHostBytes = (size_t)40 << 10;
-// The address under which kernels of the current device reach pinned host memory; false for any other memory.
-bool pinned_on_device(const void* host, const void** dev)
+// cuPointerGetAttributes of the driver; null where it cannot be had.
+using PointerGetAttributes = CUresult (*)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+PointerGetAttributes pointer_get_attributes()
 {
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, host) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    *dev = a.devicePointer;
-    return a.type == cudaMemoryTypeHost && a.devicePointer != nullptr;
+    static const PointerGetAttributes get = []() -> PointerGetAttributes {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess) cudaGetLastError();
+        return reinterpret_cast<PointerGetAttributes>(fn);
+    }();
+    return get;
+}
+// The address under which kernels of the current device reach `bytes` of pinned host memory; false for any other memory, and
+// where the allocation or registration that holds the first byte ends before the last (the copies leave that to the runtime).
+bool pinned_on_device(const void* host, size_t bytes, const void** dev)
+{
+    const PointerGetAttributes get = pointer_get_attributes();
+    if (!get) return false;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                  CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    unsigned int type = 0, managed = 1;                  // (memory that the driver does not know has type 0)
+    CUdeviceptr first = 0, start = 0;
+    size_t size = 0;
+    void* to[] = {&type, &managed, &first, &start, &size};
+    if (get(5, what, to, reinterpret_cast<CUdeviceptr>(host)) != CUDA_SUCCESS || type != CU_MEMORYTYPE_HOST || managed || !first) return false;
+    if (first < start || first - start > size || size - (first - start) < bytes) return false;
+    *dev = reinterpret_cast<const void*>(first);
+    return true;
 }
 // The device copies of cq_decode_step_host's inputs and output.
 size_t host_staging_bytes(const Shape& sh)
@@ -634,9 +654,9 @@ int cq_decode_step_host(const void* q_host, const void* k_new_host, const void* 
     // Pinned buffers of a small step: a kernel fetches the inputs (where they are more than a copy has done at once), and
     // the attention writes the result to host memory.
     const void *q_dev = nullptr, *k_dev = nullptr, *v_dev = nullptr, *sl_dev = nullptr, *out_dev = nullptr;
-    const bool direct = qb + 2 * kvb + slb + ob <= kDirectHostBytes && pinned_on_device(q_host, &q_dev) && pinned_on_device(k_new_host, &k_dev) &&
-                        pinned_on_device(v_new_host, &v_dev) && pinned_on_device(seq_lens_host, &sl_dev) &&
-                        pinned_on_device(out_host, &out_dev) && (reinterpret_cast<uintptr_t>(out_dev) & 3u) == 0;
+    const bool direct = qb + 2 * kvb + slb + ob <= kDirectHostBytes && pinned_on_device(q_host, qb, &q_dev) && pinned_on_device(k_new_host, kvb, &k_dev) &&
+                        pinned_on_device(v_new_host, kvb, &v_dev) && pinned_on_device(seq_lens_host, slb, &sl_dev) &&
+                        pinned_on_device(out_host, ob, &out_dev) && (reinterpret_cast<uintptr_t>(out_dev) & 3u) == 0;
     const bool fetch = direct && (!packed || qb + 2 * kvb + slb >= kFetchHostBytes);
     if (fetch) {
         const HostPieces pieces = {{q_dev, k_dev, v_dev, sl_dev}, {d_q, d_k, d_v, d_sl}, {qb, kvb, kvb, slb}};

@@ -166,6 +166,34 @@ def test_host_buffers_side_by_side(c, b, n_seq, n_q, n_kv):
     close(got, want)
 
 
+@pytest.mark.parametrize("part", ["q", "k_new", "v_new", "out"])
+def test_host_buffers_of_which_only_the_beginning_is_pinned(part):
+    # one page of two or more is registered: no kernel reaches the rest, the buffers are copied (or the copy is refused)
+    c, b, n_seq, n_q, n_kv, D, cap = 8, 8, 4, 8, 8, 128, 200
+    q, codes, books, new = make(c, b, n_seq, n_q, n_kv, D, cap, 31)
+    lens = torch.arange(5, 5 + 10 * n_seq, 10, dtype=torch.int32)
+    other = [x.clone() for x in codes]
+    want = cq.cq_decode_step(q, *new, lens.to(DEV), *other, *books, D ** -0.5, c, b, cap)
+    host = {"q": q.cpu(), "k_new": new[0].cpu(), "v_new": new[1].cpu(), "out": torch.empty(n_seq, n_q, D)}
+    size = host[part].numel() * host[part].element_size()
+    assert size >= 2 * mmap.PAGESIZE
+    block = torch.frombuffer(mmap.mmap(-1, size), dtype=host[part].dtype).view(host[part].shape)
+    block.copy_(host[part])
+    host = {name: block if name == part else x.pin_memory() for name, x in host.items()}
+    ws = torch.empty(cq.cq_decode_step_host_workspace_bytes(n_seq, n_q, n_kv, D, c, b, cap), dtype=torch.uint8, device=DEV)
+    rt = torch.cuda.cudart()
+    assert int(rt.cudaHostRegister(block.data_ptr(), mmap.PAGESIZE, 0)) == 0
+    try:
+        got = cq.cq_decode_step_host(host["q"], host["k_new"], host["v_new"], lens.pin_memory(), *codes, *books, D ** -0.5, c, b, cap,
+                                     host["out"], ws)
+        close(got, want)
+    except cq.CQError:
+        cq.lib().cudaGetLastError()              # (the refused copy's: torch would report it at its next launch)
+    finally:
+        torch.cuda.synchronize()
+        assert int(rt.cudaHostUnregister(block.data_ptr())) == 0
+
+
 @pytest.mark.parametrize("n_seq,cap", [(2, 64), (20, 64), (3, 9000), (14, 9000)])
 def test_steps_with_the_append_inside_right_behind_one_another(n_seq, cap):
     # decode_pair_kernel lets the next kernel go ahead at its start or at its epilogue, by its CTAs (16, 160; 96 and 448 of split
