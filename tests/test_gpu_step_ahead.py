@@ -88,27 +88,38 @@ def test_a_workspace_without_room_for_tables(c, b):
     close(got, want)
 
 
-def test_steps_right_behind_one_another():
-    # every kernel is launched ahead of the end of the one before: 12 steps without a wait between them against the same steps
-    # with one, the lengths and the caches carried on
-    c, b, n_seq, D, cap = 4, 8, 3, 128, 64
-    q, codes, books, new = make(c, b, n_seq, 2, 2, D, cap, 4)
-    ws = torch.empty(cq.cq_decode_step_workspace_bytes(n_seq, 2, 2, D, c, b, cap), dtype=torch.uint8, device=DEV)
+def back_to_back(c, b, n_seq, n_q, n_kv, cap, steps):
+    """Steps with no launch of anything else between them, so that each kernel may start before the one ahead has ended, against the
+    same steps with a wait between them.  One workspace, caches that are carried on, another query and other new tokens each time."""
+    D = 128
+    _, codes, books, _ = make(c, b, n_seq, n_q, n_kv, D, cap, c + b + n_seq)
+    g = torch.Generator().manual_seed(n_seq)
+    q = torch.randn(steps, n_seq, n_q, D, generator=g).half().to(DEV)
+    new = torch.randn(2, steps, n_seq, n_kv, D, generator=g).half().to(DEV)
+    lens = torch.clamp(lengths(n_seq, cap), max=cap - steps) + torch.arange(steps, dtype=torch.int32, device=DEV)[:, None]
+    ws = torch.empty(cq.cq_decode_step_workspace_bytes(n_seq, n_q, n_kv, D, c, b, cap), dtype=torch.uint8, device=DEV)
 
     def run(wait):
         kv = [x.clone() for x in codes]
-        lens = torch.tensor([0, 15, 40], dtype=torch.int32, device=DEV)
-        outs = []
-        for _ in range(12):
-            outs.append(cq.cq_decode_step(q, *new, lens, *kv, *books, D ** -0.5, c, b, cap, workspace=ws).clone())
-            lens.add_(1)
+        out = torch.zeros(steps, n_seq, n_q, D, device=DEV)
+        args = [(q[i], new[0, i], new[1, i], lens[i], *kv, *books, D ** -0.5, c, b, cap, out[i], ws) for i in range(steps)]
+        torch.cuda.synchronize()
+        for a in args:
+            cq.cq_decode_step(*a)
             if wait:
                 torch.cuda.synchronize()
-        return outs, kv
-    (a, ka), (w, kw) = run(False), run(True)
+        return out, kv
+    (w, kw), (a, ka) = run(True), run(False)
     assert torch.equal(ka[0], kw[0]) and torch.equal(ka[1], kw[1])
-    for x, y in zip(a, w):
-        close(x, y)
+    close(a, w)
+
+
+# tables ahead; the append ahead alone, all CTAs at once and in several waves; split contexts with a merge, with tables and without;
+# CQ-8c10b with tables and with an append of its own
+@pytest.mark.parametrize("c,b,n_seq,n_q,n_kv,cap", [(4, 8, 3, 2, 2, 64), (8, 8, 1, 1, 1, 1024), (8, 8, 8, 8, 8, 300), (4, 8, 12, 32, 32, 200), (2, 8, 9, 8, 8, 120),
+                                                    (8, 8, 4, 1, 1, 9000), (8, 8, 3, 16, 16, 9000), (8, 10, 4, 2, 2, 200), (8, 10, 8, 16, 16, 200)])
+def test_steps_right_behind_one_another(c, b, n_seq, n_q, n_kv, cap):
+    back_to_back(c, b, n_seq, n_q, n_kv, cap, 12)
 
 
 @pytest.mark.parametrize("c,b,n_seq,n_q,n_kv", [(8, 8, 3, 8, 2), (4, 8, 2, 3, 3), (4, 8, 3, 24, 24), (8, 10, 2, 2, 1), (4, 4, 2, 2, 2)])
@@ -197,22 +208,5 @@ def test_host_buffers_of_which_only_the_beginning_is_pinned(part):
 @pytest.mark.parametrize("n_seq,cap", [(2, 64), (20, 64), (3, 9000), (14, 9000)])
 def test_steps_with_the_append_inside_right_behind_one_another(n_seq, cap):
     # decode_pair_kernel lets the next kernel go ahead at its start or at its epilogue, by its CTAs (16, 160; 96 and 448 of split
-    # contexts): 8 steps without a wait between them against the same steps with one
-    c, b, D = 8, 8, 128
-    q, codes, books, new = make(c, b, n_seq, 32, 8, D, cap, n_seq)
-    ws = torch.empty(cq.cq_decode_step_workspace_bytes(n_seq, 32, 8, D, c, b, cap), dtype=torch.uint8, device=DEV)
-
-    def run(wait):
-        kv = [x.clone() for x in codes]
-        lens = torch.clamp(lengths(n_seq, cap), max=cap - 8)
-        outs = []
-        for _ in range(8):
-            outs.append(cq.cq_decode_step(q, *new, lens, *kv, *books, D ** -0.5, c, b, cap, workspace=ws).clone())
-            lens.add_(1)
-            if wait:
-                torch.cuda.synchronize()
-        return outs, kv
-    (a, ka), (w, kw) = run(False), run(True)
-    assert torch.equal(ka[0], kw[0]) and torch.equal(ka[1], kw[1])
-    for x, y in zip(a, w):
-        close(x, y)
+    # contexts)
+    back_to_back(8, 8, n_seq, 32, 8, cap, 8)
