@@ -152,6 +152,11 @@ cudaError_t launch_decode_tuned(const __half* q, const uint8_t* kc, const uint8_
                                 const AppendArgs& app = AppendArgs(), const AheadArgs& ahead = AheadArgs());
 // (app: only where decode_appends_inside; the launch then encodes the token as well and covers seq_lens[s] + 1 tokens)
 bool decode_appends_inside(const Shape& sh);
+struct DecodeCtas {
+    int64_t grid = 0;                                 // CTAs of decode_tuned_kernel (0: another kernel's shape)
+    int parts = 0, per_sm = 0;                        // CTAs to a context; CTAs that fit an SM
+};
+DecodeCtas decode_tuned_ctas(const Shape& sh);
 int decode_tuned_launches(const Shape& sh);           // 1: the attention kernel also writes the output; 2: plus the merge
 
 // The kernel ahead of the attention of a decode step (cq_decode_tables.cu; b = 8, and for the tables CQ-8c10b): encodes and

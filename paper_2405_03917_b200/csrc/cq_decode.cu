@@ -1386,6 +1386,17 @@ int decode_tuned_parts(const Shape& sh)
 // to 32 k tokens, 40 heads of CQ-8c8b: 279 -> 265): inside, every CTA took the value centroids once more for it.
 bool decode_appends_inside(const Shape& sh) { return decode_pair_supported(sh); }
 
+DecodeCtas decode_tuned_ctas(const Shape& sh)
+{
+    DecodeCtas r;
+    if (!decode_tuned_supported(sh) || wide_shape(sh)) return r;
+    const Plan pl = plan_dispatch(sh);
+    r.grid = pl.grid;
+    r.parts = pl.n_parts;
+    r.per_sm = with_instance(sh, [](auto i) { return Cfg<i.D, i.groups, i.heads>::kMinBlocks; });
+    return r;
+}
+
 int decode_tuned_launches(const Shape& sh)
 {
     const bool one = (decode_pair_supported(sh) ? decode_pair_plan(sh).n_parts : plan_dispatch(sh).n_parts) == 1;

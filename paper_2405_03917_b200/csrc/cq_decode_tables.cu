@@ -31,12 +31,13 @@ constexpr int64_t kMostEntries = 1 << 17;
 template <int kC, int kPer>
 __global__ void __launch_bounds__(kTabThreads)
 decode_ahead_kernel(const __half* __restrict__ q, const float* __restrict__ kcb, const float* __restrict__ vcb,
-                     const int32_t* __restrict__ seq_lens, float scale_log2e, Shape sh, int rows_per_cta, int n_append_ctas, int append_share,
+                     const int32_t* __restrict__ seq_lens, float scale_log2e, Shape sh, int rows_per_cta, int n_append_ctas, int append_share, int next_at_start,
                      float* __restrict__ tables, AppendArgs app)
 {
-    // launched ahead of the end of whatever lies before it; the attention behind it may be launched from here on, and waits
+    // launched ahead of the end of whatever lies before it; next_at_start: the attention behind it may be launched from here on, and
+    // waits (see the launch)
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (next_at_start) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     constexpr int kRows = 256 * kPer, kU = kC == 8 ? 4 : 8;
     constexpr int kPerCta = kTabThreads / 32 * 4 * kU;             // code values of a CTA
     static_assert(kRows % kPerCta == 0, "whole CTAs");
@@ -105,12 +106,21 @@ cudaError_t launch_ahead(const __half* q, const float* kcb, const float* vcb, co
     int64_t per = (rows * base + 2 * (int64_t)device_sm_count() - 1) / (2 * (int64_t)device_sm_count());
     per = per < 4 ? 4 : (per > kTabRows ? kTabRows : per);
     const int64_t table_ctas = tables ? base * ((rows + per - 1) / per) : 0;
-    const int64_t append_ctas = app.k_new ? 2 * few_ctas(sh, (int)sh.n_seq) : 0, grid = table_ctas + append_ctas;
+    const int share = few_share(sh, (int)sh.n_seq);
+    const int64_t append_ctas = app.k_new ? 2 * few_ctas(sh, (int)sh.n_seq, share) : 0, grid = table_ctas + append_ctas;
     if (grid > 0x7fffffff) return cudaErrorInvalidConfiguration;
+    // An attention with an SM to each CTA, of which two would fit, is launched when this kernel ends, unless both together have an SM
+    // for each of their CTAs: launched beside an append, its CTAs go where that has left most room, two to an SM, and stay there.  Steps
+    // back to back, us, launched at the start / at the end: 12 x 1000 tokens, 12 heads of CQ-8c8b 15.4 / 12.6, of CQ-4c8b 16.9 / 13.4, 1 x 4500, 36
+    // heads of CQ-4c8b 21.1 / 16.1, 64 x 1900, 2 heads on one of CQ-8c8b 26.3 / 20.3; 8 x 1900, 6 heads on 2 (64 + 48 CTAs) 12.0 / 12.2.  With more
+    // CTAs than SMs (4 x 1000, 40 heads of CQ-8c8b 15.8 / 16.1, 8 x 5000, 8 heads of CQ-4c8b 22.0 / 22.8) or one that fills an SM (8 x 1000, 8 heads
+    // of CQ-2c8b 16.3 / 16.7) the launch had better pass behind the append.
+    const DecodeCtas next = decode_tuned_ctas(sh);
+    const int next_at_start = tables || next.per_sm != 2 || next.grid > device_sm_count() || next.grid + append_ctas <= device_sm_count() ? 1 : 0;
     cudaLaunchAttribute attr;
     const cudaLaunchConfig_t cfg = overlapped_config((unsigned)grid, kTabThreads, 0, st, &attr);
     auto go = [&](auto kernel) {
-        return cudaLaunchKernelEx(&cfg, kernel, q, kcb, vcb, seq_lens, scale * kLog2e, sh, (int)per, (int)append_ctas, app.k_new ? few_share(sh, (int)sh.n_seq) : 0, tables, app);
+        return cudaLaunchKernelEx(&cfg, kernel, q, kcb, vcb, seq_lens, scale * kLog2e, sh, (int)per, (int)append_ctas, share, next_at_start, tables, app);
     };
     return go(decode_ahead_kernel<kC, kPer>);
 }

@@ -659,7 +659,7 @@ cudaError_t launch_few(const __half* x, const float* cb, const int32_t* seq_offs
     cudaLaunchAttribute attr;
     const int tensors = x2 ? 2 : 1;
     const bool by_cta = sh.b != 8 || few_by_cta(sh, n_vec, (int64_t)tensors * sh.n_kv_heads * EncCfg<kC>::G);
-    cudaLaunchConfig_t cfg = overlapped_config((unsigned)(by_cta ? sh.n_kv_heads * EncCfg<kC>::G : few_ctas(sh, n_vec)), kFewThreads, 0, st, &attr);
+    cudaLaunchConfig_t cfg = overlapped_config((unsigned)(by_cta ? sh.n_kv_heads * EncCfg<kC>::G : few_ctas(sh, n_vec, few_share(sh, n_vec))), kFewThreads, 0, st, &attr);
     cfg.gridDim.y = (unsigned)tensors;
     auto go = [&](auto kernel, auto... share) {
         return cudaLaunchKernelEx(&cfg, kernel, x, cb, seq_offsets, sh, n_vec, (int)n_tokens, token_offset, codes, x2, cb2, codes2, share...);

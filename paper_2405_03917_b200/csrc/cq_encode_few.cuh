@@ -23,9 +23,8 @@ inline int few_share(const Shape& sh, int n_vec)
     while (share < kFewVecs && 2 * (int64_t)sh.n_kv_heads * sh.G * ((n_vec + share - 1) / share) > 16 * (int64_t)device_sm_count()) ++share;
     return share;
 }
-inline int64_t few_ctas(const Shape& sh, int n_vec)
+inline int64_t few_ctas(const Shape& sh, int n_vec, int share)
 {
-    const int share = few_share(sh, n_vec);
     return ((int64_t)sh.n_kv_heads * sh.G * ((n_vec + share - 1) / share) + kFewThreads / 32 - 1) / (kFewThreads / 32);
 }
 

@@ -114,9 +114,10 @@ def back_to_back(c, b, n_seq, n_q, n_kv, cap, steps):
     close(a, w)
 
 
-# tables ahead; the append ahead alone, all CTAs at once and in several waves; split contexts with a merge, with tables and without;
+# tables ahead; the append ahead alone, with the attention launched at its end (an SM to each CTA) and at its start (an SM to each CTA of
+# both; several waves; one CTA fills an SM); split contexts with a merge, with tables and without;
 # CQ-8c10b with tables and with an append of its own
-@pytest.mark.parametrize("c,b,n_seq,n_q,n_kv,cap", [(4, 8, 3, 2, 2, 64), (8, 8, 1, 1, 1, 1024), (8, 8, 8, 8, 8, 300), (4, 8, 12, 32, 32, 200), (2, 8, 9, 8, 8, 120),
+@pytest.mark.parametrize("c,b,n_seq,n_q,n_kv,cap", [(4, 8, 3, 2, 2, 64), (8, 8, 1, 1, 1, 1024), (8, 8, 8, 8, 8, 300), (8, 8, 8, 6, 2, 300), (4, 8, 12, 32, 32, 200), (2, 8, 9, 8, 8, 120),
                                                     (8, 8, 4, 1, 1, 9000), (8, 8, 3, 16, 16, 9000), (8, 10, 4, 2, 2, 200), (8, 10, 8, 16, 16, 200)])
 def test_steps_right_behind_one_another(c, b, n_seq, n_q, n_kv, cap):
     back_to_back(c, b, n_seq, n_q, n_kv, cap, 12)
