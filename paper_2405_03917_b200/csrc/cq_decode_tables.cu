@@ -106,7 +106,14 @@ cudaError_t launch_ahead(const __half* q, const float* kcb, const float* vcb, co
     int64_t per = (rows * base + 2 * (int64_t)device_sm_count() - 1) / (2 * (int64_t)device_sm_count());
     per = per < 4 ? 4 : (per > kTabRows ? kTabRows : per);
     const int64_t table_ctas = tables ? base * ((rows + per - 1) / per) : 0;
-    const int share = few_share(sh, (int)sh.n_seq);
+    const DecodeCtas next = decode_tuned_ctas(sh);
+    // The append of CQ-2c8b takes half as many registers.  Before an attention that has nothing merged behind it, and so little of its own to
+    // do, it spreads its vectors over twice the warps, unless that attention has a last wave that is nearly empty.  12 x 1000 tokens, 12
+    // heads 20.2 -> 16.8 us, 37 x 1000, 8 heads 32.9 -> 30.9; but 8 x 5000, 8 heads, three CTAs to a context, 33.8 -> 34.4, 5 x 500, 32 on 16 (160
+    // CTAs) 25.0 -> 25.5, and 12 x 1000, 12 heads of CQ-8c8b 12.6 -> 14.5.
+    const int64_t sms = device_sm_count(), last = next.grid % sms;
+    const bool wide = kC == 2 && next.parts == 1 && (next.grid <= sms || last == 0 || 2 * last >= sms);
+    const int share = few_share(sh, (int)sh.n_seq, wide ? 2 * kFewWarpsPerSm : kFewWarpsPerSm);
     const int64_t append_ctas = app.k_new ? 2 * few_ctas(sh, (int)sh.n_seq, share) : 0, grid = table_ctas + append_ctas;
     if (grid > 0x7fffffff) return cudaErrorInvalidConfiguration;
     // An attention with an SM to each CTA, of which two would fit, is launched when this kernel ends, unless both together have an SM
@@ -115,8 +122,7 @@ cudaError_t launch_ahead(const __half* q, const float* kcb, const float* vcb, co
     // heads of CQ-4c8b 21.1 / 16.1, 64 x 1900, 2 heads on one of CQ-8c8b 26.3 / 20.3; 8 x 1900, 6 heads on 2 (64 + 48 CTAs) 12.0 / 12.2.  With more
     // CTAs than SMs (4 x 1000, 40 heads of CQ-8c8b 15.8 / 16.1, 8 x 5000, 8 heads of CQ-4c8b 22.0 / 22.8) or one that fills an SM (8 x 1000, 8 heads
     // of CQ-2c8b 16.3 / 16.7) the launch had better pass behind the append.
-    const DecodeCtas next = decode_tuned_ctas(sh);
-    const int next_at_start = tables || next.per_sm != 2 || next.grid > device_sm_count() || next.grid + append_ctas <= device_sm_count() ? 1 : 0;
+    const int next_at_start = tables || next.per_sm != 2 || next.grid > sms || next.grid + append_ctas <= sms ? 1 : 0;
     cudaLaunchAttribute attr;
     const cudaLaunchConfig_t cfg = overlapped_config((unsigned)grid, kTabThreads, 0, st, &attr);
     auto go = [&](auto kernel) {

@@ -17,10 +17,11 @@ constexpr int kFewVecs = 16;              // vectors a warp takes at most
 
 // Vectors a warp takes: as few as one wave of CTAs allows (sixteen warps an SM; key and value counted): 16 vectors of one
 // head, CQ-4c8b: 3.1 us, 4.8 with 16 to a warp.  Units of work: head, group, share of the vectors; one per warp.
-inline int few_share(const Shape& sh, int n_vec)
+constexpr int kFewWarpsPerSm = 16;
+inline int few_share(const Shape& sh, int n_vec, int warps_per_sm = kFewWarpsPerSm)
 {
     int share = 1;
-    while (share < kFewVecs && 2 * (int64_t)sh.n_kv_heads * sh.G * ((n_vec + share - 1) / share) > 16 * (int64_t)device_sm_count()) ++share;
+    while (share < kFewVecs && 2 * (int64_t)sh.n_kv_heads * sh.G * ((n_vec + share - 1) / share) > warps_per_sm * (int64_t)device_sm_count()) ++share;
     return share;
 }
 inline int64_t few_ctas(const Shape& sh, int n_vec, int share)
