@@ -169,16 +169,23 @@ __device__ __forceinline__ void pp_arm(uint64_t* bar, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.relaxed.cta.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
 }
-// Waits for the phase with the given parity; gives up after a bounded number of polls (returns false).
+// Waits for the phase with the given parity; gives up after some seconds (returns false).  The limit is one of time, since a poll may
+// suspend the thread for as long as the hardware likes; the clock is read every 256 polls (every poll: 51.4 -> 52.2 ms of the whole call).
+constexpr long long kPpWaitCycles = 1ll << 33;
 __device__ __forceinline__ bool pp_wait(uint64_t* bar, uint32_t parity)
 {
-    for (int poll = 0; poll < (1 << 22); ++poll) {
-        uint32_t done;
-        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(done) : "r"(smem_addr(bar)), "r"(parity) : "memory");
-        if (done) return true;
+    long long since = 0;
+    for (;;) {
+        for (int poll = 0; poll < 256; ++poll) {
+            uint32_t done;
+            asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                         : "=r"(done) : "r"(smem_addr(bar)), "r"(parity) : "memory");
+            if (done) return true;
+        }
+        const long long now = clock64();
+        if (since == 0) since = now;
+        if (now - since > kPpWaitCycles) return false;
     }
-    return false;
 }
 
 __device__ __forceinline__ uint32_t pp_map_shared(const void* p, int rank)
